@@ -75,8 +75,10 @@ typedef enum {
      * ops = {C, D, E, F}; B CSR; two-level schedule with the row temporary T(l) in the workspace */
     SA_EXPR_SDDMM_SPMM_GEMM = 6,
     /* kernel 3 <SpMMH,GEMM>: A(i,m) = sum_{j,l} B(i,j) C(j,l) D(j,l) E(l,m); ops = {C, D, E}; B CSR;
-     * the Description column of the Table of kernels (SpMM with a Hadamard product, then GEMM),
-     * evaluated per row as T(l) = sum_j B(i,j) C(j,l) D(j,l) followed by T . E                   */
+     * the Description column of the Table of kernels (SpMM with a Hadamard product, then GEMM).
+     * SA_SCHED_FUSED: per row T(l) = sum_j B(i,j) C(j,l) D(j,l) followed by T . E; SA_SCHED_ASSOC_RIGHT:
+     * G(j,m) = sum_l C(j,l) D(j,l) E(l,m) in the workspace, then B . G; SA_SCHED_DEFAULT: the one that
+     * moves fewer bytes                                                                         */
     SA_EXPR_SPMMH_GEMM = 7,
     /* kernel 8 <MTTKRP,GEMM>: A(i,m) = sum_{j,k,r} B(i,j,k) C(j,r) D(k,r) E(r,m); ops = {C, D, E};
      * B order-3 CSF; the MTTKRP rows T(i,:) (R floats per slice) live in the workspace              */
@@ -94,11 +96,12 @@ typedef enum {
 
 typedef enum {
     SA_SCHED_DEFAULT = 0,      /* the host table's choice for the expression; where two schedules exist
-                                  (SPMM_GEMM, SPTTM_SPTTM) the one that moves fewer bytes for this
+                                  (SPMM_GEMM, SPMMH_GEMM, SPTTM_SPTTM) the one that moves fewer bytes for this
                                   tensor among those within the auxiliary-memory cap, see sa_schedule_cost */
     SA_SCHED_FUSED = 1,        /* the fissioned / fused branched nest of the Table of kernels   */
     SA_SCHED_ASSOC_LEFT = 2,   /* SA_EXPR_SPMM_GEMM (and SPTTM_SPTTM): (B.C).D, row temporary of L floats    */
-    SA_SCHED_ASSOC_RIGHT = 3,  /* SA_EXPR_SPMM_GEMM (and SPTTM_SPTTM): B.(C.D), J x M temporary in workspace */
+    SA_SCHED_ASSOC_RIGHT = 3,  /* SA_EXPR_SPMM_GEMM (and SPTTM_SPTTM): B.(C.D), J x M temporary in workspace;
+                                  SPMMH_GEMM: B.((C o D).E)                                      */
     SA_SCHED_FISSIONED = 4,    /* one more level of kernel fission: the temporaries of the outermost producer /
                                   consumer pair pass through the workspace.  SA_EXPR_TTMC3: T(i,m,n) per slice
                                   (bitwise reproducible, which SA_SCHED_FUSED is not there: its block
@@ -277,8 +280,8 @@ sa_status sa_tensor_set_aux_limit(sa_tensor *t, size_t bytes);
  * SPTTM_SPTTM L, M in {32, 64} (out: level_counts[1] x M, see sa_expr).
  * Arithmetic: fp32 throughout; stages on tensor cores split every fp32 operand into two parts and
  * add three partial products (TF32 parts in the per-slice contractions, BF16 parts in the dense GEMM
- * stage), so every output element stays within 1e-4 of the sum of the absolute values of its terms.
- * The dense GEMM stage (SPMM_GEMM as B.(C.D), SDDMM_SPMM_GEMM) waits on on-chip hand-offs with a
+ * stage; three BF16 parts and six products in the one of SPMMH_GEMM), so every output element stays within 1e-4 of the sum of the absolute values of its terms.
+ * The dense GEMM stage (SPMM_GEMM and SPMMH_GEMM as ASSOC_RIGHT, SDDMM_SPMM_GEMM) waits on on-chip hand-offs with a
  * 2-second limit; if one runs out the kernel returns and sa_last_device_status reports SA_E_TIMEOUT.
  * Returns launch errors only; completion is observed by synchronising the stream.
  * Errors: SA_E_ARG, SA_E_SHAPE, SA_E_UNSUPPORTED, SA_E_WORKSPACE, SA_E_CUDA.

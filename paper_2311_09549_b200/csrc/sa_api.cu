@@ -203,8 +203,15 @@ void schedule_cost(const sa_tensor *t, sa_expr expr, sa_schedule sched, const sa
                  8 * I * L + 4 * L * M + 4 * I * M;
             break;
         }
-        case SA_EXPR_SPMMH_GEMM: {      // i < T(l); j', l: T += B C D , m,l: A += T E >
-            const double L = ops[0].cols, M = ops[2].cols;
+        case SA_EXPR_SPMMH_GEMM: {
+            const double J = double(t->dims[1]), L = ops[0].cols, M = ops[2].cols;
+            if (sched == SA_SCHED_ASSOC_RIGHT) {   // < G(j,m); j,l,m: G += C D E , i,j',m: A += B G >
+                it = J * L * M + nnz * M;
+                tmp = J * M;
+                by = 4 * J * (2 * L + M) + 4 * L * M + 8 * nnz + 4 * (I + 1) + table_bytes(t, J, M, nnz) + 4 * I * M;
+                break;
+            }
+            // i < T(l); j', l: T += B C D , m,l: A += T E >
             it = nnz * L + I * L * M;
             tmp = L;
             by = 8 * nnz + 4 * (I + 1) + table_bytes(t, ops[0].rows, L, nnz) + table_bytes(t, ops[1].rows, L, nnz) + 4 * L * M + 4 * I * M;
@@ -301,7 +308,6 @@ bool resolve_schedule(const sa_tensor *t, sa_expr expr, sa_schedule sched, const
         }
         case SA_EXPR_SPTTM_TTM3:
         case SA_EXPR_SDDMM_SPMM_GEMM:
-        case SA_EXPR_SPMMH_GEMM:
         case SA_EXPR_MTTKRP_GEMM:
             if (sched == SA_SCHED_DEFAULT || sched == SA_SCHED_FUSED) { *resolved = SA_SCHED_FUSED; return true; }
             return false;
@@ -310,10 +316,13 @@ bool resolve_schedule(const sa_tensor *t, sa_expr expr, sa_schedule sched, const
             if (sched == SA_SCHED_DEBUG_MATERIALIZE) { *resolved = sched; return true; }
             return false;
         case SA_EXPR_SPMM_GEMM:
-        case SA_EXPR_SPTTM_SPTTM:
+        case SA_EXPR_SPMMH_GEMM:
+        case SA_EXPR_SPTTM_SPTTM: {
+            // the row nest goes by the name ASSOC_LEFT where the expression is a plain matrix product
+            const sa_schedule nest = expr == SA_EXPR_SPMMH_GEMM ? SA_SCHED_FUSED : SA_SCHED_ASSOC_LEFT;
             if (sched == SA_SCHED_DEFAULT) {
                 sa_cost left, right;
-                schedule_cost(t, expr, SA_SCHED_ASSOC_LEFT, ops, &left);
+                schedule_cost(t, expr, nest, ops, &left);
                 schedule_cost(t, expr, SA_SCHED_ASSOC_RIGHT, ops, &right);
                 const uint64_t cap = t->aux_limit.load();
                 const bool lf = left.workspace_bytes <= cap, rf = right.workspace_bytes <= cap;
@@ -321,12 +330,13 @@ bool resolve_schedule(const sa_tensor *t, sa_expr expr, sa_schedule sched, const
                 if (lf != rf) take_left = lf;
                 else if (!lf) take_left = left.workspace_bytes <= right.workspace_bytes;
                 else take_left = left.moved_bytes <= right.moved_bytes;
-                *resolved = take_left ? SA_SCHED_ASSOC_LEFT : SA_SCHED_ASSOC_RIGHT;
+                *resolved = take_left ? nest : SA_SCHED_ASSOC_RIGHT;
                 return true;
             }
-            if (sched == SA_SCHED_FUSED || sched == SA_SCHED_ASSOC_LEFT) { *resolved = SA_SCHED_ASSOC_LEFT; return true; }
+            if (sched == SA_SCHED_FUSED || sched == nest) { *resolved = nest; return true; }
             if (sched == SA_SCHED_ASSOC_RIGHT) { *resolved = sched; return true; }
             return false;
+        }
     }
     return false;
 }
@@ -340,7 +350,7 @@ size_t workspace_bytes(const sa_tensor *t, sa_expr expr, sa_schedule sched, cons
         case SA_EXPR_SPMM_GEMM: return sa_ws_spmm_gemm(t, ops, sched == SA_SCHED_ASSOC_RIGHT);
         case SA_EXPR_TTMC3: return sa_ws_ttmc3(t, ops, sched == SA_SCHED_FISSIONED);
         case SA_EXPR_SDDMM_SPMM_GEMM: return sa_ws_sddmm_spmm_gemm(t, ops);
-        case SA_EXPR_SPMMH_GEMM: return sa_ws_spmmh_gemm(t, ops);
+        case SA_EXPR_SPMMH_GEMM: return sa_ws_spmmh_gemm(t, ops, sched == SA_SCHED_ASSOC_RIGHT);
         case SA_EXPR_MTTKRP_GEMM: return sa_ws_mttkrp_gemm(t, ops);
         case SA_EXPR_SPTTM_SPTTM: return sa_ws_spttm_spttm(t, ops, sched == SA_SCHED_ASSOC_RIGHT);
     }
@@ -555,7 +565,9 @@ sa_status sa_run(const sa_tensor *t, sa_expr expr, sa_schedule sched, const sa_d
             break;
         case SA_EXPR_TTMC3: s = sa_launch_ttmc3(t, ops, out, workspace, ws_bytes, r == SA_SCHED_FISSIONED, stream, &launches); break;
         case SA_EXPR_SDDMM_SPMM_GEMM: s = sa_launch_sddmm_spmm_gemm(t, ops, out, workspace, ws_bytes, stream, &launches); break;
-        case SA_EXPR_SPMMH_GEMM: s = sa_launch_spmmh_gemm(t, ops, out, workspace, ws_bytes, stream, &launches); break;
+        case SA_EXPR_SPMMH_GEMM: 
+            s = sa_launch_spmmh_gemm(t, ops, out, workspace, ws_bytes, r == SA_SCHED_ASSOC_RIGHT, stream, &launches);
+            break;
         case SA_EXPR_MTTKRP_GEMM: s = sa_launch_mttkrp_gemm(t, ops, out, workspace, ws_bytes, stream, &launches); break;
         case SA_EXPR_SPTTM_SPTTM:
             s = sa_launch_spttm_spttm(t, ops, out, workspace, ws_bytes, r == SA_SCHED_ASSOC_RIGHT, stream, &launches);

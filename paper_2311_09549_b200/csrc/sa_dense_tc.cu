@@ -18,6 +18,13 @@
 //   warps 0..3   read a finished accumulator with tcgen05.ld (warp w owns TMEM lanes 32w..32w+31 = tile rows),
 //                add its two halves, transpose through a swizzled shared-memory tile and store E in
 //                512-byte runs.
+// HAD (kernel 3 <SpMMH,GEMM> in the order B.((C o H).D)): the loads bring a row piece of C and one of H, the product of
+// the two is split.  That chain's row kernel sums in fp32, so here a number is split into three BF16 parts (24 bits) and
+// six products are formed.  The large one, b1.b1, gets accumulator columns of its own (M for the even and M for the odd
+// chunks: eight additions each at L = 256), the others share 2M, so that adding small terms does not round the large
+// one: the whole chain is then off by 1.9e-7 (2-norm, against fp64; with one set of columns for b1.b1 3.1e-7, the row
+// kernel 3.0e-7).  Loads go half a chunk at a time (same registers in flight); operand tiles take half as much again, so
+// two or three stages fit instead of four.  1M x 256 . 256 x 64: 363 us = 6.3 TB/s; without H 204 us = 6.2 TB/s.
 // What limits this kernel next to HBM is the shared-memory data pipe (operand writes, tensor-core operand
 // reads, epilogue), which is why C never passes through a shared-memory fp32 stage and why the two products
 // that share b1(C) are merged.
@@ -25,6 +32,7 @@
 // timer: on expiry the block raises its abort flag, all roles leave their loops, the status word is set to
 // SA_E_TIMEOUT and tensor memory is released as on the normal path.
 #include <algorithm>
+#include <type_traits>
 
 #include "sa_device.cuh"
 
@@ -32,7 +40,7 @@ namespace {
 
 constexpr int TC_BM = 128;                  // rows per tile = MMA M = TMEM lanes
 constexpr int TC_KC = 64;                   // columns of C per chunk: one 128-byte swizzled BF16 row
-constexpr int TC_OPS = 4;                   // operand stages
+constexpr int TC_OPS = 4;                   // operand stages, at most
 constexpr int TC_PF = 4;                    // chunks requested into L2 ahead of the loads into registers
 constexpr int TC_EPI_WARPS = 4;
 constexpr int TC_MMA_WARP = 4;
@@ -49,19 +57,24 @@ constexpr uint64_t TC_WAIT_NS = SA_TC_WAIT_NS;   // longest a hand-off may take 
 // completes and the bounded waits have to run out (tests/test_gpu_bounded_wait.py).
 constexpr int TC_TEST_WITHHOLD = 0x7e57;
 
-template <int L, int M>
+template <int L, int M, bool HAD>
 struct tc_cfg {
     static constexpr int KCH = L / TC_KC;
-    static constexpr uint32_t D_TILE = 2 * M * 128;                    // one chunk of D^T: M rows of b1, then M rows of b2
+    static constexpr int PARTS = HAD ? 3 : 2;                          // BF16 parts per number
+    static constexpr uint32_t OPS = !HAD ? TC_OPS : L == 256 && M == 64 ? 2 : 3;   // what shared memory has room for
+    static constexpr uint32_t D_TILE = PARTS * M * 128;                // one chunk of D^T: M rows of b1, then of b2 (and b3)
     static constexpr uint32_t OP_PART = TC_BM * 128;                   // one BF16 part of a chunk of C
+    static constexpr uint32_t OP_STAGE = PARTS * OP_PART;
     static constexpr uint32_t EPI_WARP = 32 * M * 4;                   // transposition tile of one epilogue warp
     static constexpr uint32_t OFF_D = 0, OFF_OP = uint32_t(KCH) * D_TILE;
-    static constexpr uint32_t OFF_EPI = OFF_OP + TC_OPS * 2 * OP_PART;
+    static constexpr uint32_t OFF_EPI = OFF_OP + OPS * OP_STAGE;
     static constexpr uint32_t OFF_BAR = OFF_EPI + TC_EPI_WARPS * EPI_WARP;
     static constexpr size_t SMEM = size_t(OFF_BAR) + 128 + 1024;       // barriers + slack to align the base to 1 KB
-    static constexpr uint32_t TMEM_COLS = 4 * M;                       // two fp32 accumulators of 2M columns
+    static constexpr uint32_t ACC_COLS = HAD ? 4 * M : 2 * M;          // columns of one fp32 accumulator, of which there are two
+    static constexpr uint32_t TMEM_COLS = 2 * ACC_COLS <= 128 ? 128 : 2 * ACC_COLS <= 256 ? 256 : 512;   // a power of two
     static_assert(L % TC_KC == 0 && (M == 32 || M == 64), "unsupported shape");
     static_assert(D_TILE % 1024 == 0, "swizzle atoms must stay 1 KB aligned");
+    static_assert(SMEM <= 227 * 1024, "shared memory of one block");
 };
 
 // barrier slots (8 bytes each) behind the ring
@@ -178,6 +191,13 @@ __device__ __forceinline__ void tc_split2(float x0, float x1, uint32_t &h, uint3
     l = tc_bf16x2(x0 - __uint_as_float(h << 16), x1 - __uint_as_float(h & 0xffff0000u));
 }
 
+// the same in three parts
+__device__ __forceinline__ void tc_split3(float x0, float x1, uint32_t &h, uint32_t &m, uint32_t &l)
+{
+    h = tc_bf16x2(x0, x1);
+    tc_split2(x0 - __uint_as_float(h << 16), x1 - __uint_as_float(h & 0xffff0000u), m, l);
+}
+
 // Byte offset of element (row, k) inside a K-major tile of 128-byte rows with the 128-byte swizzle: the
 // 16-byte unit index is XORed with the row index modulo 8.
 __device__ __forceinline__ uint32_t tc_sw128(uint32_t row, uint32_t k)
@@ -185,12 +205,12 @@ __device__ __forceinline__ uint32_t tc_sw128(uint32_t row, uint32_t k)
     return row * 128u + ((((k >> 3) ^ row) & 7u) << 4) + ((k & 7u) << 1);
 }
 
-template <int L, int M>
+template <int L, int M, bool HAD>
 __global__ void __launch_bounds__(TC_THREADS, 1)
-gemm_tc_kernel(int64_t J, const float *__restrict__ C, int64_t ldc, const float *__restrict__ D, int64_t ldd,
-               float *__restrict__ Eout, int32_t *__restrict__ status)
+gemm_tc_kernel(int64_t J, const float *__restrict__ C, int64_t ldc, const float *__restrict__ H, int64_t ldh,
+               const float *__restrict__ D, int64_t ldd, float *__restrict__ Eout, int32_t *__restrict__ status)
 {
-    using G = tc_cfg<L, M>;
+    using G = tc_cfg<L, M, HAD>;
     extern __shared__ uint8_t tc_smem_raw[];
     uint8_t *smem = tc_smem_raw + ((1024u - (tc_smem_u32(tc_smem_raw) & 1023u)) & 1023u);
     const uint32_t sbase = tc_smem_u32(smem);
@@ -199,19 +219,31 @@ gemm_tc_kernel(int64_t J, const float *__restrict__ C, int64_t ldc, const float 
     volatile int *abort_flag = reinterpret_cast<volatile int *>(smem + G::OFF_BAR + 8 * B_COUNT + 4);
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
 
-    // D^T as KCH operand tiles of 2M rows x 64 columns (k): rows n < M hold b1(D(k,n)), rows M + n hold b2
-    for (int x = threadIdx.x; x < L * M; x += TC_THREADS) {
-        const int k = x / M, n = x % M;
-        const float v = __ldg(D + int64_t(k) * ldd + n);
-        const uint32_t h = tc_bf16x2(v, 0.f) & 0xffffu;
-        const uint32_t l = tc_bf16x2(v - __uint_as_float(h << 16), 0.f) & 0xffffu;
-        const uint32_t off = G::OFF_D + uint32_t(k / TC_KC) * G::D_TILE + tc_sw128(n, k % TC_KC);
-        *reinterpret_cast<uint16_t *>(smem + off) = uint16_t(h);
-        *reinterpret_cast<uint16_t *>(smem + off + M * 128) = uint16_t(l);     // row n + M: same swizzle phase
+    // D^T as KCH operand tiles of PARTS M rows x 64 columns (k): rows n < M hold b1(D(k,n)), rows M + n hold b2, ...
+    // (eight k of one n per step: coalesced loads, eight in flight, and one conflict-free 16-byte store per part; element by
+    // element this took the block about 25 us)
+#pragma unroll 2
+    for (int x = threadIdx.x; x < M * (L / 8); x += TC_THREADS) {
+        const int k = x / M * 8, n = x % M;
+        float v[8];
+#pragma unroll
+        for (int i = 0; i < 8; ++i) v[i] = __ldg(D + int64_t(k + i) * ldd + n);
+        uint8_t *dst = smem + G::OFF_D + uint32_t(k / TC_KC) * G::D_TILE + tc_sw128(n, k % TC_KC);
+#pragma unroll
+        for (int z = 0; z < G::PARTS; ++z) {                                // row n + z M: same swizzle phase
+            uint32_t h[4];
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+                h[i] = tc_bf16x2(v[2 * i], v[2 * i + 1]);
+                v[2 * i] -= __uint_as_float(h[i] << 16);
+                v[2 * i + 1] -= __uint_as_float(h[i] & 0xffff0000u);
+            }
+            *reinterpret_cast<uint4 *>(dst + z * (M * 128)) = make_uint4(h[0], h[1], h[2], h[3]);
+        }
     }
     fence_async_smem();
     if (threadIdx.x == 0) {
-        for (int x = 0; x < TC_OPS; ++x) {
+        for (uint32_t x = 0; x < G::OPS; ++x) {
             mbar_init(bars + 8 * (B_FULL + x), TC_CONV_T);
             mbar_init(bars + 8 * (B_EMPTY + x), 1);
         }
@@ -240,7 +272,7 @@ gemm_tc_kernel(int64_t J, const float *__restrict__ C, int64_t ldc, const float 
     const int64_t n_chunks = my_tiles * G::KCH;
 
     if (warp < TC_EPI_WARPS) {
-        // ---- epilogue: accumulator halves -> sum -> transposition tile -> rows of E
+        // ---- epilogue: accumulator parts -> sum -> transposition tile -> rows of E
         constexpr int RC = M / 4;                                   // 16-byte units per row of E
         uint8_t *stage = smem + G::OFF_EPI + warp * G::EPI_WARP;
         for (int64_t tl = 0; tl < my_tiles; ++tl) {
@@ -248,12 +280,21 @@ gemm_tc_kernel(int64_t J, const float *__restrict__ C, int64_t ldc, const float 
             const bool ok = mbar_wait(bars + 8 * (B_ACC_FULL + a), v & 1u, abort_flag);
             if (!__all_sync(SA_FULL_MASK, ok)) break;
             tc_fence_after();
-            const uint32_t taddr = tmem_base + (uint32_t(32 * warp) << 16) + a * (2 * M);
+            const uint32_t taddr = tmem_base + (uint32_t(32 * warp) << 16) + a * G::ACC_COLS;
 #pragma unroll
             for (int c = 0; c < M / 16; ++c) {
                 float p[16], r[16];
                 tc_ld16(taddr + 16 * c, p);
                 tc_ld16(taddr + M + 16 * c, r);
+                if (HAD) {
+                    float r2[16];
+                    tc_ld16(taddr + 2 * M + 16 * c, r2);
+#pragma unroll
+                    for (int x = 0; x < 16; ++x) p[x] += r2[x];
+                    tc_ld16(taddr + 3 * M + 16 * c, r2);
+#pragma unroll
+                    for (int x = 0; x < 16; ++x) r[x] += r2[x];
+                }
 #pragma unroll
                 for (int x = 0; x < 4; ++x)                         // unit 4c + x of row `lane`, XOR-swizzled by the row
                     *reinterpret_cast<float4 *>(stage + lane * (M * 4) + (((4 * c + x) ^ (lane & 7)) << 4)) =
@@ -281,21 +322,28 @@ gemm_tc_kernel(int64_t J, const float *__restrict__ C, int64_t ldc, const float 
             const int kc = int(q % G::KCH);
             const int64_t tl = q / G::KCH;
             const uint32_t a = uint32_t(tl) & 1u, v = uint32_t(tl >> 1);
-            const uint32_t s = uint32_t(q) % TC_OPS, u = uint32_t(q / TC_OPS);
+            const uint32_t s = uint32_t(q) % G::OPS, u = uint32_t(q) / G::OPS;
             bool ok = true;
             if (kc == 0) ok = mbar_wait(bars + 8 * (B_ACC_EMPTY + a), (v & 1u) ^ 1u, abort_flag);
             if (ok) ok = mbar_wait(bars + 8 * (B_FULL + s), u & 1u, abort_flag);
             if (!__all_sync(SA_FULL_MASK, ok)) break;
             tc_fence_after();
             if (lane == 0) {
-                const uint32_t d_tmem = tmem_base + a * (2 * M);
-                const uint32_t a_hi = sbase + G::OFF_OP + s * (2 * G::OP_PART), a_lo = a_hi + G::OP_PART;
+                const uint32_t d_tmem = tmem_base + a * G::ACC_COLS;
+                const uint32_t a_hi = sbase + G::OFF_OP + s * G::OP_STAGE, a_lo = a_hi + G::OP_PART, a_3rd = a_lo + G::OP_PART;
                 const uint32_t b = sbase + G::OFF_D + uint32_t(kc) * G::D_TILE;
 #pragma unroll
                 for (int k = 0; k < TC_KC / 16; ++k) {
                     const uint32_t adv = 32u * k;                        // 16 BF16 along K inside the swizzled row
-                    tc_mma(d_tmem, tc_desc(a_hi + adv), tc_desc(b + adv), IDESC_2M, (kc | k) != 0);
-                    tc_mma(d_tmem, tc_desc(a_lo + adv), tc_desc(b + adv), IDESC_M, 1u);
+                    if (HAD) {      // columns [0,M): b1.b2 + b2.b1, [M,2M): b1.b3 + b2.b2 + b3.b1, then b1.b1 of the even and odd chunks
+                        tc_mma(d_tmem, tc_desc(a_hi + adv), tc_desc(b + M * 128 + adv), IDESC_2M, (kc | k) != 0);
+                        tc_mma(d_tmem + (2 + (kc & 1)) * M, tc_desc(a_hi + adv), tc_desc(b + adv), IDESC_M, ((kc >> 1) | k) != 0);
+                        tc_mma(d_tmem, tc_desc(a_lo + adv), tc_desc(b + adv), IDESC_2M, 1u);
+                        tc_mma(d_tmem + M, tc_desc(a_3rd + adv), tc_desc(b + adv), IDESC_M, 1u);
+                    } else {
+                        tc_mma(d_tmem, tc_desc(a_hi + adv), tc_desc(b + adv), IDESC_2M, (kc | k) != 0);
+                        tc_mma(d_tmem, tc_desc(a_lo + adv), tc_desc(b + adv), IDESC_M, 1u);
+                    }
                 }
                 tc_commit(bars + 8 * (B_EMPTY + s));
                 if (kc == G::KCH - 1) tc_commit(bars + 8 * (B_ACC_FULL + a));
@@ -308,53 +356,117 @@ gemm_tc_kernel(int64_t J, const float *__restrict__ C, int64_t ldc, const float 
         const uint32_t qf = uint32_t(t) & 15u, r0 = uint32_t(t) >> 4, sw = r0 & 7u;
         const uint32_t op_off = G::OFF_OP + r0 * 128u + (((qf >> 1) ^ sw) << 4) + ((qf & 1u) << 3);
         constexpr int NR = TC_BM / 16;
-        auto load = [&](float4 (&b)[NR], int64_t q) {
-            if (q + TC_PF < n_chunks) {                            // one 128-byte line per thread: HBM latency is paid by L2
-                const int64_t pq = q + TC_PF;
-                const int64_t row = min((int64_t(blockIdx.x) + (pq / G::KCH) * gridDim.x) * TC_BM + (t >> 1), J - 1);
-                asm volatile("prefetch.global.L2 [%0];" ::"l"(C + row * ldc + int(pq % G::KCH) * TC_KC + 32 * (t & 1)));
-            }
-            if (q < n_chunks) {
-                const int64_t row0 = (int64_t(blockIdx.x) + (q / G::KCH) * gridDim.x) * TC_BM + r0;
-                const float *src = C + int(q % G::KCH) * TC_KC + 4 * qf;
-#pragma unroll
-                for (int i = 0; i < NR; ++i) b[i] = tc_ldg4(src + min(row0 + 16 * i, J - 1) * ldc);   // rows past the end re-read the last row
-            }
-        };
 #ifdef SA_TEST_HOOKS
         const bool withhold = t == 0 && status != nullptr && status[3] == TC_TEST_WITHHOLD;
 #endif
-        auto convert = [&](const float4 (&b)[NR], int64_t q) -> bool {
-            const uint32_t s = uint32_t(q) % TC_OPS, u = uint32_t(q / TC_OPS);
-            if (!mbar_wait(bars + 8 * (B_EMPTY + s), (u & 1u) ^ 1u, abort_flag)) return false;
-            uint8_t *hi = smem + op_off + s * (2 * G::OP_PART), *lo = hi + G::OP_PART;
-#pragma unroll
-            for (int i = 0; i < NR; ++i) {
-                uint2 h, l;
-                tc_split2(b[i].x, b[i].y, h.x, l.x);
-                tc_split2(b[i].z, b[i].w, h.y, l.y);
-                *reinterpret_cast<uint2 *>(hi + i * (16 * 128)) = h;
-                *reinterpret_cast<uint2 *>(lo + i * (16 * 128)) = l;
-            }
-            fence_async_smem();
-#ifdef SA_TEST_HOOKS
-            if (withhold && q == 0) return true;
-#endif
-            mbar_arrive(bars + 8 * (B_FULL + s));
-            return true;
-        };
         float4 b0[NR], b1[NR], b2[NR];
-        load(b0, 0);
-        load(b1, 1);
-        for (int64_t q = 0; q < n_chunks; q += 3) {
-            load(b2, q + 2);
-            if (!convert(b0, q)) break;
-            if (q + 1 >= n_chunks) break;
-            load(b0, q + 3);
-            if (!convert(b1, q + 1)) break;
-            if (q + 2 >= n_chunks) break;
-            load(b1, q + 4);
-            if (!convert(b2, q + 2)) break;
+        if constexpr (!HAD) {
+            auto load = [&](float4 (&b)[NR], int64_t q) {
+                if (q + TC_PF < n_chunks) {                        // one 128-byte line per thread: HBM latency is paid by L2
+                    const int64_t pq = q + TC_PF;
+                    const int64_t row = min((int64_t(blockIdx.x) + (pq / G::KCH) * gridDim.x) * TC_BM + (t >> 1), J - 1);
+                    asm volatile("prefetch.global.L2 [%0];" ::"l"(C + row * ldc + int(pq % G::KCH) * TC_KC + 32 * (t & 1)));
+                }
+                if (q < n_chunks) {
+                    const int64_t row0 = (int64_t(blockIdx.x) + (q / G::KCH) * gridDim.x) * TC_BM + r0;
+                    const float *src = C + int(q % G::KCH) * TC_KC + 4 * qf;
+#pragma unroll
+                    for (int i = 0; i < NR; ++i) b[i] = tc_ldg4(src + min(row0 + 16 * i, J - 1) * ldc);   // rows past the end re-read the last row
+                }
+            };
+            auto convert = [&](const float4 (&b)[NR], int64_t q) -> bool {
+                const uint32_t s = uint32_t(q) % G::OPS, u = uint32_t(q / G::OPS);
+                if (!mbar_wait(bars + 8 * (B_EMPTY + s), (u & 1u) ^ 1u, abort_flag)) return false;
+                uint8_t *hi = smem + op_off + s * G::OP_STAGE, *lo = hi + G::OP_PART;
+#pragma unroll
+                for (int i = 0; i < NR; ++i) {
+                    uint2 h, l;
+                    tc_split2(b[i].x, b[i].y, h.x, l.x);
+                    tc_split2(b[i].z, b[i].w, h.y, l.y);
+                    *reinterpret_cast<uint2 *>(hi + i * (16 * 128)) = h;
+                    *reinterpret_cast<uint2 *>(lo + i * (16 * 128)) = l;
+                }
+                fence_async_smem();
+#ifdef SA_TEST_HOOKS
+                if (withhold && q == 0) return true;
+#endif
+                mbar_arrive(bars + 8 * (B_FULL + s));
+                return true;
+            };
+            load(b0, 0);
+            load(b1, 1);
+            for (int64_t q = 0; q < n_chunks; q += 3) {
+                load(b2, q + 2);
+                if (!convert(b0, q)) break;
+                if (q + 1 >= n_chunks) break;
+                load(b0, q + 3);
+                if (!convert(b1, q + 1)) break;
+                if (q + 2 >= n_chunks) break;
+                load(b1, q + 4);
+                if (!convert(b2, q + 2)) break;
+            }
+        } else {
+            // the same in half chunks of 64 rows: four float4 of C and the four of H beside them.  The half is a compile-time
+            // constant (the loop takes three chunks in six steps); as a run-time value it cost the loop 15 %.
+            constexpr int HR = NR / 2;
+            auto load = [&](float4 (&b)[NR], int64_t q, auto upper) {
+                constexpr int half = decltype(upper)::value ? 1 : 0;
+                if (q + TC_PF < n_chunks) {
+                    const int64_t pq = q + TC_PF;
+                    const int64_t row = min((int64_t(blockIdx.x) + (pq / G::KCH) * gridDim.x) * TC_BM + (t >> 1), J - 1);
+                    asm volatile("prefetch.global.L2 [%0];" ::"l"((half ? H + row * ldh : C + row * ldc) + int(pq % G::KCH) * TC_KC + 32 * (t & 1)));
+                }
+                if (q < n_chunks) {
+                    const int64_t row0 = (int64_t(blockIdx.x) + (q / G::KCH) * gridDim.x) * TC_BM + r0 + half * (TC_BM / 2);
+                    const int col = int(q % G::KCH) * TC_KC + 4 * int(qf);
+#pragma unroll
+                    for (int i = 0; i < HR; ++i) b[i] = tc_ldg4(C + col + min(row0 + 16 * i, J - 1) * ldc);
+#pragma unroll
+                    for (int i = 0; i < HR; ++i) b[HR + i] = tc_ldg4(H + col + min(row0 + 16 * i, J - 1) * ldh);
+                }
+            };
+            auto convert = [&](const float4 (&b)[NR], int64_t q, auto upper) -> bool {
+                constexpr int half = decltype(upper)::value ? 1 : 0;
+                const uint32_t s = uint32_t(q) % G::OPS, u = uint32_t(q) / G::OPS;
+                if (half == 0 && !mbar_wait(bars + 8 * (B_EMPTY + s), (u & 1u) ^ 1u, abort_flag)) return false;
+                uint8_t *hi = smem + op_off + s * G::OP_STAGE + half * (TC_BM / 2 * 128), *mid = hi + G::OP_PART, *lo = mid + G::OP_PART;
+#pragma unroll
+                for (int i = 0; i < HR; ++i) {
+                    uint2 h, m, l;
+                    tc_split3(b[i].x * b[HR + i].x, b[i].y * b[HR + i].y, h.x, m.x, l.x);
+                    tc_split3(b[i].z * b[HR + i].z, b[i].w * b[HR + i].w, h.y, m.y, l.y);
+                    *reinterpret_cast<uint2 *>(hi + i * (16 * 128)) = h;
+                    *reinterpret_cast<uint2 *>(mid + i * (16 * 128)) = m;
+                    *reinterpret_cast<uint2 *>(lo + i * (16 * 128)) = l;
+                }
+                if (half == 0) return true;
+                fence_async_smem();
+#ifdef SA_TEST_HOOKS
+                if (withhold && q == 0) return true;
+#endif
+                mbar_arrive(bars + 8 * (B_FULL + s));
+                return true;
+            };
+            const std::false_type lower{};
+            const std::true_type upper{};
+            load(b0, 0, lower);
+            load(b1, 0, upper);
+            for (int64_t q = 0; q < n_chunks; q += 3) {
+                load(b2, q + 1, lower);
+                if (!convert(b0, q, lower)) break;
+                load(b0, q + 1, upper);
+                convert(b1, q, upper);
+                if (q + 1 >= n_chunks) break;
+                load(b1, q + 2, lower);
+                if (!convert(b2, q + 1, lower)) break;
+                load(b2, q + 2, upper);
+                convert(b0, q + 1, upper);
+                if (q + 2 >= n_chunks) break;
+                load(b0, q + 3, lower);
+                if (!convert(b1, q + 2, lower)) break;
+                load(b1, q + 3, upper);
+                convert(b2, q + 2, upper);
+            }
         }
     }
 
@@ -375,17 +487,18 @@ gemm_tc_kernel(int64_t J, const float *__restrict__ C, int64_t ldc, const float 
     if (threadIdx.x == 0 && *abort_flag && status != nullptr) atomicCAS(status, 0, int(SA_E_TIMEOUT));
 }
 
-template <int L, int M>
-sa_status launch_tc(int64_t rows, const float *A, int64_t lda, const float *B, int64_t ldb, float *out, int32_t *status,
-                    cudaStream_t stream)
+template <int L, int M, bool HAD>
+sa_status launch_tc(int64_t rows, const float *A, int64_t lda, const float *H, int64_t ldh, const float *B, int64_t ldb, float *out,
+                    int32_t *status, cudaStream_t stream)
 {
-    using G = tc_cfg<L, M>;
-    auto k = gemm_tc_kernel<L, M>;
-    if (cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, int(G::SMEM)) != cudaSuccess) return SA_E_CUDA;
+    using G = tc_cfg<L, M, HAD>;
+    auto k = gemm_tc_kernel<L, M, HAD>;
+    static bool attr[SA_MAX_DEVICE_FLAGS];
+    if (!sa_set_smem_once(k, int(G::SMEM), attr)) return SA_E_CUDA;
     int dev = 0, sms = 148;
     if (cudaGetDevice(&dev) == cudaSuccess) cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     const int64_t ctas = std::min<int64_t>((rows + TC_BM - 1) / TC_BM, sms);
-    if (ctas > 0) k<<<(unsigned)ctas, TC_THREADS, G::SMEM, stream>>>(rows, A, lda, B, ldb, out, status);
+    if (ctas > 0) k<<<(unsigned)ctas, TC_THREADS, G::SMEM, stream>>>(rows, A, lda, H, ldh, B, ldb, out, status);
     return cudaGetLastError() == cudaSuccess ? SA_OK : SA_E_CUDA;
 }
 
@@ -396,8 +509,18 @@ bool sa_dense_gemm_tc_ok(int64_t L, int64_t M) { return (L == 64 || L == 128 || 
 sa_status sa_launch_dense_gemm_tc(int64_t rows, const float *A, int64_t lda, const float *B, int64_t ldb, int64_t L,
                                   int64_t M, float *out, int32_t *status, cudaStream_t stream)
 {
-#define SA_CASE(l, m) if (L == l && M == m) return launch_tc<l, m>(rows, A, lda, B, ldb, out, status, stream);
+#define SA_CASE(l, m) if (L == l && M == m) return launch_tc<l, m, false>(rows, A, lda, nullptr, 0, B, ldb, out, status, stream);
     SA_CASE(64, 32) SA_CASE(64, 64) SA_CASE(128, 32) SA_CASE(128, 64) SA_CASE(256, 32) SA_CASE(256, 64)
+#undef SA_CASE
+    return SA_E_UNSUPPORTED;
+}
+
+sa_status sa_launch_hadamard_gemm_tc(int64_t rows, const sa_dense &A, const sa_dense &H, const sa_dense &B, float *out, int32_t *status,
+                                     cudaStream_t stream)
+{
+#define SA_CASE(l, m) \
+    if (A.cols == l && B.cols == m) return launch_tc<l, m, true>(rows, A.ptr, A.ld, H.ptr, H.ld, B.ptr, B.ld, out, status, stream);
+    SA_CASE(128, 32) SA_CASE(128, 64) SA_CASE(256, 32) SA_CASE(256, 64)
 #undef SA_CASE
     return SA_E_UNSUPPORTED;
 }

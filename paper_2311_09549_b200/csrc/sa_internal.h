@@ -185,10 +185,11 @@ size_t sa_ws_sddmm_spmm(const sa_tensor *t, const sa_dense *ops, bool materializ
 sa_status sa_launch_spmm_gemm(const sa_tensor *t, const sa_dense *ops, float *out, void *ws, size_t ws_bytes,
                               bool assoc_right, cudaStream_t stream, int *launches);
 size_t sa_ws_spmm_gemm(const sa_tensor *t, const sa_dense *ops, bool assoc_right);
-// Kernel 3 <SpMMH,GEMM>: the row kernel of (B.C).D with the Hadamard product C(j,:) * D(j,:) as the gathered row.
-sa_status sa_launch_spmmh_gemm(const sa_tensor *t, const sa_dense *ops, float *out, void *ws, size_t ws_bytes,
+// Kernel 3 <SpMMH,GEMM>: the row kernel of (B.C).D with the Hadamard product C(j,:) * D(j,:) as the gathered row, or
+// (assoc_right) B.((C o D).E).
+sa_status sa_launch_spmmh_gemm(const sa_tensor *t, const sa_dense *ops, float *out, void *ws, size_t ws_bytes, bool assoc_right,
                                cudaStream_t stream, int *launches);
-size_t sa_ws_spmmh_gemm(const sa_tensor *t, const sa_dense *ops);
+size_t sa_ws_spmmh_gemm(const sa_tensor *t, const sa_dense *ops, bool assoc_right);
 
 sa_status sa_launch_ttmc3(const sa_tensor *t, const sa_dense *ops, float *out, void *ws, size_t ws_bytes, bool fissioned,
                           cudaStream_t stream, int *launches);
@@ -211,6 +212,9 @@ sa_status sa_launch_dense_gemm(int64_t rows, const float *A, int64_t lda, const 
 bool sa_dense_gemm_tc_ok(int64_t L, int64_t M);
 sa_status sa_launch_dense_gemm_tc(int64_t rows, const float *A, int64_t lda, const float *B, int64_t ldb, int64_t L,
                                   int64_t M, float *out, int32_t *status, cudaStream_t stream);
+// out (rows x M) = (A o H) (rows x L, element-wise product) . B (L x M) to fp32 accuracy, L in {128, 256}
+sa_status sa_launch_hadamard_gemm_tc(int64_t rows, const sa_dense &A, const sa_dense &H, const sa_dense &B, float *out, int32_t *status,
+                                     cudaStream_t stream);
 
 // Kernel 7 <SpTTM,SpTTM>: out = one row of M values per (i,j) fiber, in CSF order
 bool sa_ranks_ok_spttm_spttm(int64_t L, int64_t M);

@@ -421,3 +421,25 @@ def test_sddmm_spmm_gemm_rank_combinations(sa, K, L, M):
     F = configs.dense_normal(91, 3, L, M)
     w = _wl("sddmm_spmm_gemm", "csr", w0.dims, w0.coords, w0.vals, w0.dense + [F], (w0.dims[0], M))
     _check(sa, w)
+
+
+@pytest.mark.parametrize("L,M,J", [(128, 32, 1), (128, 64, 127), (256, 32, 148 * 128 + 1), (256, 64, 148 * 128 * 2 + 77)])
+def test_spmmh_gemm_right_order_ragged_tiles_and_padded_operands(sa, L, M, J):
+    """B.((C o D).E): row counts J around the dense stage's 128-row tile and its second tile per block, padded views.
+    The bound is the one of an fp32 evaluation: 2 L rounding errors of 2^-24 per term of the sum at most."""
+    import torch
+    I = 300
+    coords, vals = _random_coo(22, (I, J), min(20_000, I * J // 3))
+    dense = [configs.dense_normal(22, 0, J, L), configs.dense_normal(22, 1, J, L), configs.dense_normal(22, 2, L, M)]
+    w = _wl("spmmh_gemm", "csr", (I, J), coords, vals, dense, (I, M))
+    A_ref, S_ref = oracle.evaluate(w)
+    t = sa.SparseTensor(w.dims, w.coords, w.vals, sa.SA_FMT_CSR, device=0)
+    views = []
+    for x, pad in zip(dense, (8, 12, 4)):
+        b = torch.zeros(x.shape[0], x.shape[1] + pad, device="cuda")
+        b[:, 4:4 + x.shape[1]] = torch.from_numpy(x).cuda()
+        views.append(b[:, 4:4 + x.shape[1]])
+    out, _ = t.run("spmmh_gemm", views, sched=sa.SA_SCHED_ASSOC_RIGHT)
+    torch.cuda.synchronize()
+    assert sa.sa_last_device_status(t.handle, torch.cuda.current_stream().cuda_stream) == sa.SA_OK
+    assert_close(out.cpu().numpy().astype(np.float64), A_ref, S_ref, 2 * L * 2.0 ** -24, "spmmh right %dx%d" % (L, M))
