@@ -3,6 +3,7 @@
 // chosen schedules to compiled functions outlined in the paper's discussion of run-time overheads
 // (Section 6).
 #include <cstring>
+#include <memory>
 #include <new>
 
 #include "sa_internal.h"
@@ -402,25 +403,29 @@ sa_status sa_tensor_create(int order, const int64_t *dims, int64_t nnz, const in
         }
         if (s == SA_OK && !packed_only) s = upload(t, t->vals.data(), t->vals.size(), &t->d_vals);
         if (s == SA_OK && fmt == SA_FMT_CSF) {
-            // one bit per nonzero: set on the last nonzero of every last-level fiber
+            // per nonzero (last-level index, value); CSF: the last nonzero of every last-level fiber is marked in bit 31 of
+            // the index, and in a bit array of one bit per nonzero
             const int last = order - 1;
-            std::vector<uint32_t> bits(size_t(nnz / 32 + 1), 0u);
-            for (int64_t f = 0; f < t->count[last - 1]; ++f) {
-                const int64_t p = t->pos[last][size_t(f) + 1] - 1;
-                bits[size_t(p >> 5)] |= 1u << (p & 31);
+            std::unique_ptr<int2[]> pack(new int2[size_t(nnz) + 1]);       // filled in parallel, not set to zero first
+#pragma omp parallel for schedule(static)
+            for (int64_t p = 0; p < nnz; ++p) {
+                int32_t vb;
+                std::memcpy(&vb, &t->vals[size_t(p)], sizeof(vb));
+                pack[size_t(p)] = make_int2(t->crd[last][size_t(p)], vb);
             }
-            if (!packed_only) s = upload(t, bits.data(), bits.size(), &t->d_endbits);
-            if (s == SA_OK) {
-                std::vector<int2> pack(size_t(nnz) + 1);
-                for (int64_t p = 0; p < nnz; ++p) {
-                    const uint32_t end = (bits[size_t(p >> 5)] >> (p & 31)) & 1u;
-                    int32_t vb;
-                    std::memcpy(&vb, &t->vals[size_t(p)], sizeof(vb));
-                    pack[size_t(p)] = make_int2(int32_t(uint32_t(t->crd[last][size_t(p)]) | (end << 31)), vb);
+            pack[size_t(nnz)] = make_int2(0, 0);
+            if (fmt == SA_FMT_CSF) {
+                std::vector<uint32_t> bits(size_t(nnz / 32 + 1), 0u);
+#pragma omp parallel for schedule(static)
+                for (int64_t f = 0; f < t->count[last - 1]; ++f) {
+                    const int64_t p = t->pos[last][size_t(f) + 1] - 1;
+                    pack[size_t(p)].x |= int32_t(0x80000000u);
+#pragma omp atomic
+                    bits[size_t(p >> 5)] |= 1u << (p & 31);
                 }
-                pack[size_t(nnz)] = make_int2(0, 0);
-                s = upload(t, pack.data(), pack.size(), &t->d_nzpack);
+                if (!packed_only) s = upload(t, bits.data(), bits.size(), &t->d_endbits);
             }
+            if (s == SA_OK) s = upload(t, pack.get(), size_t(nnz) + 1, &t->d_nzpack);
         }
         const int32_t zeros[4] = {0, 0, 0, 0};
         if (s == SA_OK) s = upload(t, zeros, 4, &t->d_status);

@@ -3,6 +3,7 @@
 // lists (nonzero-balanced pieces of slices, fibers and rows) the kernels consume.
 #include <algorithm>
 #include <cstring>
+#include <memory>
 #include <omp.h>
 
 #include "sa_internal.h"
@@ -16,21 +17,24 @@ int bits_for(int64_t dim)
     return b;
 }
 
-// Stable LSD radix sort of (key, idx) pairs on the low `total_bits` bits, 11 bits per pass.
-void radix_sort(std::vector<uint64_t> &keys, std::vector<uint32_t> &idx, int total_bits)
+// Stable LSD radix sort of (key, idx) pairs on the low `total_bits` bits, 11 bits per pass.  The second pair of buffers
+// is scratch; the sorted pairs end up in keys / idx.  (Buffers that are filled in parallel are allocated without being
+// set to zero first: the one thread that would do that takes as long as a pass of the sort.)
+void radix_sort(std::unique_ptr<uint64_t[]> &keys, std::unique_ptr<uint32_t[]> &idx, size_t n, int total_bits)
 {
-    const size_t n = keys.size();
     if (n < 2) return;
     constexpr int DB = 11, NB = 1 << DB;
     const int passes = (total_bits + DB - 1) / DB;
-    std::vector<uint64_t> k2(n);
-    std::vector<uint32_t> i2(n);
+    std::unique_ptr<uint64_t[]> k2(new uint64_t[n]);
+    std::unique_ptr<uint32_t[]> i2(new uint32_t[n]);
     const int nt = std::max(1, omp_get_max_threads());
     std::vector<size_t> hist(size_t(nt) * NB);
-    uint64_t *ks = keys.data(), *kd = k2.data();
-    uint32_t *is = idx.data(), *id = i2.data();
     for (int pass = 0; pass < passes; ++pass) {
         const int shift = pass * DB;
+        const uint64_t *ks = keys.get();
+        const uint32_t *is = idx.get();
+        uint64_t *kd = k2.get();
+        uint32_t *id = i2.get();
 #pragma omp parallel num_threads(nt)
         {
             const int tid = omp_get_thread_num();
@@ -55,12 +59,8 @@ void radix_sort(std::vector<uint64_t> &keys, std::vector<uint32_t> &idx, int tot
                 id[q] = is[p];
             }
         }
-        std::swap(ks, kd);
-        std::swap(is, id);
-    }
-    if (ks != keys.data()) {
-        std::memcpy(keys.data(), ks, n * sizeof(uint64_t));
-        std::memcpy(idx.data(), is, n * sizeof(uint32_t));
+        keys.swap(k2);
+        idx.swap(i2);
     }
 }
 
@@ -76,11 +76,11 @@ sa_status sa_build_levels(sa_tensor *t, const int32_t *coords, const float *vals
     if (total > 64) return SA_E_UNSUPPORTED;
     for (int d = 0, s = total; d < order; ++d) { s -= bits[d]; shift[d] = s; }
 
-    std::vector<uint64_t> keys;
-    std::vector<uint32_t> idx;
+    std::unique_ptr<uint64_t[]> keys;
+    std::unique_ptr<uint32_t[]> idx;
     try {
-        keys.resize(size_t(nnz));
-        idx.resize(size_t(nnz));
+        keys.reset(new uint64_t[size_t(nnz)]);
+        idx.reset(new uint32_t[size_t(nnz)]);
     } catch (...) { return SA_E_ALLOC; }
 
     int bad = 0;
@@ -97,7 +97,7 @@ sa_status sa_build_levels(sa_tensor *t, const int32_t *coords, const float *vals
     }
     if (bad) return SA_E_COORD_RANGE;
 
-    radix_sort(keys, idx, total);
+    try { radix_sort(keys, idx, size_t(nnz), total); } catch (...) { return SA_E_ALLOC; }
 
     int dup = 0;
 #pragma omp parallel for reduction(| : dup) schedule(static)
@@ -109,7 +109,7 @@ sa_status sa_build_levels(sa_tensor *t, const int32_t *coords, const float *vals
         t->vals.resize(size_t(nnz));
 #pragma omp parallel for schedule(static)
         for (int64_t p = 0; p < nnz; ++p) t->vals[size_t(p)] = vals[idx[size_t(p)]];
-        std::vector<uint32_t>().swap(idx);
+        idx.reset();
 
         const int last = order - 1;
         auto coord_of = [&](uint64_t k, int d) { return int32_t((k >> shift[d]) & ((uint64_t(1) << bits[d]) - 1)); };
@@ -118,36 +118,57 @@ sa_status sa_build_levels(sa_tensor *t, const int32_t *coords, const float *vals
             const int64_t I = t->dims[0];
             t->count[0] = I;
             t->count[1] = nnz;
-            t->pos[1].assign(size_t(I) + 1, 0);
+            t->pos[1].resize(size_t(I) + 1);
             t->crd[1].resize(size_t(nnz));
-            for (int64_t p = 0; p < nnz; ++p) {
-                t->pos[1][size_t(coord_of(keys[size_t(p)], 0)) + 1]++;
-                t->crd[1][size_t(p)] = coord_of(keys[size_t(p)], 1);
+            // pos[r] = first entry of row r or of a later one: entry p sets it for the rows above the row of p - 1
+#pragma omp parallel for schedule(static)
+            for (int64_t p = 0; p <= nnz; ++p) {
+                const int64_t row = p < nnz ? coord_of(keys[size_t(p)], 0) : I;
+                for (int64_t r = p > 0 ? int64_t(coord_of(keys[size_t(p - 1)], 0)) + 1 : 0; r <= row; ++r) t->pos[1][size_t(r)] = p;
+                if (p < nnz) t->crd[1][size_t(p)] = coord_of(keys[size_t(p)], 1);
             }
-            for (int64_t i = 0; i < I; ++i) t->pos[1][size_t(i) + 1] += t->pos[1][size_t(i)];
         } else {
             // prefix of level l = key >> shift[l]; a new node opens at every level >= the first
             // level whose prefix differs from the previous entry's
-            for (int l = 0; l <= last; ++l) { t->crd[l].clear(); t->pos[l].clear(); }
-            t->crd[last].resize(size_t(nnz));
-            for (int64_t p = 0; p < nnz; ++p) {
-                const uint64_t k = keys[size_t(p)];
-                int first = 0;
-                if (p > 0) {
-                    const uint64_t diff = k ^ keys[size_t(p - 1)];
-                    first = last;
-                    for (int l = 0; l < last; ++l)
-                        if ((diff >> shift[l]) != 0) { first = l; break; }
-                }
-                for (int l = first; l < last; ++l) {
-                    t->pos[l + 1].push_back(int64_t(l + 1 == last ? p : int64_t(t->crd[l + 1].size())));
-                    t->crd[l].push_back(coord_of(k, l));
-                }
-                t->crd[last][size_t(p)] = coord_of(k, last);
+            auto first_new_level = [&](int64_t p) {
+                if (p == 0) return 0;
+                const uint64_t diff = keys[size_t(p)] ^ keys[size_t(p - 1)];
+                int l = 0;
+                while (l < last && (diff >> shift[l]) == 0) ++l;
+                return l;
+            };
+            // two passes over fixed shares of the entries: how many nodes open in a share, then where they go
+            const int nt = std::max(1, omp_get_max_threads());
+            std::vector<int64_t> opened(size_t(nt + 1) * SA_MAX_ORDER, 0);
+            auto share = [&](int w) { return nnz * w / nt; };
+#pragma omp parallel for schedule(static) num_threads(nt)
+            for (int w = 0; w < nt; ++w) {
+                int64_t cnt[SA_MAX_ORDER] = {0, 0, 0, 0};
+                for (int64_t p = share(w); p < share(w + 1); ++p)
+                    for (int l = first_new_level(p); l < last; ++l) ++cnt[l];
+                for (int l = 0; l < last; ++l) opened[size_t(w + 1) * SA_MAX_ORDER + size_t(l)] = cnt[l];
             }
-            for (int l = 0; l <= last; ++l) t->count[l] = int64_t(t->crd[l].size());
-            for (int l = 0; l < last; ++l) t->pos[l + 1].push_back(t->count[l + 1]);
+            for (int w = 0; w < nt; ++w)
+                for (int l = 0; l < last; ++l) opened[size_t(w + 1) * SA_MAX_ORDER + size_t(l)] += opened[size_t(w) * SA_MAX_ORDER + size_t(l)];
+            for (int l = 0; l <= last; ++l) {
+                t->count[l] = l == last ? nnz : opened[size_t(nt) * SA_MAX_ORDER + size_t(l)];
+                t->crd[l].resize(size_t(t->count[l]));
+                if (l < last) t->pos[l + 1].resize(size_t(t->count[l]) + 1);
+            }
+            for (int l = 0; l < last; ++l) t->pos[l + 1][size_t(t->count[l])] = t->count[l + 1];
             t->pos[0] = {0, t->count[0]};
+#pragma omp parallel for schedule(static) num_threads(nt)
+            for (int w = 0; w < nt; ++w) {
+                int64_t at[SA_MAX_ORDER] = {0, 0, 0, 0};
+                for (int l = 0; l < last; ++l) at[l] = opened[size_t(w) * SA_MAX_ORDER + size_t(l)];
+                for (int64_t p = share(w); p < share(w + 1); ++p) {
+                    const uint64_t k = keys[size_t(p)];
+                    const int first = first_new_level(p);
+                    for (int l = last - 1; l >= first; --l) t->pos[l + 1][size_t(at[l])] = l + 1 == last ? p : at[l + 1];
+                    for (int l = first; l < last; ++l) t->crd[l][size_t(at[l]++)] = coord_of(k, l);
+                    t->crd[last][size_t(p)] = coord_of(k, last);
+                }
+            }
         }
     } catch (...) { return SA_E_ALLOC; }
     return SA_OK;
