@@ -402,7 +402,7 @@ sa_status sa_tensor_create(int order, const int64_t *dims, int64_t nnz, const in
             if (s == SA_OK && !(packed_only && l == order - 1)) s = upload(t, t->crd[l].data(), t->crd[l].size(), &t->d_crd[l]);
         }
         if (s == SA_OK && !packed_only) s = upload(t, t->vals.data(), t->vals.size(), &t->d_vals);
-        if (s == SA_OK && fmt == SA_FMT_CSF) {
+        if (s == SA_OK) {
             // per nonzero (last-level index, value); CSF: the last nonzero of every last-level fiber is marked in bit 31 of
             // the index, and in a bit array of one bit per nonzero
             const int last = order - 1;

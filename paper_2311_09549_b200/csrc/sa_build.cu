@@ -564,6 +564,81 @@ void build_rows(const std::vector<int64_t> &pos, int64_t I, sa_worklist &wl, int
     wl.items.insert(wl.items.end(), ranges.begin(), ranges.end());
 }
 
+// CSR, kernel 1 (fused SDDMM -> SpMM): an item is what one group of eight lanes walks, a range of whole short rows or a
+// piece of a long row with a partial row for the fix-up kernel.
+//   Size: `target` nonzeros, at most 256, less where the tensor would not give every group of a full machine
+//     (148 SMs x 64 groups) two items, at least 16: a group needs about a microsecond per four nonzeros, and on a small tensor
+//     that chain is the whole run time (60 k nonzeros, rows of up to 1500: 28 us; with a warp per item of up to 1024
+//     nonzeros 78 us).  Ranges of short rows stay at 256; a row counts as long above 64 nonzeros.
+//   Order: D and E are gathered by column, and with J x (K + L) floats above L2 the order of the work decides what is
+//     found there.  Long rows are therefore cut where their columns cross a multiple of COL_BLOCK (a piece has at
+//     least MIN_PIECE nonzeros) and the pieces are sorted by block: whatever runs at one time then gathers from the
+//     same few blocks (32 K columns x (64 + 64) floats = 16 MB).  1M x 1M, 30 M nonzeros, K = L = 64: 1.05 ms with blocks
+//     of 32 K or 64 K columns, 1.06 with 16 K; rows long above 64 / 128 / 256 / 1024 nonzeros 1.01 / 1.03 / 1.05 / 1.09 ms.
+//     Inside a block the longest pieces come first, so that the four groups of a warp get pieces of like length.
+void build_sddmm(const std::vector<int64_t> &pos, const std::vector<int32_t> &crd, int64_t I, sa_worklist &wl)
+{
+    constexpr int64_t COL_BLOCK = 32768, MIN_PIECE = 16;
+    const int64_t target = std::min<int64_t>(256, std::max<int64_t>(16, pos[size_t(I)] / (2 * 148 * 64)));
+    const int64_t long_row = std::min<int64_t>(std::max<int64_t>(target, 48), 64), max_rows = 32;
+    struct piece_rec { uint32_t key; sa_item it; };
+    std::vector<piece_rec> pieces;
+    std::vector<sa_item> ranges;
+    int64_t r0 = 0;
+    auto flush = [&](int64_t r1) {
+        if (r1 > r0) {
+            sa_item it = empty_item();
+            it.out_row = int32_t(r0); it.row_end = int32_t(r1);
+            it.p0 = int32_t(pos[size_t(r0)]); it.p1 = int32_t(pos[size_t(r1)]);
+            ranges.push_back(it);
+        }
+        r0 = r1;
+    };
+    for (int64_t r = 0; r < I; ++r) {
+        const int64_t a = pos[size_t(r)], b = pos[size_t(r) + 1];
+        if (b - a > long_row) {
+            flush(r);
+            const size_t first = pieces.size();
+            for (int64_t p = a; p < b;) {
+                int64_t q = std::min(b, p + target);
+                // the first block boundary after MIN_PIECE nonzeros, if there is one before q
+                if (q - p > MIN_PIECE && crd[size_t(q) - 1] / COL_BLOCK != crd[size_t(p + MIN_PIECE) - 1] / COL_BLOCK) {
+                    const int32_t edge = int32_t((crd[size_t(p + MIN_PIECE) - 1] / COL_BLOCK + 1) * COL_BLOCK);
+                    q = std::lower_bound(crd.begin() + p + MIN_PIECE, crd.begin() + q, edge) - crd.begin();
+                }
+                if (b - q < MIN_PIECE) q = b;
+                sa_item it = empty_item();
+                it.out_row = int32_t(r); it.row_end = int32_t(r + 1);
+                it.p0 = int32_t(p); it.p1 = int32_t(q);
+                pieces.push_back(piece_rec{uint32_t(crd[size_t(p)] / COL_BLOCK), it});
+                p = q;
+            }
+            const int64_t np = int64_t(pieces.size() - first);
+            if (np > 1) {
+                for (size_t x = first; x < pieces.size(); ++x) pieces[x].it.dest = int32_t(wl.n_slots + int64_t(x - first));
+                wl.fix.push_back(sa_fix{int32_t(r), int32_t(wl.n_slots), int32_t(np), 0});
+                wl.n_slots += np;
+            }
+            r0 = r + 1;
+            continue;
+        }
+        if (pos[size_t(r) + 1] - pos[size_t(r0)] > target && r > r0) flush(r);
+        if (r + 1 - r0 >= max_rows) flush(r + 1);
+    }
+    flush(I);
+    std::sort(pieces.begin(), pieces.end(), [](const piece_rec &x, const piece_rec &y) {
+        if (x.key != y.key) return x.key < y.key;
+        const int32_t lx = x.it.p1 - x.it.p0, ly = y.it.p1 - y.it.p0;
+        return lx != ly ? lx > ly : x.it.p0 < y.it.p0;
+    });
+    std::stable_sort(ranges.begin(), ranges.end(), [](const sa_item &x, const sa_item &y) { return (x.p1 - x.p0) > (y.p1 - y.p0); });
+    wl.n_group_ctas = 0;
+    wl.items.clear();
+    wl.items.reserve(pieces.size() + ranges.size());
+    for (const piece_rec &x : pieces) wl.items.push_back(x.it);
+    wl.items.insert(wl.items.end(), ranges.begin(), ranges.end());
+}
+
 }  // namespace
 
 void sa_build_worklists(sa_tensor *t)
@@ -580,7 +655,11 @@ void sa_build_worklists(sa_tensor *t)
         t->wl4_main.nnz = t->nnz - t->wl4_sub.nnz;
     }
     if (t->fmt == SA_FMT_CSR) {
-        build_rows(t->pos[1], t->dims[0], t->wl_main, 256, 32, 1024, 512);    // fused SDDMM -> SpMM
+        build_sddmm(t->pos[1], t->crd[1], t->dims[0], t->wl_main);
         build_rows(t->pos[1], t->dims[0], t->wl_aux, 256, 16, 4096, 2048);    // SpMM -> GEMM (both orders)
+    }
+    for (sa_worklist *wl : {&t->wl_main, &t->wl_aux, &t->wl_sub, &t->wl4_main, &t->wl4_aux, &t->wl4_sub}) {
+        std::stable_sort(wl->fix.begin(), wl->fix.end(), [](const sa_fix &x, const sa_fix &y) { return x.count > y.count; });
+        wl->n_big_fix = std::find_if(wl->fix.begin(), wl->fix.end(), [](const sa_fix &x) { return x.count <= SA_BIG_FIX; }) - wl->fix.begin();
     }
 }

@@ -126,11 +126,50 @@ sa_fixup_kernel(const sa_fix *__restrict__ fix, const float *__restrict__ partia
     }
 }
 
+// The same for rows of at most 128 floats (8, 16 or 32 float4): the first n_big entries (the builder puts the longest
+// first) take a block each as above, the others a warp each, which is all that a few partial rows can use.
+static __global__ void __launch_bounds__(256)
+sa_fixup_rows_kernel(const sa_fix *__restrict__ fix, int n_fix, int n_big, const float *__restrict__ partial, float *__restrict__ out,
+                     int row_floats)
+{
+    __shared__ float4 red[256];
+    const bool big = int(blockIdx.x) < n_big;
+    const int W = row_floats / 4, lane = threadIdx.x & 31;
+    const int entry = big ? int(blockIdx.x) : n_big + (int(blockIdx.x) - n_big) * 8 + int(threadIdx.x >> 5);
+    if (entry >= n_fix) return;                        // whole warps of the last block
+    const sa_fix e = fix[entry];
+    const int who = big ? int(threadIdx.x) : lane, P = (big ? 256 : 32) / W;
+    const int col = who % W, phase = who / W;
+    float4 s = make_float4(0.f, 0.f, 0.f, 0.f);
+    const float *base = partial + int64_t(e.slot0) * row_floats + col * 4;
+#pragma unroll 4
+    for (int q = phase; q < e.count; q += P) {
+        const float4 v = *reinterpret_cast<const float4 *>(base + int64_t(q) * row_floats);
+        s.x += v.x; s.y += v.y; s.z += v.z; s.w += v.w;
+    }
+    red[threadIdx.x] = s;
+    if (big) __syncthreads();
+    else __syncwarp();
+    if (phase == 0) {
+        const float4 *mine = red + (big ? 0 : int(threadIdx.x) - lane);
+        for (int q = 1; q < P; ++q) {
+            const float4 v = mine[q * W + col];
+            s.x += v.x; s.y += v.y; s.z += v.z; s.w += v.w;
+        }
+        sa_st_cs4(out + int64_t(e.out_row) * row_floats + col * 4, s);
+    }
+}
+
 static inline cudaError_t sa_launch_fixup(const sa_worklist &wl, const float *partial, float *out, int tile_floats,
                                           cudaStream_t stream)
 {
     if (wl.fix.empty()) return cudaSuccess;
     const int nf4 = tile_floats / 4;
+    if (nf4 <= 32) {
+        const unsigned rows = (unsigned)wl.fix.size(), big = (unsigned)wl.n_big_fix;
+        sa_fixup_rows_kernel<<<big + (rows - big + 7) / 8, 256, 0, stream>>>(wl.d_fix, int(rows), int(big), partial, out, tile_floats);
+        return cudaGetLastError();
+    }
     const int W = nf4 < 64 ? nf4 : 64;
     dim3 grid((unsigned)wl.fix.size(), (unsigned)(nf4 / W));
     sa_fixup_kernel<<<grid, 256, 0, stream>>>(wl.d_fix, partial, out, tile_floats, W);

@@ -64,11 +64,13 @@ static inline void sa_unit3_streams(int64_t p0, int64_t p1, int64_t *lo, int64_t
     }
 }
 
+constexpr int SA_BIG_FIX = 32;
 struct sa_worklist {
     std::vector<sa_item> items;   // [n_group_ctas * SA_WARPS_PER_CTA group items][warp items]
     std::vector<sa_fix> fix;
     int64_t n_group_ctas = 0;     // leading CTAs whose 8 warps reduce into one tile
     int64_t n_slots = 0;          // partial tiles in the workspace
+    int64_t n_big_fix = 0;        // leading fix-up entries with more than SA_BIG_FIX partial tiles (longest first)
     int64_t nnz = 0;              // nonzeros the list covers (set for the order-4 lists of pass 1)
     sa_item *d_items = nullptr;
     sa_fix *d_fix = nullptr;

@@ -3,192 +3,152 @@
 // Table of kernels (Section 6): the sampled value is a scalar temporary that is consumed at once,
 // the sampled matrix is never written (auxiliary memory 1 in the paper's memory table).
 //
-// One warp per work item (a range of short rows, or a piece of a long row).  The rows D(j,:) and
-// E(j,:) of the item's nonzeros are gathered with cp.async into a per-warp ring of shared-memory
-// stages that runs ahead of the arithmetic, so that the random row reads (the HBM-bound part: D
-// and E exceed L2) stay in flight while earlier nonzeros are consumed.  K/4 lanes share one
-// nonzero (a float4 of D each, shuffle reduction of the dot product), 32/(K/4) nonzeros per step.
+// A warp is four groups of eight lanes; every group takes one work item (a range of short rows, or a piece of a long
+// row) and walks its nonzeros U at a time: a lane owns the float4 columns l, l + 8, ... of D(j,:), E(j,:), C(i,:) and of
+// the output row, so a row piece of 128 bytes is one load instruction of the group, a dot product is three shuffles per
+// four nonzeros of the warp, and nothing passes through shared memory.  Indices and values come as 8-byte records that
+// all lanes of a group read (one step ahead); C(i + 1,:) is requested while row i is being summed.
+// What bounds it: the gathered rows of D and E.  Where they exceed L2 the builder cuts long rows at column-block
+// boundaries and orders the pieces by block (build_sddmm), so that what runs at one time gathers from a few blocks that
+// L2 holds; what then limits is the L2-to-SM path (4 (K + L) bytes per nonzero), not HBM.  1M x 1M, 30 M nonzeros,
+// K = L = 64: 1.01 ms, 15.7 GB through that path and 2.8 GB of DRAM traffic, where one warp per item with the rows in a
+// cp.async ring and items in order of size took 2.24 ms and 13.2 GB.  Two nonzeros per step with 24 warps per SM: 9 % slower.
 #include "sa_device.cuh"
 
 namespace {
 
 template <int K, int L>
 struct sd_cfg {
-    static constexpr int LPN = K / 4;                 // lanes per nonzero
-    static constexpr int NPS = 32 / LPN;              // nonzeros per step
-    static constexpr int EV = L / LPN;                // floats of E(j,:) and of the output row per lane
-    static constexpr int ROWF = K + L;                // floats staged per nonzero: D(j,:) then E(j,:)
-    static constexpr int R = ROWF <= 128 ? 8 : 4;     // nonzeros per stage
-    static constexpr int NS = 3;                      // stages per warp: one being consumed, two in flight
-    static constexpr int STAGE = R * ROWF;            // floats per stage
-    static constexpr int CPL = STAGE / 4 / 32;        // 16-byte copies per lane per stage
-    static_assert(STAGE % 128 == 0 && R % NPS == 0 && 32 % R == 0, "stage shape");
+    static constexpr int DQ = K / 32, EQ = L / 32;    // float4 pieces of D(j,:) and E(j,:) per lane
+    static constexpr int U = DQ + EQ <= 4 ? 4 : 2;    // nonzeros per group and step: 16 float4 in flight per lane at most
+    static constexpr bool AHEAD = DQ + EQ < 8;        // C of the next row in registers (spills at K = L = 128)
 };
 
 template <int K, int L>
 __global__ void __launch_bounds__(256, 2)
 sddmm_spmm_kernel(const sa_item *__restrict__ items, int64_t n_items, const int32_t *__restrict__ pos,
-                  const int32_t *__restrict__ crd, const float *__restrict__ vals, const float *__restrict__ C,
-                  uint32_t ldc, const float *__restrict__ D, uint32_t ldd, const float *__restrict__ E, uint32_t lde,
-                  float *__restrict__ out, float *__restrict__ partial, float *__restrict__ sampled, const sa_limits lim)
+                  const int2 *__restrict__ nz, const float *__restrict__ C, uint32_t ldc, const float *__restrict__ D,
+                  uint32_t ldd, const float *__restrict__ E, uint32_t lde, float *__restrict__ out, float *__restrict__ partial,
+                  float *__restrict__ sampled, const sa_limits lim)
 {
     using G = sd_cfg<K, L>;
-    extern __shared__ __align__(16) float smem[];
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const int64_t idx = int64_t(blockIdx.x) * SA_WARPS_PER_CTA + warp;
-    if (idx >= n_items) return;
-    float *ring = smem + warp * (G::NS * G::STAGE);
-    const sa_item it = items[idx];
-    const int P0 = it.p0, total = it.p1 - it.p0;      // the item's nonzeros are contiguous
-    const int li = lane % G::LPN, grp = lane / G::LPN;
-
-    // column indices / values of the consumer's batch of 32 nonzeros (j0, v0) and the two after it
-    int j0, j1, j2;
-    float v0, v1, v2;
-    auto load_jv = [&](int b, int &j, float &v) {
-        const int p = 32 * b + lane;
-        j = 0;
-        v = 0.f;
-        if (p < total && SA_CHK(lim.status, P0 + p >= 0 && P0 + p < lim.nnz, 41, P0 + p)) { j = crd[P0 + p]; v = vals[P0 + p]; }
-        if (!SA_CHK(lim.status, uint32_t(j) < lim.gather_rows, 42, j)) j = 0;
-    };
-    int cb = 0;                                       // batch the consumer is in
-    // per-lane constants of the gather: copy q of a stage moves 16-byte piece x = 32 q + lane, i.e. piece
-    // cc = x % (ROWF/4) of nonzero r = x / (ROWF/4); pieces lie in the stage in the same order (byte 16 x)
-    const char *src_q[G::CPL];                        // D or E plus the piece offset
-    uint32_t rowb_q[G::CPL];                          // bytes between rows of that operand
-    int r_q[G::CPL];
-#pragma unroll
-    for (int q = 0; q < G::CPL; ++q) {
-        const int x = q * 32 + lane;
-        const int cc = x % (G::ROWF / 4);
-        r_q[q] = x / (G::ROWF / 4);
-        src_q[q] = reinterpret_cast<const char *>(cc < K / 4 ? D + cc * 4 : E + (cc - K / 4) * 4);
-        rowb_q[q] = (cc < K / 4 ? ldd : lde) * 4u;
+    constexpr int DQ = G::DQ, EQ = G::EQ, U = G::U;
+    const int l = threadIdx.x & 7;
+    const int64_t idx = (int64_t(blockIdx.x) * 256 + threadIdx.x) >> 3;
+    int r = 0, rend = 0, p = 0, end = 0, dest = -1;
+    if (idx < n_items) {
+        const int4 ia = __ldg(reinterpret_cast<const int4 *>(items + idx));          // out_row, row_end, -, -
+        const int4 ib = __ldg(reinterpret_cast<const int4 *>(items + idx) + 1);      // p0, p1, dest, -
+        if (SA_CHK(lim.status, ia.x >= 0 && ia.x <= ia.y && uint32_t(ia.y) <= lim.out_rows && ib.x >= 0 && ib.x <= ib.y && ib.y <= lim.nnz &&
+                                   ib.z < lim.n_slots, 43, idx)) {
+            r = ia.x; rend = ia.y; p = ib.x; end = ib.y; dest = ib.z;
+        }
     }
-    const uint32_t ring_lane = smem_u32(ring) + uint32_t(lane) * 16u;
-    int issue_slot = 0;                               // ring slot the next issued stage goes to
-    auto issue_stage = [&](int s) {
-        if (s * G::R < total) {
-            const uint32_t dst = ring_lane + uint32_t(issue_slot * G::STAGE) * 4u;
-            const int b = (s * G::R) >> 5;            // the stage lies inside one batch: cb or cb + 1
-            const int jsrc = b == cb ? j0 : j1;
-            const int lane0 = (s * G::R) & 31;
+    // [p, b): what is left of row r; bn: where row r + 1 ends; c, cn: C of both rows
+    float4 c[DQ], cn[DQ], acc[EQ];
+    auto row_end = [&](int row) {
+        if (dest >= 0 || row >= rend) return end;
+        int e = __ldg(pos + row + 1);
+        if (!SA_CHK(lim.status, e >= 0 && e <= end, 44, e)) e = end;
+        return e;
+    };
+    auto load_c = [&](float4 (&x)[DQ], int row) {
+        if (row < rend) {
 #pragma unroll
-            for (int q = 0; q < G::CPL; ++q) {
-                const uint32_t j = uint32_t(__shfl_sync(SA_FULL_MASK, jsrc, lane0 + r_q[q]));   // 0 beyond the item: row 0
-                cp_async16_raw(dst + q * 512u, src_q[q] + j * rowb_q[q]);
+            for (int q = 0; q < DQ; ++q) x[q] = sa_ldg4(C + (uint32_t(row) * ldc + 32u * q + 4u * l));
+        }
+    };
+    int b = row_end(r), bn = row_end(r + 1);
+    load_c(c, r);
+    if (G::AHEAD) load_c(cn, r + 1);
+#pragma unroll
+    for (int q = 0; q < EQ; ++q) acc[q] = make_float4(0.f, 0.f, 0.f, 0.f);
+    int2 rec[U];
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+        rec[u] = make_int2(0, 0);
+        if (p + u < end) rec[u] = __ldg(nz + p + u);
+    }
+    const char *Dl = reinterpret_cast<const char *>(D + 4 * l), *El = reinterpret_cast<const char *>(E + 4 * l);
+    const uint32_t d_bytes = ldd * 4u, e_bytes = lde * 4u;
+    for (;;) {
+        while (p == b && r < rend) {                  // the row is complete (or empty: +0)
+            float *dst = (dest >= 0 ? partial + int64_t(dest) * L : out + int64_t(r) * L) + 4 * l;
+#pragma unroll
+            for (int q = 0; q < EQ; ++q) {
+                *reinterpret_cast<float4 *>(dst + 32 * q) = acc[q];
+                acc[q] = make_float4(0.f, 0.f, 0.f, 0.f);
+            }
+            ++r;
+            b = bn;
+            bn = row_end(r + 1);
+            if (G::AHEAD) {
+#pragma unroll
+                for (int q = 0; q < DQ; ++q) c[q] = cn[q];
+                load_c(cn, r + 1);
+            } else {
+                load_c(c, r);
             }
         }
-        issue_slot = issue_slot == G::NS - 1 ? 0 : issue_slot + 1;
-        cp_async_commit();
-    };
-    load_jv(0, j0, v0);
-    load_jv(1, j1, v1);
-    load_jv(2, j2, v2);
+        if (!__any_sync(SA_FULL_MASK, r < rend)) break;
+        const int n = min(U, b - p);                  // 0 for a group that is done
+        float4 d[U][DQ], e[U][EQ];
+        float v[U], dot[U];
 #pragma unroll
-    for (int s = 0; s < G::NS - 1; ++s) issue_stage(s);
-    int cur_stage = -1;
-    int cur_off = -G::STAGE;                          // float offset of the consumer's stage in the ring
-    // called when the consumer first touches stage s: refill the stage it left, wait for s
-    auto enter = [&](int s) {
-        __syncwarp();
-        cur_off = cur_off == (G::NS - 1) * G::STAGE ? 0 : cur_off + G::STAGE;
-        if (s > 0 && ((s * G::R) & 31) == 0) {
-            j0 = j1; j1 = j2;
-            v0 = v1; v1 = v2;
-            ++cb;
-            load_jv(cb + 2, j2, v2);
+        for (int u = 0; u < U; ++u) {
+            dot[u] = 0.f;
+            v[u] = __int_as_float(rec[u].y);
+            if (u < n) {
+                uint32_t j = uint32_t(rec[u].x);
+                if (!SA_CHK(lim.status, j < lim.gather_rows, 42, j)) j = 0u;
+#pragma unroll
+                for (int q = 0; q < DQ; ++q) d[u][q] = __ldg(reinterpret_cast<const float4 *>(Dl + uint64_t(j) * d_bytes) + 8 * q);
+#pragma unroll
+                for (int q = 0; q < EQ; ++q) e[u][q] = __ldg(reinterpret_cast<const float4 *>(El + uint64_t(j) * e_bytes) + 8 * q);
+            }
         }
-        issue_stage(s + G::NS - 1);
-        cp_async_wait<G::NS - 1>();
-        __syncwarp();
-        cur_stage = s;
-    };
-
-    const bool piece = it.dest >= 0;
-    for (int r = it.out_row; r < it.row_end; ++r) {
-        if (!SA_CHK(lim.status, uint32_t(r) < lim.out_rows && (!piece || it.dest < lim.n_slots), 43, r)) continue;
-        const int a = piece ? 0 : pos[r] - P0;
-        const int b = piece ? total : pos[r + 1] - P0;
-        float acc[G::EV];
 #pragma unroll
-        for (int q = 0; q < G::EV; ++q) acc[q] = 0.f;
-        if (b > a) {
-            const float4 c4 = sa_ldg4(C + uint32_t(r) * ldc + 4 * li);
-            for (int base = (a / G::NPS) * G::NPS; base < b; base += G::NPS) {
-                const int st = base / G::R;
-                if (st != cur_stage) enter(st);
-                const int prel = base + grp;
-                const bool active = prel >= a && prel < b;
-                const float v = __shfl_sync(SA_FULL_MASK, v0, prel & 31);
-                const float *slot = ring + cur_off + (prel & (G::R - 1)) * G::ROWF;
-                const float4 d4 = *reinterpret_cast<const float4 *>(slot + 4 * li);
-                float dot = fmaf(c4.x, d4.x, fmaf(c4.y, d4.y, fmaf(c4.z, d4.z, c4.w * d4.w)));
+        for (int u = 0; u < U; ++u)                   // the next step's records (rows of a range lie one after the other)
+            if (p + n + u < end) rec[u] = __ldg(nz + p + n + u);
 #pragma unroll
-                for (int o = G::LPN / 2; o > 0; o >>= 1) dot += __shfl_xor_sync(SA_FULL_MASK, dot, o);
-                if (active) {
-                    const float sc = v * dot;
-                    if (sampled != nullptr && li == 0) sampled[P0 + prel] = sc;
-                    const float *e = slot + K + li * G::EV;
-                    if (G::EV >= 4) {
+        for (int u = 0; u < U; ++u)
+            if (u < n) {
 #pragma unroll
-                        for (int q = 0; q < G::EV; q += 4) {
-                            const float4 e4 = *reinterpret_cast<const float4 *>(e + q);
-                            acc[q] = fmaf(sc, e4.x, acc[q]);
-                            acc[(q + 1) % G::EV] = fmaf(sc, e4.y, acc[(q + 1) % G::EV]);
-                            acc[(q + 2) % G::EV] = fmaf(sc, e4.z, acc[(q + 2) % G::EV]);
-                            acc[(q + 3) % G::EV] = fmaf(sc, e4.w, acc[(q + 3) % G::EV]);
-                        }
-                    } else if (G::EV == 2) {
-                        const float2 e2 = *reinterpret_cast<const float2 *>(e);
-                        acc[0] = fmaf(sc, e2.x, acc[0]);
-                        acc[1 % G::EV] = fmaf(sc, e2.y, acc[1 % G::EV]);
-                    } else {
-                        acc[0] = fmaf(sc, e[0], acc[0]);
-                    }
+                for (int q = 0; q < DQ; ++q)
+                    dot[u] = fmaf(c[q].x, d[u][q].x, fmaf(c[q].y, d[u][q].y, fmaf(c[q].z, d[u][q].z, fmaf(c[q].w, d[u][q].w, dot[u]))));
+            }
+#pragma unroll
+        for (int o = 4; o > 0; o >>= 1)
+#pragma unroll
+            for (int u = 0; u < U; ++u) dot[u] += __shfl_xor_sync(SA_FULL_MASK, dot[u], o);
+#pragma unroll
+        for (int u = 0; u < U; ++u)
+            if (u < n) {
+                const float sc = v[u] * dot[u];
+                if (sampled != nullptr && l == 0) sampled[p + u] = sc;
+#pragma unroll
+                for (int q = 0; q < EQ; ++q) {
+                    acc[q].x = fmaf(sc, e[u][q].x, acc[q].x);
+                    acc[q].y = fmaf(sc, e[u][q].y, acc[q].y);
+                    acc[q].z = fmaf(sc, e[u][q].z, acc[q].z);
+                    acc[q].w = fmaf(sc, e[u][q].w, acc[q].w);
                 }
             }
-            // the NPS groups of lanes hold partial rows: add them up
-#pragma unroll
-            for (int o = 16; o >= G::LPN; o >>= 1)
-#pragma unroll
-                for (int q = 0; q < G::EV; ++q) acc[q] += __shfl_xor_sync(SA_FULL_MASK, acc[q], o);
-        }
-        if (grp == 0) {
-            float *dst = (piece ? partial + int64_t(it.dest) * L : out + int64_t(r) * L) + li * G::EV;
-            if (G::EV >= 4) {
-#pragma unroll
-                for (int q = 0; q < G::EV; q += 4)
-                    *reinterpret_cast<float4 *>(dst + q) =
-                        make_float4(acc[q], acc[(q + 1) % G::EV], acc[(q + 2) % G::EV], acc[(q + 3) % G::EV]);
-            } else if (G::EV == 2) {
-                *reinterpret_cast<float2 *>(dst) = make_float2(acc[0], acc[1 % G::EV]);
-            } else {
-                dst[0] = acc[0];
-            }
-        }
+        p += n;
     }
-    cp_async_wait<0>();
 }
 
 template <int K, int L>
 cudaError_t launch(const sa_tensor *t, const sa_dense *ops, float *out, float *partial, float *sampled,
                    cudaStream_t stream)
 {
-    using G = sd_cfg<K, L>;
     const sa_worklist &wl = t->wl_main;
     const int64_t n_items = int64_t(wl.items.size());
-    const int64_t ctas = (n_items + SA_WARPS_PER_CTA - 1) / SA_WARPS_PER_CTA;
+    const int64_t ctas = (n_items + 31) / 32;         // 32 groups per block
     if (ctas == 0) return cudaSuccess;
-    constexpr size_t smem = size_t(SA_WARPS_PER_CTA) * G::NS * G::STAGE * sizeof(float);
-    auto kern = sddmm_spmm_kernel<K, L>;
-    if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem)) != cudaSuccess)
-        return cudaGetLastError();
-    kern<<<(unsigned)ctas, 256, smem, stream>>>(wl.d_items, n_items, t->d_pos[1], t->d_crd[1], t->d_vals, ops[0].ptr,
-                                               uint32_t(ops[0].ld), ops[1].ptr, uint32_t(ops[1].ld), ops[2].ptr,
-                                               uint32_t(ops[2].ld), out, partial, sampled,
-                                               sa_make_limits(t, t->dims[1], t->dims[0], wl.n_slots));
+    sddmm_spmm_kernel<K, L><<<(unsigned)ctas, 256, 0, stream>>>(
+        wl.d_items, n_items, t->d_pos[1], t->d_nzpack, ops[0].ptr, uint32_t(ops[0].ld), ops[1].ptr, uint32_t(ops[1].ld), ops[2].ptr,
+        uint32_t(ops[2].ld), out, partial, sampled, sa_make_limits(t, t->dims[1], t->dims[0], wl.n_slots));
     return cudaGetLastError();
 }
 

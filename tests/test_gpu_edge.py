@@ -443,3 +443,19 @@ def test_spmmh_gemm_right_order_ragged_tiles_and_padded_operands(sa, L, M, J):
     torch.cuda.synchronize()
     assert sa.sa_last_device_status(t.handle, torch.cuda.current_stream().cuda_stream) == sa.SA_OK
     assert_close(out.cpu().numpy().astype(np.float64), A_ref, S_ref, 2 * L * 2.0 ** -24, "spmmh right %dx%d" % (L, M))
+
+
+@pytest.mark.parametrize("K,L", [(32, 32), (64, 128), (128, 128)])
+@pytest.mark.parametrize("deg", [1, 15, 48, 49, 64, 65, 257])
+def test_sddmm_spmm_rows_around_piece_and_column_block_limits(sa, K, L, deg):
+    """Rows just below and above the length at which they are cut, with columns on both sides of the 32 K column blocks the
+    cuts follow; empty rows between them; the fix-up of rows in a few pieces and in more than 32."""
+    rs = np.random.RandomState(deg)
+    J = 70_001
+    rows = {0: deg, 2: deg, 3: 700, 5: 1, 9: deg + 1}
+    coords = np.concatenate([np.stack([np.full(n, r), np.sort(np.concatenate([[32767, 32768, 65536][:n], rs.choice(32767, max(0, n - 3), replace=False)]))], axis=1)
+                             for r, n in rows.items()]).astype(np.int32)
+    vals = rs.uniform(-1, 1, len(coords)).astype(np.float32)
+    w = _wl("sddmm_spmm", "csr", (11, J), coords, vals,
+            [configs.dense_normal(deg, 0, 11, K), configs.dense_normal(deg, 1, J, K), configs.dense_normal(deg, 2, J, L)], (11, L))
+    _check(sa, w)
