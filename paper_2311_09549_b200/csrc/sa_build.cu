@@ -656,7 +656,10 @@ void sa_build_worklists(sa_tensor *t)
     }
     if (t->fmt == SA_FMT_CSR) {
         build_sddmm(t->pos[1], t->crd[1], t->dims[0], t->wl_main);
-        build_rows(t->pos[1], t->dims[0], t->wl_aux, 256, 16, 4096, 2048);    // SpMM -> GEMM (both orders)
+        // SpMM -> GEMM (both orders): about 256 nonzeros per item, which one lane group or warp walks as a chain; fewer where
+        // the tensor would not give every group of a full machine two items
+        const int64_t target = std::min<int64_t>(256, std::max<int64_t>(32, t->nnz / (2 * 148 * 64)));
+        build_rows(t->pos[1], t->dims[0], t->wl_aux, target, 16, 2 * target, target);
     }
     for (sa_worklist *wl : {&t->wl_main, &t->wl_aux, &t->wl_sub, &t->wl4_main, &t->wl4_aux, &t->wl4_sub}) {
         std::stable_sort(wl->fix.begin(), wl->fix.end(), [](const sa_fix &x, const sa_fix &y) { return x.count > y.count; });

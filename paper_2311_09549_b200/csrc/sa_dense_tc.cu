@@ -208,7 +208,7 @@ __device__ __forceinline__ uint32_t tc_sw128(uint32_t row, uint32_t k)
 template <int L, int M, bool HAD>
 __global__ void __launch_bounds__(TC_THREADS, 1)
 gemm_tc_kernel(int64_t J, const float *__restrict__ C, int64_t ldc, const float *__restrict__ H, int64_t ldh,
-               const float *__restrict__ D, int64_t ldd, float *__restrict__ Eout, int32_t *__restrict__ status)
+               const float *__restrict__ D, int64_t ldd, float *__restrict__ Eout, int part_shift, int32_t *__restrict__ status)
 {
     using G = tc_cfg<L, M, HAD>;
     extern __shared__ uint8_t tc_smem_raw[];
@@ -305,12 +305,13 @@ gemm_tc_kernel(int64_t J, const float *__restrict__ C, int64_t ldc, const float 
             mbar_arrive(bars + 8 * (B_ACC_EMPTY + a));               // the accumulator is free again
             __syncwarp();
             const int64_t row0 = (int64_t(blockIdx.x) + tl * gridDim.x) * TC_BM + 32 * warp;
-            float4 *dst = reinterpret_cast<float4 *>(Eout + row0 * M);
+            // E as tables of 2^part_shift float4 columns (one table: rows of E): 512-byte runs whatever the width
 #pragma unroll
             for (int i = 0; i < RC; ++i) {
-                const int idx = i * 32 + lane, r = idx / RC, j = idx % RC;
+                const int idx = i * 32 + lane, tab = idx >> (part_shift + 5), r = (idx >> part_shift) & 31;
+                const int j = (tab << part_shift) + (idx & ((1 << part_shift) - 1));
                 const float4 val = *reinterpret_cast<const float4 *>(stage + r * (M * 4) + ((j ^ (r & 7)) << 4));
-                if (row0 + r < J) dst[idx] = val;
+                if (row0 + r < J) reinterpret_cast<float4 *>(Eout)[((int64_t(tab) * J + row0) << part_shift) + (idx & ((32 << part_shift) - 1))] = val;
             }
             __syncwarp();
         }
@@ -489,7 +490,7 @@ gemm_tc_kernel(int64_t J, const float *__restrict__ C, int64_t ldc, const float 
 
 template <int L, int M, bool HAD>
 sa_status launch_tc(int64_t rows, const float *A, int64_t lda, const float *H, int64_t ldh, const float *B, int64_t ldb, float *out,
-                    int32_t *status, cudaStream_t stream)
+                    int32_t *status, cudaStream_t stream, int part)
 {
     using G = tc_cfg<L, M, HAD>;
     auto k = gemm_tc_kernel<L, M, HAD>;
@@ -498,7 +499,9 @@ sa_status launch_tc(int64_t rows, const float *A, int64_t lda, const float *H, i
     int dev = 0, sms = 148;
     if (cudaGetDevice(&dev) == cudaSuccess) cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     const int64_t ctas = std::min<int64_t>((rows + TC_BM - 1) / TC_BM, sms);
-    if (ctas > 0) k<<<(unsigned)ctas, TC_THREADS, G::SMEM, stream>>>(rows, A, lda, H, ldh, B, ldb, out, status);
+    int shift = 0;
+    while ((4 << shift) < part) ++shift;
+    if (ctas > 0) k<<<(unsigned)ctas, TC_THREADS, G::SMEM, stream>>>(rows, A, lda, H, ldh, B, ldb, out, shift, status);
     return cudaGetLastError() == cudaSuccess ? SA_OK : SA_E_CUDA;
 }
 
@@ -507,19 +510,19 @@ sa_status launch_tc(int64_t rows, const float *A, int64_t lda, const float *H, i
 bool sa_dense_gemm_tc_ok(int64_t L, int64_t M) { return (L == 64 || L == 128 || L == 256) && (M == 32 || M == 64); }
 
 sa_status sa_launch_dense_gemm_tc(int64_t rows, const float *A, int64_t lda, const float *B, int64_t ldb, int64_t L,
-                                  int64_t M, float *out, int32_t *status, cudaStream_t stream)
+                                  int64_t M, float *out, int32_t *status, cudaStream_t stream, int part)
 {
-#define SA_CASE(l, m) if (L == l && M == m) return launch_tc<l, m, false>(rows, A, lda, nullptr, 0, B, ldb, out, status, stream);
+#define SA_CASE(l, m) if (L == l && M == m) return launch_tc<l, m, false>(rows, A, lda, nullptr, 0, B, ldb, out, status, stream, part);
     SA_CASE(64, 32) SA_CASE(64, 64) SA_CASE(128, 32) SA_CASE(128, 64) SA_CASE(256, 32) SA_CASE(256, 64)
 #undef SA_CASE
     return SA_E_UNSUPPORTED;
 }
 
 sa_status sa_launch_hadamard_gemm_tc(int64_t rows, const sa_dense &A, const sa_dense &H, const sa_dense &B, float *out, int32_t *status,
-                                     cudaStream_t stream)
+                                     cudaStream_t stream, int part)
 {
 #define SA_CASE(l, m) \
-    if (A.cols == l && B.cols == m) return launch_tc<l, m, true>(rows, A.ptr, A.ld, H.ptr, H.ld, B.ptr, B.ld, out, status, stream);
+    if (A.cols == l && B.cols == m) return launch_tc<l, m, true>(rows, A.ptr, A.ld, H.ptr, H.ld, B.ptr, B.ld, out, status, stream, part);
     SA_CASE(128, 32) SA_CASE(128, 64) SA_CASE(256, 32) SA_CASE(256, 64)
 #undef SA_CASE
     return SA_E_UNSUPPORTED;

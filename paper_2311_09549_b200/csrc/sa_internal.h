@@ -208,15 +208,16 @@ sa_status sa_launch_sddmm_spmm_gemm(const sa_tensor *t, const sa_dense *ops, flo
 size_t sa_ws_sddmm_spmm_gemm(const sa_tensor *t, const sa_dense *ops);
 bool sa_dense_gemm_ok(int64_t L, int64_t M);
 // out (rows x M) = A (rows x L) . B (L x M); `status` is the tensor's device status word (a wait that runs out
-// inside the tcgen05 kernel records SA_E_TIMEOUT there).  L >= 64 runs on tcgen05, L = 32 on mma.sync.
+// inside the tcgen05 kernel records SA_E_TIMEOUT there).  L >= 64 runs on tcgen05, L = 32 on mma.sync.  part (tcgen05
+// only): `out` is written as M / part tables of rows x part floats; 0: as one.
 sa_status sa_launch_dense_gemm(int64_t rows, const float *A, int64_t lda, const float *B, int64_t ldb, int64_t L,
-                               int64_t M, float *out, int32_t *status, cudaStream_t stream);
+                               int64_t M, float *out, int32_t *status, cudaStream_t stream, int part = 0);
 bool sa_dense_gemm_tc_ok(int64_t L, int64_t M);
 sa_status sa_launch_dense_gemm_tc(int64_t rows, const float *A, int64_t lda, const float *B, int64_t ldb, int64_t L,
-                                  int64_t M, float *out, int32_t *status, cudaStream_t stream);
+                                  int64_t M, float *out, int32_t *status, cudaStream_t stream, int part);
 // out (rows x M) = (A o H) (rows x L, element-wise product) . B (L x M) to fp32 accuracy, L in {128, 256}
 sa_status sa_launch_hadamard_gemm_tc(int64_t rows, const sa_dense &A, const sa_dense &H, const sa_dense &B, float *out, int32_t *status,
-                                     cudaStream_t stream);
+                                     cudaStream_t stream, int part);
 
 // Kernel 7 <SpTTM,SpTTM>: out = one row of M values per (i,j) fiber, in CSF order
 bool sa_ranks_ok_spttm_spttm(int64_t L, int64_t M);

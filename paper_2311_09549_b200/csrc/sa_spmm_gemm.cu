@@ -259,49 +259,80 @@ gemm_bf16x3_kernel(int64_t J, const float *__restrict__ C, int64_t ldc, const fl
     asm volatile("cp.async.wait_group 0;" ::: "memory");
 }
 
-// A = B . E (the CSR SpMM nest of Fig. 1b); lane owns MV = M/32 consecutive columns.
-template <int MV>
+// A = B . E (the CSR SpMM nest of Fig. 1b), W columns of E at a time: E is stored as M / W tables of J x W (the dense
+// stage writes it so) and the grid runs one table after the other.
+// What bounds it is the gather of one row of E per nonzero, out of HBM where E exceeds L2.  W/4 lanes own a row piece as
+// one float4 each; every such lane group takes one work item and walks its nonzeros eight at a time (records one step
+// ahead, eight gathers in flight); a group that meets a row's last nonzero stores the row.  1M x 1M, 25 M nonzeros,
+// M = 64 (E 256 MB): 783 us with one table, 709 us with two, 837 us with four (more instructions per byte
+// than the misses saved are worth); a warp per row with the columns across its lanes took 981 us.
+template <int W>
 __global__ void __launch_bounds__(256)
-spmm_kernel(const sa_item *__restrict__ items, int64_t n_items, const int32_t *__restrict__ pos,
-            const int32_t *__restrict__ crd, const float *__restrict__ vals, const float *__restrict__ E,
-            float *__restrict__ out, float *__restrict__ partial, const sa_limits lim)
+spmm_kernel(const sa_item *__restrict__ items, int64_t n_items, unsigned ctas_per_part, const int32_t *__restrict__ pos,
+            const int2 *__restrict__ nz, const float *__restrict__ E, int64_t J, int M, float *__restrict__ out,
+            float *__restrict__ partial, const sa_limits lim)
 {
-    constexpr int M = MV * 32;
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const int64_t idx = int64_t(blockIdx.x) * SA_WARPS_PER_CTA + warp;
-    if (idx >= n_items) return;
-    const sa_item it = items[idx];
-    for (int r = it.out_row; r < it.row_end; ++r) {
-        if (!SA_CHK(lim.status, uint32_t(r) < lim.out_rows && it.dest < lim.n_slots, 54, r)) continue;
-        const int a = it.dest >= 0 ? it.p0 : pos[r];
-        const int b = it.dest >= 0 ? it.p1 : pos[r + 1];
-        if (!SA_CHK(lim.status, a >= 0 && a <= b && b <= lim.nnz, 55, b)) continue;
-        float acc[MV];
+    constexpr int LPR = W / 4, U = 8;                       // lanes per row, nonzeros per step
+    static_assert(LPR >= U, "one record per lane and step");
+    const unsigned part = blockIdx.x / ctas_per_part, block = blockIdx.x - part * ctas_per_part;
+    const int l = threadIdx.x % LPR;
+    const int64_t idx = (int64_t(block) * 256 + threadIdx.x) / LPR;
+    E += int64_t(part) * J * W + 4 * l;
+    int r = 0, rend = 0, p0 = 0, end = 0, dest = -1;
+    if (idx < n_items) {
+        const int4 ia = __ldg(reinterpret_cast<const int4 *>(items + idx));          // out_row, row_end, -, -
+        const int4 ib = __ldg(reinterpret_cast<const int4 *>(items + idx) + 1);      // p0, p1, dest, -
+        if (SA_CHK(lim.status, ia.x >= 0 && ia.x <= ia.y && uint32_t(ia.y) <= lim.out_rows && ib.x >= 0 && ib.x <= ib.y && ib.y <= lim.nnz &&
+                                   ib.z < lim.n_slots, 54, idx)) {
+            r = ia.x; rend = ia.y; p0 = ib.x; end = ib.y; dest = ib.z;
+        }
+    }
+    auto row_end = [&](int row) {
+        if (dest >= 0 || row >= rend) return end;
+        int e = __ldg(pos + row + 1);
+        if (!SA_CHK(lim.status, e >= 0 && e <= end, 55, e)) e = end;
+        return e;
+    };
+    float *dst0 = (dest >= 0 ? partial + int64_t(dest) * M : out) + part * W + 4 * l;
+    auto store_row = [&](float4 v) { sa_st_cs4(dst0 + (dest >= 0 ? 0 : int64_t(r) * M), v); };
+    int b = row_end(r), bn = row_end(r + 1);                // where rows r and r + 1 end
+    auto next_row = [&]() { ++r; b = bn; bn = row_end(r + 1); };
+    const float4 zero = make_float4(0.f, 0.f, 0.f, 0.f);
+    while (r < rend && b == p0) { store_row(zero); next_row(); }      // empty rows
+    const int len = end - p0, steps = __reduce_max_sync(SA_FULL_MASK, len);
+    auto fetch = [&](int c) {                                // nonzero c + lane of the group (eight lanes hold one each)
+        int2 w = make_int2(0, 0);
+        const int o = c + (l & (U - 1));
+        if (o < len) w = __ldcs(nz + p0 + o);
+        if (!SA_CHK(lim.status, uint32_t(w.x) < lim.gather_rows, 56, w.x)) w.x = 0;
+        return w;
+    };
+    float4 acc = zero;
+    int2 rec = fetch(0);
+    for (int c = 0; c < steps; c += U) {
+        float4 e[U];
+        float vs[U];
 #pragma unroll
-        for (int q = 0; q < MV; ++q) acc[q] = 0.f;
-        for (int base = a; base < b; base += 32) {
-            const int n = min(32, b - base);
-            int jj = 0;
-            float vv = 0.f;
-            if (lane < n) { jj = crd[base + lane]; vv = vals[base + lane]; }
-            if (!SA_CHK(lim.status, uint32_t(jj) < lim.gather_rows, 56, jj)) jj = 0;
-#pragma unroll 8
-            for (int s = 0; s < n; ++s) {
-                const int j = __shfl_sync(SA_FULL_MASK, jj, s);
-                const float v = __shfl_sync(SA_FULL_MASK, vv, s);
-                const float *erow = E + int64_t(j) * M + lane * MV;
-                if (MV == 2) {
-                    const float2 e = sa_ldg2(erow);
-                    acc[0] = fmaf(v, e.x, acc[0]);
-                    acc[1 % MV] = fmaf(v, e.y, acc[1 % MV]);
-                } else {
-                    acc[0] = fmaf(v, __ldg(erow), acc[0]);
-                }
+        for (int u = 0; u < U; ++u) {
+            const int k = __shfl_sync(SA_FULL_MASK, rec.x, u, LPR);
+            vs[u] = __int_as_float(__shfl_sync(SA_FULL_MASK, rec.y, u, LPR));
+            e[u] = zero;
+            if (c + u < len) e[u] = sa_ldg4(E + int64_t(k) * W);
+        }
+        rec = fetch(c + U);
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+            acc.x = fmaf(vs[u], e[u].x, acc.x);
+            acc.y = fmaf(vs[u], e[u].y, acc.y);
+            acc.z = fmaf(vs[u], e[u].z, acc.z);
+            acc.w = fmaf(vs[u], e[u].w, acc.w);
+            if (p0 + c + u + 1 == b && r < rend) {              // the last nonzero of row r
+                store_row(acc);
+                acc = zero;
+                next_row();
+                while (r < rend && b == p0 + c + u + 1) { store_row(zero); next_row(); }
             }
         }
-        float *dst = it.dest >= 0 ? partial + int64_t(it.dest) * M : out + int64_t(r) * M;
-#pragma unroll
-        for (int q = 0; q < MV; ++q) dst[lane * MV + q] = acc[q];
     }
 }
 
@@ -425,17 +456,28 @@ int resident_ctas(const void *kernel, size_t smem)
     return sms * per_sm;
 }
 
-// out = B . E with E (J x M) at the start of the workspace, the partial rows of long-row pieces behind it.
+// Columns per table of E (see spmm_kernel).  Two tables read B twice, and pay where half of E finds a good part of itself in
+// L2 while all of it does not.  Whole chain, L = 128, M = 64, 20 nonzeros per row, J columns, 2 J / 1 table, us: 250 K
+// 103 / 98; 500 K (128 MB) 204 / 215; 1 M 451 / 467; 2 M 1050 / 1000.
+int spmm_part(int64_t J, int64_t M)
+{
+    const int64_t bytes = J * M * int64_t(sizeof(float));
+    return M == 64 && bytes > (int64_t(96) << 20) && bytes <= (int64_t(320) << 20) ? 32 : int(M);
+}
+
+// out = B . E with E (J x M, in tables of spmm_part columns) at the start of the workspace, the partial rows of long-row pieces behind it.
 template <int M>
 sa_status run_spmm(const sa_tensor *t, float *E, float *out, cudaStream_t stream, int *launches)
 {
     const sa_worklist &wl = t->wl_aux;
     const int64_t n_items = int64_t(wl.items.size()), J = t->dims[1];
     float *partial = reinterpret_cast<float *>(reinterpret_cast<char *>(E) + sa_align256(size_t(J) * M * sizeof(float)));
-    const int64_t ctas = (n_items + SA_WARPS_PER_CTA - 1) / SA_WARPS_PER_CTA;
-    if (ctas > 0) {
-        spmm_kernel<M / 32><<<(unsigned)ctas, 256, 0, stream>>>(wl.d_items, n_items, t->d_pos[1], t->d_crd[1], t->d_vals, E,
-                                                               out, partial, sa_make_limits(t, J, t->dims[0], wl.n_slots));
+    if (n_items > 0) {
+        const int W = spmm_part(J, M);
+        const unsigned ctas = unsigned((n_items * (W / 4) + 255) / 256);
+        auto kern = W == 32 ? spmm_kernel<32> : spmm_kernel<64>;
+        kern<<<ctas * unsigned(M / W), 256, 0, stream>>>(wl.d_items, n_items, ctas, t->d_pos[1], t->d_nzpack, E, J, M, out, partial,
+                                                         sa_make_limits(t, J, t->dims[0], wl.n_slots));
         if (cudaGetLastError() != cudaSuccess) return SA_E_CUDA;
         *launches += 1;
     }
@@ -473,7 +515,8 @@ sa_status run(const sa_tensor *t, const sa_dense *ops, float *out, void *ws, boo
         return SA_OK;
     }
     float *E = static_cast<float *>(ws);
-    const sa_status gs = sa_launch_dense_gemm(t->dims[1], ops[0].ptr, ops[0].ld, ops[1].ptr, ops[1].ld, L, M, E, t->d_status, stream);
+    const sa_status gs = sa_launch_dense_gemm(t->dims[1], ops[0].ptr, ops[0].ld, ops[1].ptr, ops[1].ld, L, M, E, t->d_status, stream,
+                                              spmm_part(t->dims[1], M));
     if (gs != SA_OK) return gs;
     *launches += 1;
     return run_spmm<M>(t, E, out, stream, launches);
@@ -481,7 +524,7 @@ sa_status run(const sa_tensor *t, const sa_dense *ops, float *out, void *ws, boo
 
 // Kernel 3 <SpMMH,GEMM>: ops = {C, D, E}.  Left: the gathered row is C(j,:) * D(j,:), the resident matrix is E.  Right:
 // G = (C o D).E once per column j (J x M temporary), then A = B.G: one gathered row of M floats per nonzero instead of
-// two of L, for one pass over C and D.  At 1M x 1M, 25 M nonzeros, L = 256, M = 64: 9.15 ms left, 1.45 ms right.
+// two of L, for one pass over C and D.  At 1M x 1M, 25 M nonzeros, L = 256, M = 64: 9.3 ms left, 1.23 ms right.
 template <int L, int M>
 sa_status run_hadamard(const sa_tensor *t, const sa_dense *ops, float *out, void *ws, bool right, cudaStream_t stream, int *launches)
 {
@@ -491,7 +534,7 @@ sa_status run_hadamard(const sa_tensor *t, const sa_dense *ops, float *out, void
     *launches = 0;
     if (right) {
         float *G = static_cast<float *>(ws);
-        const sa_status gs = sa_launch_hadamard_gemm_tc(t->dims[1], ops[0], ops[1], ops[2], G, t->d_status, stream);
+        const sa_status gs = sa_launch_hadamard_gemm_tc(t->dims[1], ops[0], ops[1], ops[2], G, t->d_status, stream, spmm_part(t->dims[1], M));
         if (gs != SA_OK) return gs;
         *launches += 1;
         return run_spmm<M>(t, G, out, stream, launches);
@@ -582,9 +625,10 @@ static sa_status dense_gemm(int64_t rows, const float *A, int64_t lda, const flo
 bool sa_dense_gemm_ok(int64_t L, int64_t M) { return (L == 32 || L == 64 || L == 128 || L == 256) && (M == 32 || M == 64); }
 
 sa_status sa_launch_dense_gemm(int64_t rows, const float *A, int64_t lda, const float *B, int64_t ldb, int64_t L,
-                               int64_t M, float *out, int32_t *status, cudaStream_t stream)
+                               int64_t M, float *out, int32_t *status, cudaStream_t stream, int part)
 {
-    if (sa_dense_gemm_tc_ok(L, M)) return sa_launch_dense_gemm_tc(rows, A, lda, B, ldb, L, M, out, status, stream);
+    if (sa_dense_gemm_tc_ok(L, M)) return sa_launch_dense_gemm_tc(rows, A, lda, B, ldb, L, M, out, status, stream, part ? part : int(M));
+    if (part && part != M) return SA_E_UNSUPPORTED;
 #define SA_CASE(l, m) if (L == l && M == m) return dense_gemm<l, m>(rows, A, lda, B, ldb, out, stream);
     SA_CASE(32, 32) SA_CASE(32, 64)
 #undef SA_CASE

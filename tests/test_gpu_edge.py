@@ -459,3 +459,16 @@ def test_sddmm_spmm_rows_around_piece_and_column_block_limits(sa, K, L, deg):
     w = _wl("sddmm_spmm", "csr", (11, J), coords, vals,
             [configs.dense_normal(deg, 0, 11, K), configs.dense_normal(deg, 1, J, K), configs.dense_normal(deg, 2, J, L)], (11, L))
     _check(sa, w)
+
+
+@pytest.mark.parametrize("M,J", [(32, 900), (64, 900), (64, 393_217)])
+@pytest.mark.parametrize("deg", [1, 8, 31, 33, 65, 257])
+def test_spmm_gemm_right_order_rows_around_step_and_piece_limits(sa, M, J, deg):
+    """Rows around the eight-nonzero step and the length at which they are cut into pieces, empty rows at both ends of an
+    item and inside it, and the first J for which E is kept as two tables (96 MB at M = 64)."""
+    rs = np.random.RandomState(deg)
+    rows = {1: deg, 2: 1, 5: deg, 40: 8, 41: deg + 1, 77: 70}
+    coords = np.concatenate([np.stack([np.full(n, r), rs.choice(J, n, replace=False)], axis=1) for r, n in rows.items()]).astype(np.int32)
+    vals = rs.uniform(-1, 1, len(coords)).astype(np.float32)
+    w = _wl("spmm_gemm", "csr", (100, J), coords, vals, [configs.dense_normal(deg, 0, J, 128), configs.dense_normal(deg, 1, 128, M)], (100, M))
+    _check(sa, w, sched=sa.SA_SCHED_ASSOC_RIGHT)
