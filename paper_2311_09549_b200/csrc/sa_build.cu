@@ -206,6 +206,15 @@ void append_empty_slices(sa_tensor *t, sa_worklist &wl)
     }
 }
 
+// Nonzeros per unit of the order-3 kernel: 2048, less where `nnz` nonzeros would not give a full machine enough of them
+// (`slots`: at that many units the size stays 2048; a warp needs some 40 us for 2048 nonzeros, whatever else runs).
+//   Order 3, slots = 4736 (two per warp slot, 148 SMs x 16): 300 K nonzeros, ranks 16 and 32, mean fibers 1.5 to 18: 41 to
+//     97 us with units of 2048, 13 to 25 us with 256; 6 M nonzeros 78 to 204 us with 2048, 82 to 195 with 1216; a third of
+//     that size costs more partial tiles than the balance gives (87 to 217 us).
+//   Order 4, slots = 2048 of all nonzeros (the list holds the large subtrees only, whose tiles are summed in 1 KB pieces):
+//     4.2 M nonzeros 439 us with 2048, 484 us with 256.
+int64_t unit_size(int64_t nnz, int64_t slots) { return std::min<int64_t>(2048, std::max<int64_t>(256, nnz / slots / 64 * 64)); }
+
 // Order-3 CSF.  An item ("unit") is a piece [p0, p1) of one slice with the fibers [f0, f1) it touches (a
 // fiber may be cut between two units, each adds its part).  Slices above SMALL_MAX nonzeros are cut into
 // chunks; the SA_TTM3_WARPS warps of a thread block take equal pieces of a chunk and reduce their tiles on chip.
@@ -217,9 +226,10 @@ void append_empty_slices(sa_tensor *t, sa_worklist &wl)
 // the (i,j,k) fibers; output row = index of the (i,j) fiber.)
 template <typename RowOf, typename Skip>
 void build_ttm3_lists(sa_worklist &wl, int64_t n_slices, RowOf row_of, Skip skip, const std::vector<int64_t> &pos1,
-                      const std::vector<int64_t> &pos2)
+                      const std::vector<int64_t> &pos2, int64_t unit)
 {
-    constexpr int64_t SMALL_MAX = 2048, MIN_CHUNK = 8192, MAX_PARTS = 192, MAX_UNITS = 16;
+    const int64_t SMALL_MAX = unit, MIN_CHUNK = 4 * unit;
+    constexpr int64_t MAX_PARTS = 192, MAX_UNITS = 16;
     std::vector<sa_item> small;
     std::vector<group_rec> groups;
     for (int64_t s = 0; s < n_slices; ++s) {
@@ -279,9 +289,9 @@ void build_ttm3_lists(sa_worklist &wl, int64_t n_slices, RowOf row_of, Skip skip
     const int64_t max_units = std::min<int64_t>(MAX_UNITS, std::max<int64_t>(1, int64_t(small.size()) / 4096));
     for (size_t x = 0; x < small.size();) {
         wl.task_start.push_back(int32_t(wl.items.size()));
-        int64_t total = 0, cnt = 0;
-        while (x < small.size() && cnt < max_units && (cnt == 0 || total + (small[x].p1 - small[x].p0) <= SMALL_MAX)) {
-            total += small[x].p1 - small[x].p0;
+        int64_t sum = 0, cnt = 0;
+        while (x < small.size() && cnt < max_units && (cnt == 0 || sum + (small[x].p1 - small[x].p0) <= SMALL_MAX)) {
+            sum += small[x].p1 - small[x].p0;
             wl.items.push_back(small[x]);
             ++x; ++cnt;
         }
@@ -304,7 +314,7 @@ void build_ttm3_lists(sa_worklist &wl, int64_t n_slices, RowOf row_of, Skip skip
 void build_ttm3(sa_tensor *t, sa_worklist &wl)
 {
     build_ttm3_lists(wl, t->count[0], [&](int64_t s) { return t->crd[0][size_t(s)]; }, [](int64_t) { return false; }, t->pos[1],
-                     t->pos[2]);
+                     t->pos[2], unit_size(t->nnz, 4736));
     append_empty_slices(t, wl);
 }
 
@@ -325,7 +335,7 @@ static bool subtree_is_small(const sa_tensor *t, int64_t f2)
 void build_ttm4_fissioned(sa_tensor *t, sa_worklist &wl, sa_worklist &wl2)
 {
     build_ttm3_lists(wl, t->count[1], [](int64_t f) { return int32_t(f); }, [&](int64_t f) { return subtree_is_small(t, f); },
-                     t->pos[2], t->pos[3]);
+                     t->pos[2], t->pos[3], unit_size(t->nnz, 2048));
     constexpr int64_t CHUNK_F = 512;
     const auto &pos1 = t->pos[1];
     std::vector<sa_item> items;
@@ -425,7 +435,7 @@ void build_ttm4(sa_tensor *t, sa_worklist &wl, sa_worklist &wl_items, sa_worklis
         if (subtree_is_large(t, r)) large_ord[size_t(r)] = n_large++;
     t->f4_n_large = n_large;
     build_ttm3_lists(wl, F2, [&](int64_t r) { return large_ord[size_t(r)]; }, [&](int64_t r) { return large_ord[size_t(r)] < 0; },
-                     pos2, pos3);
+                     pos2, pos3, unit_size(t->nnz, 2048));
     wl.nnz = 0;
     for (const sa_item &it : wl.items) wl.nnz += it.p1 - it.p0;
 
@@ -645,8 +655,9 @@ void sa_build_worklists(sa_tensor *t)
 {
     if (t->fmt == SA_FMT_CSF && t->order == 3) {
         build_ttm3(t, t->wl_main);
-        // kernel 7 walks the tensor as a sparse matrix whose rows are the (i,j) fibers
-        build_rows(t->pos[2], t->count[1], t->wl_aux, 1024, 4096, 4096, 2048, true);
+        // kernel 7 walks the tensor as a sparse matrix whose rows are the (i,j) fibers: 1024 nonzeros per warp, fewer where
+        // that would not give every warp slot of a full machine four items
+        build_rows(t->pos[2], t->count[1], t->wl_aux, std::min<int64_t>(1024, std::max<int64_t>(128, t->nnz / (4 * 148 * 32) / 32 * 32)), 4096, 4096, 2048, true);
     }
     if (t->fmt == SA_FMT_CSF && t->order == 4) {
         build_ttm4(t, t->wl_main, t->wl_sub, t->wl_aux);
@@ -664,5 +675,6 @@ void sa_build_worklists(sa_tensor *t)
     for (sa_worklist *wl : {&t->wl_main, &t->wl_aux, &t->wl_sub, &t->wl4_main, &t->wl4_aux, &t->wl4_sub}) {
         std::stable_sort(wl->fix.begin(), wl->fix.end(), [](const sa_fix &x, const sa_fix &y) { return x.count > y.count; });
         wl->n_big_fix = std::find_if(wl->fix.begin(), wl->fix.end(), [](const sa_fix &x) { return x.count <= SA_BIG_FIX; }) - wl->fix.begin();
+        wl->n_sum_fix = std::find_if(wl->fix.begin(), wl->fix.end(), [](const sa_fix &x) { return x.count == 0; }) - wl->fix.begin();
     }
 }

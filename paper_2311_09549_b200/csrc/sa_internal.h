@@ -71,6 +71,7 @@ struct sa_worklist {
     int64_t n_group_ctas = 0;     // leading CTAs whose 8 warps reduce into one tile
     int64_t n_slots = 0;          // partial tiles in the workspace
     int64_t n_big_fix = 0;        // leading fix-up entries with more than SA_BIG_FIX partial tiles (longest first)
+    int64_t n_sum_fix = 0;        // leading fix-up entries with partial tiles at all
     int64_t nnz = 0;              // nonzeros the list covers (set for the order-4 lists of pass 1)
     sa_item *d_items = nullptr;
     sa_fix *d_fix = nullptr;

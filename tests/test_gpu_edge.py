@@ -472,3 +472,19 @@ def test_spmm_gemm_right_order_rows_around_step_and_piece_limits(sa, M, J, deg):
     vals = rs.uniform(-1, 1, len(coords)).astype(np.float32)
     w = _wl("spmm_gemm", "csr", (100, J), coords, vals, [configs.dense_normal(deg, 0, J, 128), configs.dense_normal(deg, 1, 128, M)], (100, M))
     _check(sa, w, sched=sa.SA_SCHED_ASSOC_RIGHT)
+
+
+@pytest.mark.parametrize("n", [255, 256, 257, 1023, 1024, 1025, 4097])
+@pytest.mark.parametrize("L,M", [(16, 16), (32, 32)])
+def test_ttm3_small_tensor_slices_around_the_unit_and_chunk_sizes(sa, n, L, M):
+    """A tensor small enough for units of 256 nonzeros (chunks of 1024): slices of n and of one nonzero, a fix-up entry with
+    partial tiles of several chunks."""
+    rs = np.random.RandomState(n)
+    J, K = 90, 60
+    lin = np.sort(rs.choice(J * K, n, replace=False))
+    big = np.stack([np.full(n, 4), lin // K, lin % K], axis=1)
+    ones = np.stack([np.arange(3), rs.randint(0, J, 3), rs.randint(0, K, 3)], axis=1)
+    coords = np.concatenate([big, ones]).astype(np.int32)
+    vals = rs.uniform(-1, 1, len(coords)).astype(np.float32)
+    w = _wl("spttm_ttm3", "csf", (6, J, K), coords, vals, [configs.dense_uniform(n, 0, J, L), configs.dense_uniform(n, 1, K, M)], (6, L, M))
+    _check(sa, w)
