@@ -488,3 +488,17 @@ def test_ttm3_small_tensor_slices_around_the_unit_and_chunk_sizes(sa, n, L, M):
     vals = rs.uniform(-1, 1, len(coords)).astype(np.float32)
     w = _wl("spttm_ttm3", "csf", (6, J, K), coords, vals, [configs.dense_uniform(n, 0, J, L), configs.dense_uniform(n, 1, K, M)], (6, L, M))
     _check(sa, w)
+
+
+@pytest.mark.parametrize("I", [1, 7, 9, 64, 65, 1025, 32_769])
+@pytest.mark.parametrize("L,M,N", [(16, 16, 16), (32, 16, 32), (16, 32, 32)])
+def test_ttmc3_slices_around_the_step_and_chunk_sizes(sa, I, L, M, N):
+    """Numbers of slices around the eight-row step and the chunk of slices of the reduction over i (64 slices, 65 from 32769 on)
+    and numbers of chunks around its 16 phases, with empty slices."""
+    rs = np.random.RandomState(I)
+    J, K = 30, 20
+    coords = np.stack([rs.randint(0, I, 900), rs.randint(0, J, 900), rs.randint(0, K, 900)], axis=1)
+    coords = np.unique(coords, axis=0).astype(np.int32)
+    vals = rs.uniform(-1, 1, len(coords)).astype(np.float32)
+    ops = [configs.dense_uniform(I, 0, I, L), configs.dense_uniform(I, 1, J, M), configs.dense_uniform(I, 2, K, N)]
+    _check(sa, _wl("ttmc3", "csf", (I, J, K), coords, vals, ops, (L, M, N)), sched=sa.SA_SCHED_FISSIONED)
