@@ -7,6 +7,7 @@ built (``python paper_2311_09549_b200/build.py``); there is no CPU path.
 """
 import ctypes
 import os
+import struct
 
 import numpy as np
 
@@ -72,6 +73,15 @@ _lib.sa_run_ttm3_static_scratch.argtypes = [_vp, ctypes.POINTER(SaDense), _int, 
 for _n in EXPORTED_SYMBOLS:
     if _n not in ("sa_destroy", "sa_status_string"):
         getattr(_lib, _n).restype = _int
+
+
+# sa_run for SparseTensor.run: the operand descriptors as packed bytes (a ctypes array of structures costs more to fill than
+# the call itself)
+_run_packed = _lib["sa_run"]
+_run_packed.argtypes = [_vp, _int, _int, ctypes.c_char_p, _int, _vp, _vp, ctypes.c_size_t, _vp]
+_run_packed.restype = _int
+_PACK_OPS = {n: struct.Struct("Pqqq" * n).pack for n in range(1, 5)}
+assert struct.calcsize("Pqqq") == ctypes.sizeof(SaDense)
 
 
 class SaError(RuntimeError):
@@ -245,6 +255,7 @@ class SparseTensor:
         self.handle = sa_tensor_create(self.order, self.dims, len(vals), coords, vals, fmt, device,
                                        self._allocator.struct if self._allocator else None)
         self._ws = None
+        self._fibers = int(self.info()[1][1])      # rows of a sparse output; a handle is immutable
 
     def close(self):
         if self.handle:
@@ -264,18 +275,39 @@ class SparseTensor:
         """operands: torch float32 CUDA matrices (row-major).  Returns (out, workspace)."""
         import torch
         expr = _EXPR_OF.get(expr, expr)
-        ops = [(t.data_ptr(), t.shape[0], t.shape[1], t.stride(0)) for t in operands]
-        need = sa_workspace_size(self.handle, expr, sched, ops)
-        dev = torch.device("cuda", self.device)
-        if workspace is None:
-            if self._ws is None or self._ws.numel() < need:
-                self._ws = torch.empty(max(need, 256), dtype=torch.uint8, device=dev)
-            workspace = self._ws
+        desc = []
+        for t in operands:
+            shape = t.shape
+            desc += (t.data_ptr(), shape[0], shape[1], t.stride(0))
+        n = len(operands)
+        if n not in _PACK_OPS:
+            self._size(expr, sched, desc)           # raises: no expression takes that many operands
+        own = workspace is None
+        if own:
+            workspace = self._ws if self._ws is not None else self._grow(expr, sched, desc)
         if out is None:
-            out = torch.empty(self.out_shape(expr, operands), dtype=torch.float32, device=dev)
-        s = torch.cuda.current_stream(dev) if stream is None else stream
-        sa_run(self.handle, expr, sched, ops, out.data_ptr(), workspace.data_ptr(), workspace.numel(), s.cuda_stream)
+            try:
+                shape = self.out_shape(expr, operands)
+            except IndexError:
+                self._size(expr, sched, desc)       # raises: too few operands for the expression
+                raise
+            out = torch.empty(shape, dtype=torch.float32, device=workspace.device)
+        s = torch.cuda.current_stream(self.device) if stream is None else stream
+        packed = _PACK_OPS[n](*desc)
+        st = _run_packed(self.handle, int(expr), int(sched), packed, n, out.data_ptr(), workspace.data_ptr(), workspace.numel(), s.cuda_stream)
+        if own and st == SA_E_WORKSPACE:            # nothing was enqueued: this call needs more than the ones before it
+            workspace = self._grow(expr, sched, desc)
+            st = _run_packed(self.handle, int(expr), int(sched), packed, n, out.data_ptr(), workspace.data_ptr(), workspace.numel(), s.cuda_stream)
+        _check(st, "sa_run")
         return out, workspace
+
+    def _size(self, expr, sched, desc):
+        return sa_workspace_size(self.handle, expr, sched, [tuple(desc[i:i + 4]) for i in range(0, len(desc), 4)])
+
+    def _grow(self, expr, sched, desc):
+        import torch
+        self._ws = torch.empty(max(self._size(expr, sched, desc), 256), dtype=torch.uint8, device=torch.device("cuda", self.device))
+        return self._ws
 
     def out_shape(self, expr, operands):
         expr = _EXPR_OF.get(expr, expr)
@@ -293,5 +325,5 @@ class SparseTensor:
         if expr in (SA_EXPR_SPMMH_GEMM, SA_EXPR_MTTKRP_GEMM):
             return (self.dims[0], cols[2])
         if expr == SA_EXPR_SPTTM_SPTTM:
-            return (int(self.info()[1][1]), cols[1])      # one row per (i,j) fiber, in CSF order
+            return (self._fibers, cols[1])                # one row per (i,j) fiber, in CSF order
         return (self.dims[0], cols[1])

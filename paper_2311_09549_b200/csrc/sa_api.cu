@@ -62,12 +62,14 @@ sa_status upload_worklist(sa_tensor *t, sa_worklist &wl)
 }
 
 struct device_guard {
-    int prev = -1;
+    int prev = -1;              // the device to go back to, -1: it is current already
     bool ok = false;
     explicit device_guard(int dev)
     {
-        if (cudaGetDevice(&prev) != cudaSuccess) return;
-        ok = (prev == dev) || cudaSetDevice(dev) == cudaSuccess;
+        int cur = -1;
+        if (cudaGetDevice(&cur) != cudaSuccess) return;
+        if (cur != dev) prev = cur;
+        ok = cur == dev || cudaSetDevice(dev) == cudaSuccess;
     }
     ~device_guard() { if (prev >= 0) cudaSetDevice(prev); }
 };

@@ -447,12 +447,17 @@ fiber_spmm_kernel(const sa_item *__restrict__ items, int64_t n_items, const int3
     }
 }
 
-int resident_ctas(const void *kernel, size_t smem)
+// Blocks of 256 threads that the device holds at once; asked once per kernel and device (`known`: the caller's array).
+struct resident_cache { std::atomic<int> known[SA_MAX_DEVICE_FLAGS]; };
+int resident_ctas(const void *kernel, size_t smem, resident_cache &cache)
 {
     int dev = 0, sms = 148, per_sm = 1;
     cudaGetDevice(&dev);
+    const bool keep = dev >= 0 && dev < SA_MAX_DEVICE_FLAGS;
+    if (keep && cache.known[dev].load(std::memory_order_relaxed) > 0) return cache.known[dev].load(std::memory_order_relaxed);
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel, 256, smem) != cudaSuccess || per_sm < 1) per_sm = 1;
+    if (keep) cache.known[dev].store(sms * per_sm, std::memory_order_relaxed);
     return sms * per_sm;
 }
 
@@ -498,9 +503,11 @@ sa_status run(const sa_tensor *t, const sa_dense *ops, float *out, void *ws, boo
     if (!right) {
         float *partial = static_cast<float *>(ws);
         auto kern = spmm_gemm_left_kernel<L, M, false>;
-        if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem)) != cudaSuccess) return SA_E_CUDA;
+        static bool attr[SA_MAX_DEVICE_FLAGS];
+        static resident_cache resident;
+        if (!sa_set_smem_once(kern, int(smem), attr)) return SA_E_CUDA;
         const int64_t want = (n_items + SA_WARPS_PER_CTA - 1) / SA_WARPS_PER_CTA;
-        const int64_t ctas = std::min<int64_t>(want, resident_ctas(reinterpret_cast<const void *>(kern), smem));
+        const int64_t ctas = std::min<int64_t>(want, resident_ctas(reinterpret_cast<const void *>(kern), smem, resident));
         if (ctas > 0) {
             kern<<<(unsigned)ctas, 256, smem, stream>>>(wl.d_items, n_items, t->d_pos[1], t->d_crd[1], t->d_vals, ops[0].ptr,
                                                        ops[0].ld, ops[0].ptr, ops[0].ld, ops[1].ptr, ops[1].ld, out, partial,
@@ -541,9 +548,11 @@ sa_status run_hadamard(const sa_tensor *t, const sa_dense *ops, float *out, void
     }
     float *partial = static_cast<float *>(ws);
     auto kern = spmm_gemm_left_kernel<L, M, true>;
-    if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem)) != cudaSuccess) return SA_E_CUDA;
+    static bool attr[SA_MAX_DEVICE_FLAGS];
+    static resident_cache resident;
+    if (!sa_set_smem_once(kern, int(smem), attr)) return SA_E_CUDA;
     const int64_t want = (n_items + SA_WARPS_PER_CTA - 1) / SA_WARPS_PER_CTA;
-    const int64_t ctas = std::min<int64_t>(want, resident_ctas(reinterpret_cast<const void *>(kern), smem));
+    const int64_t ctas = std::min<int64_t>(want, resident_ctas(reinterpret_cast<const void *>(kern), smem, resident));
     if (ctas > 0) {
         kern<<<(unsigned)ctas, 256, smem, stream>>>(wl.d_items, n_items, t->d_pos[1], t->d_crd[1], t->d_vals, ops[0].ptr,
                                                    ops[0].ld, ops[1].ptr, ops[1].ld, ops[2].ptr, ops[2].ld, out, partial,
@@ -616,8 +625,10 @@ static sa_status dense_gemm(int64_t rows, const float *A, int64_t lda, const flo
 {
     using GC = gemm_bf16_cfg<L, M>;
     auto gk = gemm_bf16x3_kernel<L, M>;
-    if (cudaFuncSetAttribute(gk, cudaFuncAttributeMaxDynamicSharedMemorySize, int(GC::SMEM)) != cudaSuccess) return SA_E_CUDA;
-    const int64_t ctas = std::min<int64_t>((rows + GC::BM - 1) / GC::BM, resident_ctas(reinterpret_cast<const void *>(gk), GC::SMEM));
+    static bool attr[SA_MAX_DEVICE_FLAGS];
+    static resident_cache resident;
+    if (!sa_set_smem_once(gk, int(GC::SMEM), attr)) return SA_E_CUDA;
+    const int64_t ctas = std::min<int64_t>((rows + GC::BM - 1) / GC::BM, resident_ctas(reinterpret_cast<const void *>(gk), GC::SMEM, resident));
     if (ctas > 0) gk<<<(unsigned)ctas, 256, GC::SMEM, stream>>>(rows, A, lda, B, ldb, out);
     return cudaGetLastError() == cudaSuccess ? SA_OK : SA_E_CUDA;
 }
