@@ -149,20 +149,40 @@ __device__ __forceinline__ void ttm3_flush(float (&acc)[cfg<L, M>::MT][cfg<L, M>
     }
 }
 
-// MTTKRP consumer (kernel 8): hacc(m) += sum over the parked rows row0 .. row0 + n - 1 of T(row, m) * C(j_row, m).
-// M = 32: lane = m.  M = 16: lane & 15 = m, the two half-warps take alternate rows (summed at the unit end).
+// MTTKRP consumer (kernel 8): sum over the parked rows row0 .. row0 + n - 1 of T(row, m) * C(j_row, m).  M/4 lanes per row,
+// four columns 4 (lane % (M/4)) .. + 3 per lane, so four (M = 32) or eight (M = 16) rows per step; had_total adds the lanes
+// of equal columns when the unit ends.
 template <int M>
-__device__ __forceinline__ void had_flush(float &hacc, const float *__restrict__ ring, int row0, int n,
+__device__ __forceinline__ void had_flush(float (&hacc)[4], const float *__restrict__ ring, int row0, int n,
                                           const float *__restrict__ C, int lane)
 {
-    constexpr int RS = M + 8;
-    const int m = lane & (M - 1);
+    constexpr int RS = M + 8, LANES = M / 4;
+    const int m = 4 * (lane % LANES);
 #pragma unroll
-    for (int x = 0; x < 8; ++x) {
-        const bool mine = x < n && (M == 32 || (x & 1) == (lane >> 4));
-        const float *r = ring + (row0 + x) * RS;
-        if (mine) hacc = fmaf(r[m], __ldg(C + __float_as_uint(r[M]) + m), hacc);
+    for (int x0 = 0; x0 < 8; x0 += 32 / LANES) {
+        const int x = x0 + lane / LANES;
+        if (x < n) {
+            const float *r = ring + (row0 + x) * RS;
+            const float4 c = sa_ldg4(C + __float_as_uint(r[M]) + m);
+            const float4 v = *reinterpret_cast<const float4 *>(r + m);
+            hacc[0] = fmaf(v.x, c.x, hacc[0]);
+            hacc[1] = fmaf(v.y, c.y, hacc[1]);
+            hacc[2] = fmaf(v.z, c.z, hacc[2]);
+            hacc[3] = fmaf(v.w, c.w, hacc[3]);
+        }
     }
+}
+template <int M>
+__device__ __forceinline__ float4 had_total(const float (&hacc)[4])
+{
+    float h[4];
+#pragma unroll
+    for (int x = 0; x < 4; ++x) {
+        h[x] = hacc[x];
+#pragma unroll
+        for (int d = M / 4; d < 32; d *= 2) h[x] += __shfl_xor_sync(SA_FULL_MASK, h[x], d);
+    }
+    return make_float4(h[0], h[1], h[2], h[3]);
 }
 
 // Store a slice tile held as MMA accumulator fragments (streaming stores: the output is written once).  The
@@ -260,7 +280,7 @@ __device__ __forceinline__ void ttm3_warp_task(const sa_unit3 *__restrict__ unit
                                                const float *__restrict__ vals, const uint32_t *__restrict__ endbits,
                                                const float *__restrict__ C, uint32_t ldc, const float *__restrict__ D,
                                                uint32_t ldd, unsigned char *__restrict__ wsm,
-                                               float (&acc)[cfg<L, M>::MT][cfg<L, M>::NT][4], float &hacc, const bool keep,
+                                               float (&acc)[cfg<L, M>::MT][cfg<L, M>::NT][4], float (&hacc)[4], const bool keep,
                                                float *__restrict__ out, const dbg_limits &lim, const ttmc_sink *sink = nullptr)
 {
     using K = cfg<L, M>;
@@ -456,9 +476,10 @@ __device__ __forceinline__ void ttm3_warp_task(const sa_unit3 *__restrict__ unit
         rbase = npend = 0;
         if (!keep) {
             if (HAD) {
-                if (M == 16) hacc += __shfl_xor_sync(SA_FULL_MASK, hacc, 16);
-                if (lane < M && SA_CHK(lim.status, uint32_t(crow) < lim.n_slices_dim, 8, crow)) sa_st_cs(out + int64_t(crow) * M + lane, hacc);
-                hacc = 0.f;
+                const float4 h = had_total<M>(hacc);
+                if (4 * lane < M && SA_CHK(lim.status, uint32_t(crow) < lim.n_slices_dim, 8, crow)) sa_st_cs4(out + int64_t(crow) * M + 4 * lane, h);
+#pragma unroll
+                for (int x = 0; x < 4; ++x) hacc[x] = 0.f;
             } else if (TTMC) {
                 if (SA_CHK(lim.status, uint32_t(crow) < lim.n_slices_dim, 8, crow)) ttmc_accumulate<L, M>(acc, *sink, crow, lane);
                 zero_tile<L, M>(acc);
@@ -500,7 +521,7 @@ ttm3_kernel(const sa_unit3 *__restrict__ units, const int32_t *__restrict__ task
     const int64_t task = int64_t(blockIdx.x) * SA_TTM3_WARPS + warp;
     const bool group = int(blockIdx.x) < n_group_ctas;
     float acc[K::MT][K::NT][4];
-    float hacc = 0.f;
+    float hacc[4] = {0.f, 0.f, 0.f, 0.f};
     zero_tile<L, M>(acc);
     int u0 = 0, u1 = 0;
     if (task < n_tasks) { u0 = task_start[task]; u1 = task_start[task + 1]; }
@@ -510,9 +531,9 @@ ttm3_kernel(const sa_unit3 *__restrict__ units, const int32_t *__restrict__ task
     if (HAD) {
         // the warps hold partial rows of the same slice: sum them in a fixed order
         float *rows = reinterpret_cast<float *>(smem);
-        if (M == 16) hacc += __shfl_xor_sync(SA_FULL_MASK, hacc, 16);
+        const float4 h = had_total<M>(hacc);
         __syncthreads();                // every warp is done with its shared memory
-        if (lane < M) rows[warp * M + lane] = hacc;
+        if (4 * lane < M) *reinterpret_cast<float4 *>(rows + warp * M + 4 * lane) = h;
         __syncthreads();
         const sa_unit3 lead = units[task_start[int64_t(blockIdx.x) * SA_TTM3_WARPS]];
         if (threadIdx.x < M) {
@@ -582,7 +603,7 @@ ttmc3_fused_kernel(const sa_unit3 *__restrict__ units, const int32_t *__restrict
         const int64_t task = bt * SA_TTM3_WARPS + warp;
         const bool group = bt < n_group_ctas;          // the same for all warps of the block
         float acc[K::MT][K::NT][4];
-        float hacc = 0.f;
+        float hacc[4] = {0.f, 0.f, 0.f, 0.f};
         zero_tile<L, M>(acc);
         int u0 = 0, u1 = 0;
         if (task < n_tasks) { u0 = task_start[task]; u1 = task_start[task + 1]; }
