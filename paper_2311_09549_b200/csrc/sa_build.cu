@@ -206,6 +206,25 @@ void append_empty_slices(sa_tensor *t, sa_worklist &wl)
     }
 }
 
+// Items by decreasing number of nonzeros, items of equal length in the order they have.  Lengths are bounded by the list's
+// item size, so they are counted: building a 500 K nonzero CSR tensor takes 4.5 ms, with a comparison sort 5.6.
+void longest_first(std::vector<sa_item> &items)
+{
+    auto len = [](const sa_item &x) { return size_t(x.p1 - x.p0); };
+    size_t top = 0;
+    for (const sa_item &x : items) top = std::max(top, len(x));
+    if (top > (size_t(1) << 16)) {
+        std::stable_sort(items.begin(), items.end(), [&](const sa_item &a, const sa_item &b) { return len(a) > len(b); });
+        return;
+    }
+    std::vector<size_t> at(top + 2, 0);                  // at[top - len]: where the next item of that length goes
+    for (const sa_item &x : items) ++at[top - len(x) + 1];
+    for (size_t k = 1; k < at.size(); ++k) at[k] += at[k - 1];
+    std::vector<sa_item> sorted(items.size());
+    for (const sa_item &x : items) sorted[at[top - len(x)]++] = x;
+    items.swap(sorted);
+}
+
 // Nonzeros per unit of the order-3 kernel: 2048, less where `nnz` nonzeros would not give a full machine enough of them
 // (`slots`: at that many units the size stays 2048; a warp needs some 40 us for 2048 nonzeros, whatever else runs).
 //   Order 3, slots = 4736 (two per warp slot, 148 SMs x 16): 300 K nonzeros, ranks 16 and 32, mean fibers 1.5 to 18: 41 to
@@ -275,8 +294,7 @@ void build_ttm3_lists(sa_worklist &wl, int64_t n_slices, RowOf row_of, Skip skip
         }
     }
     std::stable_sort(groups.begin(), groups.end(), [](const group_rec &a, const group_rec &b) { return a.len > b.len; });
-    std::stable_sort(small.begin(), small.end(),
-                     [](const sa_item &a, const sa_item &b) { return (a.p1 - a.p0) > (b.p1 - b.p0); });
+    longest_first(small);
     wl.n_group_ctas = int64_t(groups.size());
     wl.task_start.clear();
     for (auto &g : groups)
@@ -567,8 +585,7 @@ void build_rows(const std::vector<int64_t> &pos, int64_t I, sa_worklist &wl, int
     }
     flush(I);
     // longest first: the tail of the launch is then made of the cheapest items
-    std::stable_sort(ranges.begin(), ranges.end(),
-                     [](const sa_item &a, const sa_item &b) { return (a.p1 - a.p0) > (b.p1 - b.p0); });
+    longest_first(ranges);
     wl.n_group_ctas = 0;
     wl.items = std::move(longs);
     wl.items.insert(wl.items.end(), ranges.begin(), ranges.end());
@@ -641,7 +658,7 @@ void build_sddmm(const std::vector<int64_t> &pos, const std::vector<int32_t> &cr
         const int32_t lx = x.it.p1 - x.it.p0, ly = y.it.p1 - y.it.p0;
         return lx != ly ? lx > ly : x.it.p0 < y.it.p0;
     });
-    std::stable_sort(ranges.begin(), ranges.end(), [](const sa_item &x, const sa_item &y) { return (x.p1 - x.p0) > (y.p1 - y.p0); });
+    longest_first(ranges);
     wl.n_group_ctas = 0;
     wl.items.clear();
     wl.items.reserve(pieces.size() + ranges.size());
