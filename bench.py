@@ -34,21 +34,15 @@ FALLBACK_HBM_GBS = 6650.0
 
 # DRAM bytes (read + write) of one launch of the dominant kernel, from the ncu captures summarised under
 # profiles/ (keyed by workload, or by (workload, schedule that ran)).  A figure is reported only while the kernel's
-# source file still has the hash it had when the counters were taken; otherwise `traffic` is null.  Workloads 4 and 5
-# are captured at a quarter of their size (--scale mid) and scaled by the nonzeros, see the profiles.
+# source file still has the hash it had when the counters were taken; otherwise `traffic` is null.  Workload 5 is
+# captured at a quarter of its size (--scale mid) and scaled by the nonzeros, see the profiles.
 NCU_TRAFFIC = {
     2: {"kernel": "ttm3_kernel<32,32> (98.4 % of the step)", "source": "paper_2311_09549_b200/csrc/sa_ttm3.cu",
-        "sha256": "16c36b6ee33b033d0b7e55b20c3ade065a6d5b28ef4f8267395b734b4ada9f3f",
-        "dram_bytes": 853618688, "profile": "profiles/ttm3_kernel_cfg2.md"},
-    3: {"kernel": "sddmm_spmm_kernel<64,64> (99.6 % of the step)", "source": "paper_2311_09549_b200/csrc/sa_sddmm_spmm.cu",
-        "sha256": "7c9971e0e72e49dfbb4404b68def327568372ea956767048b5d3d830810b8ead",
-        "dram_bytes": 13186066944, "profile": "profiles/sddmm_spmm_kernel_cfg3.md"},
-    (4, "left"): {"kernel": "spmm_gemm_left_kernel<256,64> (the whole step; counters of the quarter-size case x 4)",
-                  "source": "paper_2311_09549_b200/csrc/sa_spmm_gemm.cu", "sha256": "4cbda937e034c9869d74f7b8d341eab99531152e31ca898c803c7cd6cecf2622",
-                  "dram_bytes": 4 * 24086787584, "profile": "profiles/spmm_gemm_kernels_cfg4.md"},
-    (4, "right"): {"kernel": "spmm_kernel<2> (85 % of the step; counters of the quarter-size case x 4)",
-                   "source": "paper_2311_09549_b200/csrc/sa_spmm_gemm.cu", "sha256": "4cbda937e034c9869d74f7b8d341eab99531152e31ca898c803c7cd6cecf2622",
-                   "dram_bytes": 4 * 4974276864, "profile": "profiles/spmm_gemm_kernels_cfg4.md"},
+        "sha256": "d271528bf8560d74d8ebb8f7f9ba89ac7fbdc56e9d1394806562f426a6710cd0",
+        "dram_bytes": 855337216, "profile": "profiles/ttm3_kernel_cfg2.md"},
+    3: {"kernel": "sddmm_spmm_kernel<64,64> (98 % of the step)", "source": "paper_2311_09549_b200/csrc/sa_sddmm_spmm.cu",
+        "sha256": "62d9e7c5816d3e8a68fbd66376314c713d845ab8f17485ebce0bed0d2213b159",
+        "dram_bytes": 2604608512, "profile": "profiles/sddmm_spmm_kernel_cfg3.md"},
     (5, "fused"): {"kernel": "ttm4_fused_kernel (94 % of the step; counters of the quarter-size case x 4)",
                    "source": "paper_2311_09549_b200/csrc/sa_ttm4.cu", "sha256": "77b9b58137c8e565f84a5ffd8762e5448c910f5befc50c3838442ae6007d0823",
                    "dram_bytes": 4 * 424084480, "profile": "profiles/ttm4_kernels_cfg5.md"},
@@ -56,9 +50,6 @@ NCU_TRAFFIC = {
                                  "quarter-size case x 4)",
                        "source": "paper_2311_09549_b200/csrc/sa_ttm4_fis.cu", "sha256": "be9575594a14a3633f6a12fba75381f08305534e694d350516c738ba12c2d61b",
                        "dram_bytes": 4 * 663252480, "profile": "profiles/ttm4_kernels_cfg5.md"},
-    10: {"kernel": "fiber_spmm_kernel<32> (98 % of the step)", "source": "paper_2311_09549_b200/csrc/sa_spmm_gemm.cu",
-         "sha256": "4cbda937e034c9869d74f7b8d341eab99531152e31ca898c803c7cd6cecf2622",
-         "dram_bytes": 960941824, "profile": "profiles/fiber_spmm_kernel_w10.md"},
 }
 
 
@@ -134,9 +125,13 @@ def algorithmic_work(w, counts, sched):
             return base, 2 * nnz * L + 2 * F2 * L * M
         return base, 2 * K * L * M + 2 * nnz * M
     if w.expr == "spmmh_gemm":
-        # two gathered rows of L floats per nonzero (C and its Hadamard partner), E once, the output once
+        # left: two gathered rows of L floats per nonzero (C and its Hadamard partner), E once, the output once; right:
+        # C and its partner once, the J x M temporary once, then one gathered row of M floats per nonzero
         I, J = w.dims
         L, M = w.dense[0].shape[1], w.dense[2].shape[1]
+        if sched == "right":
+            return (sum(sz(d) for d in w.dense) + J * M * 4 + 8 * nnz + 4 * (I + 1) + 4 * M * nnz + out_bytes,
+                    J * L + 2 * J * L * M + 2 * nnz * M)
         return 8 * nnz + 4 * (I + 1) + 8 * L * nnz + sz(w.dense[2]) + out_bytes, 3 * nnz * L + 2 * I * L * M
     if w.expr == "spmm_gemm":
         I, J = w.dims
