@@ -502,3 +502,18 @@ def test_ttmc3_slices_around_the_step_and_chunk_sizes(sa, I, L, M, N):
     vals = rs.uniform(-1, 1, len(coords)).astype(np.float32)
     ops = [configs.dense_uniform(I, 0, I, L), configs.dense_uniform(I, 1, J, M), configs.dense_uniform(I, 2, K, N)]
     _check(sa, _wl("ttmc3", "csf", (I, J, K), coords, vals, ops, (L, M, N)), sched=sa.SA_SCHED_FISSIONED)
+
+
+@pytest.mark.parametrize("fibers", [1, 3, 4, 5, 7, 8, 9, 65, 700])
+@pytest.mark.parametrize("per_fiber", [1, 17])
+def test_mttkrp_gemm_fibers_around_the_four_and_eight_row_steps(sa, fibers, per_fiber):
+    """Numbers of fibers per slice around the four rows of a step and the eight of a flush; the last case spans several warps
+    of a block (units of one slice) and several units."""
+    rs = np.random.RandomState(10 * fibers + per_fiber)
+    J, K = 800, 40
+    coords = np.concatenate([np.stack([np.full(fibers * per_fiber, i), np.repeat(np.sort(rs.choice(J, fibers, replace=False)), per_fiber),
+                                       np.concatenate([np.sort(rs.choice(K, per_fiber, replace=False)) for _ in range(fibers)])], axis=1)
+                             for i in (0, 2, 3)]).astype(np.int32)
+    vals = rs.uniform(-1, 1, len(coords)).astype(np.float32)
+    ops = [configs.dense_uniform(fibers, 0, J, 32), configs.dense_uniform(fibers, 1, K, 32), configs.dense_uniform(fibers, 2, 32, 32)]
+    _check(sa, _wl("mttkrp_gemm", "csf", (5, J, K), coords, vals, ops, (5, 32)))
