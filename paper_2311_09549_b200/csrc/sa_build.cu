@@ -234,6 +234,18 @@ void longest_first(std::vector<sa_item> &items)
 //     4.2 M nonzeros 439 us with 2048, 484 us with 256.
 int64_t unit_size(int64_t nnz, int64_t slots) { return std::min<int64_t>(2048, std::max<int64_t>(256, nnz / slots / 64 * 64)); }
 
+// Chunk into which a slice of n > unit nonzeros is cut (192 partial tiles per slice at most), and the partial tiles of all slices.
+int64_t ttm3_chunk(int64_t n, int64_t unit) { return chunk_for(n, 4 * unit, 192); }
+int64_t ttm3_slots(const std::vector<int64_t> &len, int64_t unit)
+{
+    int64_t slots = 0;
+    for (const int64_t n : len) {
+        const int64_t ng = n > unit ? (n - 1) / ttm3_chunk(n, unit) + 1 : 1;
+        if (ng > 1) slots += ng;
+    }
+    return slots;
+}
+
 // Order-3 CSF.  An item ("unit") is a piece [p0, p1) of one slice with the fibers [f0, f1) it touches (a
 // fiber may be cut between two units, each adds its part).  Slices above SMALL_MAX nonzeros are cut into
 // chunks; the SA_TTM3_WARPS warps of a thread block take equal pieces of a chunk and reduce their tiles on chip.
@@ -247,8 +259,8 @@ template <typename RowOf, typename Skip>
 void build_ttm3_lists(sa_worklist &wl, int64_t n_slices, RowOf row_of, Skip skip, const std::vector<int64_t> &pos1,
                       const std::vector<int64_t> &pos2, int64_t unit)
 {
-    const int64_t SMALL_MAX = unit, MIN_CHUNK = 4 * unit;
-    constexpr int64_t MAX_PARTS = 192, MAX_UNITS = 16;
+    const int64_t SMALL_MAX = unit;
+    constexpr int64_t MAX_UNITS = 16;
     std::vector<sa_item> small;
     std::vector<group_rec> groups;
     for (int64_t s = 0; s < n_slices; ++s) {
@@ -264,7 +276,7 @@ void build_ttm3_lists(sa_worklist &wl, int64_t n_slices, RowOf row_of, Skip skip
             small.push_back(it);
             continue;
         }
-        const int64_t chunk = chunk_for(n, MIN_CHUNK, MAX_PARTS);
+        const int64_t chunk = ttm3_chunk(n, unit);
         const int64_t ng = (n + chunk - 1) / chunk;
         int32_t slot0 = -1;
         if (ng > 1) {
@@ -331,8 +343,16 @@ void build_ttm3_lists(sa_worklist &wl, int64_t n_slices, RowOf row_of, Skip skip
 
 void build_ttm3(sa_tensor *t, sa_worklist &wl)
 {
+    std::vector<int64_t> len(size_t(t->count[0]));
+    for (int64_t s = 0; s < t->count[0]; ++s)
+        len[size_t(s)] = t->pos[2][size_t(t->pos[1][size_t(s) + 1])] - t->pos[2][size_t(t->pos[1][size_t(s)])];
+    // sa_run_ttm3_static_scratch has room for 1024 partial tiles of the largest ranks: smaller units than 2048 may need that
+    // many, or as many as units of 2048 need
+    int64_t unit = unit_size(t->nnz, 4736);
+    const int64_t most = std::max<int64_t>(1024, ttm3_slots(len, 2048));
+    while (unit < 2048 && ttm3_slots(len, unit) > most) unit += 64;
     build_ttm3_lists(wl, t->count[0], [&](int64_t s) { return t->crd[0][size_t(s)]; }, [](int64_t) { return false; }, t->pos[1],
-                     t->pos[2], unit_size(t->nnz, 4736));
+                     t->pos[2], unit);
     append_empty_slices(t, wl);
 }
 

@@ -481,3 +481,21 @@ def test_order4_fissioned_subtree_worklist_covers_every_subtree_once_within_its_
     sub = sa.sa_tensor_worklist(t2.handle, 6)[1]
     main = sa.sa_tensor_worklist(t2.handle, 4)[1]
     assert [tuple(x[:2]) for x in sub.tolist()] == [(1, 2)] and set(main[:, 0].tolist()) == {0}
+
+
+def uniform_slices(n_slices, per):
+    """Order-3 host handle with `n_slices` slices of `per` nonzeros each."""
+    idx = np.arange(per)
+    coords = np.stack([np.repeat(np.arange(n_slices), per), np.tile(idx // 64, n_slices), np.tile(idx % 64, n_slices)], axis=1).astype(np.int32)
+    return sa.SparseTensor((n_slices, per // 64 + 1, 64), coords, np.ones(n_slices * per, np.float32), sa.SA_FMT_CSF, device=-1)
+
+
+@pytest.mark.parametrize("n_slices,per", [(10, 120_000), (30, 133_000), (50, 40_000), (1000, 2_000), (1000, 1_100), (400, 8_000), (1025, 1_200), (600, 9_000)])
+def test_order3_partial_tiles_fit_the_built_in_scratch(n_slices, per):
+    """sa_run_ttm3_static_scratch holds 1024 partial tiles at L = M = 32, more at smaller ranks.  With the largest units a slice
+    is cut into pieces of 8192 nonzeros; smaller units may not need more tiles than that or than the 1024 that always fit."""
+    largest = n_slices * (-(-per // 8192) if per > 8192 else 0)
+    t = uniform_slices(n_slices, per)
+    for L, M in [(32, 32), (32, 16), (16, 16)]:
+        need = sa.sa_workspace_size(t.handle, sa.SA_EXPR_SPTTM_TTM3, sa.SA_SCHED_DEFAULT, [(0, t.dims[1], L, L), (0, t.dims[2], M, M)])
+        assert need <= max(1024, largest) * L * M * 4, need

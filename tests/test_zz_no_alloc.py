@@ -85,3 +85,21 @@ def test_static_scratch_rejects_what_does_not_fit():
     ref, _ = t.run("spttm_ttm3", [C, D])
     torch.cuda.synchronize()
     assert float(ref.min()) == float(ref.max()) == float(per)
+
+
+@pytest.mark.parametrize("n_slices,per", [(10, 120_000), (1000, 1_100), (50, 40_000)])
+def test_static_scratch_takes_tensors_of_medium_size(n_slices, per):
+    """Tensors whose slices would need more than 1024 partial tiles if the lists were cut as finely as their size asks for."""
+    import torch
+    import paper_2311_09549_b200 as sa
+    idx = np.arange(per)
+    i = np.repeat(np.arange(n_slices), per)
+    coords = np.stack([i, np.tile(idx // 64, n_slices), np.tile(idx % 64, n_slices)], axis=1).astype(np.int32)
+    t = sa.SparseTensor((n_slices, per // 64 + 1, 64), coords, np.ones(coords.shape[0], np.float32), sa.SA_FMT_CSF, device=0)
+    C = torch.ones(t.dims[1], 32, device="cuda")
+    D = torch.ones(64, 32, device="cuda")
+    ops = [(x.data_ptr(), x.shape[0], x.shape[1], x.stride(0)) for x in (C, D)]
+    out = torch.zeros(n_slices, 32, 32, device="cuda")
+    sa.sa_run_ttm3_static_scratch(t.handle, ops, out.data_ptr(), torch.cuda.current_stream().cuda_stream)
+    torch.cuda.synchronize()
+    assert float(out.min()) == float(out.max()) == float(per)      # sums of ones: exact in fp32
