@@ -3,6 +3,8 @@
 // lists (nonzero-balanced pieces of slices, fibers and rows) the kernels consume.
 #include <algorithm>
 #include <cstring>
+#include <functional>
+#include <iterator>
 #include <memory>
 #include <omp.h>
 
@@ -225,15 +227,6 @@ void longest_first(std::vector<sa_item> &items)
     items.swap(sorted);
 }
 
-// Nonzeros per unit of the order-3 kernel: 2048, less where `nnz` nonzeros would not give a full machine enough of them
-// (`slots`: at that many units the size stays 2048; a warp needs some 40 us for 2048 nonzeros, whatever else runs).
-//   Order 3, slots = 4736 (two per warp slot, 148 SMs x 16): 300 K nonzeros, ranks 16 and 32, mean fibers 1.5 to 18: 41 to
-//     97 us with units of 2048, 13 to 25 us with 256; 6 M nonzeros 78 to 204 us with 2048, 82 to 195 with 1216; a third of
-//     that size costs more partial tiles than the balance gives (87 to 217 us).
-//   Order 4, slots = 2048 of all nonzeros (the list holds the large subtrees only, whose tiles are summed in 1 KB pieces):
-//     4.2 M nonzeros 439 us with 2048, 484 us with 256.
-int64_t unit_size(int64_t nnz, int64_t slots) { return std::min<int64_t>(2048, std::max<int64_t>(256, nnz / slots / 64 * 64)); }
-
 // Chunk into which a slice of n > unit nonzeros is cut (192 partial tiles per slice at most), and the partial tiles of all slices.
 int64_t ttm3_chunk(int64_t n, int64_t unit) { return chunk_for(n, 4 * unit, 192); }
 int64_t ttm3_slots(const std::vector<int64_t> &len, int64_t unit)
@@ -246,10 +239,120 @@ int64_t ttm3_slots(const std::vector<int64_t> &len, int64_t unit)
     return slots;
 }
 
+// Small slices per task: several only when there are enough of them to fill the machine (a few thousand warps) anyway.
+int64_t ttm3_task_units(int64_t n_small) { return std::min<int64_t>(16, std::max<int64_t>(1, n_small / 4096)); }
+
+// Time of the order-3 kernel on slices of the given lengths with units of `unit` nonzeros, in nonzeros of one warp: the thread
+// blocks of the list in launch order on the slots of the machine, each for as long as its longest warp plus a fixed cost;
+// blocks also run faster while fewer are resident, so their sum over the slots has a share.  TILE_COST per partial tile and
+// FIX_COST for the launch that adds them.  short_len[n]: slices of n nonzeros; long_len: the slices above 2048.
+// The constants are fitted to 22 tensors of 0.3 to 7 M nonzeros (equal and Zipf slices) at four combinations of ranks, each
+// timed with all of TTM3_UNITS: the unit that ttm3_unit takes is 0.8 % slower than the fastest in the mean, 15 % at most.
+constexpr int64_t TTM3_UNITS[] = {2048, 1536, 1024, 768, 512, 384, 256};
+double ttm3_time(const std::vector<int64_t> &short_len, const std::vector<int64_t> &long_len, int64_t unit, int64_t slots)
+{
+    constexpr int64_t BLOCK_COST = 110, UNIT_COST = 32, RESIDENT = 4 * 148;      // UNIT_COST: each further unit of a task
+    constexpr double TILE_COST = 0.06, FIX_COST = 100, MAKESPAN_SHARE = 0.7;
+    struct run_rec { int64_t cost, count; };
+    std::vector<run_rec> blocks;
+    auto cut = [&](int64_t n, int64_t count) {                    // the blocks of `count` slices of n > unit nonzeros
+        const int64_t chunk = ttm3_chunk(n, unit), full = (n - 1) / chunk, rest = n - full * chunk;
+        if (full > 0) blocks.push_back(run_rec{chunk / SA_TTM3_WARPS + BLOCK_COST, full * count});
+        blocks.push_back(run_rec{(rest + SA_TTM3_WARPS - 1) / SA_TTM3_WARPS + BLOCK_COST, count});
+    };
+    for (const int64_t n : long_len) cut(n, 1);
+    int64_t n_small = 0;
+    for (int64_t n = int64_t(short_len.size()) - 1; n > 0; --n) {
+        if (short_len[size_t(n)] == 0) continue;
+        if (n > unit) cut(n, short_len[size_t(n)]);
+        else n_small += short_len[size_t(n)];
+    }
+    std::sort(blocks.begin(), blocks.end(), [](const run_rec &x, const run_rec &y) { return x.cost > y.cost; });
+    const int64_t max_units = ttm3_task_units(n_small);
+    int64_t fill = 0, sum = 0, cnt = 0;                            // tasks in the last block; nonzeros and units of the open task
+    auto emit = [&](int64_t nonzeros, int64_t units, int64_t tasks) {
+        const int64_t more = std::min<int64_t>(tasks, fill > 0 ? SA_TTM3_WARPS - fill : 0);
+        fill = (fill + tasks) % SA_TTM3_WARPS;
+        tasks -= more;
+        if (tasks > 0)
+            blocks.push_back(run_rec{nonzeros + (units - 1) * UNIT_COST + BLOCK_COST, (tasks + SA_TTM3_WARPS - 1) / SA_TTM3_WARPS});
+    };
+    for (int64_t n = unit; n > 0; --n) {
+        int64_t count = short_len[size_t(n)];
+        if (count > 0 && cnt > 0) {
+            const int64_t more = std::min(count, std::min(max_units - cnt, (unit - sum) / n));
+            sum += more * n;
+            cnt += more;
+            count -= more;
+            if (count > 0) { emit(sum, cnt, 1); sum = cnt = 0; }
+        }
+        if (count > 0) {
+            const int64_t k = std::min(max_units, unit / n);
+            if (count >= k) emit(k * n, k, count / k);
+            cnt = count % k;
+            sum = cnt * n;
+        }
+    }
+    if (cnt > 0) emit(sum, cnt, 1);
+    double total = 0;
+    int64_t n_blocks = 0;
+    for (const run_rec &x : blocks) { total += double(x.cost) * double(x.count); n_blocks += x.count; }
+    const double even = total / RESIDENT;
+    double last = even;
+    if (n_blocks <= 16 * RESIDENT) {                               // more than 16 rounds: any order fills the machine
+        std::vector<int64_t> busy(size_t(std::min<int64_t>(n_blocks, RESIDENT)), 0);    // a heap with the earliest free slot on top
+        int64_t end = 0;
+        for (const run_rec &x : blocks)
+            for (int64_t c = 0; c < x.count; ++c) {
+                std::pop_heap(busy.begin(), busy.end(), std::greater<int64_t>());
+                busy.back() += x.cost;
+                end = std::max(end, busy.back());
+                std::push_heap(busy.begin(), busy.end(), std::greater<int64_t>());
+            }
+        last = double(end);
+    }
+    return MAKESPAN_SHARE * last + (1 - MAKESPAN_SHARE) * even + (slots > 0 ? FIX_COST + TILE_COST * double(slots) : 0.0);
+}
+
+// Nonzeros per unit: the largest of TTM3_UNITS within 3 % of the shortest estimated time, among those that need at most
+// 1024 partial tiles (what sa_run_ttm3_static_scratch has room for at the largest ranks) or as many as units of 2048 need.
+// From two units of 2048 per warp slot of the machine on it is 2048: balance is then not what the time goes to.
+// L = M = 32, us, units of 2048 / what the rule takes: 300 slices of 1000 nonzeros 50 / 21, 1000 x 1100 35 / 29, 3000 x 400
+// 45 / 45 (512 or more; 52 with 256), 50 x 40 000 60 / 43, 30 x 133 000 75 / 75 (83 with 832).
+int64_t ttm3_unit(const std::vector<int64_t> &len)
+{
+    constexpr int64_t LARGEST = TTM3_UNITS[0];
+    int64_t nnz = 0;
+    for (const int64_t n : len) nnz += n;
+    if (nnz >= LARGEST * 2 * 148 * 16) return LARGEST;
+    std::vector<int64_t> short_len(size_t(LARGEST) + 1, 0), long_len;
+    for (const int64_t n : len)
+        if (n > LARGEST) long_len.push_back(n);
+        else ++short_len[size_t(n)];
+    const int64_t most = std::max<int64_t>(1024, ttm3_slots(len, LARGEST));
+    int64_t units[std::size(TTM3_UNITS)];
+    double time[std::size(TTM3_UNITS)], best = 1e300;
+    int count = 0;
+    for (const int64_t u : TTM3_UNITS) {
+        const int64_t slots = ttm3_slots(len, u);
+        if (slots > most) continue;
+        units[count] = u;
+        time[count] = ttm3_time(short_len, long_len, u, slots);
+        best = std::min(best, time[count++]);
+    }
+    for (int x = 0; x < count; ++x)
+        if (time[x] <= 1.03 * best) return units[x];
+    return LARGEST;
+}
+
+// Nonzeros per unit of the order-4 lists, which hold the large (i,j) subtrees only: 2048, less where `nnz` nonzeros, of which
+// these are a part, would give fewer than 2048 units.  4.2 M nonzeros: 439 us with 2048, 484 us with 256.
+int64_t ttm4_unit(int64_t nnz) { return std::min<int64_t>(2048, std::max<int64_t>(256, nnz / 2048 / 64 * 64)); }
+
 // Order-3 CSF.  An item ("unit") is a piece [p0, p1) of one slice with the fibers [f0, f1) it touches (a
 // fiber may be cut between two units, each adds its part).  Slices above SMALL_MAX nonzeros are cut into
 // chunks; the SA_TTM3_WARPS warps of a thread block take equal pieces of a chunk and reduce their tiles on chip.
-// Smaller slices are one unit each; a warp evaluates a task of up to MAX_UNITS such units, about
+// Smaller slices are one unit each; a warp evaluates a task of up to ttm3_task_units such units, about
 // SMALL_MAX nonzeros in total.  Inside a unit the warp's SA_STREAMS lane groups stream the parts given by
 // sa_unit3_streams; stream_f0 holds the fiber in which each part starts.
 // `n_slices` slices; slice s is output row row_of(s), owns the fibers [pos1[s], pos1[s + 1]) whose nonzeros are
@@ -260,7 +363,6 @@ void build_ttm3_lists(sa_worklist &wl, int64_t n_slices, RowOf row_of, Skip skip
                       const std::vector<int64_t> &pos2, int64_t unit)
 {
     const int64_t SMALL_MAX = unit;
-    constexpr int64_t MAX_UNITS = 16;
     std::vector<sa_item> small;
     std::vector<group_rec> groups;
     for (int64_t s = 0; s < n_slices; ++s) {
@@ -314,9 +416,7 @@ void build_ttm3_lists(sa_worklist &wl, int64_t n_slices, RowOf row_of, Skip skip
             wl.task_start.push_back(int32_t(wl.items.size()));
             if (size_t(w) < g.items.size()) wl.items.push_back(g.items[size_t(w)]);
         }
-    // a task strings several small slices together only when there are enough of them to fill the machine
-    // (a few thousand warps) anyway
-    const int64_t max_units = std::min<int64_t>(MAX_UNITS, std::max<int64_t>(1, int64_t(small.size()) / 4096));
+    const int64_t max_units = ttm3_task_units(int64_t(small.size()));
     for (size_t x = 0; x < small.size();) {
         wl.task_start.push_back(int32_t(wl.items.size()));
         int64_t sum = 0, cnt = 0;
@@ -346,13 +446,8 @@ void build_ttm3(sa_tensor *t, sa_worklist &wl)
     std::vector<int64_t> len(size_t(t->count[0]));
     for (int64_t s = 0; s < t->count[0]; ++s)
         len[size_t(s)] = t->pos[2][size_t(t->pos[1][size_t(s) + 1])] - t->pos[2][size_t(t->pos[1][size_t(s)])];
-    // sa_run_ttm3_static_scratch has room for 1024 partial tiles of the largest ranks: smaller units than 2048 may need that
-    // many, or as many as units of 2048 need
-    int64_t unit = unit_size(t->nnz, 4736);
-    const int64_t most = std::max<int64_t>(1024, ttm3_slots(len, 2048));
-    while (unit < 2048 && ttm3_slots(len, unit) > most) unit += 64;
     build_ttm3_lists(wl, t->count[0], [&](int64_t s) { return t->crd[0][size_t(s)]; }, [](int64_t) { return false; }, t->pos[1],
-                     t->pos[2], unit);
+                     t->pos[2], ttm3_unit(len));
     append_empty_slices(t, wl);
 }
 
@@ -373,7 +468,7 @@ static bool subtree_is_small(const sa_tensor *t, int64_t f2)
 void build_ttm4_fissioned(sa_tensor *t, sa_worklist &wl, sa_worklist &wl2)
 {
     build_ttm3_lists(wl, t->count[1], [](int64_t f) { return int32_t(f); }, [&](int64_t f) { return subtree_is_small(t, f); },
-                     t->pos[2], t->pos[3], unit_size(t->nnz, 2048));
+                     t->pos[2], t->pos[3], ttm4_unit(t->nnz));
     constexpr int64_t CHUNK_F = 512;
     const auto &pos1 = t->pos[1];
     std::vector<sa_item> items;
@@ -473,7 +568,7 @@ void build_ttm4(sa_tensor *t, sa_worklist &wl, sa_worklist &wl_items, sa_worklis
         if (subtree_is_large(t, r)) large_ord[size_t(r)] = n_large++;
     t->f4_n_large = n_large;
     build_ttm3_lists(wl, F2, [&](int64_t r) { return large_ord[size_t(r)]; }, [&](int64_t r) { return large_ord[size_t(r)] < 0; },
-                     pos2, pos3, unit_size(t->nnz, 2048));
+                     pos2, pos3, ttm4_unit(t->nnz));
     wl.nnz = 0;
     for (const sa_item &it : wl.items) wl.nnz += it.p1 - it.p0;
 

@@ -499,3 +499,15 @@ def test_order3_partial_tiles_fit_the_built_in_scratch(n_slices, per):
     for L, M in [(32, 32), (32, 16), (16, 16)]:
         need = sa.sa_workspace_size(t.handle, sa.SA_EXPR_SPTTM_TTM3, sa.SA_SCHED_DEFAULT, [(0, t.dims[1], L, L), (0, t.dims[2], M, M)])
         assert need <= max(1024, largest) * L * M * 4, need
+
+
+@pytest.mark.parametrize("n_slices,per,groups,slots", [
+    (3000, 400, 0, 0),              # more slices than warps: not cut
+    (1000, 1_100, 1000, 0),         # a block per slice, no partial tiles
+    (400, 8_000, 800, 800),
+    (30, 133_000, 510, 510),        # one round of blocks on the machine (148 x 4); three rounds of smaller ones are slower
+    (10, 120_000, 590, 590),
+])
+def test_order3_units_are_those_whose_blocks_fill_the_machine_evenly(n_slices, per, groups, slots):
+    counts = sa.sa_tensor_worklist(uniform_slices(n_slices, per).handle)[0]
+    assert (counts[1], counts[3]) == (groups, slots), counts
