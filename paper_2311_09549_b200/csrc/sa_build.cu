@@ -243,15 +243,15 @@ int64_t ttm3_slots(const std::vector<int64_t> &len, int64_t unit)
 int64_t ttm3_task_units(int64_t n_small) { return std::min<int64_t>(16, std::max<int64_t>(1, n_small / 4096)); }
 
 // Time of the order-3 kernel on slices of the given lengths with units of `unit` nonzeros, in nonzeros of one warp: the thread
-// blocks of the list in launch order on the slots of the machine, each for as long as its longest warp plus a fixed cost;
+// blocks of the list in launch order on the `resident` slots of the machine, each for as long as its longest warp plus a fixed cost;
 // blocks also run faster while fewer are resident, so their sum over the slots has a share.  TILE_COST per partial tile and
 // FIX_COST for the launch that adds them.  short_len[n]: slices of n nonzeros; long_len: the slices above 2048.
 // The constants are fitted to 22 tensors of 0.3 to 7 M nonzeros (equal and Zipf slices) at four combinations of ranks, each
 // timed with all of TTM3_UNITS: the unit that ttm3_unit takes is 0.8 % slower than the fastest in the mean, 15 % at most.
 constexpr int64_t TTM3_UNITS[] = {2048, 1536, 1024, 768, 512, 384, 256};
-double ttm3_time(const std::vector<int64_t> &short_len, const std::vector<int64_t> &long_len, int64_t unit, int64_t slots)
+double ttm3_time(const std::vector<int64_t> &short_len, const std::vector<int64_t> &long_len, int64_t unit, int64_t slots, int64_t resident)
 {
-    constexpr int64_t BLOCK_COST = 110, UNIT_COST = 32, RESIDENT = 4 * 148;      // UNIT_COST: each further unit of a task
+    constexpr int64_t BLOCK_COST = 110, UNIT_COST = 32;              // UNIT_COST: each further unit of a task
     constexpr double TILE_COST = 0.06, FIX_COST = 100, MAKESPAN_SHARE = 0.7;
     struct run_rec { int64_t cost, count; };
     std::vector<run_rec> blocks;
@@ -297,10 +297,10 @@ double ttm3_time(const std::vector<int64_t> &short_len, const std::vector<int64_
     double total = 0;
     int64_t n_blocks = 0;
     for (const run_rec &x : blocks) { total += double(x.cost) * double(x.count); n_blocks += x.count; }
-    const double even = total / RESIDENT;
+    const double even = total / double(resident);
     double last = even;
-    if (n_blocks <= 16 * RESIDENT) {                               // more than 16 rounds: any order fills the machine
-        std::vector<int64_t> busy(size_t(std::min<int64_t>(n_blocks, RESIDENT)), 0);    // a heap with the earliest free slot on top
+    if (n_blocks <= 16 * resident) {                               // more than 16 rounds: any order fills the machine
+        std::vector<int64_t> busy(size_t(std::min<int64_t>(n_blocks, resident)), 0);    // a heap with the earliest free slot on top
         int64_t end = 0;
         for (const run_rec &x : blocks)
             for (int64_t c = 0; c < x.count; ++c) {
@@ -319,7 +319,10 @@ double ttm3_time(const std::vector<int64_t> &short_len, const std::vector<int64_
 // From two units of 2048 per warp slot of the machine on it is 2048: balance is then not what the time goes to.
 // L = M = 32, us, units of 2048 / what the rule takes: 300 slices of 1000 nonzeros 50 / 21, 1000 x 1100 35 / 29, 3000 x 400
 // 45 / 45 (512 or more; 52 with 256), 50 x 40 000 60 / 43, 30 x 133 000 75 / 75 (83 with 832).
-int64_t ttm3_unit(const std::vector<int64_t> &len)
+// *six_blocks: the 16 x 16 kernel compiled for six blocks per SM (fewer registers, each block 1.3 times as long) is through
+// sooner than the one for four; left alone for large tensors.  16 x 16, us, four / six blocks: 1000 slices of 2000 nonzeros
+// 33 / 39, 10 x 120 000 23 / 25, 400 x 8000 47 / 55, 3000 x 400 34 / 27, 800 x 700 21 / 15, 3000 x 2000 159 / 139.
+int64_t ttm3_unit(const std::vector<int64_t> &len, int *six_blocks)
 {
     constexpr int64_t LARGEST = TTM3_UNITS[0];
     int64_t nnz = 0;
@@ -337,12 +340,13 @@ int64_t ttm3_unit(const std::vector<int64_t> &len)
         const int64_t slots = ttm3_slots(len, u);
         if (slots > most) continue;
         units[count] = u;
-        time[count] = ttm3_time(short_len, long_len, u, slots);
+        time[count] = ttm3_time(short_len, long_len, u, slots, 4 * 148);
         best = std::min(best, time[count++]);
     }
-    for (int x = 0; x < count; ++x)
-        if (time[x] <= 1.03 * best) return units[x];
-    return LARGEST;
+    int x = 0;
+    while (time[x] > 1.03 * best) ++x;
+    *six_blocks = 1.3 * ttm3_time(short_len, long_len, units[x], ttm3_slots(len, units[x]), 6 * 148) < time[x];
+    return units[x];
 }
 
 // Nonzeros per unit of the order-4 lists, which hold the large (i,j) subtrees only: 2048, less where `nnz` nonzeros, of which
@@ -447,7 +451,7 @@ void build_ttm3(sa_tensor *t, sa_worklist &wl)
     for (int64_t s = 0; s < t->count[0]; ++s)
         len[size_t(s)] = t->pos[2][size_t(t->pos[1][size_t(s) + 1])] - t->pos[2][size_t(t->pos[1][size_t(s)])];
     build_ttm3_lists(wl, t->count[0], [&](int64_t s) { return t->crd[0][size_t(s)]; }, [](int64_t) { return false; }, t->pos[1],
-                     t->pos[2], ttm3_unit(len));
+                     t->pos[2], ttm3_unit(len, &wl.six_blocks));
     append_empty_slices(t, wl);
 }
 

@@ -73,6 +73,7 @@ struct sa_worklist {
     int64_t n_big_fix = 0;        // leading fix-up entries with more than SA_BIG_FIX partial tiles (longest first)
     int64_t n_sum_fix = 0;        // leading fix-up entries with partial tiles at all
     int64_t nnz = 0;              // nonzeros the list covers (set for the order-4 lists of pass 1)
+    int six_blocks = -1;          // order-3 CSF: whether the 16 x 16 kernel for six blocks per SM takes the list; -1: by its mean unit
     sa_item *d_items = nullptr;
     sa_fix *d_fix = nullptr;
     // order-3 CSF: warp w evaluates items [task_start[w], task_start[w + 1]); the first

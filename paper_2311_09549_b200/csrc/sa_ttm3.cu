@@ -33,10 +33,11 @@ struct dbg_limits {
 template <int L, int M>
 struct cfg {
     // Thread blocks per SM the register budget is set for: 4 (16 warps, 128 registers).  The 16 x 16 kernel also
-    // compiles without spills for 6 blocks (24 warps, 80 registers); that variant is slower on long units but
-    // faster when the units are short (many unit switches, whose latencies more warps hide): the launcher picks.
+    // compiles without spills for 6 blocks (24 warps, 80 registers); a block of that variant takes longer, but more of them
+    // run at a time: the builder picks by the rounds of blocks (ttm3_unit), for lists too large for rounds to matter the
+    // launcher does: short units mean many unit switches, whose latencies more warps hide.
     static constexpr int MINCTAS = 4;
-    static constexpr int MINCTAS_SHORT = (L == 16 && M == 16) ? 6 : 4;
+    static constexpr int MINCTAS_SIX = (L == 16 && M == 16) ? 6 : 4;
     static constexpr int MT = L / 16;            // m16 tiles over l
     static constexpr int NT = M / 8;             // n8 tiles over m
     static constexpr int NS = SA_STREAMS;        // streams per warp
@@ -661,10 +662,10 @@ cudaError_t launch(const sa_ttm3_view &v, const sa_dense &first, const sa_dense 
     const int64_t ctas = (n_tasks + SA_TTM3_WARPS - 1) / SA_TTM3_WARPS;
     if (ctas <= 0) return cudaSuccess;
     constexpr size_t smem = size_t(SA_TTM3_WARPS) * cfg<L, M>::WARP_BYTES;
-    const bool short_units = v.nnz < int64_t(512) * int64_t(wl.items.size());          // mean unit below 512 nonzeros
-    auto kern = short_units ? ttm3_kernel<L, M, cfg<L, M>::MINCTAS_SHORT, HAD> : ttm3_kernel<L, M, cfg<L, M>::MINCTAS, HAD>;
-    static bool attr_long[SA_MAX_DEVICE_FLAGS], attr_short[SA_MAX_DEVICE_FLAGS];     // per instantiation of this launcher
-    if (!sa_set_smem_once(kern, int(smem), short_units ? attr_short : attr_long)) return cudaGetLastError();
+    const bool six = wl.six_blocks >= 0 ? wl.six_blocks != 0 : v.nnz < int64_t(512) * int64_t(wl.items.size());   // mean unit below 512 nonzeros
+    auto kern = six ? ttm3_kernel<L, M, cfg<L, M>::MINCTAS_SIX, HAD> : ttm3_kernel<L, M, cfg<L, M>::MINCTAS, HAD>;
+    static bool attr_four[SA_MAX_DEVICE_FLAGS], attr_six[SA_MAX_DEVICE_FLAGS];     // per instantiation of this launcher
+    if (!sa_set_smem_once(kern, int(smem), six ? attr_six : attr_four)) return cudaGetLastError();
     dbg_limits lim;
     lim.status = v.status;
     lim.c_rows = uint32_t(first.rows); lim.d_rows = uint32_t(second.rows);
