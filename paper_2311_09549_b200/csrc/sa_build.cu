@@ -715,18 +715,22 @@ void build_rows(const std::vector<int64_t> &pos, int64_t I, sa_worklist &wl, int
 //   Size: `target` nonzeros, at most 256, less where the tensor would not give every group of a full machine
 //     (148 SMs x 64 groups) two items, at least 16: a group needs about a microsecond per four nonzeros, and on a small tensor
 //     that chain is the whole run time (60 k nonzeros, rows of up to 1500: 28 us; with a warp per item of up to 1024
-//     nonzeros 78 us).  A row counts as long above 64 nonzeros.  Rows per range: 32, at least 4, by the same rule, since a
+//     nonzeros 78 us).  A row counts as long above 64 nonzeros (1M x 1M, 30 M nonzeros: above 64 / 128 / 256 / 1024
+//     1.01 / 1.03 / 1.05 / 1.09 ms).  Rows per range: 32, at least 4, by the same rule, since a
 //     range of nearly empty rows is a chain of row loads and stores (whole call with the dense stage, 60 k nonzeros on 6 K
 //     rows 24.6 us with 32 rows, 18.2 with 4; 1.3 M nonzeros on 229 K rows, L = 128, 212 us with 32, 186 with 12).
 //   Order: D and E are gathered by column, and with J x (K + L) floats above L2 the order of the work decides what is
-//     found there.  Long rows are therefore cut where their columns cross a multiple of COL_BLOCK (a piece has at
-//     least MIN_PIECE nonzeros) and the pieces are sorted by block: whatever runs at one time then gathers from the
-//     same few blocks (32 K columns x (64 + 64) floats = 16 MB).  1M x 1M, 30 M nonzeros, K = L = 64: 1.05 ms with blocks
-//     of 32 K or 64 K columns, 1.06 with 16 K; rows long above 64 / 128 / 256 / 1024 nonzeros 1.01 / 1.03 / 1.05 / 1.09 ms.
+//     found there.  Rows above CUT_ROW nonzeros are therefore cut where their columns cross a multiple of COL_BLOCK (a piece
+//     has at least MIN_PIECE nonzeros, since each costs a partial row) and the pieces are sorted by block: whatever runs at one
+//     time then gathers from the same few blocks (32 K columns x (64 + 64) floats = 16 MB).  1M x 1M, 30 M nonzeros,
+//     K = L = 64: 1.05 ms with blocks of 32 K or 64 K columns, 1.06 with 16 K.  Shorter rows stay whole: their pieces would be
+//     mostly partial rows.  K = L = 64, us, cut / whole: rows of 100 nonzeros, 1 M columns 526 / 516, 200 K 382 / 311, 100 K
+//     343 / 273; rows of 200, 1 M columns 329 / 345, 200 K 246 / 251.  Pieces of at least 16 instead of 32 nonzeros need up to
+//     twice the workspace: rows of 300, 1 M columns 249 / 222, K = L = 128 687 / 699.
 //     Inside a block the longest pieces come first, so that the four groups of a warp get pieces of like length.
 void build_sddmm(const std::vector<int64_t> &pos, const std::vector<int32_t> &crd, int64_t I, sa_worklist &wl)
 {
-    constexpr int64_t COL_BLOCK = 32768, MIN_PIECE = 16;
+    constexpr int64_t COL_BLOCK = 32768, MIN_PIECE = 32, CUT_ROW = 128, MIN_REST = 16;
     const int64_t target = std::min<int64_t>(256, std::max<int64_t>(16, pos[size_t(I)] / (2 * 148 * 64)));
     const int64_t long_row = std::min<int64_t>(std::max<int64_t>(target, 48), 64);
     const int64_t max_rows = std::min<int64_t>(32, std::max<int64_t>(4, I / (2 * 148 * 64)));
@@ -751,11 +755,11 @@ void build_sddmm(const std::vector<int64_t> &pos, const std::vector<int32_t> &cr
             for (int64_t p = a; p < b;) {
                 int64_t q = std::min(b, p + target);
                 // the first block boundary after MIN_PIECE nonzeros, if there is one before q
-                if (q - p > MIN_PIECE && crd[size_t(q) - 1] / COL_BLOCK != crd[size_t(p + MIN_PIECE) - 1] / COL_BLOCK) {
+                if (b - a > CUT_ROW && q - p > MIN_PIECE && crd[size_t(q) - 1] / COL_BLOCK != crd[size_t(p + MIN_PIECE) - 1] / COL_BLOCK) {
                     const int32_t edge = int32_t((crd[size_t(p + MIN_PIECE) - 1] / COL_BLOCK + 1) * COL_BLOCK);
                     q = std::lower_bound(crd.begin() + p + MIN_PIECE, crd.begin() + q, edge) - crd.begin();
                 }
-                if (b - q < MIN_PIECE) q = b;
+                if (b - q < MIN_REST) q = b;
                 sa_item it = empty_item();
                 it.out_row = int32_t(r); it.row_end = int32_t(r + 1);
                 it.p0 = int32_t(p); it.p1 = int32_t(q);

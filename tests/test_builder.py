@@ -511,3 +511,15 @@ def test_order3_partial_tiles_fit_the_built_in_scratch(n_slices, per):
 def test_order3_units_are_those_whose_blocks_fill_the_machine_evenly(n_slices, per, groups, slots):
     counts = sa.sa_tensor_worklist(uniform_slices(n_slices, per).handle)[0]
     assert (counts[1], counts[3]) == (groups, slots), counts
+
+
+@pytest.mark.parametrize("rows,deg", [(50_000, 100), (40_000, 128), (17_000, 300)])
+def test_csr_rows_are_cut_by_column_blocks_only_where_the_pieces_stay_long(rows, deg):
+    """Kernel 1 on one million columns: rows of up to 128 nonzeros need no partial rows, longer ones one per 32 nonzeros at most."""
+    rng = np.random.default_rng(3)
+    cols = (np.sort(rng.integers(0, 1_000_000 - deg, (rows, deg)), axis=1) + np.arange(deg)).astype(np.int32)      # distinct per row
+    coords = np.stack([np.repeat(np.arange(rows, dtype=np.int32), deg), cols.ravel()], axis=1)
+    t = sa.SparseTensor((rows, 1_000_000), coords, np.ones(rows * deg, np.float32), sa.SA_FMT_CSR, device=-1)
+    need = sa.sa_workspace_size(t.handle, sa.SA_EXPR_SDDMM_SPMM, sa.SA_SCHED_DEFAULT,
+                                [(0, rows, 128, 128), (0, 1_000_000, 128, 128), (0, 1_000_000, 128, 128)])
+    assert need <= (0 if deg <= 128 else rows * (deg // 32) * 128 * 4 + 255), need
