@@ -22,10 +22,13 @@ struct sd_cfg {
     static constexpr int DQ = K / 32, EQ = L / 32;    // float4 pieces of D(j,:) and E(j,:) per lane
     static constexpr int U = DQ + EQ <= 4 ? 4 : 2;    // nonzeros per group and step: 16 float4 in flight per lane at most
     static constexpr bool AHEAD = DQ + EQ < 8;        // C of the next row in registers (spills at K = L = 128)
+    // Blocks per SM.  K = L = 32 has half the bytes in flight per lane and needs the warps: 100 K rows of 100 nonzeros on 1 M
+    // columns 337 us with two blocks, 273 with three, 489 (spills) with four; eight nonzeros per step with two blocks 307.
+    static constexpr int CTAS = DQ + EQ <= 2 ? 3 : 2;
 };
 
 template <int K, int L>
-__global__ void __launch_bounds__(256, 2)
+__global__ void __launch_bounds__(256, (sd_cfg<K, L>::CTAS))
 sddmm_spmm_kernel(const sa_item *__restrict__ items, int64_t n_items, const int32_t *__restrict__ pos,
                   const int2 *__restrict__ nz, const float *__restrict__ C, uint32_t ldc, const float *__restrict__ D,
                   uint32_t ldd, const float *__restrict__ E, uint32_t lde, float *__restrict__ out, float *__restrict__ partial,
