@@ -716,9 +716,10 @@ void build_rows(const std::vector<int64_t> &pos, int64_t I, sa_worklist &wl, int
 //     (148 SMs x 64 groups) two items, at least 16: a group needs about a microsecond per four nonzeros, and on a small tensor
 //     that chain is the whole run time (60 k nonzeros, rows of up to 1500: 28 us; with a warp per item of up to 1024
 //     nonzeros 78 us).  A row counts as long above 64 nonzeros (1M x 1M, 30 M nonzeros: above 64 / 128 / 256 / 1024
-//     1.01 / 1.03 / 1.05 / 1.09 ms).  Rows per range: 32, at least 4, by the same rule, since a
+//     1.01 / 1.03 / 1.05 / 1.09 ms).  Rows per range: 8, at least 4, by the same rule, since a
 //     range of nearly empty rows is a chain of row loads and stores (whole call with the dense stage, 60 k nonzeros on 6 K
-//     rows 24.6 us with 32 rows, 18.2 with 4; 1.3 M nonzeros on 229 K rows, L = 128, 212 us with 32, 186 with 12).
+//     rows 24.6 us with 32 rows, 18.2 with 4; 3 M nonzeros on 1 M rows and columns, Zipf(1.2), K = L = 32 236 us with 32, 213
+//     with 16, 200 with 8; K = 64, L = 32 309, 291, 278).
 //   Order: D and E are gathered by column, and with J x (K + L) floats above L2 the order of the work decides what is
 //     found there.  Rows above CUT_ROW nonzeros are therefore cut where their columns cross a multiple of COL_BLOCK (a piece
 //     has at least MIN_PIECE nonzeros, since each costs a partial row) and the pieces are sorted by block: whatever runs at one
@@ -733,7 +734,7 @@ void build_sddmm(const std::vector<int64_t> &pos, const std::vector<int32_t> &cr
     constexpr int64_t COL_BLOCK = 32768, MIN_PIECE = 32, CUT_ROW = 128, MIN_REST = 16;
     const int64_t target = std::min<int64_t>(256, std::max<int64_t>(16, pos[size_t(I)] / (2 * 148 * 64)));
     const int64_t long_row = std::min<int64_t>(std::max<int64_t>(target, 48), 64);
-    const int64_t max_rows = std::min<int64_t>(32, std::max<int64_t>(4, I / (2 * 148 * 64)));
+    const int64_t max_rows = std::min<int64_t>(8, std::max<int64_t>(4, I / (2 * 148 * 64)));
     struct piece_rec { uint32_t key; sa_item it; };
     std::vector<piece_rec> pieces;
     std::vector<sa_item> ranges;

@@ -523,3 +523,11 @@ def test_csr_rows_are_cut_by_column_blocks_only_where_the_pieces_stay_long(rows,
     need = sa.sa_workspace_size(t.handle, sa.SA_EXPR_SDDMM_SPMM, sa.SA_SCHED_DEFAULT,
                                 [(0, rows, 128, 128), (0, 1_000_000, 128, 128), (0, 1_000_000, 128, 128)])
     assert need <= (0 if deg <= 128 else rows * (deg // 32) * 128 * 4 + 255), need
+
+
+def test_csr_ranges_of_short_rows_hold_at_most_eight():
+    """Kernel 1: a lane group walks a range row by row, so nearly empty rows make it a chain of latencies."""
+    rows = 400_000
+    coords = np.stack([np.arange(rows), np.arange(rows) % 1000], axis=1).astype(np.int32)
+    items = sa.sa_tensor_worklist(sa.SparseTensor((rows, 1000), coords, np.ones(rows, np.float32), sa.SA_FMT_CSR, device=-1).handle)[1]
+    assert (items[:, 1] - items[:, 0]).max() <= 8
