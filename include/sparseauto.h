@@ -280,7 +280,10 @@ sa_status sa_tensor_set_aux_limit(sa_tensor *t, size_t bytes);
  * SPTTM_SPTTM L, M in {32, 64} (out: level_counts[1] x M, see sa_expr).
  * Arithmetic: fp32 throughout; stages on tensor cores split every fp32 operand into two parts and
  * add three partial products (TF32 parts in the per-slice contractions, BF16 parts in the dense GEMM
- * stage; three BF16 parts and six products in the one of SPMMH_GEMM), so every output element stays within 1e-4 of the sum of the absolute values of its terms.
+ * stage; three BF16 parts and six products in the one of SPMMH_GEMM), so every output element stays within 1e-4
+ * of the sum of the absolute values of its terms.  Infinities, NaN and finite operands above the largest BF16
+ * number (3.39e38) give what fp32 arithmetic in the schedule's order gives in SDDMM_SPMM, SPMMH_GEMM and the
+ * ASSOC_LEFT orders; where an operand is split into two parts they give NaN.
  * The dense GEMM stage (SPMM_GEMM and SPMMH_GEMM as ASSOC_RIGHT, SDDMM_SPMM_GEMM) waits on on-chip hand-offs with a
  * 2-second limit; if one runs out the kernel returns and sa_last_device_status reports SA_E_TIMEOUT.
  * Returns launch errors only; completion is observed by synchronising the stream.

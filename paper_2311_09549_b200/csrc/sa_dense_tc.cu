@@ -281,6 +281,7 @@ gemm_tc_kernel(int64_t J, const float *__restrict__ C, int64_t ldc, const float 
             if (!__all_sync(SA_FULL_MASK, ok)) break;
             tc_fence_after();
             const uint32_t taddr = tmem_base + (uint32_t(32 * warp) << 16) + a * G::ACC_COLS;
+            float zero = 0.f;                                        // HAD: NaN once an element of this row is not finite
 #pragma unroll
             for (int c = 0; c < M / 16; ++c) {
                 float p[16], r[16];
@@ -294,6 +295,8 @@ gemm_tc_kernel(int64_t J, const float *__restrict__ C, int64_t ldc, const float 
                     tc_ld16(taddr + 3 * M + 16 * c, r2);
 #pragma unroll
                     for (int x = 0; x < 16; ++x) r[x] += r2[x];
+#pragma unroll
+                    for (int x = 0; x < 16; ++x) zero = fmaf(p[x] + r[x], 0.f, zero);
                 }
 #pragma unroll
                 for (int x = 0; x < 4; ++x)                         // unit 4c + x of row `lane`, XOR-swizzled by the row
@@ -305,6 +308,27 @@ gemm_tc_kernel(int64_t J, const float *__restrict__ C, int64_t ldc, const float 
             mbar_arrive(bars + 8 * (B_ACC_EMPTY + a));               // the accumulator is free again
             __syncwarp();
             const int64_t row0 = (int64_t(blockIdx.x) + tl * gridDim.x) * TC_BM + 32 * warp;
+            if constexpr (HAD) {
+                // An infinity, a NaN or a number that rounds to a BF16 infinity has no BF16 parts (x - bf16(x) is NaN or infinite)
+                // and leaves NaN in its whole row: such rows are summed once more in fp32 arithmetic, which has the right value.
+                for (unsigned bad = __ballot_sync(SA_FULL_MASK, zero != 0.f); bad != 0; bad &= bad - 1) {
+                    const int r = __ffs(bad) - 1;
+                    const int64_t row = min(row0 + r, J - 1);
+                    float acc[M / 32];
+#pragma unroll
+                    for (int q = 0; q < M / 32; ++q) acc[q] = 0.f;
+#pragma unroll 8
+                    for (int k = 0; k < L; ++k) {
+                        const float x = __ldg(C + row * ldc + k) * __ldg(H + row * ldh + k);
+#pragma unroll
+                        for (int q = 0; q < M / 32; ++q) acc[q] = fmaf(x, __ldg(D + int64_t(k) * ldd + 32 * q + lane), acc[q]);
+                    }
+#pragma unroll
+                    for (int q = 0; q < M / 32; ++q)
+                        *reinterpret_cast<float *>(stage + r * (M * 4) + (((8 * q + (lane >> 2)) ^ (r & 7)) << 4) + 4 * (lane & 3)) = acc[q];
+                }
+                __syncwarp();
+            }
             // E as tables of 2^part_shift float4 columns (one table: rows of E): 512-byte runs whatever the width
 #pragma unroll
             for (int i = 0; i < RC; ++i) {

@@ -517,3 +517,60 @@ def test_mttkrp_gemm_fibers_around_the_four_and_eight_row_steps(sa, fibers, per_
     vals = rs.uniform(-1, 1, len(coords)).astype(np.float32)
     ops = [configs.dense_uniform(fibers, 0, J, 32), configs.dense_uniform(fibers, 1, K, 32), configs.dense_uniform(fibers, 2, 32, 32)]
     _check(sa, _wl("mttkrp_gemm", "csf", (5, J, K), coords, vals, ops, (5, 32)))
+
+
+@pytest.mark.parametrize("L,M,J", [(128, 32, 200), (128, 64, 1), (256, 32, 148 * 128 + 33), (256, 64, 5_000)])
+def test_spmmh_gemm_right_order_keeps_infinities_nan_and_the_largest_numbers(sa, L, M, J):
+    """The dense stage of B.((C o D).E) splits its operands into BF16 parts; numbers that have no such parts (infinities, NaN,
+    finite ones that round to a BF16 infinity) must give what the row nest in fp32 arithmetic gives.  All operands are positive
+    apart from one negative infinity and every row has nonzeros, so that the two orders of summation meet the same cases."""
+    import torch
+    rng = np.random.default_rng(7)
+    I, deg = 700, min(4, J)
+    cols = np.stack([rng.choice(J, deg, replace=False) for _ in range(I)])
+    cols[:4, 0] = [0, J - 1, J // 2, J // 3]
+    cols = np.stack([np.pad(np.unique(c), (0, deg - len(np.unique(c))), constant_values=-1) for c in cols])
+    keep = cols.ravel() >= 0
+    coords = np.stack([np.repeat(np.arange(I), deg)[keep], cols.ravel()[keep]], axis=1).astype(np.int32)
+    vals = rng.uniform(0.5, 1.0, coords.shape[0]).astype(np.float32)
+    t = sa.SparseTensor((I, J), coords, vals, sa.SA_FMT_CSR, device=0)
+    C, D = (rng.uniform(0.5, 1.0, (J, L)).astype(np.float32) for _ in range(2))
+    E = rng.uniform(0.5, 1.0, (L, M)).astype(np.float32)
+
+    def both(C, D, E):
+        ops = [torch.from_numpy(x).cuda() for x in (C, D, E)]
+        out = [t.run("spmmh_gemm", ops, sched=s)[0].cpu().numpy() for s in (sa.SA_SCHED_ASSOC_RIGHT, sa.SA_SCHED_FUSED)]
+        assert sa.sa_last_device_status(t.handle, torch.cuda.current_stream().cuda_stream) == sa.SA_OK
+        return out
+
+    def same(right, nest):
+        assert np.array_equal(np.isnan(right), np.isnan(nest))
+        inf = np.isinf(nest)
+        assert np.array_equal(np.isinf(right), inf) and np.array_equal(right[inf], nest[inf])
+        fin = np.isfinite(nest)
+        assert fin.sum() == 0 or np.abs(right[fin] / nest[fin] - 1).max() < 2 * L * 2.0 ** -24      # fp32 sums of L positive terms
+        return nest
+
+    tiny = np.float32(1e-3)
+    for where in {0, J - 1, J // 2, J // 3}:
+        for value in (np.inf, -np.inf, np.nan):
+            for hit in (0, 1):
+                X = [C.copy(), D.copy()]
+                X[hit][where, L // 3] = value
+                nest = same(*both(X[0], X[1], E))
+                assert np.isfinite(nest).any() or J < 5
+                assert not np.isfinite(nest).all()
+        X = C.copy()
+        X[where, L - 1] = np.float32(3.4e38)                       # finite, rounds to a BF16 infinity; the sums stay finite
+        Y = D.copy()
+        Y[where, L - 1] = 1
+        F = E.copy()
+        F[L - 1] = tiny
+        assert np.isfinite(same(*both(X, Y, F))).all()
+        Y[where, L - 1] = 8                                        # the product itself overflows
+        assert np.isinf(same(*both(X, Y, F))).any()
+    for value in (np.inf, np.nan, np.float32(3.4e38)):
+        F = E.copy()
+        F[L // 2, M - 1] = value
+        nest = same(*both(C * tiny, D, F))
+        assert np.isfinite(nest[:, :M - 1]).all()
