@@ -509,7 +509,8 @@ def test_order3_partial_tiles_fit_the_built_in_scratch(n_slices, per):
     (10, 120_000, 590, 590),
 ])
 def test_order3_units_are_those_whose_blocks_fill_the_machine_evenly(n_slices, per, groups, slots):
-    counts = sa.sa_tensor_worklist(uniform_slices(n_slices, per).handle)[0]
+    t = uniform_slices(n_slices, per)
+    counts = sa.sa_tensor_worklist(t.handle)[0]
     assert (counts[1], counts[3]) == (groups, slots), counts
 
 
@@ -529,5 +530,6 @@ def test_csr_ranges_of_short_rows_hold_at_most_eight():
     """Kernel 1: a lane group walks a range row by row, so nearly empty rows make it a chain of latencies."""
     rows = 400_000
     coords = np.stack([np.arange(rows), np.arange(rows) % 1000], axis=1).astype(np.int32)
-    items = sa.sa_tensor_worklist(sa.SparseTensor((rows, 1000), coords, np.ones(rows, np.float32), sa.SA_FMT_CSR, device=-1).handle)[1]
+    t = sa.SparseTensor((rows, 1000), coords, np.ones(rows, np.float32), sa.SA_FMT_CSR, device=-1)
+    items = sa.sa_tensor_worklist(t.handle)[1]
     assert (items[:, 1] - items[:, 0]).max() <= 8
