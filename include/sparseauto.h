@@ -77,8 +77,9 @@ typedef enum {
     /* kernel 3 <SpMMH,GEMM>: A(i,m) = sum_{j,l} B(i,j) C(j,l) D(j,l) E(l,m); ops = {C, D, E}; B CSR;
      * the Description column of the Table of kernels (SpMM with a Hadamard product, then GEMM).
      * SA_SCHED_FUSED: per row T(l) = sum_j B(i,j) C(j,l) D(j,l) followed by T . E; SA_SCHED_ASSOC_RIGHT:
-     * G(j,m) = sum_l C(j,l) D(j,l) E(l,m) in the workspace, then B . G; SA_SCHED_DEFAULT: the one that
-     * moves fewer bytes                                                                         */
+     * G(j,m) = sum_l C(j,l) D(j,l) E(l,m) in the workspace (dims[1] x M floats), then B . G;
+     * SA_SCHED_DEFAULT: the one that moves fewer bytes.  sa_workspace_size gives what that one needs; sa_run with
+     * a smaller workspace, or none, runs SA_SCHED_FUSED instead if that fits (up to several times slower) */
     SA_EXPR_SPMMH_GEMM = 7,
     /* kernel 8 <MTTKRP,GEMM>: A(i,m) = sum_{j,k,r} B(i,j,k) C(j,r) D(k,r) E(r,m); ops = {C, D, E};
      * B order-3 CSF; the MTTKRP rows T(i,:) (R floats per slice) live in the workspace              */
@@ -271,7 +272,8 @@ sa_status sa_tensor_set_aux_limit(sa_tensor *t, size_t bytes);
  *   out        DEVICE fp32, dense row-major, contiguous, 16-byte aligned; FULLY OVERWRITTEN
  *              (the statement is an assignment; empty slices / rows become +0.0)
  *   workspace  DEVICE scratch of at least sa_workspace_size bytes, 256-byte aligned; may be
- *              NULL when that size is 0.  Contents on entry are ignored.
+ *              NULL when that size is 0.  Contents on entry are ignored.  Ask for the size: it follows the
+ *              lists of the tensor (how its slices and rows are cut), not only the operand shapes.
  *   cuda_stream  a cudaStream_t (NULL = default stream)
  * Compiled dense ranks (anything else is SA_E_UNSUPPORTED): SPTTM_TTM3 L, M in {16, 32};
  * SPTTM_TTM4 L = M = N = 16; SDDMM_SPMM K, L in {32, 64, 128}; SPMM_GEMM L in {128, 256},
@@ -282,8 +284,8 @@ sa_status sa_tensor_set_aux_limit(sa_tensor *t, size_t bytes);
  * add three partial products (TF32 parts in the per-slice contractions, BF16 parts in the dense GEMM
  * stage; three BF16 parts and six products in the one of SPMMH_GEMM), so every output element stays within 1e-4
  * of the sum of the absolute values of its terms.  Infinities, NaN and finite operands above the largest BF16
- * number (3.39e38) give what fp32 arithmetic in the schedule's order gives in SDDMM_SPMM, SPMMH_GEMM and the
- * ASSOC_LEFT orders; where an operand is split into two parts they give NaN.
+ * number (3.39e38) give what fp32 arithmetic in the schedule's order gives in SDDMM_SPMM, SPMMH_GEMM and
+ * SPMM_GEMM as ASSOC_LEFT; where an operand is split into two parts they give NaN.
  * The dense GEMM stage (SPMM_GEMM and SPMMH_GEMM as ASSOC_RIGHT, SDDMM_SPMM_GEMM) waits on on-chip hand-offs with a
  * 2-second limit; if one runs out the kernel returns and sa_last_device_status reports SA_E_TIMEOUT.
  * Returns launch errors only; completion is observed by synchronising the stream.

@@ -75,11 +75,14 @@ for _n in EXPORTED_SYMBOLS:
         getattr(_lib, _n).restype = _int
 
 
-# sa_run for SparseTensor.run: the operand descriptors as packed bytes (a ctypes array of structures costs more to fill than
-# the call itself)
+# sa_run and sa_workspace_size for SparseTensor.run: the operand descriptors as packed bytes (a ctypes array of structures
+# costs more to fill than the call itself)
 _run_packed = _lib["sa_run"]
 _run_packed.argtypes = [_vp, _int, _int, ctypes.c_char_p, _int, _vp, _vp, ctypes.c_size_t, _vp]
 _run_packed.restype = _int
+_size_packed = _lib["sa_workspace_size"]
+_size_packed.argtypes = [_vp, _int, _int, ctypes.c_char_p, _int, _vp]
+_size_packed.restype = _int
 _PACK_OPS = {n: struct.Struct("Pqqq" * n).pack for n in range(1, 5)}
 assert struct.calcsize("Pqqq") == ctypes.sizeof(SaDense)
 
@@ -282,9 +285,13 @@ class SparseTensor:
         n = len(operands)
         if n not in _PACK_OPS:
             self._size(expr, sched, desc)           # raises: no expression takes that many operands
+        packed = _PACK_OPS[n](*desc)
         own = workspace is None
         if own:
-            workspace = self._ws if self._ws is not None else self._grow(expr, sched, desc)
+            workspace = self._ws
+            # kernel 3 by default runs a slower schedule in a small workspace, where the others report SA_E_WORKSPACE
+            if workspace is None or (expr == SA_EXPR_SPMMH_GEMM and workspace.numel() < self._packed_size(expr, sched, packed, n)):
+                workspace = self._grow(expr, sched, desc)
         if out is None:
             try:
                 shape = self.out_shape(expr, operands)
@@ -293,7 +300,6 @@ class SparseTensor:
                 raise
             out = torch.empty(shape, dtype=torch.float32, device=workspace.device)
         s = torch.cuda.current_stream(self.device) if stream is None else stream
-        packed = _PACK_OPS[n](*desc)
         st = _run_packed(self.handle, int(expr), int(sched), packed, n, out.data_ptr(), workspace.data_ptr(), workspace.numel(), s.cuda_stream)
         if own and st == SA_E_WORKSPACE:            # nothing was enqueued: this call needs more than the ones before it
             workspace = self._grow(expr, sched, desc)
@@ -304,9 +310,21 @@ class SparseTensor:
     def _size(self, expr, sched, desc):
         return sa_workspace_size(self.handle, expr, sched, [tuple(desc[i:i + 4]) for i in range(0, len(desc), 4)])
 
+    def _packed_size(self, expr, sched, packed, n):
+        need = ctypes.c_size_t()
+        _check(_size_packed(self.handle, int(expr), int(sched), packed, n, ctypes.byref(need)), "sa_workspace_size")
+        return need.value
+
     def _grow(self, expr, sched, desc):
         import torch
-        self._ws = torch.empty(max(self._size(expr, sched, desc), 256), dtype=torch.uint8, device=torch.device("cuda", self.device))
+        need, dev = self._size(expr, sched, desc), torch.device("cuda", self.device)
+        try:
+            self._ws = torch.empty(max(need, 256), dtype=torch.uint8, device=dev)
+        except torch.OutOfMemoryError:
+            if expr != SA_EXPR_SPMMH_GEMM or sched != SA_SCHED_DEFAULT:
+                raise
+            # no room for the J x M temporary of kernel 3's faster order: sa_run takes the row nest
+            self._ws = torch.empty(max(self._size(expr, SA_SCHED_FUSED, desc), 256), dtype=torch.uint8, device=dev)
         return self._ws
 
     def out_shape(self, expr, operands):

@@ -551,9 +551,13 @@ sa_status sa_run(const sa_tensor *t, sa_expr expr, sa_schedule sched, const sa_d
     if (s != SA_OK) return s;
     sa_schedule r;
     if (!resolve_schedule(t, expr, sched, ops, &r)) return SA_E_UNSUPPORTED;
-    const size_t need = workspace_bytes(t, expr, r, ops);
-    if (need > 0 && (!workspace || ws_bytes < need || reinterpret_cast<uintptr_t>(workspace) % 256))
-        return SA_E_WORKSPACE;
+    auto fits = [&]() {
+        const size_t need = workspace_bytes(t, expr, r, ops);
+        return need == 0 || (workspace && ws_bytes >= need && reinterpret_cast<uintptr_t>(workspace) % 256 == 0);
+    };
+    // kernel 3: the row nest takes the call if the J x M temporary of the faster order has no room
+    if (expr == SA_EXPR_SPMMH_GEMM && sched == SA_SCHED_DEFAULT && !fits()) r = SA_SCHED_FUSED;
+    if (!fits()) return SA_E_WORKSPACE;
     device_guard g(t->device);
     if (!g.ok) return SA_E_CUDA;
     cudaStream_t stream = static_cast<cudaStream_t>(cuda_stream);
@@ -572,7 +576,7 @@ sa_status sa_run(const sa_tensor *t, sa_expr expr, sa_schedule sched, const sa_d
             break;
         case SA_EXPR_TTMC3: s = sa_launch_ttmc3(t, ops, out, workspace, ws_bytes, r == SA_SCHED_FISSIONED, stream, &launches); break;
         case SA_EXPR_SDDMM_SPMM_GEMM: s = sa_launch_sddmm_spmm_gemm(t, ops, out, workspace, ws_bytes, stream, &launches); break;
-        case SA_EXPR_SPMMH_GEMM: 
+        case SA_EXPR_SPMMH_GEMM:
             s = sa_launch_spmmh_gemm(t, ops, out, workspace, ws_bytes, r == SA_SCHED_ASSOC_RIGHT, stream, &launches);
             break;
         case SA_EXPR_MTTKRP_GEMM: s = sa_launch_mttkrp_gemm(t, ops, out, workspace, ws_bytes, stream, &launches); break;

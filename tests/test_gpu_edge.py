@@ -574,3 +574,41 @@ def test_spmmh_gemm_right_order_keeps_infinities_nan_and_the_largest_numbers(sa,
         F[L // 2, M - 1] = value
         nest = same(*both(C * tiny, D, F))
         assert np.isfinite(nest[:, :M - 1]).all()
+
+
+def test_spmmh_gemm_default_runs_in_the_workspace_it_is_given(sa):
+    """Without room for the J x M temporary of its faster order the default of kernel 3 is the row nest: from a caller that has
+    no workspace to give, and where the device has no memory left for one."""
+    import torch
+    I, J, L, M = 300, 200_000, 128, 64
+    coords, vals = _random_coo(31, (I, J), 600_000)
+    t = sa.SparseTensor((I, J), coords, vals, sa.SA_FMT_CSR, device=0)
+    g = torch.Generator(device="cuda")
+    g.manual_seed(5)
+    ops = [torch.randn(s, device="cuda", generator=g) for s in ((J, L), (J, L), (L, M))]
+    tuples = [(x.data_ptr(), x.shape[0], x.shape[1], x.stride(0)) for x in ops]
+    E, F, D = sa.SA_EXPR_SPMMH_GEMM, sa.SA_SCHED_FUSED, sa.SA_SCHED_DEFAULT
+    need, nest = (sa.sa_workspace_size(t.handle, E, s, tuples) for s in (D, F))
+    assert sa.sa_schedule_cost(t.handle, E, D, tuples)["resolved"] == sa.SA_SCHED_ASSOC_RIGHT and need >= J * M * 4 > 4 * nest
+    ref, _ = t.run("spmmh_gemm", ops, sched=F)                     # leaves a workspace with too little room for the default
+    stream = torch.cuda.current_stream().cuda_stream
+    ws = torch.empty(max(nest, 256), dtype=torch.uint8, device="cuda")
+    out = torch.full_like(ref, float("nan"))
+    sa.sa_run(t.handle, E, D, tuples, out.data_ptr(), ws.data_ptr() if nest else None, nest, stream)
+    assert torch.equal(out, ref)
+    for s in (sa.SA_SCHED_ASSOC_RIGHT, F if nest else sa.SA_SCHED_ASSOC_RIGHT):        # named schedules say what they lack
+        with pytest.raises(sa.SaError) as e:
+            sa.sa_run(t.handle, E, s, tuples, out.data_ptr(), None, 0, stream)
+        assert e.value.status == sa.SA_E_WORKSPACE
+    total = torch.cuda.get_device_properties(0).total_memory
+    torch.cuda.synchronize()
+    torch.cuda.empty_cache()
+    try:
+        torch.cuda.set_per_process_memory_fraction((torch.cuda.memory_reserved() + need // 2) / total)
+        out, _ = t.run("spmmh_gemm", ops)
+        assert torch.equal(out, ref)
+    finally:
+        torch.cuda.set_per_process_memory_fraction(1.0)
+    out, ws = t.run("spmmh_gemm", ops)                             # and with memory the faster order, after the smaller workspace
+    assert ws.numel() >= need and not torch.equal(out, ref)
+    assert float((out - ref).norm() / ref.norm()) < 1e-5
