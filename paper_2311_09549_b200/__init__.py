@@ -8,6 +8,8 @@ built (``python paper_2311_09549_b200/build.py``); there is no CPU path.
 import ctypes
 import os
 import struct
+import threading
+from threading import get_ident
 
 import numpy as np
 
@@ -110,6 +112,7 @@ class TorchAllocator:
         self._torch = torch
         self.device = torch.device("cuda", device)
         self.live = {}
+        self.stream = torch.cuda.current_stream(device).cuda_stream       # of the allocations: sa_tensor_create makes them all
         self._alloc = _ALLOC_FN(self._do_alloc)
         self._release = _RELEASE_FN(self._do_release)
         self.struct = SaAllocator(self._alloc, self._release, None)
@@ -124,6 +127,11 @@ class TorchAllocator:
 
     def _do_release(self, ptr, _ctx):
         self.live.pop(ptr, None)
+
+    def record_stream(self, stream):
+        """The arrays are about to be used on `stream`: once released they are not handed out before its work is done."""
+        for buf in list(self.live.values()):
+            buf.record_stream(stream)
 
 
 def sa_tensor_create(order, dims, nnz, coords, vals, fmt, device, dev_alloc=None):
@@ -257,13 +265,17 @@ class SparseTensor:
         self._allocator = TorchAllocator(device) if device >= 0 else None
         self.handle = sa_tensor_create(self.order, self.dims, len(vals), coords, vals, fmt, device,
                                        self._allocator.struct if self._allocator else None)
-        self._ws = None
+        self._torch = self._allocator._torch if self._allocator else None
+        self._ws = {}                              # workspaces by (thread, stream): calls that may overlap share none
+        self._ws_lock = threading.Lock()
+        self._streams = {self._allocator.stream} if self._allocator else set()     # streams the device arrays are known to be used on
         self._fibers = int(self.info()[1][1])      # rows of a sparse output; a handle is immutable
 
     def close(self):
         if self.handle:
             sa_destroy(self.handle)
             self.handle = None
+            self._ws.clear()
 
     def __del__(self):
         try:
@@ -275,8 +287,14 @@ class SparseTensor:
         return sa_tensor_info(self.handle, self.order)
 
     def run(self, expr, operands, out=None, sched=SA_SCHED_DEFAULT, stream=None, workspace=None):
-        """operands: torch float32 CUDA matrices (row-major).  Returns (out, workspace)."""
-        import torch
+        """operands: torch float32 CUDA matrices (row-major).  Returns (out, workspace).
+
+        The call is enqueued on ``stream`` (default: torch's current one), which has to be ordered behind whatever writes the
+        operands.  ``out`` and the workspace are allocated there unless given; the workspace is kept for later calls from the same
+        thread on the same stream, at most ``MAX_WORKSPACES`` of them per tensor."""
+        torch = self._torch
+        if torch is None:
+            raise SaError(SA_E_ARG, "sa_run")       # a host-only handle
         expr = _EXPR_OF.get(expr, expr)
         desc = []
         for t in operands:
@@ -286,26 +304,40 @@ class SparseTensor:
         if n not in _PACK_OPS:
             self._size(expr, sched, desc)           # raises: no expression takes that many operands
         packed = _PACK_OPS[n](*desc)
+        here = torch._C._cuda_getCurrentRawStream(self.device)
+        sid = here if stream is None else stream.cuda_stream
         own = workspace is None
         if own:
-            workspace = self._ws
+            key = (get_ident(), sid)
+            workspace = self._ws.get(key)
             # kernel 3 by default runs a slower schedule in a small workspace, where the others report SA_E_WORKSPACE
             if workspace is None or (expr == SA_EXPR_SPMMH_GEMM and workspace.numel() < self._packed_size(expr, sched, packed, n)):
-                workspace = self._grow(expr, sched, desc)
+                workspace = self._grow(expr, sched, desc, key, stream)
         if out is None:
             try:
                 shape = self.out_shape(expr, operands)
             except IndexError:
                 self._size(expr, sched, desc)       # raises: too few operands for the expression
                 raise
-            out = torch.empty(shape, dtype=torch.float32, device=workspace.device)
-        s = torch.cuda.current_stream(self.device) if stream is None else stream
-        st = _run_packed(self.handle, int(expr), int(sched), packed, n, out.data_ptr(), workspace.data_ptr(), workspace.numel(), s.cuda_stream)
+            if sid == here:
+                out = torch.empty(shape, dtype=torch.float32, device=workspace.device)
+            else:
+                out = self._empty(shape, torch.float32, stream)
+                out.record_stream(torch.cuda.current_stream(self.device))
+        if sid not in self._streams:
+            self._streams.add(sid)
+            s = torch.cuda.current_stream(self.device) if stream is None else self._torch_stream(stream)
+            if not isinstance(s, torch.cuda.ExternalStream):       # (such a stream may be gone before the tensor is)
+                self._allocator.record_stream(s)
+        st = _run_packed(self.handle, int(expr), int(sched), packed, n, out.data_ptr(), workspace.data_ptr(), workspace.numel(), sid)
         if own and st == SA_E_WORKSPACE:            # nothing was enqueued: this call needs more than the ones before it
-            workspace = self._grow(expr, sched, desc)
-            st = _run_packed(self.handle, int(expr), int(sched), packed, n, out.data_ptr(), workspace.data_ptr(), workspace.numel(), s.cuda_stream)
+            workspace = self._grow(expr, sched, desc, key, stream)
+            st = _run_packed(self.handle, int(expr), int(sched), packed, n, out.data_ptr(), workspace.data_ptr(), workspace.numel(), sid)
         _check(st, "sa_run")
         return out, workspace
+
+    #: Workspaces a tensor keeps; beyond that the oldest goes back to torch's allocator.
+    MAX_WORKSPACES = 8
 
     def _size(self, expr, sched, desc):
         return sa_workspace_size(self.handle, expr, sched, [tuple(desc[i:i + 4]) for i in range(0, len(desc), 4)])
@@ -315,17 +347,35 @@ class SparseTensor:
         _check(_size_packed(self.handle, int(expr), int(sched), packed, n, ctypes.byref(need)), "sa_workspace_size")
         return need.value
 
-    def _grow(self, expr, sched, desc):
-        import torch
-        need, dev = self._size(expr, sched, desc), torch.device("cuda", self.device)
+    def _torch_stream(self, stream):
+        torch = self._torch
+        return stream if isinstance(stream, torch.cuda.Stream) else torch.cuda.ExternalStream(stream.cuda_stream, device=self.device)
+
+    def _empty(self, shape, dtype, stream):
+        """torch.empty on a stream (None: the current one)."""
+        torch = self._torch
+        if stream is None:
+            return torch.empty(shape, dtype=dtype, device=self.device)
+        with torch.cuda.stream(self._torch_stream(stream)):
+            return torch.empty(shape, dtype=dtype, device=self.device)
+
+    def _grow(self, expr, sched, desc, key, stream):
+        """A new workspace for `key`, from that stream's share of torch's allocator: what it replaces is given back in that
+        stream's order."""
+        torch = self._torch
         try:
-            self._ws = torch.empty(max(need, 256), dtype=torch.uint8, device=dev)
+            ws = self._empty(max(self._size(expr, sched, desc), 256), torch.uint8, stream)
         except torch.OutOfMemoryError:
             if expr != SA_EXPR_SPMMH_GEMM or sched != SA_SCHED_DEFAULT:
                 raise
             # no room for the J x M temporary of kernel 3's faster order: sa_run takes the row nest
-            self._ws = torch.empty(max(self._size(expr, SA_SCHED_FUSED, desc), 256), dtype=torch.uint8, device=dev)
-        return self._ws
+            ws = self._empty(max(self._size(expr, SA_SCHED_FUSED, desc), 256), torch.uint8, stream)
+        with self._ws_lock:
+            self._ws.pop(key, None)
+            while len(self._ws) >= self.MAX_WORKSPACES:
+                del self._ws[next(iter(self._ws))]
+            self._ws[key] = ws
+        return ws
 
     def out_shape(self, expr, operands):
         expr = _EXPR_OF.get(expr, expr)

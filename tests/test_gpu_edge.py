@@ -612,3 +612,86 @@ def test_spmmh_gemm_default_runs_in_the_workspace_it_is_given(sa):
     out, ws = t.run("spmmh_gemm", ops)                             # and with memory the faster order, after the smaller workspace
     assert ws.numel() >= need and not torch.equal(out, ref)
     assert float((out - ref).norm() / ref.norm()) < 1e-5
+
+
+def _cut_rows_case(sa, J=3000):
+    """Matrix whose long rows are summed from partial rows in the workspace, its operands for kernel 1, and the result."""
+    import torch
+    w = configs.make_sddmm_spmm("streams", 51, 2_000, J, 60_000, 1.5, 1_500, 64, 64)
+    t = sa.SparseTensor(w.dims, w.coords, w.vals, sa.SA_FMT_CSR, device=0)
+    ops = [torch.from_numpy(x).cuda() for x in w.dense]
+    ref, ws = t.run("sddmm_spmm", ops)
+    torch.cuda.synchronize()
+    assert sa.sa_tensor_worklist(t.handle)[0][3] > 0
+    return t, ops, ref, ws
+
+
+def test_calls_on_two_streams_share_no_workspace(sa):
+    import torch
+    t, ops, ref, ws = _cut_rows_case(sa)
+    streams = [torch.cuda.Stream() for _ in range(2)]
+    outs, spaces = [], [ws]
+    for s in streams:
+        s.wait_stream(torch.cuda.current_stream())
+    for rep in range(50):
+        for s in streams:
+            out, w = t.run("sddmm_spmm", ops, stream=s)
+            outs.append(out)
+            spaces.append(w)
+    torch.cuda.synchronize()
+    assert len({w.data_ptr() for w in spaces}) == 3
+    assert all(torch.equal(o, ref) for o in outs)
+
+
+def test_calls_from_two_threads_share_no_workspace(sa):
+    import threading
+    import torch
+    t, ops, ref, ws = _cut_rows_case(sa)
+    spaces, outs, meet = [ws], [], threading.Barrier(2)
+
+    def work():
+        meet.wait()
+        got = [t.run("sddmm_spmm", ops) for _ in range(50)]
+        outs.extend(o for o, _ in got)
+        spaces.extend(w for _, w in got)
+
+    threads = [threading.Thread(target=work) for _ in range(2)]
+    for x in threads:
+        x.start()
+    for x in threads:
+        x.join()
+    torch.cuda.synchronize()
+    assert len({w.data_ptr() for w in spaces}) == 3
+    assert all(torch.equal(o, ref) for o in outs)
+    assert len(t._ws) <= t.MAX_WORKSPACES
+
+
+def test_workspaces_kept_by_a_tensor_are_bounded_and_given_back(sa):
+    import torch
+    t, ops, ref, _ = _cut_rows_case(sa)
+    before = torch.cuda.memory_allocated()
+    for _ in range(3 * t.MAX_WORKSPACES):
+        out, _ws = t.run("sddmm_spmm", ops, stream=torch.cuda.Stream())
+        torch.cuda.synchronize()
+        assert torch.equal(out, ref)
+    assert len(t._ws) == t.MAX_WORKSPACES
+    del out, _ws
+    t.close()
+    assert not t._ws and torch.cuda.memory_allocated() < before
+
+
+def test_workspace_grows_after_a_smaller_call_on_a_side_stream(sa):
+    import torch
+    t, ops, ref, _ = _cut_rows_case(sa)
+    F = torch.ones(64, 32, device="cuda")
+    full, _ = t.run("sddmm_spmm_gemm", ops + [F])
+    s = torch.cuda.Stream()
+    s.wait_stream(torch.cuda.current_stream())
+    small, w1 = t.run("sddmm_spmm", ops, stream=s)
+    n1 = w1.numel()
+    del w1
+    big, w2 = t.run("sddmm_spmm_gemm", ops + [F], stream=s)        # needs the row temporary as well
+    again, w3 = t.run("sddmm_spmm", ops, stream=s)
+    s.synchronize()
+    assert w2.numel() > n1 and w3 is w2
+    assert torch.equal(small, ref) and torch.equal(again, ref) and torch.equal(big, full)
