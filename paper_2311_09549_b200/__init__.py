@@ -319,11 +319,15 @@ class SparseTensor:
             except IndexError:
                 self._size(expr, sched, desc)       # raises: too few operands for the expression
                 raise
-            if sid == here:
-                out = torch.empty(shape, dtype=torch.float32, device=workspace.device)
-            else:
-                out = self._empty(shape, torch.float32, stream)
-                out.record_stream(torch.cuda.current_stream(self.device))
+            try:
+                if sid == here:
+                    out = torch.empty(shape, dtype=torch.float32, device=self.device)
+                else:
+                    out = self._empty(shape, torch.float32, stream)
+                    out.record_stream(torch.cuda.current_stream(self.device))
+            except RuntimeError:
+                self._size(expr, sched, desc)       # raises if the operands make no sense, which may be why there is no room
+                raise
         if sid not in self._streams:
             self._streams.add(sid)
             s = torch.cuda.current_stream(self.device) if stream is None else self._torch_stream(stream)

@@ -695,3 +695,25 @@ def test_workspace_grows_after_a_smaller_call_on_a_side_stream(sa):
     s.synchronize()
     assert w2.numel() > n1 and w3 is w2
     assert torch.equal(small, ref) and torch.equal(again, ref) and torch.equal(big, full)
+
+
+def test_output_is_on_the_tensor_device_whatever_the_workspace_is(sa, monkeypatch):
+    """A caller's workspace may be pinned host memory; the output that run allocates may not.  Nothing is launched here."""
+    import torch
+    t, ops, ref, _ = _cut_rows_case(sa)
+    monkeypatch.setattr(sa, "_run_packed", lambda *a: sa.SA_OK)
+    out, _ = t.run("sddmm_spmm", ops, workspace=torch.empty(1 << 20, dtype=torch.uint8).pin_memory())
+    assert out.device == ref.device
+
+
+def test_operands_that_make_no_sense_are_refused_before_their_output_is_too_large(sa):
+    import torch
+    t = sa.SparseTensor((2_000_000, 50, 60), np.array([[5, 6, 7]], np.int32), np.ones(1, np.float32), sa.SA_FMT_CSF, device=0)
+    ops = [torch.ones(50, 512, device="cuda"), torch.ones(60, 512, device="cuda")]     # 2.1 TB of output at ranks it is not built for
+    good = [torch.ones(50, 16, device="cuda"), torch.ones(60, 16, device="cuda")]
+    for _ in range(2):
+        with pytest.raises(sa.SaError) as e:
+            t.run("spttm_ttm3", ops)
+        assert e.value.status == sa.SA_E_UNSUPPORTED
+        out, _ws = t.run("spttm_ttm3", good)       # leaves a workspace, so that the second round does not ask for its size first
+        assert float(out[5, 0, 0]) == 1.0
