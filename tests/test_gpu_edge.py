@@ -600,15 +600,17 @@ def test_spmmh_gemm_default_runs_in_the_workspace_it_is_given(sa):
         with pytest.raises(sa.SaError) as e:
             sa.sa_run(t.handle, E, s, tuples, out.data_ptr(), None, 0, stream)
         assert e.value.status == sa.SA_E_WORKSPACE
-    total = torch.cuda.get_device_properties(0).total_memory
-    torch.cuda.synchronize()
-    torch.cuda.empty_cache()
-    try:
-        torch.cuda.set_per_process_memory_fraction((torch.cuda.memory_reserved() + need // 2) / total)
-        out, _ = t.run("spmmh_gemm", ops)
-        assert torch.equal(out, ref)
-    finally:
-        torch.cuda.set_per_process_memory_fraction(1.0)
+    empty = t._empty
+
+    def no_room(shape, *a):
+        if shape == need:
+            raise torch.OutOfMemoryError("as the allocator says it")
+        return empty(shape, *a)
+
+    t._empty = no_room
+    out, _ = t.run("spmmh_gemm", ops)
+    assert torch.equal(out, ref)
+    t._empty = empty
     out, ws = t.run("spmmh_gemm", ops)                             # and with memory the faster order, after the smaller workspace
     assert ws.numel() >= need and not torch.equal(out, ref)
     assert float((out - ref).norm() / ref.norm()) < 1e-5
