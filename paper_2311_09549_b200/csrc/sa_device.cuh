@@ -72,13 +72,13 @@ static inline bool sa_set_smem_once(Kernel kernel, int bytes, bool (&done)[SA_MA
 
 // ---- PTX helpers shared by the kernels
 
-// x = hi + lo with hi the upper 19 bits of x (a TF32 number) and lo = x - hi (exact in fp32), of which the tensor core
-// reads the upper 19 bits.  hi.hi + hi.lo + lo.hi then misses the true product by about 2^-20 relative.  (cvt.rna.tf32
-// costs several instructions per value on this target; plain masking is one.)
+// x = hi + lo + rest in TF32 numbers: hi the upper 19 bits of x, lo the upper 19 bits of x - hi (exact in fp32).  hi.hi +
+// hi.lo + lo.hi then misses the true product by about 2^-20 relative.  (cvt.rna.tf32 costs several instructions per value on
+// this target; plain masking is one.)
 __device__ __forceinline__ void split_tf32(float x, uint32_t &hi, uint32_t &lo)
 {
     hi = __float_as_uint(x) & 0xffffe000u;
-    lo = __float_as_uint(x - __uint_as_float(hi));
+    lo = __float_as_uint(x - __uint_as_float(hi)) & 0xffffe000u;
 }
 
 __device__ __forceinline__ void mma_m16n8k8_tf32(float (&c)[4], const uint32_t (&a)[4], const uint32_t (&b)[2])
