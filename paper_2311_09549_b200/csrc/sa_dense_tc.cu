@@ -518,7 +518,7 @@ sa_status launch_tc(int64_t rows, const float *A, int64_t lda, const float *H, i
 {
     using G = tc_cfg<L, M, HAD>;
     auto k = gemm_tc_kernel<L, M, HAD>;
-    static bool attr[SA_MAX_DEVICE_FLAGS];
+    static sa_device_flags attr;
     if (!sa_set_smem_once(k, int(G::SMEM), attr)) return SA_E_CUDA;
     int dev = 0, sms = 148;
     if (cudaGetDevice(&dev) == cudaSuccess) cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);

@@ -3,6 +3,7 @@
 
 #include <cuda_runtime.h>
 #include <algorithm>
+#include <atomic>
 #include <cstdint>
 
 #include "sa_internal.h"
@@ -57,16 +58,19 @@ static inline sa_limits sa_make_limits(const sa_tensor *t, int64_t gather_rows, 
 }
 
 // Opt a kernel into `bytes` of dynamic shared memory once per device instead of once per launch (the attribute is
-// per device; `done` is the caller's flag array, one entry per device ordinal).
+// per device; `done` is the caller's flags, one per device ordinal).  Host threads may launch at the same time: the
+// attribute may then be set more than once, to the same value.
 constexpr int SA_MAX_DEVICE_FLAGS = 64;
+struct sa_device_flags { std::atomic<bool> set[SA_MAX_DEVICE_FLAGS]; };
 template <typename Kernel>
-static inline bool sa_set_smem_once(Kernel kernel, int bytes, bool (&done)[SA_MAX_DEVICE_FLAGS])
+static inline bool sa_set_smem_once(Kernel kernel, int bytes, sa_device_flags &done)
 {
     int dev = 0;
     if (cudaGetDevice(&dev) != cudaSuccess) return false;
-    if (dev >= 0 && dev < SA_MAX_DEVICE_FLAGS && done[dev]) return true;
+    const bool keep = dev >= 0 && dev < SA_MAX_DEVICE_FLAGS;
+    if (keep && done.set[dev].load(std::memory_order_acquire)) return true;
     if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes) != cudaSuccess) return false;
-    if (dev >= 0 && dev < SA_MAX_DEVICE_FLAGS) done[dev] = true;
+    if (keep) done.set[dev].store(true, std::memory_order_release);
     return true;
 }
 

@@ -503,7 +503,7 @@ sa_status run(const sa_tensor *t, const sa_dense *ops, float *out, void *ws, boo
     if (!right) {
         float *partial = static_cast<float *>(ws);
         auto kern = spmm_gemm_left_kernel<L, M, false>;
-        static bool attr[SA_MAX_DEVICE_FLAGS];
+        static sa_device_flags attr;
         static resident_cache resident;
         if (!sa_set_smem_once(kern, int(smem), attr)) return SA_E_CUDA;
         const int64_t want = (n_items + SA_WARPS_PER_CTA - 1) / SA_WARPS_PER_CTA;
@@ -548,7 +548,7 @@ sa_status run_hadamard(const sa_tensor *t, const sa_dense *ops, float *out, void
     }
     float *partial = static_cast<float *>(ws);
     auto kern = spmm_gemm_left_kernel<L, M, true>;
-    static bool attr[SA_MAX_DEVICE_FLAGS];
+    static sa_device_flags attr;
     static resident_cache resident;
     if (!sa_set_smem_once(kern, int(smem), attr)) return SA_E_CUDA;
     const int64_t want = (n_items + SA_WARPS_PER_CTA - 1) / SA_WARPS_PER_CTA;
@@ -625,7 +625,7 @@ static sa_status dense_gemm(int64_t rows, const float *A, int64_t lda, const flo
 {
     using GC = gemm_bf16_cfg<L, M>;
     auto gk = gemm_bf16x3_kernel<L, M>;
-    static bool attr[SA_MAX_DEVICE_FLAGS];
+    static sa_device_flags attr;
     static resident_cache resident;
     if (!sa_set_smem_once(gk, int(GC::SMEM), attr)) return SA_E_CUDA;
     const int64_t ctas = std::min<int64_t>((rows + GC::BM - 1) / GC::BM, resident_ctas(reinterpret_cast<const void *>(gk), GC::SMEM, resident));

@@ -664,7 +664,7 @@ cudaError_t launch(const sa_ttm3_view &v, const sa_dense &first, const sa_dense 
     constexpr size_t smem = size_t(SA_TTM3_WARPS) * cfg<L, M>::WARP_BYTES;
     const bool six = wl.six_blocks >= 0 ? wl.six_blocks != 0 : v.nnz < int64_t(512) * int64_t(wl.items.size());   // mean unit below 512 nonzeros
     auto kern = six ? ttm3_kernel<L, M, cfg<L, M>::MINCTAS_SIX, HAD> : ttm3_kernel<L, M, cfg<L, M>::MINCTAS, HAD>;
-    static bool attr_four[SA_MAX_DEVICE_FLAGS], attr_six[SA_MAX_DEVICE_FLAGS];     // per instantiation of this launcher
+    static sa_device_flags attr_four, attr_six;     // per instantiation of this launcher
     if (!sa_set_smem_once(kern, int(smem), six ? attr_six : attr_four)) return cudaGetLastError();
     dbg_limits lim;
     lim.status = v.status;
@@ -826,7 +826,7 @@ static __device__ __align__(256) float sa_static_scratch[SA_STATIC_SCRATCH_BYTES
 namespace {
 
 constexpr int SA_MAX_DEVICES = 64;
-float *g_static_scratch_addr[SA_MAX_DEVICES];   // device address of sa_static_scratch, per device; set once
+std::atomic<float *> g_static_scratch_addr[SA_MAX_DEVICES];   // device address of sa_static_scratch, per device; set once
 
 // In host code `sa_static_scratch` only names the symbol; the address a kernel can use has to be
 // asked for, with the owning device current.

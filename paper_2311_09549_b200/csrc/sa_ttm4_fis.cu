@@ -442,7 +442,7 @@ sa_status sa_launch_ttm4_fissioned(const sa_tensor *t, const sa_dense *ops, floa
     if (n_sub > 0) {
         const bool contig = ops[1].ld == R && ops[2].ld == R;
         auto kern = contig ? ttm4_subtree_kernel<true> : ttm4_subtree_kernel<false>;
-        static bool attr_contig[SA_MAX_DEVICE_FLAGS], attr_strided[SA_MAX_DEVICE_FLAGS];
+        static sa_device_flags attr_contig, attr_strided;
         if (!sa_set_smem_once(kern, SUB_SMEM, contig ? attr_contig : attr_strided)) return SA_E_CUDA;
         const int64_t ctas = (n_sub + SA_WARPS_PER_CTA - 1) / SA_WARPS_PER_CTA;
         kern<<<(unsigned)ctas, 256, SUB_SMEM, stream>>>(t->wl4_sub.d_items, n_sub, t->d_pos[2], t->d_pos[3], t->d_crd[2],
@@ -463,7 +463,7 @@ sa_status sa_launch_ttm4_fissioned(const sa_tensor *t, const sa_dense *ops, floa
         int dev = 0, sms = 148;
         if (cudaGetDevice(&dev) == cudaSuccess) cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
         const int64_t ctas = std::min<int64_t>((n_items + SA_WARPS_PER_CTA - 1) / SA_WARPS_PER_CTA, int64_t(sms) * 2);
-        static bool attr_slice[SA_MAX_DEVICE_FLAGS];
+        static sa_device_flags attr_slice;
         if (!sa_set_smem_once(ttm4_slice_kernel, SL_SMEM, attr_slice)) return SA_E_CUDA;
         ttm4_slice_kernel<<<(unsigned)ctas, 256, SL_SMEM, stream>>>(wl.d_items, n_items, t->d_crd[1], T2, ops[0].ptr, uint32_t(ops[0].ld),
                                                                   out, part2, lim);
