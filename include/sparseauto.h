@@ -216,8 +216,8 @@ sa_status sa_tensor_worklist(const sa_tensor *t, int which, int64_t *counts, int
  *               consecutive ones are the pieces of one chunk of a large slice, summed by one thread
  *               block.  Every later task holds up to 16 whole small slices.
  *   stream_f0   HOST [n_items * 4]: inside an item the warp's four groups of eight lanes each stream a
- *               contiguous part of the nonzeros [p0, p1).  With b = p0 rounded down to a multiple of 8
- *               and s = ceil((p1 - b) / 4) rounded up to a multiple of 8, part q is
+ *               contiguous part of the nonzeros [p0, p1).  With b = p0 rounded down to a multiple of 16
+ *               and s = ceil((p1 - b) / 4) rounded up to a multiple of 16, part q is
  *               [b + q s, b + (q + 1) s) clipped to [p0, p1); stream_f0[4 n + q] is the level-1 fiber
  *               that holds the first nonzero of part q of item n (f0 of the item if the part is empty).
  * NULL outputs are skipped.  Errors: SA_E_ARG, SA_E_FORMAT (not a CSF tensor).
@@ -240,7 +240,7 @@ sa_status sa_workspace_size(const sa_tensor *t, sa_expr expr, sa_schedule sched,
  *   moved_bytes     bytes the schedule's kernels load and store: streams of B once, the output once, dense
  *                   operands that are read in order once, gathered rows once per use (a row served by the
  *                   last-level cache still occupies the load path), temporaries in the workspace written and
- *                   read.  This is the time term the default schedule is chosen by (the chains are bound by
+ *                   read (partial tiles and rows of cut slices and rows are not counted).  This is the time term the default schedule is chosen by (the chains are bound by
  *                   memory traffic here, not by loop iterations).
  *   temp_elements   dense temporaries that pass values from producer to consumer nests, in elements: the
  *                   paper's auxiliary memory (Section 4.2; table of auxiliary memory requirements, Section 6),

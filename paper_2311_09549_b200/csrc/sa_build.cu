@@ -208,17 +208,13 @@ void append_empty_slices(sa_tensor *t, sa_worklist &wl)
     }
 }
 
-// Items by decreasing number of nonzeros, items of equal length in the order they have.  Lengths are bounded by the list's
-// item size, so they are counted: building a 500 K nonzero CSR tensor takes 4.5 ms, with a comparison sort 5.6.
+// Items by decreasing number of nonzeros, items of equal length in the order they have.  Lengths are at most 4096 in all lists,
+// so they are counted: building a 500 K nonzero CSR tensor takes 4.5 ms, with a comparison sort 5.6.
 void longest_first(std::vector<sa_item> &items)
 {
     auto len = [](const sa_item &x) { return size_t(x.p1 - x.p0); };
     size_t top = 0;
     for (const sa_item &x : items) top = std::max(top, len(x));
-    if (top > (size_t(1) << 16)) {
-        std::stable_sort(items.begin(), items.end(), [&](const sa_item &a, const sa_item &b) { return len(a) > len(b); });
-        return;
-    }
     std::vector<size_t> at(top + 2, 0);                  // at[top - len]: where the next item of that length goes
     for (const sa_item &x : items) ++at[top - len(x) + 1];
     for (size_t k = 1; k < at.size(); ++k) at[k] += at[k - 1];
@@ -327,7 +323,7 @@ int64_t ttm3_unit(const std::vector<int64_t> &len, int *six_blocks)
     constexpr int64_t LARGEST = TTM3_UNITS[0];
     int64_t nnz = 0;
     for (const int64_t n : len) nnz += n;
-    if (nnz >= LARGEST * 2 * 148 * 16) return LARGEST;
+    if (nnz >= LARGEST * 2 * SA_SMS * 16) return LARGEST;
     std::vector<int64_t> short_len(size_t(LARGEST) + 1, 0), long_len;
     for (const int64_t n : len)
         if (n > LARGEST) long_len.push_back(n);
@@ -340,12 +336,12 @@ int64_t ttm3_unit(const std::vector<int64_t> &len, int *six_blocks)
         const int64_t slots = ttm3_slots(len, u);
         if (slots > most) continue;
         units[count] = u;
-        time[count] = ttm3_time(short_len, long_len, u, slots, 4 * 148);
+        time[count] = ttm3_time(short_len, long_len, u, slots, 4 * SA_SMS);
         best = std::min(best, time[count++]);
     }
     int x = 0;
     while (time[x] > 1.03 * best) ++x;
-    *six_blocks = 1.3 * ttm3_time(short_len, long_len, units[x], ttm3_slots(len, units[x]), 6 * 148) < time[x];
+    *six_blocks = 1.3 * ttm3_time(short_len, long_len, units[x], ttm3_slots(len, units[x]), 6 * SA_SMS) < time[x];
     return units[x];
 }
 
@@ -713,7 +709,7 @@ void build_rows(const std::vector<int64_t> &pos, int64_t I, sa_worklist &wl, int
 // CSR, kernel 1 (fused SDDMM -> SpMM): an item is what one group of eight lanes walks, a range of whole short rows or a
 // piece of a long row with a partial row for the fix-up kernel.
 //   Size: `target` nonzeros, at most 256, less where the tensor would not give every group of a full machine
-//     (148 SMs x 64 groups) two items, at least 16: a group needs about a microsecond per four nonzeros, and on a small tensor
+//     (64 groups per SM) two items, at least 16: a group needs about a microsecond per four nonzeros, and on a small tensor
 //     that chain is the whole run time (60 k nonzeros, rows of up to 1500: 28 us; with a warp per item of up to 1024
 //     nonzeros 78 us).  A row counts as long above 64 nonzeros (1M x 1M, 30 M nonzeros: above 64 / 128 / 256 / 1024
 //     1.01 / 1.03 / 1.05 / 1.09 ms).  Rows per range: 8, at least 4, by the same rule, since a
@@ -732,9 +728,9 @@ void build_rows(const std::vector<int64_t> &pos, int64_t I, sa_worklist &wl, int
 void build_sddmm(const std::vector<int64_t> &pos, const std::vector<int32_t> &crd, int64_t I, sa_worklist &wl)
 {
     constexpr int64_t COL_BLOCK = 32768, MIN_PIECE = 32, CUT_ROW = 128, MIN_REST = 16;
-    const int64_t target = std::min<int64_t>(256, std::max<int64_t>(16, pos[size_t(I)] / (2 * 148 * 64)));
+    const int64_t target = std::min<int64_t>(256, std::max<int64_t>(16, pos[size_t(I)] / (2 * SA_SMS * 64)));
     const int64_t long_row = std::min<int64_t>(std::max<int64_t>(target, 48), 64);
-    const int64_t max_rows = std::min<int64_t>(8, std::max<int64_t>(4, I / (2 * 148 * 64)));
+    const int64_t max_rows = std::min<int64_t>(8, std::max<int64_t>(4, I / (2 * SA_SMS * 64)));
     struct piece_rec { uint32_t key; sa_item it; };
     std::vector<piece_rec> pieces;
     std::vector<sa_item> ranges;
@@ -801,7 +797,7 @@ void sa_build_worklists(sa_tensor *t)
         build_ttm3(t, t->wl_main);
         // kernel 7 walks the tensor as a sparse matrix whose rows are the (i,j) fibers: 1024 nonzeros per warp, fewer where
         // that would not give every warp slot of a full machine four items
-        build_rows(t->pos[2], t->count[1], t->wl_aux, std::min<int64_t>(1024, std::max<int64_t>(128, t->nnz / (4 * 148 * 32) / 32 * 32)), 4096, 4096, 2048, true);
+        build_rows(t->pos[2], t->count[1], t->wl_aux, std::min<int64_t>(1024, std::max<int64_t>(128, t->nnz / (4 * SA_SMS * 32) / 32 * 32)), 4096, 4096, 2048, true);
     }
     if (t->fmt == SA_FMT_CSF && t->order == 4) {
         build_ttm4(t, t->wl_main, t->wl_sub, t->wl_aux);
@@ -813,7 +809,7 @@ void sa_build_worklists(sa_tensor *t)
         build_sddmm(t->pos[1], t->crd[1], t->dims[0], t->wl_main);
         // SpMM -> GEMM (both orders): about 256 nonzeros per item, which one lane group or warp walks as a chain; fewer where
         // the tensor would not give every group of a full machine two items
-        const int64_t target = std::min<int64_t>(256, std::max<int64_t>(32, t->nnz / (2 * 148 * 64)));
+        const int64_t target = std::min<int64_t>(256, std::max<int64_t>(32, t->nnz / (2 * SA_SMS * 64)));
         build_rows(t->pos[1], t->dims[0], t->wl_aux, target, 16, 2 * target, target);
     }
     for (sa_worklist *wl : {&t->wl_main, &t->wl_aux, &t->wl_sub, &t->wl4_main, &t->wl4_aux, &t->wl4_sub}) {

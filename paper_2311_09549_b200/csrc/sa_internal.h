@@ -9,6 +9,7 @@
 #include "sparseauto.h"
 
 constexpr int SA_MAX_ORDER = 4;
+constexpr int SA_SMS = 148;          // SMs of the target; the lists are made for it whether or not a device is there
 constexpr int SA_WARPS_PER_CTA = 8;
 constexpr int SA_TTM3_WARPS = 4;     // warps per thread block of the order-3 kernel (they share one chunk of a large slice)
 
@@ -64,7 +65,7 @@ static inline void sa_unit3_streams(int64_t p0, int64_t p1, int64_t *lo, int64_t
     }
 }
 
-constexpr int SA_BIG_FIX = 32;
+constexpr int SA_BIG_FIX = 32;       // partial tiles from which the fix-up kernels give an entry more threads
 struct sa_worklist {
     std::vector<sa_item> items;   // [n_group_ctas * SA_WARPS_PER_CTA group items][warp items]
     std::vector<sa_fix> fix;
@@ -105,8 +106,9 @@ struct sa_tensor {
     float *d_vals = nullptr;
     uint32_t *d_endbits = nullptr;            // CSF: bit (p & 31) of word p / 32 is set when nonzero p is the last of
                                               // its last-level fiber ((i,j) for order 3, (i,j,k) for order 4)
-    int2 *d_nzpack = nullptr;                 // CSF: per nonzero (last-level index | end-of-fiber bit << 31, value bits): what the
-                                              // group-per-fiber kernels (kernel 7, order-4 subtree kernel) stream, one 8-byte load
+    int2 *d_nzpack = nullptr;                 // per nonzero (last-level index, value bits), one 8-byte load; CSF: end-of-fiber bit in
+                                              // bit 31 of the index.  What kernels 1 and 7, the SpMM stage of kernels 3 and 4 and the
+                                              // order-4 subtree kernel stream
     int32_t *d_status = nullptr;              // [4] device status word
 
     sa_worklist wl_main;                      // TTM3 / SDDMM-SpMM; order-4 CSF: the order-3 lists over the large (i,j) subtrees

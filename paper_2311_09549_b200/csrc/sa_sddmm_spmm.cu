@@ -1,7 +1,8 @@
 // Kernel 1 <SDDMM,SpMM>:  A(i,l) = sum_j B(i,j) (sum_k C(i,k) D(j,k)) E(j,l), scheduled as the
 // fused nest  i, j' < t ; k: t += B(i,j) C(i,k) D(j,k) , l: A(i,l) += t E(j,l) >  of the paper's
 // Table of kernels (Section 6): the sampled value is a scalar temporary that is consumed at once,
-// the sampled matrix is never written (auxiliary memory 1 in the paper's memory table).
+// the sampled matrix is never written (auxiliary memory 1 in the paper's memory table; what the workspace holds are partial
+// rows of long rows: L floats per 32 nonzeros at most, per 16 where the matrix is small).
 //
 // A warp is four groups of eight lanes; every group takes one work item (a range of short rows, or a piece of a long
 // row) and walks its nonzeros U at a time: a lane owns the float4 columns l, l + 8, ... of D(j,:), E(j,:), C(i,:) and of
@@ -175,7 +176,7 @@ sa_status sa_launch_sddmm_spmm(const sa_tensor *t, const sa_dense *ops, float *o
     const int64_t K = ops[0].cols, L = ops[2].cols;
     float *partial = static_cast<float *>(ws);
     float *sampled = nullptr;
-    for (int i = 0; i < 3; ++i)                       // the kernel addresses dense rows with 32-bit byte offsets
+    for (int i = 0; i < 3; ++i)                       // rows of C are found by 32-bit offsets; one limit for all operands
         if (ops[i].rows * ops[i].ld >= (int64_t(1) << 30)) return SA_E_UNSUPPORTED;
     if (materialize)
         sampled = reinterpret_cast<float *>(static_cast<char *>(ws) + sa_align256(size_t(t->wl_main.n_slots) * size_t(L) * sizeof(float)));

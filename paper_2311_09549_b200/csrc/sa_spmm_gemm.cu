@@ -462,8 +462,8 @@ int resident_ctas(const void *kernel, size_t smem, resident_cache &cache)
 }
 
 // Columns per table of E (see spmm_kernel).  Two tables read B twice, and pay where half of E finds a good part of itself in
-// L2 while all of it does not.  Whole chain, L = 128, M = 64, 20 nonzeros per row, J columns, 2 J / 1 table, us: 250 K
-// 103 / 98; 500 K (128 MB) 204 / 215; 1 M 451 / 467; 2 M 1050 / 1000.
+// the 126 MB of L2 while all of it does not: from 96 MB to 320 MB.  Whole chain, L = 128, M = 64, 20 nonzeros per row, J
+// columns, us with two tables / one: 250 K 103 / 98; 500 K (128 MB) 204 / 215; 1 M 451 / 467; 2 M 1050 / 1000.
 int spmm_part(int64_t J, int64_t M)
 {
     const int64_t bytes = J * M * int64_t(sizeof(float));

@@ -747,7 +747,7 @@ static bool ttmc3_fused_shape(int L3, int *grid, size_t *smem_bytes)
 // Accumulator elements the fused schedule of kernel 5 keeps per block; beyond this only the fissioned schedule runs.
 constexpr int64_t SA_TTMC3_FUSED_MAX = 8192;
 // Upper bound on the blocks of the fused schedule (sizes the workspace without asking the device).
-constexpr int SA_TTMC3_MAX_BLOCKS = 148 * 6 * 2;
+constexpr int SA_TTMC3_MAX_BLOCKS = SA_SMS * 6 * 2;
 
 bool sa_ttmc3_fused_ok(int64_t L3, int64_t M, int64_t N) { return L3 * M * N <= SA_TTMC3_FUSED_MAX; }
 size_t sa_ws_ttmc3_fused(int64_t L3, int64_t M, int64_t N) { return sa_align256(size_t(SA_TTMC3_MAX_BLOCKS) * size_t(L3 * M * N) * sizeof(float)); }
