@@ -6,7 +6,8 @@
 
 One "step" is one pass of the whole hot path (sa_run: main kernel(s) + fix-up) over the
 synthetic workload.  Default workload: config 2, the order-3 <SpTTM,TTM> chain at scale.
-Prints ONE JSON line (rank 0).  With N > 1 (torchrun, one rank per GPU) every rank runs an
+Prints ONE JSON line (rank 0), last; the default run prints a `per_config {...}` line per workload and
+schedule before it.  With N > 1 (torchrun, one rank per GPU) every rank runs an
 independent replica of the same workload -- the path has no exchange step -- and `value`
 is the aggregate over ranks, timed as the max over ranks.
 """
@@ -38,18 +39,18 @@ FALLBACK_HBM_GBS = 6650.0
 # captured at a quarter of its size (--scale mid) and scaled by the nonzeros, see the profiles.
 NCU_TRAFFIC = {
     2: {"kernel": "ttm3_kernel<32,32> (98.4 % of the step)", "source": "paper_2311_09549_b200/csrc/sa_ttm3.cu",
-        "sha256": "d271528bf8560d74d8ebb8f7f9ba89ac7fbdc56e9d1394806562f426a6710cd0",
-        "dram_bytes": 855337216, "profile": "profiles/ttm3_kernel_cfg2.md"},
+        "sha256": "698a23dccef6f7b97f8f186486a5099dcbfeac67c71cbc936d0910db206a0725",
+        "dram_bytes": 484427776 + 368994816},
     3: {"kernel": "sddmm_spmm_kernel<64,64> (98 % of the step)", "source": "paper_2311_09549_b200/csrc/sa_sddmm_spmm.cu",
-        "sha256": "62d9e7c5816d3e8a68fbd66376314c713d845ab8f17485ebce0bed0d2213b159",
-        "dram_bytes": 2604608512, "profile": "profiles/sddmm_spmm_kernel_cfg3.md"},
+        "sha256": "a34375e5f1a10c4348634a90868f17ecb43f9bf96e3c3fc5d932295c26bcd3d8",
+        "dram_bytes": 2580615168 + 278981632},
     (5, "fused"): {"kernel": "ttm4_fused_kernel (94 % of the step; counters of the quarter-size case x 4)",
-                   "source": "paper_2311_09549_b200/csrc/sa_ttm4.cu", "sha256": "77b9b58137c8e565f84a5ffd8762e5448c910f5befc50c3838442ae6007d0823",
-                   "dram_bytes": 4 * 424084480, "profile": "profiles/ttm4_kernels_cfg5.md"},
+                   "source": "paper_2311_09549_b200/csrc/sa_ttm4.cu", "sha256": "f6e8316914ad48188dfc5417cdd93bf51bb6a64f1611b1dbc1ba407ab5eabb08",
+                   "dram_bytes": 4 * (244847104 + 178882816)},
     (5, "fissioned"): {"kernel": "ttm4_subtree_kernel (pass 1 on the small subtrees, 51 % of the step; counters of the "
                                  "quarter-size case x 4)",
-                       "source": "paper_2311_09549_b200/csrc/sa_ttm4_fis.cu", "sha256": "be9575594a14a3633f6a12fba75381f08305534e694d350516c738ba12c2d61b",
-                       "dram_bytes": 4 * 663252480, "profile": "profiles/ttm4_kernels_cfg5.md"},
+                       "source": "paper_2311_09549_b200/csrc/sa_ttm4_fis.cu", "sha256": "9408bfd279ea3310255ff443d7c23c1b70f130301738ba229049381d419f39ee",
+                       "dram_bytes": 4 * (211818752 + 450940160)},
 }
 
 
@@ -409,7 +410,7 @@ def workload_label(cfg, sched):
              9: "kernel 8 <MTTKRP,GEMM> on the config-2 tensor, R=32 M=32",
              10: "kernel 7 <SpTTM,SpTTM> on the config-2 tensor, L=M=32, sparse output (one row per (i,j) fiber)",
              11: "kernel 5 <3D TTMC> on a flickr-3d-shaped tensor 320000x2820000x1600000 112.89M nnz L=M=N=16"}
-    return names[cfg] + (" (%s)" % sched if cfg in (4, 5, 6, 10, 11) else "")
+    return names[cfg] + (" (%s)" % sched if cfg in (4, 5, 6, 8, 10, 11) else "")
 
 
 def label(args):
@@ -450,7 +451,7 @@ def measure(sa, torch, dist, w, sched_name, steps, warmup, e2e_steps, dev, rank,
     tensor = sa.SparseTensor(w.dims, w.coords, w.vals, fmt, device=dev.index)
     build_s = time.perf_counter() - t0
     nnz, counts, n_chunks = tensor.info()
-    two_schedules = w.expr in ("spttm_ttm4", "ttmc3")          # fused / fissioned
+    two_schedules = w.expr in ("spttm_ttm4", "ttmc3", "spmmh_gemm")          # fused / fissioned, fused / right
     sched = {"left": sa.SA_SCHED_ASSOC_LEFT, "right": sa.SA_SCHED_ASSOC_RIGHT, "default": sa.SA_SCHED_DEFAULT,
              "fused": sa.SA_SCHED_FUSED if two_schedules else sa.SA_SCHED_DEFAULT, "fissioned": sa.SA_SCHED_FISSIONED}[sched_name]
     host_ops = [torch.from_numpy(np.ascontiguousarray(x)).pin_memory() for x in w.dense]
@@ -569,7 +570,7 @@ def main():
                     help="one workload only; without it: config 2 as the headline plus a per_config list of all five configs")
     ap.add_argument("--scale", default="full", choices=["full", "mid", "mini"])
     ap.add_argument("--sched", default=None, choices=["left", "right", "fused", "fissioned", "default"],
-                    help="schedule: left / right (association order, workloads 4 and 10), fused / fissioned (workloads 5, 6, 11), "
+                    help="schedule: left / right (association order, workloads 4 and 10), fused / fissioned (workloads 5, 6, 11), fused / right (workload 8), "
                          "default (the library's choice; also the default here, except workloads 4 and 10: right)")
     ap.add_argument("--no-cpu-baseline", action="store_true")
     ap.add_argument("--no-per-config", action="store_true")
@@ -614,6 +615,8 @@ def main():
     w = configs.make(args.workload, args.scale)
     if w.expr in ("spmm_gemm", "spttm_spttm"):
         sched_name = args.sched if args.sched in ("left", "right", "default") else "right"
+    elif w.expr == "spmmh_gemm":
+        sched_name = args.sched if args.sched in ("fused", "right", "default") else "default"
     elif w.expr in ("spttm_ttm4", "ttmc3"):
         sched_name = args.sched if args.sched in ("fused", "fissioned", "default") else "default"
     else:
@@ -634,7 +637,9 @@ def main():
             "e2e": rec["e2e"], "gpu_launches": rec["gpu_launches"], "clocks": rec["clocks"],
         }
         if "l2_gather_ceiling" in rec:
-            line["l2_gather_ceiling"] = rec["l2_gather_ceiling"]
+            # in full in the workload's own line
+            g = rec["l2_gather_ceiling"]
+            line["l2_gather_ceiling"] = {"what": g["what"], "ms": g["ms"], "gbs": g["gbs"], "copy_engine_ms": g["copy_engine_gather4"]["ms"]}
         kept = {args.workload: w}
         records = [dict(rec, config=args.workload)]
         if all_configs:
@@ -660,8 +665,11 @@ def main():
             nest = nest_sample(kept[args.workload])
             if nest is not None:
                 line["cpu_scheduled_nest"] = nest
+        # the records first, a line each, and the one JSON line of the run last and short
+        for r in records:
+            print("per_config " + json.dumps(r), flush=True)
         if all_configs:
-            line["per_config"] = records
+            line["per_config"] = [[r["config"], r["schedule"], round(r["value"], 4), round(r["ms_per_step"], 4)] for r in records]
         print(json.dumps(line), flush=True)
     if world > 1:
         dist.destroy_process_group()
