@@ -28,8 +28,8 @@ struct sd_cfg {
     static constexpr int CTAS = DQ + EQ <= 2 ? 3 : 2;
 };
 
-template <int K, int L>
-__global__ void __launch_bounds__(256, (sd_cfg<K, L>::CTAS))
+template <int K, int L, int CTAS>
+__global__ void __launch_bounds__(256, CTAS)
 sddmm_spmm_kernel(const sa_item *__restrict__ items, int64_t n_items, const int32_t *__restrict__ pos,
                   const int2 *__restrict__ nz, const float *__restrict__ C, uint32_t ldc, const float *__restrict__ D,
                   uint32_t ldd, const float *__restrict__ E, uint32_t lde, float *__restrict__ out, float *__restrict__ partial,
@@ -150,7 +150,11 @@ cudaError_t launch(const sa_tensor *t, const sa_dense *ops, float *out, float *p
     const int64_t n_items = int64_t(wl.items.size());
     const int64_t ctas = (n_items + 31) / 32;         // 32 groups per block
     if (ctas == 0) return cudaSuccess;
-    sddmm_spmm_kernel<K, L><<<(unsigned)ctas, 256, 0, stream>>>(
+    // Up to two and a half rounds of items the length of one is the run time, and two blocks per SM walk it faster (registers for
+    // more loads at a time).  K = L = 32, us, two / three blocks: 60 K nonzeros (4.7 K items) 14.4 / 16.5, 1 M on 20 K rows
+    // (22 K items) 29.3 / 31.8, 1 M on 300 K rows (38 K items) 61 / 53, on 200 K rows and 700 K columns (42 K) 83 / 69.
+    auto kern = n_items <= int64_t(5) * SA_SMS * 32 ? sddmm_spmm_kernel<K, L, 2> : sddmm_spmm_kernel<K, L, sd_cfg<K, L>::CTAS>;
+    kern<<<(unsigned)ctas, 256, 0, stream>>>(
         wl.d_items, n_items, t->d_pos[1], t->d_nzpack, ops[0].ptr, uint32_t(ops[0].ld), ops[1].ptr, uint32_t(ops[1].ld), ops[2].ptr,
         uint32_t(ops[2].ld), out, partial, sampled, sa_make_limits(t, t->dims[1], t->dims[0], wl.n_slots));
     return cudaGetLastError();
