@@ -176,9 +176,10 @@ sa_status sa_tensor_export(const sa_tensor *t, int level, int64_t *pos, int32_t 
  *   0  main list (order-3 CSF: units of kernel 6, grouped into tasks, see sa_tensor_tasks; CSR: rows for
  *      SA_EXPR_SDDMM_SPMM; order-4 CSF: the same kind of list over the (i,j) subtrees above 4096 nonzeros,
  *      out_row = index among those subtrees, [f0,f1) level-2 nodes)
- *   1  second list (CSR: rows for SA_EXPR_SPMM_GEMM; order-3 CSF: fiber rows for SA_EXPR_SPTTM_SPTTM, rows =
+ *   1  second list (CSR: rows for SA_EXPR_SPMM_GEMM and SPMMH_GEMM as ASSOC_RIGHT; order-3 CSF: fiber rows for SA_EXPR_SPTTM_SPTTM, rows =
  *      level-1 fibers; order-4 CSF: no items, only the fix-up entries and partial-tile slots of the fused kernel)
- *   2  order-4 CSF: the items of the fused kernel, runs of (i,j) subtrees: out_row / row_end = first subtree /
+ *   2  CSR: rows for the orders that form a row temporary first and gather 256 floats or more per nonzero
+ *      (SPMM_GEMM with L = 256 as ASSOC_LEFT, SPMMH_GEMM as FUSED); order-4 CSF: the items of the fused kernel, runs of (i,j) subtrees: out_row / row_end = first subtree /
  *      one past the last (at most 32), last field = kind.  Kind 0: the kernel evaluates them, [f0,f1) their
  *      level-2 fibers, [p0,p1) their nonzeros.  Kind 1: subtrees above 4096 nonzeros (at most 8), whose
  *      temporaries the main list's kernel writes first; f0 = index of the first among those subtrees.
@@ -192,7 +193,8 @@ sa_status sa_tensor_export(const sa_tensor *t, int level, int64_t *pos, int32_t 
  *      of at most 512 level-1 fibers [f0,f1) of slice out_row, quarter of the 256 columns (m,n) in the last field;
  *      a piece of at most eight fibers is a single item with 4 there: all quarters),
  *      with the fix-up entries of slices cut into pieces; 6 = first pass on whole small subtrees: rows
- *      [out_row,row_end) = level-1 fibers, [f0,f1) their level-2 fibers (at most 64), [p0,p1) their nonzeros
+ *      [out_row,row_end) = level-1 fibers, [f0,f1) their level-2 fibers (at most 64), [p0,p1) their nonzeros.
+ *      6, CSR: like list 2 where 128 floats are gathered per nonzero (SPMM_GEMM with L = 128 as ASSOC_LEFT)
  * For which = 0..2 and 4..6:
  *   counts [4]: number of items, number of leading groups that one thread block reduces into a
  *               single tile (8 items each; order-3 tensors: 4 tasks each, see sa_tensor_tasks),

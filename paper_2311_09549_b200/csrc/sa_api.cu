@@ -434,10 +434,10 @@ sa_status sa_tensor_create(int order, const int64_t *dims, int64_t nnz, const in
         if (s == SA_OK) s = upload_worklist(t, t->wl_main);
         if (s == SA_OK) s = upload_worklist(t, t->wl_aux);
         if (s == SA_OK) s = upload_worklist(t, t->wl_sub);
+        if (s == SA_OK && (fmt == SA_FMT_CSR || order == 4)) s = upload_worklist(t, t->wl4_sub);
         if (s == SA_OK && fmt == SA_FMT_CSF && order == 4) {
             s = upload_worklist(t, t->wl4_main);
             if (s == SA_OK) s = upload_worklist(t, t->wl4_aux);
-            if (s == SA_OK) s = upload_worklist(t, t->wl4_sub);
             if (s == SA_OK) s = upload(t, t->f4_supers.data(), t->f4_supers.size(), &t->d_f4_supers);
             if (s == SA_OK) s = upload(t, t->f4_pieces.data(), t->f4_pieces.size(), &t->d_f4_pieces);
         }

@@ -650,10 +650,11 @@ void build_ttm4(sa_tensor *t, sa_worklist &wl, sa_worklist &wl_items, sa_worklis
 
 // Rows of a sparse matrix given by its pos array: row ranges of about target_nnz nonzeros (at most max_rows rows); rows longer than
 // long_thresh are cut into pieces of `piece` nonzeros whose partial rows the fix-up kernel sums.
+// equal_parts: the pieces of a row have equal lengths, `piece` at most, and the list starts with the longest pieces.
 // quarter_rows: a range item also records the rows that hold its nonzeros p0 + q ceil((p1 - p0) / 4), q = 1, 2, 3
 // (fields f0, f1, pad), for kernels whose lane groups take equal counts of nonzeros rather than of rows.
 void build_rows(const std::vector<int64_t> &pos, int64_t I, sa_worklist &wl, int64_t target_nnz, int64_t max_rows,
-                int64_t long_thresh, int64_t piece, bool quarter_rows = false)
+                int64_t long_thresh, int64_t piece, bool quarter_rows = false, bool equal_parts = false)
 {
     std::vector<sa_item> longs, ranges;
     int64_t r0 = 0;
@@ -681,14 +682,14 @@ void build_rows(const std::vector<int64_t> &pos, int64_t I, sa_worklist &wl, int
         const int64_t a = pos[size_t(r)], b = pos[size_t(r) + 1];
         if (b - a > long_thresh) {
             flush(r);
-            const int64_t np = (b - a + piece - 1) / piece;
+            const int64_t np = (b - a + piece - 1) / piece, part = equal_parts ? (b - a + np - 1) / np : piece;
             const int32_t slot0 = int32_t(wl.n_slots);
             wl.fix.push_back(sa_fix{int32_t(r), slot0, int32_t(np), 0});
             wl.n_slots += np;
             for (int64_t q = 0; q < np; ++q) {
                 sa_item it = empty_item();
                 it.out_row = int32_t(r); it.row_end = int32_t(r + 1);
-                it.p0 = int32_t(a + q * piece); it.p1 = int32_t(std::min(b, a + (q + 1) * piece));
+                it.p0 = int32_t(std::min(b, a + q * part)); it.p1 = int32_t(std::min(b, a + (q + 1) * part));
                 it.dest = slot0 + int32_t(q);
                 longs.push_back(it);
             }
@@ -701,9 +702,68 @@ void build_rows(const std::vector<int64_t> &pos, int64_t I, sa_worklist &wl, int
     flush(I);
     // longest first: the tail of the launch is then made of the cheapest items
     longest_first(ranges);
+    if (equal_parts) longest_first(longs);
     wl.n_group_ctas = 0;
     wl.items = std::move(longs);
     wl.items.insert(wl.items.end(), ranges.begin(), ranges.end());
+}
+
+// CSR, row kernel of the left orders (spmm_gemm_left_kernel): the most nonzeros a row may have without being cut.  Cutting a
+// row costs a product of its part with D (row_cost nonzeros' time) per piece, and the gathers of the pieces run at the rate of
+// HBM, which is what cut_warps warps reach; so do those of whole rows unless columns are used several times (nnz > 2 J): then
+// all warps walk through the columns together and find C in L2.  Cutting pays where few or very unequal rows leave warps
+// idle.  Time in nonzeros of one warp: the kernel's warps take items in turn, longest first, so the first one of each round
+// counts.  Rows stay whole if no cut is 2 % faster, else the largest limit within 2 % of the shortest time is taken.
+// L = 256, M = 64, us, rows of up to 4096 whole / cut at nnz / 18944 nonzeros / by this rule: 2000 rows of 600 nonzeros 130 /
+// 200 / 130 (kernel 3: 211 / 417 / 211), 3000 of 1000 215 / 430 / 215, 500 of 1000 231 / 103 / 94, 500 of 3000 555 / 242 / 182,
+// 3 M nonzeros on 100 K rows, Zipf(1.2) 1230 / 650 / 680.
+int64_t left_row_limit(const std::vector<int64_t> &pos, int64_t I, int64_t J, int64_t target, int64_t row_cost, int64_t cut_warps)
+{
+    constexpr int64_t LIMITS[] = {4096, 2048, 1024, 512, 256, 128, 64, 32}, WARPS = SA_SMS * 24, FIX_COST = 40;   // FIX_COST: the launch that adds the pieces
+    std::vector<int64_t> count(size_t(LIMITS[0]) + 1, 0), over;
+    for (int64_t r = 0; r < I; ++r) {
+        const int64_t n = pos[size_t(r) + 1] - pos[size_t(r)];
+        if (n > LIMITS[0]) over.push_back(n);
+        else ++count[size_t(n)];
+    }
+    const int64_t nnz = pos[size_t(I)];
+    double best = 1e300, time[std::size(LIMITS)];
+    for (size_t x = 0; x < std::size(LIMITS); ++x) {
+        const int64_t limit = LIMITS[x], piece = std::min<int64_t>(limit, 2048);
+        std::vector<int64_t> len(count.begin(), count.begin() + limit + 1);      // items by length (short rows as if one each)
+        bool cut = false;
+        auto add = [&](int64_t n, int64_t rows) {
+            cut = true;
+            const int64_t parts = (n + piece - 1) / piece;
+            len[size_t((n + parts - 1) / parts)] += rows * parts;
+        };
+        for (int64_t n = limit + 1; n <= LIMITS[0]; ++n)
+            if (count[size_t(n)] > 0) add(n, count[size_t(n)]);
+        for (const int64_t n : over) add(n, 1);
+        double first = 0, short_nnz = 0, short_rows = 0;
+        int64_t at = 0;                                                         // items longer than `target` so far
+        for (int64_t n = limit; n >= 0; --n) {
+            const int64_t c = len[size_t(n)];
+            if (n <= target) {
+                short_nnz += double(c * n);
+                short_rows += double(c);
+                continue;
+            }
+            first += double((at + c + WARPS - 1) / WARPS - (at + WARPS - 1) / WARPS) * double(n + row_cost);
+            at += c;
+        }
+        // ranges of short rows: `target` nonzeros or 16 rows; they begin in the last round of the long items
+        const double rows_each = std::min(16.0, std::max(1.0, double(target) * short_rows / std::max(1.0, short_nnz)));
+        const double each = std::max(1.0, rows_each * (short_nnz / std::max(1.0, short_rows) + double(row_cost)));
+        const double ranges = short_rows / rows_each, room = double((at + WARPS - 1) / WARPS * WARPS - at);
+        time[x] = std::max(first + std::max(0.0, ranges - room) / WARPS * each, short_rows > 0 ? each : 0.0) + (cut ? FIX_COST : 0);
+        best = std::min(best, time[x]);
+    }
+    const double from_hbm = double(nnz) / double(cut_warps);
+    if (std::max(time[0], nnz > 2 * J ? 0.0 : from_hbm) <= 1.02 * std::max(best, from_hbm)) return LIMITS[0];
+    size_t x = 1;
+    while (time[x] > 1.02 * best) ++x;
+    return LIMITS[x];
 }
 
 // CSR, kernel 1 (fused SDDMM -> SpMM): an item is what one group of eight lanes walks, a range of whole short rows or a
@@ -807,10 +867,14 @@ void sa_build_worklists(sa_tensor *t)
     }
     if (t->fmt == SA_FMT_CSR) {
         build_sddmm(t->pos[1], t->crd[1], t->dims[0], t->wl_main);
-        // SpMM -> GEMM (both orders): about 256 nonzeros per item, which one lane group or warp walks as a chain; fewer where
+        // SpMM -> GEMM, the SpMM stage of the right orders (wl_aux) and the row kernel of the left ones (wl_sub, wl4_sub): about 256 nonzeros per item, which one lane group or warp walks as a chain; fewer where
         // the tensor would not give every group of a full machine two items
         const int64_t target = std::min<int64_t>(256, std::max<int64_t>(32, t->nnz / (2 * SA_SMS * 64)));
         build_rows(t->pos[1], t->dims[0], t->wl_aux, target, 16, 2 * target, target);
+        const int64_t wide = left_row_limit(t->pos[1], t->dims[0], t->dims[1], target, 50, 1200);     // 1 KB or more gathered per nonzero
+        const int64_t narrow = left_row_limit(t->pos[1], t->dims[0], t->dims[1], target, 20, 2400);   // 512 bytes
+        build_rows(t->pos[1], t->dims[0], t->wl_sub, target, 16, wide, std::min<int64_t>(wide, 2048), false, true);
+        build_rows(t->pos[1], t->dims[0], t->wl4_sub, target, 16, narrow, std::min<int64_t>(narrow, 2048), false, true);
     }
     for (sa_worklist *wl : {&t->wl_main, &t->wl_aux, &t->wl_sub, &t->wl4_main, &t->wl4_aux, &t->wl4_sub}) {
         std::stable_sort(wl->fix.begin(), wl->fix.end(), [](const sa_fix &x, const sa_fix &y) { return x.count > y.count; });

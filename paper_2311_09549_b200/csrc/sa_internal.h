@@ -112,9 +112,10 @@ struct sa_tensor {
     int32_t *d_status = nullptr;              // [4] device status word
 
     sa_worklist wl_main;                      // TTM3 / SDDMM-SpMM; order-4 CSF: the order-3 lists over the large (i,j) subtrees
-    sa_worklist wl_aux;                       // CSR: SpMM-GEMM row items; order-3 CSF: fiber rows (kernel 7); order-4 CSF: partial
+    sa_worklist wl_aux;                       // CSR: row items of the SpMM stage of SpMM-GEMM and SpMMH-GEMM; order-3 CSF: fiber rows (kernel 7); order-4 CSF: partial
                                               // slice tiles and fix-up entries of the fused kernel
-    sa_worklist wl_sub;                       // order-4 CSF: items of the fused kernel (runs of (i,j) subtrees)
+    sa_worklist wl_sub;                       // order-4 CSF: items of the fused kernel (runs of (i,j) subtrees); CSR: row items of the
+                                              // left orders that gather 256 floats or more per nonzero (wl4_sub: 128)
     // order-4 CSF, schedule SA_SCHED_FISSIONED (sa_ttm4_fis.cu): order-3 lists over the (i,j) subtrees the subtree kernel
     // does not take, pass-2 items (piece of a slice x quarter of the columns) with their fix-up entries, and ranges of
     // whole small subtrees for the subtree kernel

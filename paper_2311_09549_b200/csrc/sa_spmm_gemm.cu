@@ -493,10 +493,13 @@ sa_status run_spmm(const sa_tensor *t, float *E, float *out, cudaStream_t stream
     return SA_OK;
 }
 
+// Items of the row kernel: the list made for the floats that it gathers per nonzero (`tables` rows of L).
+const sa_worklist &left_list(const sa_tensor *t, int64_t L, int tables) { return L * tables >= 256 ? t->wl_sub : t->wl4_sub; }
+
 template <int L, int M>
 sa_status run(const sa_tensor *t, const sa_dense *ops, float *out, void *ws, bool right, cudaStream_t stream, int *launches)
 {
-    const sa_worklist &wl = t->wl_aux;
+    const sa_worklist &wl = left_list(t, L, 1);       // run_spmm has its own
     const int64_t n_items = int64_t(wl.items.size());
     const size_t smem = size_t(L * M + SA_WARPS_PER_CTA * L) * sizeof(float);
     *launches = 0;
@@ -535,7 +538,7 @@ sa_status run(const sa_tensor *t, const sa_dense *ops, float *out, void *ws, boo
 template <int L, int M>
 sa_status run_hadamard(const sa_tensor *t, const sa_dense *ops, float *out, void *ws, bool right, cudaStream_t stream, int *launches)
 {
-    const sa_worklist &wl = t->wl_aux;
+    const sa_worklist &wl = left_list(t, L, 2);       // run_spmm has its own
     const int64_t n_items = int64_t(wl.items.size());
     const size_t smem = size_t(L * M + SA_WARPS_PER_CTA * L) * sizeof(float);
     *launches = 0;
@@ -652,7 +655,7 @@ bool sa_ranks_ok_spmm_gemm(int64_t L, int64_t M) { return (L == 128 || L == 256)
 size_t sa_ws_spmm_gemm(const sa_tensor *t, const sa_dense *ops, bool right)
 {
     const size_t M = size_t(ops[1].cols);
-    size_t b = sa_align256(size_t(t->wl_aux.n_slots) * M * sizeof(float));
+    size_t b = sa_align256(size_t((right ? t->wl_aux : left_list(t, ops[0].cols, 1)).n_slots) * M * sizeof(float));
     if (right) b += sa_align256(size_t(t->dims[1]) * M * sizeof(float));
     return b;
 }
@@ -672,7 +675,7 @@ sa_status sa_launch_spmm_gemm(const sa_tensor *t, const sa_dense *ops, float *ou
 size_t sa_ws_spmmh_gemm(const sa_tensor *t, const sa_dense *ops, bool right)
 {
     const size_t M = size_t(ops[2].cols);
-    size_t b = sa_align256(size_t(t->wl_aux.n_slots) * M * sizeof(float));
+    size_t b = sa_align256(size_t((right ? t->wl_aux : left_list(t, ops[0].cols, 2)).n_slots) * M * sizeof(float));
     if (right) b += sa_align256(size_t(t->dims[1]) * M * sizeof(float));
     return b;
 }

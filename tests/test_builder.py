@@ -533,3 +533,30 @@ def test_csr_ranges_of_short_rows_hold_at_most_eight():
     t = sa.SparseTensor((rows, 1000), coords, np.ones(rows, np.float32), sa.SA_FMT_CSR, device=-1)
     items = sa.sa_tensor_worklist(t.handle)[1]
     assert (items[:, 1] - items[:, 0]).max() <= 8
+
+
+@pytest.mark.parametrize("rows,deg,cols,longest", [
+    (2000, 600, 200_000, 600),       # C is found in L2 while all rows walk through the columns together: whole
+    (3000, 1000, 200_000, 1000),
+    (500, 1000, 200_000, 250),       # too few rows for the machine
+    (100, 4000, 100_000, 125),
+    (200, 200, 100_000, 29),
+])
+def test_csr_row_kernel_list_cuts_rows_only_where_warps_would_idle(rows, deg, cols, longest):
+    coords = np.stack([np.repeat(np.arange(rows), deg), np.tile(np.arange(deg) * (cols // deg), rows)], axis=1).astype(np.int32)
+    t = sa.SparseTensor((rows, cols), coords, np.ones(rows * deg, np.float32), sa.SA_FMT_CSR, device=-1)
+    pos = np.arange(rows + 1) * deg
+    for which in (2, 6):
+        counts, items, fix = sa.sa_tensor_worklist(t.handle, which)
+        length = items[:, 5] - items[:, 4]
+        if which == 2:
+            assert length.max() == longest
+        assert np.all(length[items[:, 6] >= 0][:-1] >= length[items[:, 6] >= 0][1:])
+        # every nonzero once; pieces of a row fill slots in a row of their own
+        start = np.sort(items[:, 4])
+        assert start[0] == 0 and length.sum() == rows * deg and np.array_equal(np.sort(items[:, 5])[:-1], start[1:])
+        cut = items[items[:, 6] >= 0]
+        assert np.array_equal(np.sort(cut[:, 6]), np.arange(counts[3])) and np.all(cut[:, 1] == cut[:, 0] + 1)
+        assert fix[:, 2].sum() == counts[3] and set(fix[:, 0]) == set(cut[:, 0])
+        whole = items[items[:, 6] < 0]
+        assert np.array_equal(pos[whole[:, 0]], whole[:, 4]) and np.array_equal(pos[whole[:, 1]], whole[:, 5])
