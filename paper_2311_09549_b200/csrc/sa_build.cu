@@ -239,16 +239,20 @@ int64_t ttm3_slots(const std::vector<int64_t> &len, int64_t unit)
 int64_t ttm3_task_units(int64_t n_small) { return std::min<int64_t>(16, std::max<int64_t>(1, n_small / 4096)); }
 
 // Time of the order-3 kernel on slices of the given lengths with units of `unit` nonzeros, in nonzeros of one warp: the thread
-// blocks of the list in launch order on the `resident` slots of the machine, each for as long as its longest warp plus a fixed cost;
-// blocks also run faster while fewer are resident, so their sum over the slots has a share.  TILE_COST per partial tile and
-// FIX_COST for the launch that adds them.  short_len[n]: slices of n nonzeros; long_len: the slices above 2048.
-// The constants are fitted to 22 tensors of 0.3 to 7 M nonzeros (equal and Zipf slices) at four combinations of ranks, each
-// timed with all of TTM3_UNITS: the unit that ttm3_unit takes is 0.8 % slower than the fastest in the mean, 15 % at most.
-constexpr int64_t TTM3_UNITS[] = {2048, 1536, 1024, 768, 512, 384, 256};
-double ttm3_time(const std::vector<int64_t> &short_len, const std::vector<int64_t> &long_len, int64_t unit, int64_t slots, int64_t resident)
+// blocks of the list in launch order on the `resident` slots of the machine, each for as long as its longest warp plus a fixed
+// cost; blocks also run faster while fewer are resident, so their sum over the slots has a share.  A partial tile and the
+// launch that adds them cost something too.  short_len[n]: slices of n nonzeros; long_len: the slices above 2048.
+// `fibers` per nonzero: a nonzero takes the longer the more of them end a fiber, and the fixed costs count the less.
+// The constants are fitted to 32 tensors of 0.15 to 7 M nonzeros (equal and Zipf slices, mean fibers of 1.5 to 20) at up to six
+// combinations of ranks, each timed with seven unit sizes: the one that ttm3_unit takes is 1.3 % slower than the fastest in the
+// mean, 16 % at most.
+constexpr int64_t TTM3_UNITS[] = {2048, 1536, 1280, 1024, 896, 768, 640, 512, 384, 256};
+double ttm3_time(const std::vector<int64_t> &short_len, const std::vector<int64_t> &long_len, double fibers, int64_t unit, int64_t slots, int64_t resident)
 {
-    constexpr int64_t BLOCK_COST = 110, UNIT_COST = 32;              // UNIT_COST: each further unit of a task
-    constexpr double TILE_COST = 0.06, FIX_COST = 100, MAKESPAN_SHARE = 0.7;
+    constexpr double MAKESPAN_SHARE = 0.8;
+    const double weight = 1.25 / (1 + 2 * fibers);                 // 1 for fibers of eight nonzeros
+    const int64_t BLOCK_COST = int64_t(65 * weight), UNIT_COST = int64_t(32 * weight);      // UNIT_COST: each further unit of a task
+    const double TILE_COST = 0.06 * weight, FIX_COST = 100 * weight;
     struct run_rec { int64_t cost, count; };
     std::vector<run_rec> blocks;
     auto cut = [&](int64_t n, int64_t count) {                    // the blocks of `count` slices of n > unit nonzeros
@@ -310,7 +314,7 @@ double ttm3_time(const std::vector<int64_t> &short_len, const std::vector<int64_
     return MAKESPAN_SHARE * last + (1 - MAKESPAN_SHARE) * even + (slots > 0 ? FIX_COST + TILE_COST * double(slots) : 0.0);
 }
 
-// Nonzeros per unit: the largest of TTM3_UNITS within 3 % of the shortest estimated time, among those that need at most
+// Nonzeros per unit: the largest of TTM3_UNITS within 1 % of the shortest estimated time, among those that need at most
 // 1024 partial tiles (what sa_run_ttm3_static_scratch has room for at the largest ranks) or as many as units of 2048 need.
 // From two units of 2048 per warp slot of the machine on it is 2048: balance is then not what the time goes to.
 // L = M = 32, us, units of 2048 / what the rule takes: 300 slices of 1000 nonzeros 50 / 21, 1000 x 1100 35 / 29, 3000 x 400
@@ -318,7 +322,7 @@ double ttm3_time(const std::vector<int64_t> &short_len, const std::vector<int64_
 // *six_blocks: the 16 x 16 kernel compiled for six blocks per SM (fewer registers, each block 1.3 times as long) is through
 // sooner than the one for four; left alone for large tensors.  16 x 16, us, four / six blocks: 1000 slices of 2000 nonzeros
 // 33 / 39, 10 x 120 000 23 / 25, 400 x 8000 47 / 55, 3000 x 400 34 / 27, 800 x 700 21 / 15, 3000 x 2000 159 / 139.
-int64_t ttm3_unit(const std::vector<int64_t> &len, int *six_blocks)
+int64_t ttm3_unit(const std::vector<int64_t> &len, int64_t n_fibers, int *six_blocks)
 {
     constexpr int64_t LARGEST = TTM3_UNITS[0];
     int64_t nnz = 0;
@@ -329,6 +333,7 @@ int64_t ttm3_unit(const std::vector<int64_t> &len, int *six_blocks)
         if (n > LARGEST) long_len.push_back(n);
         else ++short_len[size_t(n)];
     const int64_t most = std::max<int64_t>(1024, ttm3_slots(len, LARGEST));
+    const double fibers = double(n_fibers) / double(std::max<int64_t>(1, nnz));
     int64_t units[std::size(TTM3_UNITS)];
     double time[std::size(TTM3_UNITS)], best = 1e300;
     int count = 0;
@@ -336,12 +341,12 @@ int64_t ttm3_unit(const std::vector<int64_t> &len, int *six_blocks)
         const int64_t slots = ttm3_slots(len, u);
         if (slots > most) continue;
         units[count] = u;
-        time[count] = ttm3_time(short_len, long_len, u, slots, 4 * SA_SMS);
+        time[count] = ttm3_time(short_len, long_len, fibers, u, slots, 4 * SA_SMS);
         best = std::min(best, time[count++]);
     }
     int x = 0;
-    while (time[x] > 1.03 * best) ++x;
-    *six_blocks = 1.3 * ttm3_time(short_len, long_len, units[x], ttm3_slots(len, units[x]), 6 * SA_SMS) < time[x];
+    while (time[x] > 1.01 * best) ++x;
+    *six_blocks = 1.3 * ttm3_time(short_len, long_len, fibers, units[x], ttm3_slots(len, units[x]), 6 * SA_SMS) < time[x];
     return units[x];
 }
 
@@ -447,7 +452,7 @@ void build_ttm3(sa_tensor *t, sa_worklist &wl)
     for (int64_t s = 0; s < t->count[0]; ++s)
         len[size_t(s)] = t->pos[2][size_t(t->pos[1][size_t(s) + 1])] - t->pos[2][size_t(t->pos[1][size_t(s)])];
     build_ttm3_lists(wl, t->count[0], [&](int64_t s) { return t->crd[0][size_t(s)]; }, [](int64_t) { return false; }, t->pos[1],
-                     t->pos[2], ttm3_unit(len, &wl.six_blocks));
+                     t->pos[2], ttm3_unit(len, t->count[1], &wl.six_blocks));
     append_empty_slices(t, wl);
 }
 
