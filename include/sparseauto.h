@@ -194,7 +194,8 @@ sa_status sa_tensor_export(const sa_tensor *t, int level, int64_t *pos, int32_t 
  *      a piece of at most eight fibers is a single item with 4 there: all quarters),
  *      with the fix-up entries of slices cut into pieces; 6 = first pass on whole small subtrees: rows
  *      [out_row,row_end) = level-1 fibers, [f0,f1) their level-2 fibers (at most 64), [p0,p1) their nonzeros.
- *      6, CSR: like list 2 where 128 floats are gathered per nonzero (SPMM_GEMM with L = 128 as ASSOC_LEFT)
+ *      6, CSR: like list 2 where 128 floats are gathered per nonzero (SPMM_GEMM with L = 128 as ASSOC_LEFT);
+ *      empty where list 2 serves both
  * For which = 0..2 and 4..6:
  *   counts [4]: number of items, number of leading groups that one thread block reduces into a
  *               single tile (8 items each; order-3 tensors: 4 tasks each, see sa_tensor_tasks),

@@ -2,10 +2,12 @@
 // tree of levels, arrays named pos / crd / vals as in Fig. 1b) and of the load-balancing work
 // lists (nonzero-balanced pieces of slices, fibers and rows) the kernels consume.
 #include <algorithm>
+#include <atomic>
 #include <cstring>
 #include <functional>
 #include <iterator>
 #include <memory>
+#include <new>
 #include <omp.h>
 
 #include "sa_internal.h"
@@ -871,15 +873,24 @@ void sa_build_worklists(sa_tensor *t)
         t->wl4_main.nnz = t->nnz - t->wl4_sub.nnz;
     }
     if (t->fmt == SA_FMT_CSR) {
-        build_sddmm(t->pos[1], t->crd[1], t->dims[0], t->wl_main);
-        // SpMM -> GEMM, the SpMM stage of the right orders (wl_aux) and the row kernel of the left ones (wl_sub, wl4_sub): about 256 nonzeros per item, which one lane group or warp walks as a chain; fewer where
-        // the tensor would not give every group of a full machine two items
-        const int64_t target = std::min<int64_t>(256, std::max<int64_t>(32, t->nnz / (2 * SA_SMS * 64)));
-        build_rows(t->pos[1], t->dims[0], t->wl_aux, target, 16, 2 * target, target);
-        const int64_t wide = left_row_limit(t->pos[1], t->dims[0], t->dims[1], target, 50, 1200);     // 1 KB or more gathered per nonzero
-        const int64_t narrow = left_row_limit(t->pos[1], t->dims[0], t->dims[1], target, 20, 2400);   // 512 bytes
-        build_rows(t->pos[1], t->dims[0], t->wl_sub, target, 16, wide, std::min<int64_t>(wide, 2048), false, true);
-        build_rows(t->pos[1], t->dims[0], t->wl4_sub, target, 16, narrow, std::min<int64_t>(narrow, 2048), false, true);
+        // SpMM -> GEMM, the SpMM stage of the right orders (wl_aux) and the row kernel of the left ones (wl_sub, wl4_sub): about
+        // 256 nonzeros per item, which one lane group or warp walks as a chain; fewer where the tensor would not give every
+        // group of a full machine two items
+        const std::vector<int64_t> &pos = t->pos[1];
+        const int64_t I = t->dims[0], J = t->dims[1], target = std::min<int64_t>(256, std::max<int64_t>(32, t->nnz / (2 * SA_SMS * 64)));
+        const int64_t wide = left_row_limit(pos, I, J, target, 50, 1200);      // 1 KB or more gathered per nonzero
+        const int64_t narrow = left_row_limit(pos, I, J, target, 20, 2400);    // 512 bytes; no list of its own at the same limit
+        std::atomic<bool> failed{false};
+#pragma omp parallel for schedule(dynamic, 1)
+        for (int list = 0; list < 4; ++list) {
+            try {
+                if (list == 0) build_sddmm(pos, t->crd[1], I, t->wl_main);
+                if (list == 1) build_rows(pos, I, t->wl_aux, target, 16, 2 * target, target);
+                if (list == 2) build_rows(pos, I, t->wl_sub, target, 16, wide, std::min<int64_t>(wide, 2048), false, true);
+                if (list == 3 && narrow != wide) build_rows(pos, I, t->wl4_sub, target, 16, narrow, std::min<int64_t>(narrow, 2048), false, true);
+            } catch (...) { failed = true; }
+        }
+        if (failed) throw std::bad_alloc();
     }
     for (sa_worklist *wl : {&t->wl_main, &t->wl_aux, &t->wl_sub, &t->wl4_main, &t->wl4_aux, &t->wl4_sub}) {
         std::stable_sort(wl->fix.begin(), wl->fix.end(), [](const sa_fix &x, const sa_fix &y) { return x.count > y.count; });

@@ -494,7 +494,11 @@ sa_status run_spmm(const sa_tensor *t, float *E, float *out, cudaStream_t stream
 }
 
 // Items of the row kernel: the list made for the floats that it gathers per nonzero (`tables` rows of L).
-const sa_worklist &left_list(const sa_tensor *t, int64_t L, int tables) { return L * tables >= 256 ? t->wl_sub : t->wl4_sub; }
+// (One list where the rule cuts rows alike for both widths.)
+const sa_worklist &left_list(const sa_tensor *t, int64_t L, int tables)
+{
+    return L * tables >= 256 || t->wl4_sub.items.empty() ? t->wl_sub : t->wl4_sub;
+}
 
 template <int L, int M>
 sa_status run(const sa_tensor *t, const sa_dense *ops, float *out, void *ws, bool right, cudaStream_t stream, int *launches)
