@@ -336,20 +336,22 @@ int64_t ttm3_unit(const std::vector<int64_t> &len, int64_t n_fibers, int *six_bl
         else ++short_len[size_t(n)];
     const int64_t most = std::max<int64_t>(1024, ttm3_slots(len, LARGEST));
     const double fibers = double(n_fibers) / double(std::max<int64_t>(1, nnz));
-    int64_t units[std::size(TTM3_UNITS)];
-    double time[std::size(TTM3_UNITS)], best = 1e300;
-    int count = 0;
-    for (const int64_t u : TTM3_UNITS) {
-        const int64_t slots = ttm3_slots(len, u);
-        if (slots > most) continue;
-        units[count] = u;
-        time[count] = ttm3_time(short_len, long_len, fibers, u, slots, 4 * SA_SMS);
-        best = std::min(best, time[count++]);
+    constexpr int COUNT = int(std::size(TTM3_UNITS));
+    double time[COUNT], best = 1e300;
+    std::atomic<bool> failed{false};
+#pragma omp parallel for schedule(dynamic, 1)
+    for (int x = 0; x < COUNT; ++x) {
+        try {
+            const int64_t slots = ttm3_slots(len, TTM3_UNITS[x]);
+            time[x] = slots > most ? 1e300 : ttm3_time(short_len, long_len, fibers, TTM3_UNITS[x], slots, 4 * SA_SMS);
+        } catch (...) { failed = true; }
     }
+    if (failed) throw std::bad_alloc();
+    for (const double x : time) best = std::min(best, x);
     int x = 0;
     while (time[x] > 1.01 * best) ++x;
-    *six_blocks = 1.3 * ttm3_time(short_len, long_len, fibers, units[x], ttm3_slots(len, units[x]), 6 * SA_SMS) < time[x];
-    return units[x];
+    *six_blocks = 1.3 * ttm3_time(short_len, long_len, fibers, TTM3_UNITS[x], ttm3_slots(len, TTM3_UNITS[x]), 6 * SA_SMS) < time[x];
+    return TTM3_UNITS[x];
 }
 
 // Nonzeros per unit of the order-4 lists, which hold the large (i,j) subtrees only: 2048, less where `nnz` nonzeros, of which
