@@ -25,6 +25,7 @@
 // one: the whole chain is then off by 1.9e-7 (2-norm, against fp64; with one set of columns for b1.b1 3.1e-7, the row
 // kernel 3.0e-7).  Loads go half a chunk at a time (same registers in flight); operand tiles take half as much again, so
 // two or three stages fit instead of four.  1M x 256 . 256 x 64: 363 us = 6.3 TB/s; without H 204 us = 6.2 TB/s.
+// Rows with numbers that have no BF16 parts come out as NaN and are summed once more in fp32 by the epilogue.
 // What limits this kernel next to HBM is the shared-memory data pipe (operand writes, tensor-core operand
 // reads, epilogue), which is why C never passes through a shared-memory fp32 stage and why the two products
 // that share b1(C) are merged.
