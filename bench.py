@@ -42,8 +42,8 @@ NCU_TRAFFIC = {
         "sha256": "698a23dccef6f7b97f8f186486a5099dcbfeac67c71cbc936d0910db206a0725",
         "dram_bytes": 484427776 + 368994816},
     3: {"kernel": "sddmm_spmm_kernel<64,64> (98 % of the step)", "source": "paper_2311_09549_b200/csrc/sa_sddmm_spmm.cu",
-        "sha256": "7d300585ca589d56f3795e257106157cc664663e6b8f45605ef23957106afd48",
-        "dram_bytes": 2580707072 + 277291008},
+        "sha256": "794f12987d2bfe30728df7f0547b2774d1049eacebb59236b608f535538ecff7",
+        "dram_bytes": 2580282112 + 277797376},
     (5, "fused"): {"kernel": "ttm4_fused_kernel (94 % of the step; counters of the quarter-size case x 4)",
                    "source": "paper_2311_09549_b200/csrc/sa_ttm4.cu", "sha256": "f6e8316914ad48188dfc5417cdd93bf51bb6a64f1611b1dbc1ba407ab5eabb08",
                    "dram_bytes": 4 * (244847104 + 178882816)},

@@ -150,10 +150,11 @@ cudaError_t launch(const sa_tensor *t, const sa_dense *ops, float *out, float *p
     const int64_t n_items = int64_t(wl.items.size());
     const int64_t ctas = (n_items + 31) / 32;         // 32 groups per block
     if (ctas == 0) return cudaSuccess;
-    // Up to two and a half rounds of items the length of one is the run time, and two blocks per SM walk it faster (registers for
+    // Up to three rounds of items the length of one is the run time, and two blocks per SM walk it faster (registers for
     // more loads at a time).  K = L = 32, us, two / three blocks: 60 K nonzeros (4.7 K items) 14.4 / 16.5, 1 M on 20 K rows
-    // (22 K items) 29.3 / 31.8, 1 M on 300 K rows (38 K items) 61 / 53, on 200 K rows and 700 K columns (42 K) 83 / 69.
-    auto kern = n_items <= int64_t(5) * SA_SMS * 32 ? sddmm_spmm_kernel<K, L, 2> : sddmm_spmm_kernel<K, L, sd_cfg<K, L>::CTAS>;
+    // (22 K items) 29.3 / 31.8, 400 K on 40 K rows (26 K) 29.1 / 30.9, 1.5 M on 50 K rows (30 K) 48.3 / 47.5, 1 M on 300 K rows
+    // (38 K) 61 / 53, on 200 K rows and 700 K columns (42 K) 83 / 69.
+    auto kern = n_items <= int64_t(3) * 2 * SA_SMS * 32 ? sddmm_spmm_kernel<K, L, 2> : sddmm_spmm_kernel<K, L, sd_cfg<K, L>::CTAS>;
     kern<<<(unsigned)ctas, 256, 0, stream>>>(
         wl.d_items, n_items, t->d_pos[1], t->d_nzpack, ops[0].ptr, uint32_t(ops[0].ld), ops[1].ptr, uint32_t(ops[1].ld), ops[2].ptr,
         uint32_t(ops[2].ld), out, partial, sampled, sa_make_limits(t, t->dims[1], t->dims[0], wl.n_slots));

@@ -721,10 +721,10 @@ def test_operands_that_make_no_sense_are_refused_before_their_output_is_too_larg
         assert float(out[5, 0, 0]) == 1.0
 
 
-@pytest.mark.parametrize("rows", [23_680 * 8 - 3, 23_680 * 8 + 3])
+@pytest.mark.parametrize("rows", [28_416 * 8 - 3, 28_416 * 8 + 3])
 def test_sddmm_spmm_ranks_32_on_both_sides_of_the_two_and_three_block_kernels(sa, rows):
-    """One nonzero per row, ranges of eight rows: 23 680 items are the last that the kernel for two blocks per SM takes."""
+    """One nonzero per row, ranges of eight rows: 28 416 items are the last that the kernel for two blocks per SM takes."""
     coords, vals = np.stack([np.arange(rows), np.arange(rows) % 40], axis=1), rng.uniform_f32(61, 1, np.arange(rows), -1.0, 1.0)
     w = _wl("sddmm_spmm", "csr", (rows, 40), coords, vals, [_dense(61, 0, rows, 32), _dense(61, 1, 40, 32), _dense(61, 2, 40, 32)], (rows, 32))
     _, t = _check(sa, w)
-    assert (len(sa.sa_tensor_worklist(t.handle)[1]) <= 23_680) == (rows < 23_680 * 8)
+    assert (len(sa.sa_tensor_worklist(t.handle)[1]) <= 28_416) == (rows < 28_416 * 8)
