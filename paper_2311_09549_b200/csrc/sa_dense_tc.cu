@@ -219,6 +219,7 @@ gemm_tc_kernel(int64_t J, const float *__restrict__ C, int64_t ldc, const float 
     uint32_t *tmem_slot = reinterpret_cast<uint32_t *>(smem + G::OFF_BAR + 8 * B_COUNT);
     volatile int *abort_flag = reinterpret_cast<volatile int *>(smem + G::OFF_BAR + 8 * B_COUNT + 4);
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    sa_after_previous();
 
     // D^T as KCH operand tiles of PARTS M rows x 64 columns (k): rows n < M hold b1(D(k,n)), rows M + n hold b2, ...
     // (eight k of one n per step: coalesced loads, eight in flight, and one conflict-free 16-byte store per part; element by
@@ -526,7 +527,7 @@ sa_status launch_tc(int64_t rows, const float *A, int64_t lda, const float *H, i
     const int64_t ctas = std::min<int64_t>((rows + TC_BM - 1) / TC_BM, sms);
     int shift = 0;
     while ((4 << shift) < part) ++shift;
-    if (ctas > 0) k<<<(unsigned)ctas, TC_THREADS, G::SMEM, stream>>>(rows, A, lda, H, ldh, B, ldb, out, shift, status);
+    if (ctas > 0) sa_launch(k, (unsigned)ctas, TC_THREADS, G::SMEM, stream, rows, A, lda, H, ldh, B, ldb, out, shift, status);
     return cudaGetLastError() == cudaSuccess ? SA_OK : SA_E_CUDA;
 }
 

@@ -57,6 +57,36 @@ static inline sa_limits sa_make_limits(const sa_tensor *t, int64_t gather_rows, 
     return lim;
 }
 
+// Kernels are launched so that they may start while the one before them on the stream still runs (programmatic dependent
+// launch): their blocks take the places that the other's last round leaves, read what no kernel ever writes (work lists, the
+// tensor's arrays) and then wait, in sa_after_previous, until the other is through and its results can be seen.  Nothing else may
+// be read or written before that, and some thread of every launch has to wait, or a kernel further back could still be running.
+// Then they let the next kernel on the stream start in the same way.  Back to back, us, without / with: order-3 tensor of 20 K
+// nonzeros (one launch) 10.2 / 9.5, of 2.3 M (two) 49.6 / 45.6, kernel 2 on 60 K nonzeros (two) 18.1 / 16.0.
+__device__ __forceinline__ void sa_after_previous()
+{
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+}
+template <bool EARLY = true, typename... Params, typename... Args>
+static inline cudaError_t sa_launch(void (*kernel)(Params...), dim3 grid, unsigned threads, size_t smem, cudaStream_t stream, Args... args)
+{
+    // EARLY = false: an SM keeps its split of shared memory and L1 as long as blocks are on it, so a kernel that lives on L1
+    // (or needs more shared memory) must not start beside one with another split: gather of kernel 7 (12.5 M nonzeros) behind
+    // the dense stage 140 us, early 164.
+    cudaLaunchAttribute attr;
+    attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr.val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = grid;
+    cfg.blockDim = dim3(threads);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = stream;
+    cfg.attrs = &attr;
+    cfg.numAttrs = EARLY ? 1 : 0;
+    return cudaLaunchKernelEx(&cfg, kernel, Params(args)...);
+}
+
 // Opt a kernel into `bytes` of dynamic shared memory once per device instead of once per launch (the attribute is
 // per device; `done` is the caller's flags, one per device ordinal).  Host threads may launch at the same time: the
 // attribute may then be set more than once, to the same value.
@@ -111,6 +141,7 @@ sa_fixup_kernel(const sa_fix *__restrict__ fix, unsigned n_big, unsigned n_sum, 
                 float *__restrict__ out, int shift)
 {
     __shared__ float4 red[256];
+    sa_after_previous();
     const unsigned big_blocks = n_big << (shift - 4), sum_blocks = (n_sum - n_big) << (shift - 6);
     unsigned b = blockIdx.x;
     if (b >= big_blocks + sum_blocks) {
@@ -155,6 +186,7 @@ sa_fixup_rows_kernel(const sa_fix *__restrict__ fix, int n_fix, int n_big, const
     const int entry = big ? int(blockIdx.x) : n_big + (int(blockIdx.x) - n_big) * 8 + int(threadIdx.x >> 5);
     if (entry >= n_fix) return;                        // whole warps of the last block
     const sa_fix e = fix[entry];
+    sa_after_previous();
     const int who = big ? int(threadIdx.x) : lane, P = (big ? 256 : 32) / W;
     const int col = who % W, phase = who / W;
     float4 s = make_float4(0.f, 0.f, 0.f, 0.f);
@@ -184,14 +216,12 @@ static inline cudaError_t sa_launch_fixup(const sa_worklist &wl, const float *pa
     const int nf4 = tile_floats / 4;
     if (nf4 <= 32) {
         const unsigned rows = (unsigned)wl.fix.size(), big = (unsigned)wl.n_big_fix;
-        sa_fixup_rows_kernel<<<big + (rows - big + 7) / 8, 256, 0, stream>>>(wl.d_fix, int(rows), int(big), partial, out, tile_floats);
-        return cudaGetLastError();
+        return sa_launch(sa_fixup_rows_kernel, big + (rows - big + 7) / 8, 256, 0, stream, wl.d_fix, int(rows), int(big), partial, out, tile_floats);
     }
     int shift = 0;
     while ((4 << shift) < tile_floats) ++shift;
     const int64_t zeros = int64_t(wl.fix.size()) - wl.n_sum_fix;
     const int64_t blocks = (wl.n_big_fix << (shift - 4)) + ((wl.n_sum_fix - wl.n_big_fix) << (shift - 6)) + (((zeros << shift) + 255) >> 8);
-    sa_fixup_kernel<<<(unsigned)blocks, 256, 0, stream>>>(wl.d_fix, unsigned(wl.n_big_fix), unsigned(wl.n_sum_fix), unsigned(wl.fix.size()), partial,
-                                                          out, shift);
-    return cudaGetLastError();
+    return sa_launch(sa_fixup_kernel, unsigned(blocks), 256, 0, stream, wl.d_fix, unsigned(wl.n_big_fix), unsigned(wl.n_sum_fix), unsigned(wl.fix.size()),
+                     partial, out, shift);
 }

@@ -172,6 +172,7 @@ struct sa_ttm3_view {
     int64_t nnz;                  // nonzeros the lists cover (chooses the register budget)
     int64_t nnz_total;            // length of the index / value arrays (bounds of the self-checking build)
     int32_t *status;              // the tensor's device status word
+    bool early = true;            // may start beside the kernel before it (sa_launch)
 };
 sa_status sa_launch_ttm3_view(const sa_ttm3_view &v, const sa_dense &first, const sa_dense &second, float *out,
                               float *partial, cudaStream_t stream, int *launches);

@@ -63,16 +63,17 @@ sddmm_spmm_kernel(const sa_item *__restrict__ items, int64_t n_items, const int3
         }
     };
     int b = row_end(r), bn = row_end(r + 1);
-    load_c(c, r);
-    if (G::AHEAD) load_c(cn, r + 1);
-#pragma unroll
-    for (int q = 0; q < EQ; ++q) acc[q] = make_float4(0.f, 0.f, 0.f, 0.f);
     int2 rec[U];
 #pragma unroll
     for (int u = 0; u < U; ++u) {
         rec[u] = make_int2(0, 0);
         if (p + u < end) rec[u] = __ldg(nz + p + u);
     }
+    sa_after_previous();
+    load_c(c, r);
+    if (G::AHEAD) load_c(cn, r + 1);
+#pragma unroll
+    for (int q = 0; q < EQ; ++q) acc[q] = make_float4(0.f, 0.f, 0.f, 0.f);
     const char *Dl = reinterpret_cast<const char *>(D + 4 * l), *El = reinterpret_cast<const char *>(E + 4 * l);
     const uint32_t d_bytes = ldd * 4u, e_bytes = lde * 4u;
     for (;;) {
@@ -155,8 +156,7 @@ cudaError_t launch(const sa_tensor *t, const sa_dense *ops, float *out, float *p
     // (22 K items) 29.3 / 31.8, 400 K on 40 K rows (26 K) 29.1 / 30.9, 1.5 M on 50 K rows (30 K) 48.3 / 47.5, 1 M on 300 K rows
     // (38 K) 61 / 53, on 200 K rows and 700 K columns (42 K) 83 / 69.
     auto kern = n_items <= int64_t(3) * 2 * SA_SMS * 32 ? sddmm_spmm_kernel<K, L, 2> : sddmm_spmm_kernel<K, L, sd_cfg<K, L>::CTAS>;
-    kern<<<(unsigned)ctas, 256, 0, stream>>>(
-        wl.d_items, n_items, t->d_pos[1], t->d_nzpack, ops[0].ptr, uint32_t(ops[0].ld), ops[1].ptr, uint32_t(ops[1].ld), ops[2].ptr,
+    sa_launch(kern, (unsigned)ctas, 256, 0, stream, wl.d_items, n_items, t->d_pos[1], t->d_nzpack, ops[0].ptr, uint32_t(ops[0].ld), ops[1].ptr, uint32_t(ops[1].ld), ops[2].ptr,
         uint32_t(ops[2].ld), out, partial, sampled, sa_make_limits(t, t->dims[1], t->dims[0], wl.n_slots));
     return cudaGetLastError();
 }

@@ -57,6 +57,7 @@ spmm_gemm_left_kernel(const sa_item *__restrict__ items, int64_t n_items, const 
     float *Ds = smem;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     float *Ts = smem + L * M + warp * L;
+    sa_after_previous();
     load_D<L, M>(Ds, D, ldd);
     __syncthreads();
     for (int64_t idx = int64_t(blockIdx.x) * SA_WARPS_PER_CTA + warp; idx < n_items;
@@ -170,6 +171,7 @@ gemm_bf16x3_kernel(int64_t J, const float *__restrict__ C, int64_t ldc, const fl
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int g = lane >> 2, t = lane & 3;
     const int wr = warp >> 1, wc = warp & 1;           // warp tile: rows 32*wr.., columns (M/2)*wc..
+    sa_after_previous();
     for (int x = threadIdx.x; x < (L / 2) * M; x += 256) {
         const int p = x / M, m = x % M;
         uint32_t h, l;
@@ -298,7 +300,6 @@ spmm_kernel(const sa_item *__restrict__ items, int64_t n_items, unsigned ctas_pe
     int b = row_end(r), bn = row_end(r + 1);                // where rows r and r + 1 end
     auto next_row = [&]() { ++r; b = bn; bn = row_end(r + 1); };
     const float4 zero = make_float4(0.f, 0.f, 0.f, 0.f);
-    while (r < rend && b == p0) { store_row(zero); next_row(); }      // empty rows
     const int len = end - p0, steps = __reduce_max_sync(SA_FULL_MASK, len);
     auto fetch = [&](int c) {                                // nonzero c + lane of the group (eight lanes hold one each)
         int2 w = make_int2(0, 0);
@@ -309,6 +310,8 @@ spmm_kernel(const sa_item *__restrict__ items, int64_t n_items, unsigned ctas_pe
     };
     float4 acc = zero;
     int2 rec = fetch(0);
+    sa_after_previous();
+    while (r < rend && b == p0) { store_row(zero); next_row(); }      // empty rows
     for (int c = 0; c < steps; c += U) {
         float4 e[U];
         float vs[U];
@@ -390,6 +393,7 @@ fiber_spmm_kernel(const sa_item *__restrict__ items, int64_t n_items, const int3
     int xn;
     float vn;
     fetch(0, xn, vn);
+    sa_after_previous();
     for (int c = 0; c < maxlen; c += 8) {
         const int x = xn;
         const float v = vn;
@@ -481,7 +485,7 @@ sa_status run_spmm(const sa_tensor *t, float *E, float *out, cudaStream_t stream
         const int W = spmm_part(J, M);
         const unsigned ctas = unsigned((n_items * (W / 4) + 255) / 256);
         auto kern = W == 32 ? spmm_kernel<32> : spmm_kernel<64>;
-        kern<<<ctas * unsigned(M / W), 256, 0, stream>>>(wl.d_items, n_items, ctas, t->d_pos[1], t->d_nzpack, E, J, M, out, partial,
+        sa_launch<false>(kern, ctas * unsigned(M / W), 256, 0, stream, wl.d_items, n_items, ctas, t->d_pos[1], t->d_nzpack, E, J, M, out, partial,
                                                          sa_make_limits(t, J, t->dims[0], wl.n_slots));
         if (cudaGetLastError() != cudaSuccess) return SA_E_CUDA;
         *launches += 1;
@@ -516,7 +520,7 @@ sa_status run(const sa_tensor *t, const sa_dense *ops, float *out, void *ws, boo
         const int64_t want = (n_items + SA_WARPS_PER_CTA - 1) / SA_WARPS_PER_CTA;
         const int64_t ctas = std::min<int64_t>(want, resident_ctas(reinterpret_cast<const void *>(kern), smem, resident));
         if (ctas > 0) {
-            kern<<<(unsigned)ctas, 256, smem, stream>>>(wl.d_items, n_items, t->d_pos[1], t->d_crd[1], t->d_vals, ops[0].ptr,
+            sa_launch(kern, (unsigned)ctas, 256, smem, stream, wl.d_items, n_items, t->d_pos[1], t->d_crd[1], t->d_vals, ops[0].ptr,
                                                        ops[0].ld, ops[0].ptr, ops[0].ld, ops[1].ptr, ops[1].ld, out, partial,
                                                        sa_make_limits(t, t->dims[1], t->dims[0], wl.n_slots));
             if (cudaGetLastError() != cudaSuccess) return SA_E_CUDA;
@@ -561,7 +565,7 @@ sa_status run_hadamard(const sa_tensor *t, const sa_dense *ops, float *out, void
     const int64_t want = (n_items + SA_WARPS_PER_CTA - 1) / SA_WARPS_PER_CTA;
     const int64_t ctas = std::min<int64_t>(want, resident_ctas(reinterpret_cast<const void *>(kern), smem, resident));
     if (ctas > 0) {
-        kern<<<(unsigned)ctas, 256, smem, stream>>>(wl.d_items, n_items, t->d_pos[1], t->d_crd[1], t->d_vals, ops[0].ptr,
+        sa_launch(kern, (unsigned)ctas, 256, smem, stream, wl.d_items, n_items, t->d_pos[1], t->d_crd[1], t->d_vals, ops[0].ptr,
                                                    ops[0].ld, ops[1].ptr, ops[1].ld, ops[2].ptr, ops[2].ld, out, partial,
                                                    sa_make_limits(t, t->dims[1], t->dims[0], wl.n_slots));
         if (cudaGetLastError() != cudaSuccess) return SA_E_CUDA;
@@ -593,7 +597,7 @@ sa_status run_fibers(const sa_tensor *t, const sa_dense *ops, float *out, void *
         if (gs != SA_OK) return gs;
         *launches += 1;
         if (ctas > 0) {
-            fiber_spmm_kernel<M><<<(unsigned)ctas, 256, 0, stream>>>(wl.d_items, n_items, t->d_pos[2], t->d_nzpack, E, M, out, partial,
+            sa_launch<false>(fiber_spmm_kernel<M>, (unsigned)ctas, 256, 0, stream, wl.d_items, n_items, t->d_pos[2], t->d_nzpack, E, M, out, partial,
                                                                      sa_make_limits(t, K, F2, wl.n_slots));
             if (cudaGetLastError() != cudaSuccess) return SA_E_CUDA;
             *launches += 1;
@@ -607,7 +611,7 @@ sa_status run_fibers(const sa_tensor *t, const sa_dense *ops, float *out, void *
     float *T = static_cast<float *>(ws);
     float *partial = reinterpret_cast<float *>(static_cast<char *>(ws) + sa_align256(size_t(F2) * L * sizeof(float)));
     if (ctas > 0) {
-        fiber_spmm_kernel<L><<<(unsigned)ctas, 256, 0, stream>>>(wl.d_items, n_items, t->d_pos[2], t->d_nzpack, ops[0].ptr, ops[0].ld,
+        sa_launch<false>(fiber_spmm_kernel<L>, (unsigned)ctas, 256, 0, stream, wl.d_items, n_items, t->d_pos[2], t->d_nzpack, ops[0].ptr, ops[0].ld,
                                                                 T, partial, sa_make_limits(t, K, F2, wl.n_slots));
         if (cudaGetLastError() != cudaSuccess) return SA_E_CUDA;
         *launches += 1;
@@ -636,7 +640,7 @@ static sa_status dense_gemm(int64_t rows, const float *A, int64_t lda, const flo
     static resident_cache resident;
     if (!sa_set_smem_once(gk, int(GC::SMEM), attr)) return SA_E_CUDA;
     const int64_t ctas = std::min<int64_t>((rows + GC::BM - 1) / GC::BM, resident_ctas(reinterpret_cast<const void *>(gk), GC::SMEM, resident));
-    if (ctas > 0) gk<<<(unsigned)ctas, 256, GC::SMEM, stream>>>(rows, A, lda, B, ldb, out);
+    if (ctas > 0) sa_launch(gk, (unsigned)ctas, 256, GC::SMEM, stream, rows, A, lda, B, ldb, out);
     return cudaGetLastError() == cudaSuccess ? SA_OK : SA_E_CUDA;
 }
 

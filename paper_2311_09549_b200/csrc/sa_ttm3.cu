@@ -283,7 +283,7 @@ __device__ __forceinline__ void ttm3_warp_task(const sa_unit3 *__restrict__ unit
                                                const float *__restrict__ C, uint32_t ldc, const float *__restrict__ D,
                                                uint32_t ldd, unsigned char *__restrict__ wsm,
                                                float (&acc)[cfg<L, M>::MT][cfg<L, M>::NT][4], float (&hacc)[4], const bool keep,
-                                               float *__restrict__ out, const dbg_limits &lim, const ttmc_sink *sink = nullptr)
+                                               float *__restrict__ out, const dbg_limits &lim, const bool first, const ttmc_sink *sink = nullptr)
 {
     using K = cfg<L, M>;
     constexpr int VEC = K::VEC, DEPTH = K::DEPTH;
@@ -346,6 +346,7 @@ __device__ __forceinline__ void ttm3_warp_task(const sa_unit3 *__restrict__ unit
     const uint32_t row_bytes = ldd * 4u;
     cp_async_wait<DEPTH - 2>();
     __syncwarp();
+    if (first) sa_after_previous();                      // up to here only the tensor and its lists were read
     rowvec<VEC> buf[8];                                  // rows of the round about to be consumed
     {
         const uint4 ka = lds128(s_kv), kb = lds128(s_kv + 16);
@@ -528,7 +529,7 @@ ttm3_kernel(const sa_unit3 *__restrict__ units, const int32_t *__restrict__ task
     int u0 = 0, u1 = 0;
     if (task < n_tasks) { u0 = task_start[task]; u1 = task_start[task + 1]; }
     if (u1 > u0)
-        ttm3_warp_task<L, M, HAD>(units, u0, u1 - u0, crd_j, crd_k, vals, endbits, C, ldc, D, ldd, wsm, acc, hacc, group, out, lim);
+        ttm3_warp_task<L, M, HAD>(units, u0, u1 - u0, crd_j, crd_k, vals, endbits, C, ldc, D, ldd, wsm, acc, hacc, group, out, lim, true);
     if (!group) return;                 // whole small slices: every tile was stored when its unit ended
     if (HAD) {
         // the warps hold partial rows of the same slice: sum them in a fixed order
@@ -597,6 +598,7 @@ ttmc3_fused_kernel(const sa_unit3 *__restrict__ units, const int32_t *__restrict
     float *accs = reinterpret_cast<float *>(smem + SA_TTM3_WARPS * K::WARP_BYTES);
     const int n_acc = L3 * TILE;
     for (int x = threadIdx.x; x < n_acc; x += 32 * SA_TTM3_WARPS) accs[x] = 0.f;
+    sa_after_previous();
     __syncthreads();
     ttmc_sink sink;
     sink.C3 = C3; sink.ldc3 = ldc3; sink.L3 = L3; sink.accs = accs;
@@ -611,7 +613,7 @@ ttmc3_fused_kernel(const sa_unit3 *__restrict__ units, const int32_t *__restrict
         if (task < n_tasks) { u0 = task_start[task]; u1 = task_start[task + 1]; }
         if (u1 > u0)
             ttm3_warp_task<L, M, false, true>(units, u0, u1 - u0, crd_j, crd_k, vals, endbits, C, ldc, D, ldd, wsm, acc, hacc, group,
-                                              nullptr, lim, &sink);
+                                              nullptr, lim, false, &sink);
         if (!group) continue;              // whole small slices: added to the accumulator when their units ended
         // the block's warps hold partial temporaries of the same slice: sum them, then one rank-1 update
         __syncthreads();                   // every warp is done with its shared-memory region
@@ -671,9 +673,13 @@ cudaError_t launch(const sa_ttm3_view &v, const sa_dense &first, const sa_dense 
     lim.c_rows = uint32_t(first.rows); lim.d_rows = uint32_t(second.rows);
     lim.n_fibers = uint32_t(v.n_fibers); lim.n_slices_dim = uint32_t(v.n_out_rows);
     lim.nnz = v.nnz_total;
-    kern<<<(unsigned)ctas, 32 * SA_TTM3_WARPS, smem, stream>>>(wl.d_units3, wl.d_task_start, n_tasks, int(wl.n_group_ctas), v.crd_fiber,
-                                                              v.crd_nz, v.vals, v.endbits, first.ptr, uint32_t(first.ld), second.ptr,
-                                                              uint32_t(second.ld), out, partial, lim);
+    auto start = [&](auto early) {
+        sa_launch<decltype(early)::value>(kern, (unsigned)ctas, 32 * SA_TTM3_WARPS, smem, stream, wl.d_units3, wl.d_task_start, n_tasks,
+                                          int(wl.n_group_ctas), v.crd_fiber, v.crd_nz, v.vals, v.endbits, first.ptr, uint32_t(first.ld),
+                                          second.ptr, uint32_t(second.ld), out, partial, lim);
+    };
+    if (v.early) start(std::true_type{});
+    else start(std::false_type{});
     return cudaGetLastError();
 }
 
@@ -775,7 +781,7 @@ sa_status sa_launch_ttmc3_fused_stage(const sa_tensor *t, const sa_dense &C3, co
     if (M == m && N == n) {                                                                                                       \
         if (!ttmc3_fused_shape<m, n>(int(C3.cols), &grid, &smem)) return SA_E_CUDA;                                               \
         grid = int(std::min<int64_t>(std::min<int64_t>(grid, SA_TTMC3_MAX_BLOCKS), n_block_tasks));                               \
-        ttmc3_fused_kernel<m, n, 4><<<unsigned(grid), 32 * SA_TTM3_WARPS, smem, stream>>>(                                        \
+        sa_launch(ttmc3_fused_kernel<m, n, 4>, unsigned(grid), 32 * SA_TTM3_WARPS, smem, stream, \
             wl.d_units3, wl.d_task_start, n_tasks, int(wl.n_group_ctas), t->d_crd[1], t->d_crd[2], t->d_vals, t->d_endbits, D.ptr, \
             uint32_t(D.ld), E.ptr, uint32_t(E.ld), C3.ptr, uint32_t(C3.ld), int(C3.cols), partials, lim);                         \
         if (cudaGetLastError() != cudaSuccess) return SA_E_CUDA;                                                                  \

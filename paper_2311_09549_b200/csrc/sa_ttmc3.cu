@@ -33,6 +33,7 @@ ttmc3_partial_kernel(int64_t I, int chunk, int cols, const float *__restrict__ T
                      uint32_t ldc, float *__restrict__ P)
 {
     __shared__ __align__(16) float cs[TTMC_STEP * L];
+    sa_after_previous();
     const int col = blockIdx.x * 256 + threadIdx.x;
     const int64_t i0 = int64_t(blockIdx.y) * chunk, i1 = min(I, i0 + chunk);
     float acc[L];
@@ -75,6 +76,7 @@ __global__ void __launch_bounds__(256)
 ttmc3_final_kernel(int n_chunks, int64_t n_out, const float *__restrict__ P, float *__restrict__ A)
 {
     __shared__ float4 red[256];
+    sa_after_previous();
     const int col = threadIdx.x & 15, phase = threadIdx.x >> 4;
     const int64_t x = (int64_t(blockIdx.x) * 16 + col) * 4;               // n_out is a multiple of 64
     float4 s = make_float4(0.f, 0.f, 0.f, 0.f);
@@ -137,7 +139,7 @@ sa_status sa_launch_ttmc3(const sa_tensor *t, const sa_dense *ops, float *out, v
         if (s != SA_OK) return s;
         const int64_t n_out = L * cols;
         // n_blocks == 0 (a tensor without nonzeros): the sum over no accumulators writes zeros
-        ttmc3_final_kernel<<<(unsigned)(n_out / 64), 256, 0, stream>>>(n_blocks, n_out, partials, out);
+        sa_launch(ttmc3_final_kernel, (unsigned)(n_out / 64), 256, 0, stream, n_blocks, n_out, partials, out);
         if (cudaGetLastError() != cudaSuccess) return SA_E_CUDA;
         *launches = (n_blocks > 0 ? 1 : 0) + 1;
         return SA_OK;
@@ -152,11 +154,11 @@ sa_status sa_launch_ttmc3(const sa_tensor *t, const sa_dense *ops, float *out, v
     if (s != SA_OK) return s;
     *launches = n3;
     dim3 grid((unsigned)(cols / 256), (unsigned)p.n_chunks);              // cols is 256, 512 or 1024
-    if (L == 16) ttmc3_partial_kernel<16><<<grid, 256, 0, stream>>>(I, p.chunk, cols, T, ops[0].ptr, uint32_t(ops[0].ld), P);
-    else ttmc3_partial_kernel<32><<<grid, 256, 0, stream>>>(I, p.chunk, cols, T, ops[0].ptr, uint32_t(ops[0].ld), P);
+    if (L == 16) sa_launch(ttmc3_partial_kernel<16>, grid, 256, 0, stream, I, p.chunk, cols, T, ops[0].ptr, uint32_t(ops[0].ld), P);
+    else sa_launch(ttmc3_partial_kernel<32>, grid, 256, 0, stream, I, p.chunk, cols, T, ops[0].ptr, uint32_t(ops[0].ld), P);
     if (cudaGetLastError() != cudaSuccess) return SA_E_CUDA;
     const int64_t n_out = L * cols;
-    ttmc3_final_kernel<<<(unsigned)(n_out / 64), 256, 0, stream>>>(p.n_chunks, n_out, P, out);
+    sa_launch(ttmc3_final_kernel, (unsigned)(n_out / 64), 256, 0, stream, p.n_chunks, n_out, P, out);
     if (cudaGetLastError() != cudaSuccess) return SA_E_CUDA;
     *launches += 2;
     return SA_OK;
