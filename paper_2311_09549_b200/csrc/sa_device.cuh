@@ -57,23 +57,29 @@ static inline sa_limits sa_make_limits(const sa_tensor *t, int64_t gather_rows, 
     return lim;
 }
 
-// Kernels are launched so that they may start while the one before them on the stream still runs (programmatic dependent
-// launch): their blocks take the places that the other's last round leaves, read what no kernel ever writes (work lists, the
-// tensor's arrays) and then wait, in sa_after_previous, until the other is through and its results can be seen.  Nothing else may
-// be read or written before that, and some thread of every launch has to wait, or a kernel further back could still be running.
-// Then they let the next kernel on the stream start in the same way.  Back to back, us, without / with: order-3 tensor of 20 K
-// nonzeros (one launch) 10.2 / 9.5, of 2.3 M (two) 49.6 / 45.6, kernel 2 on 60 K nonzeros (two) 18.1 / 16.0.
+// Kernels may start while the one before them on the stream still runs (programmatic dependent launch): their blocks take the
+// places that the other's last round leaves, read what no kernel ever writes (work lists, the tensor's arrays) and then wait, in
+// sa_after_previous, until the other is through and its results can be seen.  Nothing else may be read or written before that,
+// and some thread of every launch has to wait, or a kernel further back could still be running.  Then they let the next kernel
+// on the stream start in the same way.  Back to back, us, without / with: order-3 tensor of 20 K nonzeros (one launch)
+// 10.2 / 9.5, kernel 2 on 60 K nonzeros (two) 18.1 / 16.0.
 __device__ __forceinline__ void sa_after_previous()
 {
     asm volatile("griddepcontrol.wait;" ::: "memory");
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
 }
-template <bool EARLY = true, typename... Params, typename... Args>
+// Which launches may: an SM keeps its split of shared memory and L1 as long as blocks are on it, so a kernel that starts beside
+// one with another split runs with that split to its end: with little L1 (gather of kernel 7, 12.5 M nonzeros, behind the dense
+// stage: 140 us, early 164; kernel 2 on a large graph 984 us, early 1486) or with fewer blocks per SM than it has room for.
+enum class sa_start {
+    FOLLOWS,        // behind a kernel of the same call that leaves it what it needs: early
+    FIRST,          // first of its call, behind anything: early where every block can have an SM to itself
+    ALONE           // lives on L1, behind a kernel with much shared memory: never early
+};
+template <sa_start START, typename... Params, typename... Args>
 static inline cudaError_t sa_launch(void (*kernel)(Params...), dim3 grid, unsigned threads, size_t smem, cudaStream_t stream, Args... args)
 {
-    // EARLY = false: an SM keeps its split of shared memory and L1 as long as blocks are on it, so a kernel that lives on L1
-    // (or needs more shared memory) must not start beside one with another split: gather of kernel 7 (12.5 M nonzeros) behind
-    // the dense stage 140 us, early 164.
+    const bool early = START == sa_start::FOLLOWS || (START == sa_start::FIRST && int64_t(grid.x) * grid.y <= SA_SMS);
     cudaLaunchAttribute attr;
     attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr.val.programmaticStreamSerializationAllowed = 1;
@@ -83,7 +89,7 @@ static inline cudaError_t sa_launch(void (*kernel)(Params...), dim3 grid, unsign
     cfg.dynamicSmemBytes = smem;
     cfg.stream = stream;
     cfg.attrs = &attr;
-    cfg.numAttrs = EARLY ? 1 : 0;
+    cfg.numAttrs = early ? 1 : 0;
     return cudaLaunchKernelEx(&cfg, kernel, Params(args)...);
 }
 
@@ -216,12 +222,12 @@ static inline cudaError_t sa_launch_fixup(const sa_worklist &wl, const float *pa
     const int nf4 = tile_floats / 4;
     if (nf4 <= 32) {
         const unsigned rows = (unsigned)wl.fix.size(), big = (unsigned)wl.n_big_fix;
-        return sa_launch(sa_fixup_rows_kernel, big + (rows - big + 7) / 8, 256, 0, stream, wl.d_fix, int(rows), int(big), partial, out, tile_floats);
+        return sa_launch<sa_start::FOLLOWS>(sa_fixup_rows_kernel, big + (rows - big + 7) / 8, 256, 0, stream, wl.d_fix, int(rows), int(big), partial, out, tile_floats);
     }
     int shift = 0;
     while ((4 << shift) < tile_floats) ++shift;
     const int64_t zeros = int64_t(wl.fix.size()) - wl.n_sum_fix;
     const int64_t blocks = (wl.n_big_fix << (shift - 4)) + ((wl.n_sum_fix - wl.n_big_fix) << (shift - 6)) + (((zeros << shift) + 255) >> 8);
-    return sa_launch(sa_fixup_kernel, unsigned(blocks), 256, 0, stream, wl.d_fix, unsigned(wl.n_big_fix), unsigned(wl.n_sum_fix), unsigned(wl.fix.size()),
+    return sa_launch<sa_start::FOLLOWS>(sa_fixup_kernel, unsigned(blocks), 256, 0, stream, wl.d_fix, unsigned(wl.n_big_fix), unsigned(wl.n_sum_fix), unsigned(wl.fix.size()),
                      partial, out, shift);
 }

@@ -239,6 +239,7 @@ ttm4_subtree_kernel(const sa_item *__restrict__ items, int64_t n_items, const in
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int64_t idx = int64_t(blockIdx.x) * SA_WARPS_PER_CTA + warp;
     if (idx >= n_items) return;
+    sa_after_previous();                    // here: further down it would part loads that are in flight together (2 us)
     const sa_item it = items[idx];
     if (!SA_CHK(lim.status, it.f0 >= 0 && it.f1 - it.f0 <= SA_SUB_MAX_F3 && it.f1 <= lim.n_fibers && it.out_row >= 0 &&
                                 it.row_end - it.out_row <= SA_SUB_MAX_ROWS && it.row_end <= lim.n_subtrees && it.p0 >= 0 && it.p1 <= lim.nnz,
@@ -253,7 +254,6 @@ ttm4_subtree_kernel(const sa_item *__restrict__ items, int64_t n_items, const in
     int kk0 = lane < nf3 ? __ldg(crd_k + it.f0 + lane) : 0;
     int kk1 = lane + 32 < nf3 ? __ldg(crd_k + it.f0 + 32 + lane) : 0;
     if (!SA_CHK(lim.status, uint32_t(kk0) < lim.d_rows && uint32_t(kk1) < lim.d_rows, 74, kk0)) kk0 = kk1 = 0;
-    sa_after_previous();
     // word 16 of a fiber's parked row: the element offset of its row of D
     pk[lane * SUB_RS + R] = __uint_as_float(uint32_t(kk0) * ld_d);
     pk[(lane + 32) * SUB_RS + R] = __uint_as_float(uint32_t(kk1) * ld_d);
@@ -432,7 +432,7 @@ sa_status sa_launch_ttm4_fissioned(const sa_tensor *t, const sa_dense *ops, floa
     v.nnz = t->wl4_main.nnz;
     v.nnz_total = t->nnz;
     v.status = t->d_status;
-    v.early = false;
+    v.first = false;
     fis_limits lim;
     lim.status = t->d_status;
     lim.c_rows = uint32_t(ops[0].rows); lim.d_rows = uint32_t(ops[1].rows); lim.e_rows = uint32_t(ops[2].rows);
@@ -448,7 +448,7 @@ sa_status sa_launch_ttm4_fissioned(const sa_tensor *t, const sa_dense *ops, floa
         static sa_device_flags attr_contig, attr_strided;
         if (!sa_set_smem_once(kern, SUB_SMEM, contig ? attr_contig : attr_strided)) return SA_E_CUDA;
         const int64_t ctas = (n_sub + SA_WARPS_PER_CTA - 1) / SA_WARPS_PER_CTA;
-        sa_launch<false>(kern, (unsigned)ctas, 256, SUB_SMEM, stream, t->wl4_sub.d_items, n_sub, t->d_pos[2], t->d_pos[3], t->d_crd[2],
+        sa_launch<sa_start::ALONE>(kern, (unsigned)ctas, 256, SUB_SMEM, stream, t->wl4_sub.d_items, n_sub, t->d_pos[2], t->d_pos[3], t->d_crd[2],
                                                                        t->d_nzpack, ops[1].ptr, ops[1].ld, ops[2].ptr, ops[2].ld, T2, lim);
         if (cudaGetLastError() != cudaSuccess) return SA_E_CUDA;
         *launches += 1;
@@ -468,7 +468,7 @@ sa_status sa_launch_ttm4_fissioned(const sa_tensor *t, const sa_dense *ops, floa
         const int64_t ctas = std::min<int64_t>((n_items + SA_WARPS_PER_CTA - 1) / SA_WARPS_PER_CTA, int64_t(sms) * 2);
         static sa_device_flags attr_slice;
         if (!sa_set_smem_once(ttm4_slice_kernel, SL_SMEM, attr_slice)) return SA_E_CUDA;
-        sa_launch<false>(ttm4_slice_kernel, (unsigned)ctas, 256, SL_SMEM, stream, wl.d_items, n_items, t->d_crd[1], T2, ops[0].ptr, uint32_t(ops[0].ld),
+        sa_launch<sa_start::ALONE>(ttm4_slice_kernel, (unsigned)ctas, 256, SL_SMEM, stream, wl.d_items, n_items, t->d_crd[1], T2, ops[0].ptr, uint32_t(ops[0].ld),
                                                                   out, part2, lim);
         if (cudaGetLastError() != cudaSuccess) return SA_E_CUDA;
         *launches += 1;
