@@ -76,8 +76,12 @@ enum class sa_start {
     FIRST,          // first of its call, behind anything: early where every block can have an SM to itself
     ALONE           // lives on L1, behind a kernel with much shared memory: never early
 };
-template <sa_start START, typename... Params, typename... Args>
-static inline cudaError_t sa_launch(void (*kernel)(Params...), dim3 grid, unsigned threads, size_t smem, cudaStream_t stream, Args... args)
+// The arguments convert as they do in a call (not by a cast: a pointer in the wrong place does not compile).
+template <typename T>
+struct sa_arg { using type = T; };
+template <sa_start START, typename... Params>
+static inline cudaError_t sa_launch(void (*kernel)(Params...), dim3 grid, unsigned threads, size_t smem, cudaStream_t stream,
+                                    typename sa_arg<Params>::type... args)
 {
     const bool early = START == sa_start::FOLLOWS || (START == sa_start::FIRST && int64_t(grid.x) * grid.y <= SA_SMS);
     cudaLaunchAttribute attr;
@@ -90,7 +94,7 @@ static inline cudaError_t sa_launch(void (*kernel)(Params...), dim3 grid, unsign
     cfg.stream = stream;
     cfg.attrs = &attr;
     cfg.numAttrs = early ? 1 : 0;
-    return cudaLaunchKernelEx(&cfg, kernel, Params(args)...);
+    return cudaLaunchKernelEx(&cfg, kernel, args...);
 }
 
 // Opt a kernel into `bytes` of dynamic shared memory once per device instead of once per launch (the attribute is

@@ -1,0 +1,41 @@
+"""What the launch wrapper of the kernels (sa_launch) takes and refuses at compile time.  Needs nvcc, no GPU."""
+import os
+import subprocess
+
+import pytest
+
+ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+
+SOURCE = """
+#include "sa_device.cuh"
+__global__ void kernel(const int32_t *index, int32_t *status, float *out, int64_t n)
+{
+    sa_after_previous();
+    if (n > 0) out[0] = float(index[0] + status[0]);
+}
+cudaError_t launch(const int32_t *index, int32_t *status, float *out)
+{
+    return sa_launch<sa_start::FIRST>(kernel, 1u, 32u, 0, nullptr, %s);
+}
+"""
+
+
+def _compiles(tmp_path, args):
+    src = tmp_path / "launch.cu"
+    src.write_text(SOURCE % args)
+    nvcc = os.environ.get("NVCC", "/usr/local/cuda/bin/nvcc")
+    r = subprocess.run([nvcc, "-gencode", "arch=compute_100a,code=sm_100a", "-std=c++17", "-I", os.path.join(ROOT, "include"),
+                        "-I", os.path.join(ROOT, "paper_2311_09549_b200", "csrc"), "-c", str(src), "-o", str(tmp_path / "launch.o")],
+                       capture_output=True, text=True, timeout=300)
+    return r.returncode == 0, r.stderr
+
+
+@pytest.mark.parametrize("args, right", [
+    ("index, status, out, 7", True),                  # int -> int64_t, as in a call
+    ("index, out, status, int64_t(7)", False),        # two arguments swapped
+    ("index, index, out, int64_t(7)", False),         # a constant array where the kernel writes
+    ("index, status, int64_t(7), out", False),        # a number for a pointer
+])
+def test_arguments_convert_only_as_in_a_call(tmp_path, args, right):
+    ok, log = _compiles(tmp_path, args)
+    assert ok == right, log
