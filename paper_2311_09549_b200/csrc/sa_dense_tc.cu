@@ -172,13 +172,6 @@ __device__ __forceinline__ void tc_ld16(uint32_t taddr, float (&v)[16])
     for (int x = 0; x < 16; ++x) v[x] = __uint_as_float(r[x]);
 }
 
-__device__ __forceinline__ float4 tc_ldg4(const float *p)
-{
-    float4 v;
-    asm volatile("ld.global.nc.L1::no_allocate.v4.f32 {%0,%1,%2,%3}, [%4];" : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w) : "l"(p));
-    return v;
-}
-
 // packed BF16 pair, element `lo` in the low half
 __device__ __forceinline__ uint32_t tc_bf16x2(float lo, float hi)
 {
@@ -208,8 +201,7 @@ __device__ __forceinline__ uint32_t tc_sw128(uint32_t row, uint32_t k)
 
 template <int L, int M, bool HAD>
 __global__ void __launch_bounds__(TC_THREADS, 1)
-gemm_tc_kernel(int64_t J, const float *__restrict__ C, int64_t ldc, const float *__restrict__ H, int64_t ldh,
-               const float *__restrict__ D, int64_t ldd, float *__restrict__ Eout, int part_shift, int32_t *__restrict__ status)
+gemm_tc_kernel(int64_t J, sa_data C, int64_t ldc, sa_data H, int64_t ldh, sa_data D, int64_t ldd, float *__restrict__ Eout, int part_shift, int32_t *__restrict__ status)
 {
     using G = tc_cfg<L, M, HAD>;
     extern __shared__ uint8_t tc_smem_raw[];
@@ -229,7 +221,7 @@ gemm_tc_kernel(int64_t J, const float *__restrict__ C, int64_t ldc, const float 
         const int k = x / M * 8, n = x % M;
         float v[8];
 #pragma unroll
-        for (int i = 0; i < 8; ++i) v[i] = __ldg(D + int64_t(k + i) * ldd + n);
+        for (int i = 0; i < 8; ++i) v[i] = (D + (int64_t(k + i) * ldd + n)).ld();
         uint8_t *dst = smem + G::OFF_D + uint32_t(k / TC_KC) * G::D_TILE + tc_sw128(n, k % TC_KC);
 #pragma unroll
         for (int z = 0; z < G::PARTS; ++z) {                                // row n + z M: same swizzle phase
@@ -321,9 +313,9 @@ gemm_tc_kernel(int64_t J, const float *__restrict__ C, int64_t ldc, const float 
                     for (int q = 0; q < M / 32; ++q) acc[q] = 0.f;
 #pragma unroll 8
                     for (int k = 0; k < L; ++k) {
-                        const float x = __ldg(C + row * ldc + k) * __ldg(H + row * ldh + k);
+                        const float x = (C + (row * ldc + k)).ld() * (H + (row * ldh + k)).ld();
 #pragma unroll
-                        for (int q = 0; q < M / 32; ++q) acc[q] = fmaf(x, __ldg(D + int64_t(k) * ldd + 32 * q + lane), acc[q]);
+                        for (int q = 0; q < M / 32; ++q) acc[q] = fmaf(x, (D + (int64_t(k) * ldd + 32 * q + lane)).ld(), acc[q]);
                     }
 #pragma unroll
                     for (int q = 0; q < M / 32; ++q)
@@ -392,13 +384,13 @@ gemm_tc_kernel(int64_t J, const float *__restrict__ C, int64_t ldc, const float 
                 if (q + TC_PF < n_chunks) {                        // one 128-byte line per thread: HBM latency is paid by L2
                     const int64_t pq = q + TC_PF;
                     const int64_t row = min((int64_t(blockIdx.x) + (pq / G::KCH) * gridDim.x) * TC_BM + (t >> 1), J - 1);
-                    asm volatile("prefetch.global.L2 [%0];" ::"l"(C + row * ldc + int(pq % G::KCH) * TC_KC + 32 * (t & 1)));
+                    asm volatile("prefetch.global.L2 [%0];" ::"l"((C + (row * ldc + int(pq % G::KCH) * TC_KC + 32 * (t & 1))).p));
                 }
                 if (q < n_chunks) {
                     const int64_t row0 = (int64_t(blockIdx.x) + (q / G::KCH) * gridDim.x) * TC_BM + r0;
-                    const float *src = C + int(q % G::KCH) * TC_KC + 4 * qf;
+                    const sa_data src = C + (int(q % G::KCH) * TC_KC + 4 * int(qf));
 #pragma unroll
-                    for (int i = 0; i < NR; ++i) b[i] = tc_ldg4(src + min(row0 + 16 * i, J - 1) * ldc);   // rows past the end re-read the last row
+                    for (int i = 0; i < NR; ++i) b[i] = (src + min(row0 + 16 * i, J - 1) * ldc).ld4_once();   // rows past the end re-read the last row
                 }
             };
             auto convert = [&](const float4 (&b)[NR], int64_t q) -> bool {
@@ -441,15 +433,15 @@ gemm_tc_kernel(int64_t J, const float *__restrict__ C, int64_t ldc, const float 
                 if (q + TC_PF < n_chunks) {
                     const int64_t pq = q + TC_PF;
                     const int64_t row = min((int64_t(blockIdx.x) + (pq / G::KCH) * gridDim.x) * TC_BM + (t >> 1), J - 1);
-                    asm volatile("prefetch.global.L2 [%0];" ::"l"((half ? H + row * ldh : C + row * ldc) + int(pq % G::KCH) * TC_KC + 32 * (t & 1)));
+                    asm volatile("prefetch.global.L2 [%0];" ::"l"(((half ? H + row * ldh : C + row * ldc) + (int(pq % G::KCH) * TC_KC + 32 * (t & 1))).p));
                 }
                 if (q < n_chunks) {
                     const int64_t row0 = (int64_t(blockIdx.x) + (q / G::KCH) * gridDim.x) * TC_BM + r0 + half * (TC_BM / 2);
                     const int col = int(q % G::KCH) * TC_KC + 4 * int(qf);
 #pragma unroll
-                    for (int i = 0; i < HR; ++i) b[i] = tc_ldg4(C + col + min(row0 + 16 * i, J - 1) * ldc);
+                    for (int i = 0; i < HR; ++i) b[i] = (C + (col + min(row0 + 16 * i, J - 1) * ldc)).ld4_once();
 #pragma unroll
-                    for (int i = 0; i < HR; ++i) b[HR + i] = tc_ldg4(H + col + min(row0 + 16 * i, J - 1) * ldh);
+                    for (int i = 0; i < HR; ++i) b[HR + i] = (H + (col + min(row0 + 16 * i, J - 1) * ldh)).ld4_once();
                 }
             };
             auto convert = [&](const float4 (&b)[NR], int64_t q, auto upper) -> bool {

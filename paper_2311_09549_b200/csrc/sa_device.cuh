@@ -5,13 +5,63 @@
 #include <algorithm>
 #include <atomic>
 #include <cstdint>
+#include <type_traits>
 
 #include "sa_internal.h"
 
 #define SA_FULL_MASK 0xffffffffu
 
-__device__ __forceinline__ float4 sa_ldg4(const float *p) { return __ldg(reinterpret_cast<const float4 *>(p)); }
-__device__ __forceinline__ float2 sa_ldg2(const float *p) { return __ldg(reinterpret_cast<const float2 *>(p)); }
+// fp32 numbers that an earlier kernel on the stream may have written: dense operands, temporaries, partial sums.  A kernel may
+// start while that one is still running (sa_launch), so they are not constant for its lifetime, which is what __ldg,
+// ld.global.nc and `const float *__restrict__` promise: the compiler may move such loads up across the wait, and the read-only
+// path need not see the new values.  These loads are coherent, and volatile like the wait, so that they stay behind it.  Work
+// lists and the tensor's arrays (sa_values: its values) are never written by a kernel; they take the read-only path.
+struct sa_data {
+    const float *p;
+    __host__ __device__ __forceinline__ sa_data(const float *q = nullptr) : p(q) {}
+    __device__ __forceinline__ sa_data operator+(int64_t n) const { return p + n; }
+    __device__ __forceinline__ sa_data plus_bytes(uint64_t n) const { return reinterpret_cast<const float *>(reinterpret_cast<const char *>(p) + n); }
+    __device__ __forceinline__ float ld() const
+    {
+        float v;
+        asm volatile("ld.global.f32 %0, [%1];" : "=f"(v) : "l"(p));
+        return v;
+    }
+    __device__ __forceinline__ float ld_cs() const             // read once: evict first
+    {
+        float v;
+        asm volatile("ld.global.cs.f32 %0, [%1];" : "=f"(v) : "l"(p));
+        return v;
+    }
+    __device__ __forceinline__ float2 ld2() const
+    {
+        float2 v;
+        asm volatile("ld.global.v2.f32 {%0,%1}, [%2];" : "=f"(v.x), "=f"(v.y) : "l"(p));
+        return v;
+    }
+    __device__ __forceinline__ float4 ld4() const
+    {
+        float4 v;
+        asm volatile("ld.global.v4.f32 {%0,%1,%2,%3}, [%4];" : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w) : "l"(p));
+        return v;
+    }
+    __device__ __forceinline__ float4 ld4_cs() const
+    {
+        float4 v;
+        asm volatile("ld.global.cs.v4.f32 {%0,%1,%2,%3}, [%4];" : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w) : "l"(p));
+        return v;
+    }
+    __device__ __forceinline__ float4 ld4_once() const         // not kept in L1
+    {
+        float4 v;
+        asm volatile("ld.global.L1::no_allocate.v4.f32 {%0,%1,%2,%3}, [%4];" : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w) : "l"(p));
+        return v;
+    }
+};
+struct sa_values {
+    const float *p;
+    __host__ __device__ __forceinline__ sa_values(const float *q) : p(q) {}
+};
 
 // Streaming (evict-first) stores for output tiles that are written once and never re-read, so
 // they do not displace the factor matrices held in L2.
@@ -94,6 +144,7 @@ static inline cudaError_t sa_launch(void (*kernel)(Params...), dim3 grid, unsign
     cfg.stream = stream;
     cfg.attrs = &attr;
     cfg.numAttrs = early ? 1 : 0;
+    static_assert(!(std::is_same<Params, const float *>::value || ...), "fp32 inputs are sa_data or sa_values");
     return cudaLaunchKernelEx(&cfg, kernel, args...);
 }
 
@@ -147,7 +198,7 @@ __device__ __forceinline__ void cp_async_wait() { asm volatile("cp.async.wait_gr
 // are zeroed 256 float4 per block.  Fixed summation order: deterministic.  192 partials of 4 KB: 13 us with 64 columns per
 // block throughout, 7.5 us.
 static __global__ void __launch_bounds__(256)
-sa_fixup_kernel(const sa_fix *__restrict__ fix, unsigned n_big, unsigned n_sum, unsigned n_fix, const float *__restrict__ partial,
+sa_fixup_kernel(const sa_fix *__restrict__ fix, unsigned n_big, unsigned n_sum, unsigned n_fix, sa_data partial,
                 float *__restrict__ out, int shift)
 {
     __shared__ float4 red[256];
@@ -167,10 +218,10 @@ sa_fixup_kernel(const sa_fix *__restrict__ fix, unsigned n_big, unsigned n_sum, 
     const int col = threadIdx.x & (W - 1), phase = threadIdx.x >> wlog;
     const int64_t f4 = int64_t(b & ((1u << (shift - wlog)) - 1)) * W + col;
     float4 s = make_float4(0.f, 0.f, 0.f, 0.f);
-    const float *base = partial + ((int64_t(e.slot0) << shift) + f4) * 4;
+    const sa_data base = partial + ((int64_t(e.slot0) << shift) + f4) * 4;
 #pragma unroll 4
     for (int q = phase; q < e.count; q += P) {
-        const float4 v = *reinterpret_cast<const float4 *>(base + ((int64_t(q) << shift) * 4));
+        const float4 v = (base + ((int64_t(q) << shift) * 4)).ld4();
         s.x += v.x; s.y += v.y; s.z += v.z; s.w += v.w;
     }
     red[threadIdx.x] = s;
@@ -187,7 +238,7 @@ sa_fixup_kernel(const sa_fix *__restrict__ fix, unsigned n_big, unsigned n_sum, 
 // The same for rows of at most 128 floats (8, 16 or 32 float4): the first n_big entries (the builder puts the longest
 // first) take a block each as above, the others a warp each, which is all that a few partial rows can use.
 static __global__ void __launch_bounds__(256)
-sa_fixup_rows_kernel(const sa_fix *__restrict__ fix, int n_fix, int n_big, const float *__restrict__ partial, float *__restrict__ out,
+sa_fixup_rows_kernel(const sa_fix *__restrict__ fix, int n_fix, int n_big, sa_data partial, float *__restrict__ out,
                      int row_floats)
 {
     __shared__ float4 red[256];
@@ -200,10 +251,10 @@ sa_fixup_rows_kernel(const sa_fix *__restrict__ fix, int n_fix, int n_big, const
     const int who = big ? int(threadIdx.x) : lane, P = (big ? 256 : 32) / W;
     const int col = who % W, phase = who / W;
     float4 s = make_float4(0.f, 0.f, 0.f, 0.f);
-    const float *base = partial + int64_t(e.slot0) * row_floats + col * 4;
+    const sa_data base = partial + (int64_t(e.slot0) * row_floats + col * 4);
 #pragma unroll 4
     for (int q = phase; q < e.count; q += P) {
-        const float4 v = *reinterpret_cast<const float4 *>(base + int64_t(q) * row_floats);
+        const float4 v = (base + int64_t(q) * row_floats).ld4();
         s.x += v.x; s.y += v.y; s.z += v.z; s.w += v.w;
     }
     red[threadIdx.x] = s;

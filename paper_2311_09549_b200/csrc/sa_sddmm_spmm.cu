@@ -31,9 +31,8 @@ struct sd_cfg {
 template <int K, int L, int CTAS>
 __global__ void __launch_bounds__(256, CTAS)
 sddmm_spmm_kernel(const sa_item *__restrict__ items, int64_t n_items, const int32_t *__restrict__ pos,
-                  const int2 *__restrict__ nz, const float *__restrict__ C, uint32_t ldc, const float *__restrict__ D,
-                  uint32_t ldd, const float *__restrict__ E, uint32_t lde, float *__restrict__ out, float *__restrict__ partial,
-                  float *__restrict__ sampled, const sa_limits lim)
+                  const int2 *__restrict__ nz, sa_data C, uint32_t ldc, sa_data D, uint32_t ldd, sa_data E, uint32_t lde,
+                  float *__restrict__ out, float *__restrict__ partial, float *__restrict__ sampled, const sa_limits lim)
 {
     using G = sd_cfg<K, L>;
     constexpr int DQ = G::DQ, EQ = G::EQ, U = G::U;
@@ -59,7 +58,7 @@ sddmm_spmm_kernel(const sa_item *__restrict__ items, int64_t n_items, const int3
     auto load_c = [&](float4 (&x)[DQ], int row) {
         if (row < rend) {
 #pragma unroll
-            for (int q = 0; q < DQ; ++q) x[q] = sa_ldg4(C + (uint32_t(row) * ldc + 32u * q + 4u * l));
+            for (int q = 0; q < DQ; ++q) x[q] = (C + (uint32_t(row) * ldc + 32u * q + 4u * l)).ld4();
         }
     };
     int b = row_end(r), bn = row_end(r + 1);
@@ -74,7 +73,7 @@ sddmm_spmm_kernel(const sa_item *__restrict__ items, int64_t n_items, const int3
     if (G::AHEAD) load_c(cn, r + 1);
 #pragma unroll
     for (int q = 0; q < EQ; ++q) acc[q] = make_float4(0.f, 0.f, 0.f, 0.f);
-    const char *Dl = reinterpret_cast<const char *>(D + 4 * l), *El = reinterpret_cast<const char *>(E + 4 * l);
+    const sa_data Dl = D + 4 * l, El = E + 4 * l;
     const uint32_t d_bytes = ldd * 4u, e_bytes = lde * 4u;
     for (;;) {
         while (p == b && r < rend) {                  // the row is complete (or empty: +0)
@@ -107,9 +106,9 @@ sddmm_spmm_kernel(const sa_item *__restrict__ items, int64_t n_items, const int3
                 uint32_t j = uint32_t(rec[u].x);
                 if (!SA_CHK(lim.status, j < lim.gather_rows, 42, j)) j = 0u;
 #pragma unroll
-                for (int q = 0; q < DQ; ++q) d[u][q] = __ldg(reinterpret_cast<const float4 *>(Dl + uint64_t(j) * d_bytes) + 8 * q);
+                for (int q = 0; q < DQ; ++q) d[u][q] = (Dl.plus_bytes(uint64_t(j) * d_bytes) + 32 * q).ld4();
 #pragma unroll
-                for (int q = 0; q < EQ; ++q) e[u][q] = __ldg(reinterpret_cast<const float4 *>(El + uint64_t(j) * e_bytes) + 8 * q);
+                for (int q = 0; q < EQ; ++q) e[u][q] = (El.plus_bytes(uint64_t(j) * e_bytes) + 32 * q).ld4();
             }
         }
 #pragma unroll

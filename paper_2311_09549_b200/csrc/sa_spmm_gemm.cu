@@ -37,20 +37,19 @@ __device__ __forceinline__ void row_times_D(const float *__restrict__ Ts, const 
 }
 
 template <int L, int M>
-__device__ __forceinline__ void load_D(float *Ds, const float *__restrict__ D, int64_t ldd)
+__device__ __forceinline__ void load_D(float *Ds, sa_data D, int64_t ldd)
 {
     for (int x = threadIdx.x * 4; x < L * M; x += blockDim.x * 4) {
         const int l = x / M, m = x % M;
-        *reinterpret_cast<float4 *>(Ds + x) = sa_ldg4(D + int64_t(l) * ldd + m);
+        *reinterpret_cast<float4 *>(Ds + x) = (D + (int64_t(l) * ldd + m)).ld4();
     }
 }
 
 template <int L, int M, bool HAD>
 __global__ void __launch_bounds__(256, 3)
 spmm_gemm_left_kernel(const sa_item *__restrict__ items, int64_t n_items, const int32_t *__restrict__ pos,
-                      const int32_t *__restrict__ crd, const float *__restrict__ vals, const float *__restrict__ C,
-                      int64_t ldc, const float *__restrict__ H, int64_t ldh, const float *__restrict__ D, int64_t ldd,
-                      float *__restrict__ out, float *__restrict__ partial, const sa_limits lim)
+                      const int32_t *__restrict__ crd, sa_values vals, sa_data C, int64_t ldc, sa_data H, int64_t ldh, sa_data D,
+                      int64_t ldd, float *__restrict__ out, float *__restrict__ partial, const sa_limits lim)
 {
     constexpr int LV4 = L / 128, MV = M / 32;
     extern __shared__ __align__(16) float smem[];
@@ -75,19 +74,19 @@ spmm_gemm_left_kernel(const sa_item *__restrict__ items, int64_t n_items, const 
                 const int n = min(32, b - base);
                 int jj = 0;
                 float vv = 0.f;
-                if (lane < n) { jj = crd[base + lane]; vv = vals[base + lane]; }
+                if (lane < n) { jj = crd[base + lane]; vv = __ldg(vals.p + base + lane); }
                 if (!SA_CHK(lim.status, uint32_t(jj) < lim.gather_rows, 53, jj)) jj = 0;
 #pragma unroll LEFT_UNROLL
                 for (int s = 0; s < n; ++s) {
                     const int j = __shfl_sync(SA_FULL_MASK, jj, s);
                     const float v = __shfl_sync(SA_FULL_MASK, vv, s);
-                    const float *crow = C + int64_t(j) * ldc + lane * 4;
-                    const float *hrow = H + int64_t(j) * ldh + lane * 4;     // HAD: the row of the Hadamard partner
+                    const sa_data crow = C + (int64_t(j) * ldc + lane * 4);
+                    const sa_data hrow = H + (int64_t(j) * ldh + lane * 4);     // HAD: the row of the Hadamard partner
 #pragma unroll
                     for (int q = 0; q < LV4; ++q) {
-                        float4 c = sa_ldg4(crow + q * 128);
+                        float4 c = (crow + q * 128).ld4();
                         if (HAD) {
-                            const float4 h = sa_ldg4(hrow + q * 128);
+                            const float4 h = (hrow + q * 128).ld4();
                             c.x *= h.x; c.y *= h.y; c.z *= h.z; c.w *= h.w;
                         }
                         t[q].x = fmaf(v, c.x, t[q].x); t[q].y = fmaf(v, c.y, t[q].y);
@@ -160,8 +159,7 @@ struct gemm_bf16_cfg {
 
 template <int L, int M>
 __global__ void __launch_bounds__(256, 1)
-gemm_bf16x3_kernel(int64_t J, const float *__restrict__ C, int64_t ldc, const float *__restrict__ D, int64_t ldd,
-                   float *__restrict__ Eout)
+gemm_bf16x3_kernel(int64_t J, sa_data C, int64_t ldc, sa_data D, int64_t ldd, float *__restrict__ Eout)
 {
     using G = gemm_bf16_cfg<L, M>;
     extern __shared__ __align__(16) float smem[];
@@ -175,7 +173,7 @@ gemm_bf16x3_kernel(int64_t J, const float *__restrict__ C, int64_t ldc, const fl
     for (int x = threadIdx.x; x < (L / 2) * M; x += 256) {
         const int p = x / M, m = x % M;
         uint32_t h, l;
-        bf16_split2(__ldg(D + int64_t(2 * p) * ldd + m), __ldg(D + int64_t(2 * p + 1) * ldd + m), h, l);
+        bf16_split2((D + (int64_t(2 * p) * ldd + m)).ld(), (D + (int64_t(2 * p + 1) * ldd + m)).ld(), h, l);
         Dh[p * G::DS + m] = h;
         Dl[p * G::DS + m] = l;
     }
@@ -192,7 +190,7 @@ gemm_bf16x3_kernel(int64_t J, const float *__restrict__ C, int64_t ldc, const fl
             for (int x = threadIdx.x; x < G::BM * (G::KC / 4); x += 256) {
                 const int r = x / (G::KC / 4), c4 = x % (G::KC / 4);
                 const int64_t row = min(row0 + r, J - 1);            // rows past the end re-read the last row
-                g_cp_async16(dst + r * G::CS + c4 * 4, C + row * ldc + k0 + c4 * 4);
+                g_cp_async16(dst + r * G::CS + c4 * 4, (C + (row * ldc + k0 + c4 * 4)).p);
             }
         }
         asm volatile("cp.async.commit_group;" ::: "memory");
@@ -271,15 +269,15 @@ gemm_bf16x3_kernel(int64_t J, const float *__restrict__ C, int64_t ldc, const fl
 template <int W>
 __global__ void __launch_bounds__(256)
 spmm_kernel(const sa_item *__restrict__ items, int64_t n_items, unsigned ctas_per_part, const int32_t *__restrict__ pos,
-            const int2 *__restrict__ nz, const float *__restrict__ E, int64_t J, int M, float *__restrict__ out,
-            float *__restrict__ partial, const sa_limits lim)
+            const int2 *__restrict__ nz, sa_data E, int64_t J, int M, float *__restrict__ out, float *__restrict__ partial,
+            const sa_limits lim)
 {
     constexpr int LPR = W / 4, U = 8;                       // lanes per row, nonzeros per step
     static_assert(LPR >= U, "one record per lane and step");
     const unsigned part = blockIdx.x / ctas_per_part, block = blockIdx.x - part * ctas_per_part;
     const int l = threadIdx.x % LPR;
     const int64_t idx = (int64_t(block) * 256 + threadIdx.x) / LPR;
-    E += int64_t(part) * J * W + 4 * l;
+    E = E + (int64_t(part) * J * W + 4 * l);
     int r = 0, rend = 0, p0 = 0, end = 0, dest = -1;
     if (idx < n_items) {
         const int4 ia = __ldg(reinterpret_cast<const int4 *>(items + idx));          // out_row, row_end, -, -
@@ -320,7 +318,7 @@ spmm_kernel(const sa_item *__restrict__ items, int64_t n_items, unsigned ctas_pe
             const int k = __shfl_sync(SA_FULL_MASK, rec.x, u, LPR);
             vs[u] = __int_as_float(__shfl_sync(SA_FULL_MASK, rec.y, u, LPR));
             e[u] = zero;
-            if (c + u < len) e[u] = sa_ldg4(E + int64_t(k) * W);
+            if (c + u < len) e[u] = (E + int64_t(k) * W).ld4();
         }
         rec = fetch(c + U);
 #pragma unroll
@@ -351,8 +349,8 @@ spmm_kernel(const sa_item *__restrict__ items, int64_t n_items, unsigned ctas_pe
 template <int M>
 __global__ void __launch_bounds__(256)
 fiber_spmm_kernel(const sa_item *__restrict__ items, int64_t n_items, const int32_t *__restrict__ pos,
-                  const int2 *__restrict__ nz, const float *__restrict__ E, int64_t lde, float *__restrict__ out,
-                  float *__restrict__ partial, const sa_limits lim)
+                  const int2 *__restrict__ nz, sa_data E, int64_t lde, float *__restrict__ out, float *__restrict__ partial,
+                  const sa_limits lim)
 {
     constexpr int LPR = M / 4, NG = 32 / LPR;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -407,7 +405,7 @@ fiber_spmm_kernel(const sa_item *__restrict__ items, int64_t n_items, const int3
             vs[u] = __shfl_sync(SA_FULL_MASK, v, u, LPR);
             uint32_t k = uint32_t(xs[u]) & 0x7fffffffu;
             if (!SA_CHK(lim.status, k < lim.gather_rows, 62, k)) k = 0u;
-            e[u] = sa_ldg4(E + int64_t(k) * lde + 4 * l);
+            e[u] = (E + (int64_t(k) * lde + 4 * l)).ld4();
         }
 #pragma unroll
         for (int u = 0; u < 8; ++u) {

@@ -75,16 +75,17 @@ __device__ __forceinline__ uint4 lds128(uint32_t a)
 __device__ __forceinline__ void sts32(uint32_t a, uint32_t v) { asm volatile("st.shared.u32 [%0], %1;" ::"r"(a), "r"(v) : "memory"); }
 __device__ __forceinline__ void prefetch_l1(const void *p) { asm volatile("prefetch.global.L1 [%0];" ::"l"(p)); }
 
-// A lane's piece of a factor row: VEC = 4 or 2 consecutive floats.  Plain read-only loads: with the
-// L1::no_allocate qualifier the rows also lost their place in L2 (hit rate 57 % instead of 87 %).
+// A lane's piece of a factor row: VEC = 4 or 2 consecutive floats.  Plain loads: with the L1::no_allocate qualifier the
+// rows also lost their place in L2 (hit rate 57 % instead of 87 %).
 template <int VEC>
 struct rowvec;
 template <>
 struct rowvec<4> {
     float x[4];
-    __device__ __forceinline__ void load(const char *p)
+    __device__ __forceinline__ void load(sa_data p)
     {
-        asm volatile("ld.global.nc.v4.f32 {%0,%1,%2,%3}, [%4];" : "=f"(x[0]), "=f"(x[1]), "=f"(x[2]), "=f"(x[3]) : "l"(p));
+        const float4 v = p.ld4();
+        x[0] = v.x; x[1] = v.y; x[2] = v.z; x[3] = v.w;
     }
     __device__ __forceinline__ void store_shared(uint32_t a) const
     {
@@ -94,9 +95,10 @@ struct rowvec<4> {
 template <>
 struct rowvec<2> {
     float x[2];
-    __device__ __forceinline__ void load(const char *p)
+    __device__ __forceinline__ void load(sa_data p)
     {
-        asm volatile("ld.global.nc.v2.f32 {%0,%1}, [%2];" : "=f"(x[0]), "=f"(x[1]) : "l"(p));
+        const float2 v = p.ld2();
+        x[0] = v.x; x[1] = v.y;
     }
     __device__ __forceinline__ void store_shared(uint32_t a) const
     {
@@ -107,7 +109,7 @@ struct rowvec<2> {
 // acc += Cg^T . T for the parked rows row0 + x, x = 0 .. 7, of which the first n are in use.
 template <int L, int M>
 __device__ __forceinline__ void ttm3_flush(float (&acc)[cfg<L, M>::MT][cfg<L, M>::NT][4], const float *__restrict__ ring,
-                                           int row0, int n, const float *__restrict__ C, int lane, const dbg_limits &lim, uint32_t ldc)
+                                           int row0, int n, sa_data C, int lane, const dbg_limits &lim, uint32_t ldc)
 {
     using K = cfg<L, M>;
     const int g = lane >> 2, t = lane & 3;
@@ -120,14 +122,13 @@ __device__ __forceinline__ void ttm3_flush(float (&acc)[cfg<L, M>::MT][cfg<L, M>
         uint32_t oa = va ? __float_as_uint(ra[M]) : 0u, ob = vb ? __float_as_uint(rb[M]) : 0u;
         if (!SA_CHK(lim.status, oa < lim.c_rows * ldc, 1, oa)) oa = 0u;
         if (!SA_CHK(lim.status, ob < lim.c_rows * ldc, 2, ob)) ob = 0u;
-        const float *ca = C + oa + g;
-        const float *cb = C + ob + g;
+        const sa_data ca = C + oa + g, cb = C + ob + g;
 #pragma unroll
         for (int mt = 0; mt < K::MT; ++mt) {
-            cf[mt][0] = va ? __ldg(ca + 16 * mt) : 0.f;
-            cf[mt][1] = va ? __ldg(ca + 16 * mt + 8) : 0.f;
-            cf[mt][2] = vb ? __ldg(cb + 16 * mt) : 0.f;
-            cf[mt][3] = vb ? __ldg(cb + 16 * mt + 8) : 0.f;
+            cf[mt][0] = va ? (ca + 16 * mt).ld() : 0.f;
+            cf[mt][1] = va ? (ca + (16 * mt + 8)).ld() : 0.f;
+            cf[mt][2] = vb ? (cb + 16 * mt).ld() : 0.f;
+            cf[mt][3] = vb ? (cb + (16 * mt + 8)).ld() : 0.f;
         }
     }
     uint32_t bh[K::NT][2], bl[K::NT][2];
@@ -156,7 +157,7 @@ __device__ __forceinline__ void ttm3_flush(float (&acc)[cfg<L, M>::MT][cfg<L, M>
 // lanes of equal columns when the unit ends.
 template <int M>
 __device__ __forceinline__ void had_flush(float (&hacc)[4], const float *__restrict__ ring, int row0, int n,
-                                          const float *__restrict__ C, int lane)
+                                          sa_data C, int lane)
 {
     constexpr int RS = M + 8, LANES = M / 4;
     const int m = 4 * (lane % LANES);
@@ -165,7 +166,7 @@ __device__ __forceinline__ void had_flush(float (&hacc)[4], const float *__restr
         const int x = x0 + lane / LANES;
         if (x < n) {
             const float *r = ring + (row0 + x) * RS;
-            const float4 c = sa_ldg4(C + __float_as_uint(r[M]) + m);
+            const float4 c = (C + __float_as_uint(r[M]) + m).ld4();
             const float4 v = *reinterpret_cast<const float4 *>(r + m);
             hacc[0] = fmaf(v.x, c.x, hacc[0]);
             hacc[1] = fmaf(v.y, c.y, hacc[1]);
@@ -247,7 +248,7 @@ __device__ __forceinline__ stream_range stream_of(int p0, int p1, int q)
 // What kernel 5 adds at the end of a unit (TTMC = true): the slice temporary T(i; m,n) in `acc` is not stored but
 // contracted with C(i,:) into the block's accumulator of the whole output, accs[l][m][n] += C(i,l) T(i; m,n).
 struct ttmc_sink {
-    const float *C3;        // C of kernel 5 (rows by i)
+    sa_data C3;             // C of kernel 5 (rows by i)
     uint32_t ldc3;
     int L3;                 // its columns
     float *accs;            // shared memory, L3 x L x M floats
@@ -259,9 +260,9 @@ __device__ __forceinline__ void ttmc_accumulate(const float (&acc)[cfg<L, M>::MT
 {
     using K = cfg<L, M>;
     const int g = lane >> 2, t = lane & 3;
-    const float *crow = sk.C3 + uint32_t(row) * sk.ldc3;
+    const sa_data crow = sk.C3 + uint32_t(row) * sk.ldc3;
     for (int l = 0; l < sk.L3; ++l) {
-        const float c = __ldg(crow + l);
+        const float c = (crow + l).ld();
         float *base = sk.accs + l * (L * M) + g * M + 2 * t;
 #pragma unroll
         for (int mt = 0; mt < K::MT; ++mt)
@@ -279,9 +280,8 @@ __device__ __forceinline__ void ttmc_accumulate(const float (&acc)[cfg<L, M>::MT
 template <int L, int M, bool HAD, bool TTMC = false>
 __device__ __forceinline__ void ttm3_warp_task(const sa_unit3 *__restrict__ units, int u0, int nu,
                                                const int32_t *__restrict__ crd_j, const int32_t *__restrict__ crd_k,
-                                               const float *__restrict__ vals, const uint32_t *__restrict__ endbits,
-                                               const float *__restrict__ C, uint32_t ldc, const float *__restrict__ D,
-                                               uint32_t ldd, unsigned char *__restrict__ wsm,
+                                               sa_values vals, const uint32_t *__restrict__ endbits, sa_data C, uint32_t ldc,
+                                               sa_data D, uint32_t ldd, unsigned char *__restrict__ wsm,
                                                float (&acc)[cfg<L, M>::MT][cfg<L, M>::NT][4], float (&hacc)[4], const bool keep,
                                                float *__restrict__ out, const dbg_limits &lim, const bool first, const ttmc_sink *sink = nullptr)
 {
@@ -317,7 +317,7 @@ __device__ __forceinline__ void ttm3_warp_task(const sa_unit3 *__restrict__ unit
             if (pg < fs.hi && pg + K::STEPS > fs.lo && SA_CHK(lim.status, pg >= 0 && pg <= lim.nnz, 3, pg)) {
                 const uint32_t dst = s_kv + slot * (K::NS * K::SLOT);
                 // lanes 0 .. 3 of the stream copy the sixteen indices, lanes 4 .. 7 the sixteen values
-                cp_async16_raw(dst + 16 * c, (c < 4 ? reinterpret_cast<const char *>(crd_k) : reinterpret_cast<const char *>(vals)) + 4 * int64_t(pg) + 16 * (c & 3));
+                cp_async16_raw(dst + 16 * c, (c < 4 ? reinterpret_cast<const char *>(crd_k) : reinterpret_cast<const char *>(vals.p)) + 4 * int64_t(pg) + 16 * (c & 3));
                 if (c == 0) cp_async4_raw(dst + 8 * K::STEPS, endbits + (pg >> 5));
             }
             if (++fr == fs.rounds) {
@@ -342,7 +342,7 @@ __device__ __forceinline__ void ttm3_warp_task(const sa_unit3 *__restrict__ unit
     int fq = load_sf(0);                                // next fiber this stream parks
     if (!SA_CHK(lim.status, uint32_t(fq) <= lim.n_fibers, 4, fq)) fq = 0;
     int jreg = __ldg(crd_j + fq + c);                   // C rows of the next eight fibers of the stream, one per lane
-    const char *dlane = reinterpret_cast<const char *>(D + c * VEC);
+    const sa_data dlane = D + c * VEC;
     const uint32_t row_bytes = ldd * 4u;
     cp_async_wait<DEPTH - 2>();
     __syncwarp();
@@ -352,7 +352,7 @@ __device__ __forceinline__ void ttm3_warp_task(const sa_unit3 *__restrict__ unit
         const uint4 ka = lds128(s_kv), kb = lds128(s_kv + 16);
         const uint32_t k8[8] = {ka.x, ka.y, ka.z, ka.w, kb.x, kb.y, kb.z, kb.w};
 #pragma unroll
-        for (int s = 0; s < 8; ++s) buf[s].load(dlane + uint64_t(SA_CHK(lim.status, k8[s] < lim.d_rows, 5, k8[s]) ? k8[s] : 0u) * row_bytes);
+        for (int s = 0; s < 8; ++s) buf[s].load(dlane.plus_bytes(uint64_t(SA_CHK(lim.status, k8[s] < lim.d_rows, 5, k8[s]) ? k8[s] : 0u) * row_bytes));
     }
     float T[VEC];
 #pragma unroll
@@ -411,7 +411,7 @@ __device__ __forceinline__ void ttm3_warp_task(const sa_unit3 *__restrict__ unit
         if (c < cnt) {
             const uint32_t off = uint32_t(jreg) * ldc;
             sts32(s_ring + ((slot + c) * K::RS + M) * 4, off);
-            prefetch_l1(C + off);
+            prefetch_l1((C + off).p);
             if (c + 8 < cnt)                                  // more than eight fibers of one stream end in this round
                 sts32(s_ring + ((slot + c + 8) * K::RS + M) * 4, uint32_t(__ldg(crd_j + fq + c + 8)) * ldc);
         }
@@ -439,7 +439,7 @@ __device__ __forceinline__ void ttm3_warp_task(const sa_unit3 *__restrict__ unit
 #pragma unroll
                         for (int x = 0; x < VEC; ++x) T[x] = fmaf(v4[s4], buf[b].x[x], T[x]);
                     }
-                    buf[b].load(dlane + uint64_t(SA_CHK(lim.status, k4[s4] < lim.d_rows, 7, k4[s4]) ? k4[s4] : 0u) * row_bytes);
+                    buf[b].load(dlane.plus_bytes(uint64_t(SA_CHK(lim.status, k4[s4] < lim.d_rows, 7, k4[s4]) ? k4[s4] : 0u) * row_bytes));
                     if (e8 & (1u << s)) {
                         rowvec<VEC> tv;
 #pragma unroll
@@ -510,9 +510,8 @@ __device__ __forceinline__ void ttm3_warp_task(const sa_unit3 *__restrict__ unit
 template <int L, int M, int NCTA, bool HAD>
 __global__ void __launch_bounds__(32 * SA_TTM3_WARPS, NCTA)
 ttm3_kernel(const sa_unit3 *__restrict__ units, const int32_t *__restrict__ task_start, int64_t n_tasks, int n_group_ctas,
-            const int32_t *__restrict__ crd_j, const int32_t *__restrict__ crd_k, const float *__restrict__ vals,
-            const uint32_t *__restrict__ endbits, const float *__restrict__ C, uint32_t ldc,
-            const float *__restrict__ D, uint32_t ldd, float *__restrict__ out, float *__restrict__ partial,
+            const int32_t *__restrict__ crd_j, const int32_t *__restrict__ crd_k, sa_values vals,
+            const uint32_t *__restrict__ endbits, sa_data C, uint32_t ldc, sa_data D, uint32_t ldd, float *__restrict__ out, float *__restrict__ partial,
             const dbg_limits lim)
 {
     using K = cfg<L, M>;
@@ -584,10 +583,9 @@ ttm3_kernel(const sa_unit3 *__restrict__ units, const int32_t *__restrict__ task
 template <int L, int M, int NCTA>
 __global__ void __launch_bounds__(32 * SA_TTM3_WARPS, NCTA)
 ttmc3_fused_kernel(const sa_unit3 *__restrict__ units, const int32_t *__restrict__ task_start, int64_t n_tasks, int n_group_ctas,
-                   const int32_t *__restrict__ crd_j, const int32_t *__restrict__ crd_k, const float *__restrict__ vals,
-                   const uint32_t *__restrict__ endbits, const float *__restrict__ C, uint32_t ldc,
-                   const float *__restrict__ D, uint32_t ldd, const float *__restrict__ C3, uint32_t ldc3, int L3,
-                   float *__restrict__ partials, const dbg_limits lim)
+                   const int32_t *__restrict__ crd_j, const int32_t *__restrict__ crd_k, sa_values vals,
+                   const uint32_t *__restrict__ endbits, sa_data C, uint32_t ldc, sa_data D, uint32_t ldd, sa_data C3, uint32_t ldc3,
+                   int L3, float *__restrict__ partials, const dbg_limits lim)
 {
     using K = cfg<L, M>;
     constexpr int TILE = L * M;
@@ -630,7 +628,7 @@ ttmc3_fused_kernel(const sa_unit3 *__restrict__ units, const int32_t *__restrict
         const int row = units[task_start[bt * SA_TTM3_WARPS]].out_row;       // warp 0 always has a unit
         const float *all = reinterpret_cast<const float *>(smem);
         if (SA_CHK(lim.status, uint32_t(row) < lim.n_slices_dim, 8, row)) {
-            const float *crow = C3 + uint32_t(row) * ldc3;
+            const sa_data crow = C3 + uint32_t(row) * ldc3;
             for (int x = threadIdx.x * 4; x < TILE; x += 32 * SA_TTM3_WARPS * 4) {
                 const int off = (x / M) * K::RS + (x % M);
                 float4 s = *reinterpret_cast<const float4 *>(all + off);
@@ -640,7 +638,7 @@ ttmc3_fused_kernel(const sa_unit3 *__restrict__ units, const int32_t *__restrict
                     s.x += v.x; s.y += v.y; s.z += v.z; s.w += v.w;
                 }
                 for (int l = 0; l < L3; ++l) {          // no other warp touches the accumulator during a chunk
-                    const float c = __ldg(crow + l);
+                    const float c = (crow + l).ld();
                     float4 *a = reinterpret_cast<float4 *>(accs + l * TILE + x);
                     float4 o = *a;
                     o.x = fmaf(c, s.x, o.x); o.y = fmaf(c, s.y, o.y); o.z = fmaf(c, s.z, o.z); o.w = fmaf(c, s.w, o.w);

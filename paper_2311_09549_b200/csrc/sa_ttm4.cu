@@ -66,7 +66,7 @@ __device__ __forceinline__ int f4_rowpos(int r, int pos) { return r * F4_RS + ((
 // parks it at every end-of-fiber bit (no reset: a predicated store and a pointer bump per step); the rows are
 // turned into per-fiber sums afterwards by subtracting the previous row inside each group's share.
 __device__ __forceinline__ void f4_stage_a(float *pk, uint32_t pk_s, int nf, int s3, int pe, const int2 *__restrict__ nz,
-                                           const float *__restrict__ E, uint32_t ld_e, int lane, const f4_limits &lim)
+                                           sa_data E, uint32_t ld_e, int lane, const f4_limits &lim)
 {
     const int g = lane >> 2, l = lane & 3;
     const int pb0 = __shfl_sync(SA_FULL_MASK, s3, 0);
@@ -117,7 +117,7 @@ __device__ __forceinline__ void f4_stage_a(float *pk, uint32_t pk_s, int nf, int
             vs[u] = __shfl_sync(SA_FULL_MASK, v[u >> 2], u & 3, 4);
             uint32_t o = uint32_t(xs[u]) & 0x7fffffffu;
             if (!SA_CHK(lim.status, o < lim.e_rows, 22, o)) o = 0u;
-            e[u] = sa_ldg4(E + (o * ld_e + 4u * l));
+            e[u] = (E + (o * ld_e + 4u * l)).ld4();
         }
 #pragma unroll
         for (int u = 0; u < 8; ++u) {
@@ -161,8 +161,8 @@ __device__ __forceinline__ void f4_stage_a(float *pk, uint32_t pk_s, int nf, int
 // slot0 + (subtree - it.out_row).
 __device__ __forceinline__ void f4_small_item(const sa_item &it, float *pk, float *pool_slot0, const int32_t *__restrict__ pos2,
                                               const int32_t *__restrict__ pos3, const int32_t *__restrict__ crd_k,
-                                              const int2 *__restrict__ nz, const float *__restrict__ D, uint32_t ld_d,
-                                              const float *__restrict__ E, uint32_t ld_e, int lane, const f4_limits &lim)
+                                              const int2 *__restrict__ nz, sa_data D, uint32_t ld_d, sa_data E, uint32_t ld_e,
+                                              int lane, const f4_limits &lim)
 {
     const int g = lane >> 2, t = lane & 3;
     const int nsub = it.row_end - it.out_row;
@@ -199,7 +199,7 @@ __device__ __forceinline__ void f4_small_item(const sa_item &it, float *pk, floa
         for (int i = 0; i < SA_F4_ROWS / 8; ++i) {
             const int row = g + 8 * i;
             const int k = __shfl_sync(SA_FULL_MASK, kk, row);
-            if (row < nf) cp_async16_raw(pk_s + uint32_t(f4_rowpos(row, R + 4 * t)) * 4u, D + (uint32_t(k) * ld_d + 4u * t));
+            if (row < nf) cp_async16_raw(pk_s + uint32_t(f4_rowpos(row, R + 4 * t)) * 4u, (D + (uint32_t(k) * ld_d + 4u * t)).p);
         }
         cp_async_commit();
         f4_stage_a(pk, pk_s, nf, m.s3, m.pe, nz, E, ld_e, lane, lim);
@@ -253,17 +253,17 @@ __device__ __forceinline__ void f4_small_item(const sa_item &it, float *pk, floa
 
 // One item of kind 1: the temporaries of the large subtrees [it.out_row, it.row_end) were written by the order-3
 // kernel to T2L[it.f0 ...]; copy them into the pool.
-__device__ __forceinline__ void f4_large_item(const sa_item &it, float *pool_slot0, const float *__restrict__ T2L, int lane,
+__device__ __forceinline__ void f4_large_item(const sa_item &it, float *pool_slot0, sa_data T2L, int lane,
                                               const f4_limits &lim)
 {
     for (int r = 0; r < it.row_end - it.out_row; ++r) {
         if (!SA_CHK(lim.status, it.f0 + r >= 0 && it.f0 + r < lim.n_large, 26, it.f0 + r)) continue;
-        const float *src = T2L + int64_t(it.f0 + r) * T2F;
+        const sa_data src = T2L + int64_t(it.f0 + r) * T2F;
         float *dst = pool_slot0 + r * F4_TS;
 #pragma unroll
         for (int i = 0; i < 2; ++i) {
             const int e = 4 * (lane + 32 * i);
-            const float4 v = __ldcs(reinterpret_cast<const float4 *>(src + e));
+            const float4 v = (src + e).ld4_cs();
             *reinterpret_cast<float4 *>(dst + f4_pos(e >> 4, e & 15)) = v;
         }
     }
@@ -318,9 +318,8 @@ __global__ void __launch_bounds__(32 * F4_WARPS, SA_F4_CTAS)
 ttm4_fused_kernel(const int4 *__restrict__ pieces, const int4 *__restrict__ supers, const sa_item *__restrict__ items,
                   const int32_t *__restrict__ pos1, const int32_t *__restrict__ crd0, const int32_t *__restrict__ crd_j,
                   const int32_t *__restrict__ pos2, const int32_t *__restrict__ pos3, const int32_t *__restrict__ crd_k,
-                  const int2 *__restrict__ nz, const float *__restrict__ C, uint32_t ldc, const float *__restrict__ D, uint32_t ldd,
-                  const float *__restrict__ E, uint32_t lde, const float *__restrict__ T2L, float *__restrict__ out,
-                  float *__restrict__ partial, const f4_limits lim)
+                  const int2 *__restrict__ nz, sa_data C, uint32_t ldc, sa_data D, uint32_t ldd, sa_data E, uint32_t lde,
+                  sa_data T2L, float *__restrict__ out, float *__restrict__ partial, const f4_limits lim)
 {
     extern __shared__ __align__(16) unsigned char f4_smem[];
     float *park = reinterpret_cast<float *>(f4_smem);
@@ -350,7 +349,7 @@ ttm4_fused_kernel(const int4 *__restrict__ pieces, const int4 *__restrict__ supe
             if (slot < S.w - S.z) {
                 uint32_t j = uint32_t(__ldg(crd_j + S.z + slot));
                 if (!SA_CHK(lim.status, j < lim.c_rows, 27, j)) j = 0u;
-                *reinterpret_cast<float4 *>(cs + slot * F4_CS + 4 * part) = sa_ldg4(C + (j * ldc + 4u * part));
+                *reinterpret_cast<float4 *>(cs + slot * F4_CS + 4 * part) = (C + (j * ldc + 4u * part)).ld4();
             }
         }
         // ---- produce

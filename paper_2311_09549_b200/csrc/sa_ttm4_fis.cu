@@ -96,30 +96,29 @@ __device__ __forceinline__ void sl_load_j(uint32_t (&j)[2], const sl_cursor &cur
     if (!SA_CHK(lim.status, j[1] < lim.c_rows, 71, j[1])) j[1] = 0u;
 }
 __device__ __forceinline__ void sl_load_c(float (&c)[4], const uint32_t (&j)[2], const sl_cursor &cur, int lane,
-                                          const float *__restrict__ C, uint32_t ldc)
+                                          sa_data C, uint32_t ldc)
 {
     const int g = lane >> 2, t = lane & 3;
     const bool va = cur.live && cur.f + t < cur.f1, vb = cur.live && cur.f + t + 4 < cur.f1;
-    const float *ca = C + j[0] * ldc + g;
-    const float *cb = C + j[1] * ldc + g;
-    c[0] = va ? __ldg(ca) : 0.f;
-    c[1] = va ? __ldg(ca + 8) : 0.f;
-    c[2] = vb ? __ldg(cb) : 0.f;
-    c[3] = vb ? __ldg(cb + 8) : 0.f;
+    const sa_data ca = C + j[0] * ldc + g, cb = C + j[1] * ldc + g;
+    c[0] = va ? ca.ld() : 0.f;
+    c[1] = va ? (ca + 8).ld() : 0.f;
+    c[2] = vb ? cb.ld() : 0.f;
+    c[3] = vb ? (cb + 8).ld() : 0.f;
 }
 
 // Copies of the group's eight quarter rows into a stage: 128 pieces of 16 bytes, four per lane; rows past the end of
 // the item are filled with zeros (their C entries are zero too, but what the stage held before need not be finite).
-__device__ __forceinline__ void sl_issue(const sl_cursor &cur, uint32_t stage, int lane, const float *__restrict__ T2)
+__device__ __forceinline__ void sl_issue(const sl_cursor &cur, uint32_t stage, int lane, sa_data T2)
 {
     if (cur.live) {
         const int piece = lane & 15;
-        const float *src = T2 + int64_t(cur.f) * T2F + cur.qc * QC + 4 * piece;
+        const sa_data src = T2 + (int64_t(cur.f) * T2F + cur.qc * QC + 4 * piece);
 #pragma unroll
         for (int i = 0; i < 4; ++i) {
             const int r = (lane >> 4) + 2 * i;
             const uint32_t dst = stage + uint32_t(r * SL_RS + 4 * piece) * 4u;
-            if (cur.f + r < cur.f1) cp_async16_raw(dst, src + int64_t(r) * T2F);
+            if (cur.f + r < cur.f1) cp_async16_raw(dst, (src + int64_t(r) * T2F).p);
             else asm volatile("st.shared.v4.f32 [%0], {%1,%1,%1,%1};" ::"r"(dst), "f"(0.f) : "memory");
         }
     }
@@ -128,8 +127,7 @@ __device__ __forceinline__ void sl_issue(const sl_cursor &cur, uint32_t stage, i
 
 __global__ void __launch_bounds__(256, 2)
 ttm4_slice_kernel(const sa_item *__restrict__ items, int64_t n_items, const int32_t *__restrict__ crd_j,
-                  const float *__restrict__ T2, const float *__restrict__ C, uint32_t ldc, float *__restrict__ out,
-                  float *__restrict__ partial, const fis_limits lim)
+                  sa_data T2, sa_data C, uint32_t ldc, float *__restrict__ out, float *__restrict__ partial, const fis_limits lim)
 {
     extern __shared__ __align__(16) float sl_smem[];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, g = lane >> 2, t = lane & 3;
@@ -232,8 +230,7 @@ template <bool CONTIG>
 __global__ void __launch_bounds__(256, 4)
 ttm4_subtree_kernel(const sa_item *__restrict__ items, int64_t n_items, const int32_t *__restrict__ pos2,
                     const int32_t *__restrict__ pos3, const int32_t *__restrict__ crd_k, const int2 *__restrict__ nz,
-                    const float *__restrict__ D, int64_t ldd, const float *__restrict__ E, int64_t lde, float *__restrict__ T2,
-                    const fis_limits lim)
+                    sa_data D, int64_t ldd, sa_data E, int64_t lde, float *__restrict__ T2, const fis_limits lim)
 {
     extern __shared__ __align__(16) float sub_smem[];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -308,7 +305,7 @@ ttm4_subtree_kernel(const sa_item *__restrict__ items, int64_t n_items, const in
                     vs[u] = __shfl_sync(SA_FULL_MASK, v[h], u, 4);
                     uint32_t o = uint32_t(xs[u]) & 0x7fffffffu;
                     if (!SA_CHK(lim.status, o < lim.e_rows, 76, o)) o = 0u;
-                    e[u] = sa_ldg4(E + (o * ld_e + 4u * l));
+                    e[u] = (E + (o * ld_e + 4u * l)).ld4();
                 }
 #pragma unroll
                 for (int u = 0; u < 4; ++u) {
@@ -355,13 +352,12 @@ ttm4_subtree_kernel(const sa_item *__restrict__ items, int64_t n_items, const in
                 const bool va = fg + t < fend, vb = fg + t + 4 < fend;
                 const float *ra = pk + (va ? fg + t : fbeg) * SUB_RS;
                 const float *rb = pk + (vb ? fg + t + 4 : fbeg) * SUB_RS;
-                const float *da = D + __float_as_uint(ra[R]) + g;
-                const float *db = D + __float_as_uint(rb[R]) + g;
+                const sa_data da = D + __float_as_uint(ra[R]) + g, db = D + __float_as_uint(rb[R]) + g;
                 float av[4];
-                av[0] = va ? __ldg(da) : 0.f;
-                av[1] = va ? __ldg(da + 8) : 0.f;
-                av[2] = vb ? __ldg(db) : 0.f;
-                av[3] = vb ? __ldg(db + 8) : 0.f;
+                av[0] = va ? da.ld() : 0.f;
+                av[1] = va ? (da + 8).ld() : 0.f;
+                av[2] = vb ? db.ld() : 0.f;
+                av[3] = vb ? (db + 8).ld() : 0.f;
                 uint32_t ah[4], al[4];
 #pragma unroll
                 for (int x = 0; x < 4; ++x) split_tf32(av[x], ah[x], al[x]);

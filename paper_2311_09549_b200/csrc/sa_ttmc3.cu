@@ -29,8 +29,7 @@ constexpr int TTMC_MAX_CHUNKS = 512;
 constexpr int TTMC_STEP = 64;
 template <int L>
 __global__ void __launch_bounds__(256)
-ttmc3_partial_kernel(int64_t I, int chunk, int cols, const float *__restrict__ T, const float *__restrict__ C,
-                     uint32_t ldc, float *__restrict__ P)
+ttmc3_partial_kernel(int64_t I, int chunk, int cols, sa_data T, sa_data C, uint32_t ldc, float *__restrict__ P)
 {
     __shared__ __align__(16) float cs[TTMC_STEP * L];
     sa_after_previous();
@@ -43,13 +42,13 @@ ttmc3_partial_kernel(int64_t I, int chunk, int cols, const float *__restrict__ T
         const int n = int(min(int64_t(TTMC_STEP), i1 - base));
         __syncthreads();
         for (int x = threadIdx.x * 4; x < n * L; x += 1024)
-            *reinterpret_cast<float4 *>(cs + x) = sa_ldg4(C + (base + x / L) * ldc + x % L);
+            *reinterpret_cast<float4 *>(cs + x) = (C + ((base + x / L) * ldc + x % L)).ld4();
         __syncthreads();
-        const float *t0 = T + base * cols + col;
+        const sa_data t0 = T + (base * cols + col);
         for (int s = 0; s < n; s += 8) {
             float t[8];
 #pragma unroll
-            for (int u = 0; u < 8; ++u) t[u] = s + u < n ? __ldcs(t0 + int64_t(s + u) * cols) : 0.f;
+            for (int u = 0; u < 8; ++u) t[u] = s + u < n ? (t0 + int64_t(s + u) * cols).ld_cs() : 0.f;
 #pragma unroll
             for (int u = 0; u < 8; ++u) {
                 if (s + u >= n) break;
@@ -73,7 +72,7 @@ ttmc3_partial_kernel(int64_t I, int chunk, int cols, const float *__restrict__ T
 // A(x) = sum over chunks c of P(c, x), x = l * cols + col, in a fixed order: 16 phases over the chunks (64 outputs per block),
 // then the phases.  188 chunks of 4096: 17 us as one sum per thread, 8 us now.
 __global__ void __launch_bounds__(256)
-ttmc3_final_kernel(int n_chunks, int64_t n_out, const float *__restrict__ P, float *__restrict__ A)
+ttmc3_final_kernel(int n_chunks, int64_t n_out, sa_data P, float *__restrict__ A)
 {
     __shared__ float4 red[256];
     sa_after_previous();
@@ -82,7 +81,7 @@ ttmc3_final_kernel(int n_chunks, int64_t n_out, const float *__restrict__ P, flo
     float4 s = make_float4(0.f, 0.f, 0.f, 0.f);
 #pragma unroll 4
     for (int c = phase; c < n_chunks; c += 16) {
-        const float4 v = *reinterpret_cast<const float4 *>(P + int64_t(c) * n_out + x);
+        const float4 v = (P + (int64_t(c) * n_out + x)).ld4();
         s.x += v.x; s.y += v.y; s.z += v.z; s.w += v.w;
     }
     red[threadIdx.x] = s;
