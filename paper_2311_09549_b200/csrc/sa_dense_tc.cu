@@ -519,7 +519,7 @@ sa_status launch_tc(int64_t rows, const float *A, int64_t lda, const float *H, i
     const int64_t ctas = std::min<int64_t>((rows + TC_BM - 1) / TC_BM, sms);
     int shift = 0;
     while ((4 << shift) < part) ++shift;
-    if (ctas > 0) sa_launch<sa_start::FOLLOWS>(k, (unsigned)ctas, TC_THREADS, G::SMEM, stream, rows, A, lda, H, ldh, B, ldb, out, shift, status);
+    if (ctas > 0) sa_launch(k, (unsigned)ctas, TC_THREADS, G::SMEM, stream, rows, A, lda, H, ldh, B, ldb, out, shift, status);
     return cudaGetLastError() == cudaSuccess ? SA_OK : SA_E_CUDA;
 }
 

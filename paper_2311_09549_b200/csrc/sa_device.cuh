@@ -107,33 +107,26 @@ static inline sa_limits sa_make_limits(const sa_tensor *t, int64_t gather_rows, 
     return lim;
 }
 
-// Kernels may start while the one before them on the stream still runs (programmatic dependent launch): their blocks take the
-// places that the other's last round leaves, read what no kernel ever writes (work lists, the tensor's arrays) and then wait, in
-// sa_after_previous, until the other is through and its results can be seen.  Nothing else may be read or written before that,
-// and some thread of every launch has to wait, or a kernel further back could still be running.  Then they let the next kernel
-// on the stream start in the same way.  Back to back, us, without / with: order-3 tensor of 20 K nonzeros (one launch)
-// 10.2 / 9.5, kernel 2 on 60 K nonzeros (two) 18.1 / 16.0.
-__device__ __forceinline__ void sa_after_previous()
-{
-    asm volatile("griddepcontrol.wait;" ::: "memory");
-    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-}
-// Which launches may: an SM keeps its split of shared memory and L1 as long as blocks are on it, so a kernel that starts beside
-// one with another split runs with that split to its end: with little L1 (gather of kernel 7, 12.5 M nonzeros, behind the dense
-// stage: 140 us, early 164; kernel 2 on a large graph 984 us, early 1486) or with fewer blocks per SM than it has room for.
-enum class sa_start {
-    FOLLOWS,        // behind a kernel of the same call that leaves it what it needs: early
-    FIRST,          // first of its call, behind anything: early where every block can have an SM to itself
-    ALONE           // lives on L1, behind a kernel with much shared memory: never early
-};
+// Programmatic dependent launch: a kernel's blocks come onto the SMs when the last block of the kernel before it has left, read
+// there what no kernel ever writes (work lists, the tensor's arrays) and wait, in sa_after_previous, until that kernel is through
+// and its results can be seen.  Nothing else may be read or written before that, and some thread of every launch has to wait,
+// or a kernel further back could still be running.
+// No kernel lets the next one start before its own blocks have left (griddepcontrol.launch_dependents): the next one's blocks
+// then came onto the SMs as these emptied, several onto the first ones, and ran to their end with the split of L1 and shared
+// memory that they found there.  Two calls in turn, us, ordinary launches / with launch_dependents behind the wait (and only
+// kernels of a block per SM, or with no need of L1, starting early) / as it is: row kernel on 60 K nonzeros and kernel 1 on
+// 100 K (K = L = 128) 55 / 87 / 51, order 3 on 8 M nonzeros and the same kernel 1 176 / 194 / 169.  One call after another:
+// kernel 1 on 6 M nonzeros 234 / 236 / 233, kernel 2 on 60 K (three launches) 18.4 / 13.8 / 12.3, kernel 7 on 60 K 12.6 / 11.9 /
+// 9.5, order 3 on 20 K (one launch, the one that is slower so) 10.3 / 7.7 / 8.1.
+__device__ __forceinline__ void sa_after_previous() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+
 // The arguments convert as they do in a call (not by a cast: a pointer in the wrong place does not compile).
 template <typename T>
 struct sa_arg { using type = T; };
-template <sa_start START, typename... Params>
+template <typename... Params>
 static inline cudaError_t sa_launch(void (*kernel)(Params...), dim3 grid, unsigned threads, size_t smem, cudaStream_t stream,
                                     typename sa_arg<Params>::type... args)
 {
-    const bool early = START == sa_start::FOLLOWS || (START == sa_start::FIRST && int64_t(grid.x) * grid.y <= SA_SMS);
     cudaLaunchAttribute attr;
     attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr.val.programmaticStreamSerializationAllowed = 1;
@@ -143,7 +136,7 @@ static inline cudaError_t sa_launch(void (*kernel)(Params...), dim3 grid, unsign
     cfg.dynamicSmemBytes = smem;
     cfg.stream = stream;
     cfg.attrs = &attr;
-    cfg.numAttrs = early ? 1 : 0;
+    cfg.numAttrs = 1;
     static_assert(!(std::is_same<Params, const float *>::value || ...), "fp32 inputs are sa_data or sa_values");
     return cudaLaunchKernelEx(&cfg, kernel, args...);
 }
@@ -277,12 +270,13 @@ static inline cudaError_t sa_launch_fixup(const sa_worklist &wl, const float *pa
     const int nf4 = tile_floats / 4;
     if (nf4 <= 32) {
         const unsigned rows = (unsigned)wl.fix.size(), big = (unsigned)wl.n_big_fix;
-        return sa_launch<sa_start::FOLLOWS>(sa_fixup_rows_kernel, big + (rows - big + 7) / 8, 256, 0, stream, wl.d_fix, int(rows), int(big), partial, out, tile_floats);
+        return sa_launch(sa_fixup_rows_kernel, big + (rows - big + 7) / 8, 256, 0, stream, wl.d_fix, int(rows), int(big), partial, out,
+                         tile_floats);
     }
     int shift = 0;
     while ((4 << shift) < tile_floats) ++shift;
     const int64_t zeros = int64_t(wl.fix.size()) - wl.n_sum_fix;
     const int64_t blocks = (wl.n_big_fix << (shift - 4)) + ((wl.n_sum_fix - wl.n_big_fix) << (shift - 6)) + (((zeros << shift) + 255) >> 8);
-    return sa_launch<sa_start::FOLLOWS>(sa_fixup_kernel, unsigned(blocks), 256, 0, stream, wl.d_fix, unsigned(wl.n_big_fix), unsigned(wl.n_sum_fix), unsigned(wl.fix.size()),
-                     partial, out, shift);
+    return sa_launch(sa_fixup_kernel, unsigned(blocks), 256, 0, stream, wl.d_fix, unsigned(wl.n_big_fix), unsigned(wl.n_sum_fix),
+                     unsigned(wl.fix.size()), partial, out, shift);
 }

@@ -172,7 +172,6 @@ struct sa_ttm3_view {
     int64_t nnz;                  // nonzeros the lists cover (chooses the register budget)
     int64_t nnz_total;            // length of the index / value arrays (bounds of the self-checking build)
     int32_t *status;              // the tensor's device status word
-    bool first = true;            // the launch is the first of its call (sa_launch)
 };
 sa_status sa_launch_ttm3_view(const sa_ttm3_view &v, const sa_dense &first, const sa_dense &second, float *out,
                               float *partial, cudaStream_t stream, int *launches);
@@ -215,9 +214,9 @@ size_t sa_ws_sddmm_spmm_gemm(const sa_tensor *t, const sa_dense *ops);
 bool sa_dense_gemm_ok(int64_t L, int64_t M);
 // out (rows x M) = A (rows x L) . B (L x M); `status` is the tensor's device status word (a wait that runs out
 // inside the tcgen05 kernel records SA_E_TIMEOUT there).  L >= 64 runs on tcgen05, L = 32 on mma.sync.  part (tcgen05
-// only): `out` is written as M / part tables of rows x part floats; 0: as one.  first: of the call's launches (sa_launch).
+// only): `out` is written as M / part tables of rows x part floats; 0: as one.
 sa_status sa_launch_dense_gemm(int64_t rows, const float *A, int64_t lda, const float *B, int64_t ldb, int64_t L,
-                               int64_t M, float *out, int32_t *status, cudaStream_t stream, bool first, int part = 0);
+                               int64_t M, float *out, int32_t *status, cudaStream_t stream, int part = 0);
 bool sa_dense_gemm_tc_ok(int64_t L, int64_t M);
 sa_status sa_launch_dense_gemm_tc(int64_t rows, const float *A, int64_t lda, const float *B, int64_t ldb, int64_t L,
                                   int64_t M, float *out, int32_t *status, cudaStream_t stream, int part);

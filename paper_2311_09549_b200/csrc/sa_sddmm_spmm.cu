@@ -155,8 +155,9 @@ cudaError_t launch(const sa_tensor *t, const sa_dense *ops, float *out, float *p
     // (22 K items) 29.3 / 31.8, 400 K on 40 K rows (26 K) 29.1 / 30.9, 1.5 M on 50 K rows (30 K) 48.3 / 47.5, 1 M on 300 K rows
     // (38 K) 61 / 53, on 200 K rows and 700 K columns (42 K) 83 / 69.
     auto kern = n_items <= int64_t(3) * 2 * SA_SMS * 32 ? sddmm_spmm_kernel<K, L, 2> : sddmm_spmm_kernel<K, L, sd_cfg<K, L>::CTAS>;
-    sa_launch<sa_start::FIRST>(kern, (unsigned)ctas, 256, 0, stream, wl.d_items, n_items, t->d_pos[1], t->d_nzpack, ops[0].ptr, uint32_t(ops[0].ld), ops[1].ptr, uint32_t(ops[1].ld), ops[2].ptr,
-        uint32_t(ops[2].ld), out, partial, sampled, sa_make_limits(t, t->dims[1], t->dims[0], wl.n_slots));
+    sa_launch(kern, (unsigned)ctas, 256, 0, stream, wl.d_items, n_items, t->d_pos[1], t->d_nzpack, ops[0].ptr, uint32_t(ops[0].ld),
+              ops[1].ptr, uint32_t(ops[1].ld), ops[2].ptr, uint32_t(ops[2].ld), out, partial, sampled,
+              sa_make_limits(t, t->dims[1], t->dims[0], wl.n_slots));
     return cudaGetLastError();
 }
 
@@ -217,7 +218,7 @@ sa_status sa_launch_sddmm_spmm_gemm(const sa_tensor *t, const sa_dense *ops, flo
     int n1 = 0;
     const sa_status s = sa_launch_sddmm_spmm(t, ops, T, static_cast<char *>(ws) + t_bytes, ws_bytes - t_bytes, false, stream, &n1);
     if (s != SA_OK) return s;
-    const sa_status g = sa_launch_dense_gemm(I, T, L, ops[3].ptr, ops[3].ld, L, M, out, t->d_status, stream, false);
+    const sa_status g = sa_launch_dense_gemm(I, T, L, ops[3].ptr, ops[3].ld, L, M, out, t->d_status, stream);
     if (g != SA_OK) return g;
     *launches = n1 + 1;
     return SA_OK;

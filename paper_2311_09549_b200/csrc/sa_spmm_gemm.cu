@@ -483,8 +483,8 @@ sa_status run_spmm(const sa_tensor *t, float *E, float *out, cudaStream_t stream
         const int W = spmm_part(J, M);
         const unsigned ctas = unsigned((n_items * (W / 4) + 255) / 256);
         auto kern = W == 32 ? spmm_kernel<32> : spmm_kernel<64>;
-        sa_launch<sa_start::ALONE>(kern, ctas * unsigned(M / W), 256, 0, stream, wl.d_items, n_items, ctas, t->d_pos[1], t->d_nzpack, E, J, M, out, partial,
-                                                         sa_make_limits(t, J, t->dims[0], wl.n_slots));
+        sa_launch(kern, ctas * unsigned(M / W), 256, 0, stream, wl.d_items, n_items, ctas, t->d_pos[1], t->d_nzpack, E, J, M, out,
+                  partial, sa_make_limits(t, J, t->dims[0], wl.n_slots));
         if (cudaGetLastError() != cudaSuccess) return SA_E_CUDA;
         *launches += 1;
     }
@@ -518,9 +518,9 @@ sa_status run(const sa_tensor *t, const sa_dense *ops, float *out, void *ws, boo
         const int64_t want = (n_items + SA_WARPS_PER_CTA - 1) / SA_WARPS_PER_CTA;
         const int64_t ctas = std::min<int64_t>(want, resident_ctas(reinterpret_cast<const void *>(kern), smem, resident));
         if (ctas > 0) {
-            sa_launch<sa_start::FIRST>(kern, (unsigned)ctas, 256, smem, stream, wl.d_items, n_items, t->d_pos[1], t->d_crd[1], t->d_vals, ops[0].ptr,
-                                                       ops[0].ld, ops[0].ptr, ops[0].ld, ops[1].ptr, ops[1].ld, out, partial,
-                                                       sa_make_limits(t, t->dims[1], t->dims[0], wl.n_slots));
+            sa_launch(kern, (unsigned)ctas, 256, smem, stream, wl.d_items, n_items, t->d_pos[1], t->d_crd[1], t->d_vals, ops[0].ptr,
+                      ops[0].ld, ops[0].ptr, ops[0].ld, ops[1].ptr, ops[1].ld, out, partial,
+                      sa_make_limits(t, t->dims[1], t->dims[0], wl.n_slots));
             if (cudaGetLastError() != cudaSuccess) return SA_E_CUDA;
             *launches += 1;
         }
@@ -531,7 +531,7 @@ sa_status run(const sa_tensor *t, const sa_dense *ops, float *out, void *ws, boo
         return SA_OK;
     }
     float *E = static_cast<float *>(ws);
-    const sa_status gs = sa_launch_dense_gemm(t->dims[1], ops[0].ptr, ops[0].ld, ops[1].ptr, ops[1].ld, L, M, E, t->d_status, stream, true,
+    const sa_status gs = sa_launch_dense_gemm(t->dims[1], ops[0].ptr, ops[0].ld, ops[1].ptr, ops[1].ld, L, M, E, t->d_status, stream,
                                               spmm_part(t->dims[1], M));
     if (gs != SA_OK) return gs;
     *launches += 1;
@@ -563,9 +563,9 @@ sa_status run_hadamard(const sa_tensor *t, const sa_dense *ops, float *out, void
     const int64_t want = (n_items + SA_WARPS_PER_CTA - 1) / SA_WARPS_PER_CTA;
     const int64_t ctas = std::min<int64_t>(want, resident_ctas(reinterpret_cast<const void *>(kern), smem, resident));
     if (ctas > 0) {
-        sa_launch<sa_start::FIRST>(kern, (unsigned)ctas, 256, smem, stream, wl.d_items, n_items, t->d_pos[1], t->d_crd[1], t->d_vals, ops[0].ptr,
-                                                   ops[0].ld, ops[1].ptr, ops[1].ld, ops[2].ptr, ops[2].ld, out, partial,
-                                                   sa_make_limits(t, t->dims[1], t->dims[0], wl.n_slots));
+        sa_launch(kern, (unsigned)ctas, 256, smem, stream, wl.d_items, n_items, t->d_pos[1], t->d_crd[1], t->d_vals, ops[0].ptr,
+                  ops[0].ld, ops[1].ptr, ops[1].ld, ops[2].ptr, ops[2].ld, out, partial,
+                  sa_make_limits(t, t->dims[1], t->dims[0], wl.n_slots));
         if (cudaGetLastError() != cudaSuccess) return SA_E_CUDA;
         *launches += 1;
     }
@@ -591,12 +591,12 @@ sa_status run_fibers(const sa_tensor *t, const sa_dense *ops, float *out, void *
     if (right) {
         float *E = static_cast<float *>(ws);
         float *partial = reinterpret_cast<float *>(static_cast<char *>(ws) + sa_align256(size_t(K) * M * sizeof(float)));
-        const sa_status gs = sa_launch_dense_gemm(K, ops[0].ptr, ops[0].ld, ops[1].ptr, ops[1].ld, L, M, E, t->d_status, stream, true);
+        const sa_status gs = sa_launch_dense_gemm(K, ops[0].ptr, ops[0].ld, ops[1].ptr, ops[1].ld, L, M, E, t->d_status, stream);
         if (gs != SA_OK) return gs;
         *launches += 1;
         if (ctas > 0) {
-            sa_launch<sa_start::ALONE>(fiber_spmm_kernel<M>, (unsigned)ctas, 256, 0, stream, wl.d_items, n_items, t->d_pos[2], t->d_nzpack, E, M, out, partial,
-                                                                     sa_make_limits(t, K, F2, wl.n_slots));
+            sa_launch(fiber_spmm_kernel<M>, (unsigned)ctas, 256, 0, stream, wl.d_items, n_items, t->d_pos[2], t->d_nzpack, E, M, out,
+                      partial, sa_make_limits(t, K, F2, wl.n_slots));
             if (cudaGetLastError() != cudaSuccess) return SA_E_CUDA;
             *launches += 1;
         }
@@ -609,8 +609,8 @@ sa_status run_fibers(const sa_tensor *t, const sa_dense *ops, float *out, void *
     float *T = static_cast<float *>(ws);
     float *partial = reinterpret_cast<float *>(static_cast<char *>(ws) + sa_align256(size_t(F2) * L * sizeof(float)));
     if (ctas > 0) {
-        sa_launch<sa_start::ALONE>(fiber_spmm_kernel<L>, (unsigned)ctas, 256, 0, stream, wl.d_items, n_items, t->d_pos[2], t->d_nzpack, ops[0].ptr, ops[0].ld,
-                                                                T, partial, sa_make_limits(t, K, F2, wl.n_slots));
+        sa_launch(fiber_spmm_kernel<L>, (unsigned)ctas, 256, 0, stream, wl.d_items, n_items, t->d_pos[2], t->d_nzpack, ops[0].ptr,
+                  ops[0].ld, T, partial, sa_make_limits(t, K, F2, wl.n_slots));
         if (cudaGetLastError() != cudaSuccess) return SA_E_CUDA;
         *launches += 1;
     }
@@ -618,7 +618,7 @@ sa_status run_fibers(const sa_tensor *t, const sa_dense *ops, float *out, void *
         if (sa_launch_fixup(wl, partial, T, L, stream) != cudaSuccess) return SA_E_CUDA;
         *launches += 1;
     }
-    const sa_status gs = sa_launch_dense_gemm(F2, T, L, ops[1].ptr, ops[1].ld, L, M, out, t->d_status, stream, false);
+    const sa_status gs = sa_launch_dense_gemm(F2, T, L, ops[1].ptr, ops[1].ld, L, M, out, t->d_status, stream);
     if (gs != SA_OK) return gs;
     *launches += 1;
     return SA_OK;
@@ -630,7 +630,7 @@ sa_status run_fibers(const sa_tensor *t, const sa_dense *ops, float *out, void *
 // dense stage of other chains.  L in {32, 64, 128, 256}, M in {32, 64}.
 template <int L, int M>
 static sa_status dense_gemm(int64_t rows, const float *A, int64_t lda, const float *B, int64_t ldb, float *out,
-                            cudaStream_t stream, bool first)
+                            cudaStream_t stream)
 {
     using GC = gemm_bf16_cfg<L, M>;
     auto gk = gemm_bf16x3_kernel<L, M>;
@@ -638,19 +638,18 @@ static sa_status dense_gemm(int64_t rows, const float *A, int64_t lda, const flo
     static resident_cache resident;
     if (!sa_set_smem_once(gk, int(GC::SMEM), attr)) return SA_E_CUDA;
     const int64_t ctas = std::min<int64_t>((rows + GC::BM - 1) / GC::BM, resident_ctas(reinterpret_cast<const void *>(gk), GC::SMEM, resident));
-    if (ctas > 0 && first) sa_launch<sa_start::FIRST>(gk, (unsigned)ctas, 256, GC::SMEM, stream, rows, A, lda, B, ldb, out);
-    else if (ctas > 0) sa_launch<sa_start::FOLLOWS>(gk, (unsigned)ctas, 256, GC::SMEM, stream, rows, A, lda, B, ldb, out);
+    if (ctas > 0) sa_launch(gk, (unsigned)ctas, 256, GC::SMEM, stream, rows, A, lda, B, ldb, out);
     return cudaGetLastError() == cudaSuccess ? SA_OK : SA_E_CUDA;
 }
 
 bool sa_dense_gemm_ok(int64_t L, int64_t M) { return (L == 32 || L == 64 || L == 128 || L == 256) && (M == 32 || M == 64); }
 
 sa_status sa_launch_dense_gemm(int64_t rows, const float *A, int64_t lda, const float *B, int64_t ldb, int64_t L,
-                               int64_t M, float *out, int32_t *status, cudaStream_t stream, bool first, int part)
+                               int64_t M, float *out, int32_t *status, cudaStream_t stream, int part)
 {
     if (sa_dense_gemm_tc_ok(L, M)) return sa_launch_dense_gemm_tc(rows, A, lda, B, ldb, L, M, out, status, stream, part ? part : int(M));
     if (part && part != M) return SA_E_UNSUPPORTED;
-#define SA_CASE(l, m) if (L == l && M == m) return dense_gemm<l, m>(rows, A, lda, B, ldb, out, stream, first);
+#define SA_CASE(l, m) if (L == l && M == m) return dense_gemm<l, m>(rows, A, lda, B, ldb, out, stream);
     SA_CASE(32, 32) SA_CASE(32, 64)
 #undef SA_CASE
     return SA_E_UNSUPPORTED;

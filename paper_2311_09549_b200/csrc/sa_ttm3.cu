@@ -671,13 +671,9 @@ cudaError_t launch(const sa_ttm3_view &v, const sa_dense &first, const sa_dense 
     lim.c_rows = uint32_t(first.rows); lim.d_rows = uint32_t(second.rows);
     lim.n_fibers = uint32_t(v.n_fibers); lim.n_slices_dim = uint32_t(v.n_out_rows);
     lim.nnz = v.nnz_total;
-    auto start = [&](auto first_of_call) {
-        sa_launch<decltype(first_of_call)::value ? sa_start::FIRST : sa_start::ALONE>(kern, (unsigned)ctas, 32 * SA_TTM3_WARPS, smem, stream, wl.d_units3, wl.d_task_start, n_tasks,
-                                          int(wl.n_group_ctas), v.crd_fiber, v.crd_nz, v.vals, v.endbits, first.ptr, uint32_t(first.ld),
-                                          second.ptr, uint32_t(second.ld), out, partial, lim);
-    };
-    if (v.first) start(std::true_type{});
-    else start(std::false_type{});
+    sa_launch(kern, (unsigned)ctas, 32 * SA_TTM3_WARPS, smem, stream, wl.d_units3, wl.d_task_start, n_tasks, int(wl.n_group_ctas),
+              v.crd_fiber, v.crd_nz, v.vals, v.endbits, first.ptr, uint32_t(first.ld), second.ptr, uint32_t(second.ld), out, partial,
+              lim);
     return cudaGetLastError();
 }
 
@@ -779,7 +775,7 @@ sa_status sa_launch_ttmc3_fused_stage(const sa_tensor *t, const sa_dense &C3, co
     if (M == m && N == n) {                                                                                                       \
         if (!ttmc3_fused_shape<m, n>(int(C3.cols), &grid, &smem)) return SA_E_CUDA;                                               \
         grid = int(std::min<int64_t>(std::min<int64_t>(grid, SA_TTMC3_MAX_BLOCKS), n_block_tasks));                               \
-        sa_launch<sa_start::FIRST>(ttmc3_fused_kernel<m, n, 4>, unsigned(grid), 32 * SA_TTM3_WARPS, smem, stream, \
+        sa_launch(ttmc3_fused_kernel<m, n, 4>, unsigned(grid), 32 * SA_TTM3_WARPS, smem, stream,                                  \
             wl.d_units3, wl.d_task_start, n_tasks, int(wl.n_group_ctas), t->d_crd[1], t->d_crd[2], t->d_vals, t->d_endbits, D.ptr, \
             uint32_t(D.ld), E.ptr, uint32_t(E.ld), C3.ptr, uint32_t(C3.ld), int(C3.cols), partials, lim);                         \
         if (cudaGetLastError() != cudaSuccess) return SA_E_CUDA;                                                                  \

@@ -453,7 +453,6 @@ sa_status sa_launch_ttm4(const sa_tensor *t, const sa_dense *ops, float *out, vo
         v.nnz = t->wl_main.nnz;
         v.nnz_total = t->nnz;
         v.status = t->d_status;
-    v.first = false;
         int n1 = 0;
         const sa_status s = sa_launch_ttm3_view(v, ops[1], ops[2], T2L, part1, stream, &n1);
         if (s != SA_OK) return s;
@@ -471,9 +470,10 @@ sa_status sa_launch_ttm4(const sa_tensor *t, const sa_dense *ops, float *out, vo
         lim.n_slices = uint32_t(t->dims[0]);
         lim.n_subtrees = int32_t(t->count[1]); lim.n_fibers = int32_t(t->count[2]); lim.n_large = t->f4_n_large;
         lim.n_slots = int32_t(t->wl_aux.n_slots); lim.nnz = int32_t(t->nnz);
-        sa_launch<sa_start::ALONE>(kern, (unsigned)n_pieces, 32 * F4_WARPS, F4_SMEM, stream, reinterpret_cast<const int4 *>(t->d_f4_pieces), reinterpret_cast<const int4 *>(t->d_f4_supers), t->wl_sub.d_items,
-            t->d_pos[1], t->d_crd[0], t->d_crd[1], t->d_pos[2], t->d_pos[3], t->d_crd[2], t->d_nzpack, ops[0].ptr,
-            uint32_t(ops[0].ld), ops[1].ptr, uint32_t(ops[1].ld), ops[2].ptr, uint32_t(ops[2].ld), T2L, out, part2, lim);
+        sa_launch(kern, (unsigned)n_pieces, 32 * F4_WARPS, F4_SMEM, stream, reinterpret_cast<const int4 *>(t->d_f4_pieces),
+                  reinterpret_cast<const int4 *>(t->d_f4_supers), t->wl_sub.d_items, t->d_pos[1], t->d_crd[0], t->d_crd[1],
+                  t->d_pos[2], t->d_pos[3], t->d_crd[2], t->d_nzpack, ops[0].ptr, uint32_t(ops[0].ld), ops[1].ptr,
+                  uint32_t(ops[1].ld), ops[2].ptr, uint32_t(ops[2].ld), T2L, out, part2, lim);
         if (cudaGetLastError() != cudaSuccess) return SA_E_CUDA;
         *launches += 1;
     }

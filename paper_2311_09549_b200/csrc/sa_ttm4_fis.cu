@@ -428,7 +428,6 @@ sa_status sa_launch_ttm4_fissioned(const sa_tensor *t, const sa_dense *ops, floa
     v.nnz = t->wl4_main.nnz;
     v.nnz_total = t->nnz;
     v.status = t->d_status;
-    v.first = false;
     fis_limits lim;
     lim.status = t->d_status;
     lim.c_rows = uint32_t(ops[0].rows); lim.d_rows = uint32_t(ops[1].rows); lim.e_rows = uint32_t(ops[2].rows);
@@ -444,8 +443,8 @@ sa_status sa_launch_ttm4_fissioned(const sa_tensor *t, const sa_dense *ops, floa
         static sa_device_flags attr_contig, attr_strided;
         if (!sa_set_smem_once(kern, SUB_SMEM, contig ? attr_contig : attr_strided)) return SA_E_CUDA;
         const int64_t ctas = (n_sub + SA_WARPS_PER_CTA - 1) / SA_WARPS_PER_CTA;
-        sa_launch<sa_start::ALONE>(kern, (unsigned)ctas, 256, SUB_SMEM, stream, t->wl4_sub.d_items, n_sub, t->d_pos[2], t->d_pos[3], t->d_crd[2],
-                                                                       t->d_nzpack, ops[1].ptr, ops[1].ld, ops[2].ptr, ops[2].ld, T2, lim);
+        sa_launch(kern, (unsigned)ctas, 256, SUB_SMEM, stream, t->wl4_sub.d_items, n_sub, t->d_pos[2], t->d_pos[3], t->d_crd[2],
+                  t->d_nzpack, ops[1].ptr, ops[1].ld, ops[2].ptr, ops[2].ld, T2, lim);
         if (cudaGetLastError() != cudaSuccess) return SA_E_CUDA;
         *launches += 1;
     }
@@ -464,8 +463,8 @@ sa_status sa_launch_ttm4_fissioned(const sa_tensor *t, const sa_dense *ops, floa
         const int64_t ctas = std::min<int64_t>((n_items + SA_WARPS_PER_CTA - 1) / SA_WARPS_PER_CTA, int64_t(sms) * 2);
         static sa_device_flags attr_slice;
         if (!sa_set_smem_once(ttm4_slice_kernel, SL_SMEM, attr_slice)) return SA_E_CUDA;
-        sa_launch<sa_start::ALONE>(ttm4_slice_kernel, (unsigned)ctas, 256, SL_SMEM, stream, wl.d_items, n_items, t->d_crd[1], T2, ops[0].ptr, uint32_t(ops[0].ld),
-                                                                  out, part2, lim);
+        sa_launch(ttm4_slice_kernel, (unsigned)ctas, 256, SL_SMEM, stream, wl.d_items, n_items, t->d_crd[1], T2, ops[0].ptr,
+                  uint32_t(ops[0].ld), out, part2, lim);
         if (cudaGetLastError() != cudaSuccess) return SA_E_CUDA;
         *launches += 1;
     }

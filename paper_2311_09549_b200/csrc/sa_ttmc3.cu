@@ -138,7 +138,7 @@ sa_status sa_launch_ttmc3(const sa_tensor *t, const sa_dense *ops, float *out, v
         if (s != SA_OK) return s;
         const int64_t n_out = L * cols;
         // n_blocks == 0 (a tensor without nonzeros): the sum over no accumulators writes zeros
-        sa_launch<sa_start::FOLLOWS>(ttmc3_final_kernel, (unsigned)(n_out / 64), 256, 0, stream, n_blocks, n_out, partials, out);
+        sa_launch(ttmc3_final_kernel, (unsigned)(n_out / 64), 256, 0, stream, n_blocks, n_out, partials, out);
         if (cudaGetLastError() != cudaSuccess) return SA_E_CUDA;
         *launches = (n_blocks > 0 ? 1 : 0) + 1;
         return SA_OK;
@@ -153,11 +153,11 @@ sa_status sa_launch_ttmc3(const sa_tensor *t, const sa_dense *ops, float *out, v
     if (s != SA_OK) return s;
     *launches = n3;
     dim3 grid((unsigned)(cols / 256), (unsigned)p.n_chunks);              // cols is 256, 512 or 1024
-    if (L == 16) sa_launch<sa_start::FOLLOWS>(ttmc3_partial_kernel<16>, grid, 256, 0, stream, I, p.chunk, cols, T, ops[0].ptr, uint32_t(ops[0].ld), P);
-    else sa_launch<sa_start::FOLLOWS>(ttmc3_partial_kernel<32>, grid, 256, 0, stream, I, p.chunk, cols, T, ops[0].ptr, uint32_t(ops[0].ld), P);
+    auto kern = L == 16 ? ttmc3_partial_kernel<16> : ttmc3_partial_kernel<32>;
+    sa_launch(kern, grid, 256, 0, stream, I, p.chunk, cols, T, ops[0].ptr, uint32_t(ops[0].ld), P);
     if (cudaGetLastError() != cudaSuccess) return SA_E_CUDA;
     const int64_t n_out = L * cols;
-    sa_launch<sa_start::FOLLOWS>(ttmc3_final_kernel, (unsigned)(n_out / 64), 256, 0, stream, p.n_chunks, n_out, P, out);
+    sa_launch(ttmc3_final_kernel, (unsigned)(n_out / 64), 256, 0, stream, p.n_chunks, n_out, P, out);
     if (cudaGetLastError() != cudaSuccess) return SA_E_CUDA;
     *launches += 2;
     return SA_OK;

@@ -20,9 +20,9 @@ __global__ void copy(%s in, float *out)
 }
 cudaError_t launch(const int32_t *index, int32_t *status, float *out, const float *in)
 {
-    cudaError_t e = sa_launch<sa_start::FIRST>(copy, 1u, 32u, 0, nullptr, in, out);
+    cudaError_t e = sa_launch(copy, 1u, 32u, 0, nullptr, in, out);
     if (e != cudaSuccess) return e;
-    return sa_launch<sa_start::FIRST>(kernel, 1u, 32u, 0, nullptr, %s);
+    return sa_launch(kernel, 1u, 32u, 0, nullptr, %s);
 }
 """
 
