@@ -201,7 +201,7 @@ __device__ __forceinline__ uint32_t tc_sw128(uint32_t row, uint32_t k)
 
 template <int L, int M, bool HAD>
 __global__ void __launch_bounds__(TC_THREADS, 1)
-gemm_tc_kernel(int64_t J, sa_data C, int64_t ldc, sa_data H, int64_t ldh, sa_data D, int64_t ldd, float *__restrict__ Eout, int part_shift, int32_t *__restrict__ status)
+gemm_tc_kernel(int64_t J, sa_input C_in, int64_t ldc, sa_input H_in, int64_t ldh, sa_input D_in, int64_t ldd, float *__restrict__ Eout, int part_shift, int32_t *__restrict__ status)
 {
     using G = tc_cfg<L, M, HAD>;
     extern __shared__ uint8_t tc_smem_raw[];
@@ -211,7 +211,8 @@ gemm_tc_kernel(int64_t J, sa_data C, int64_t ldc, sa_data H, int64_t ldh, sa_dat
     uint32_t *tmem_slot = reinterpret_cast<uint32_t *>(smem + G::OFF_BAR + 8 * B_COUNT);
     volatile int *abort_flag = reinterpret_cast<volatile int *>(smem + G::OFF_BAR + 8 * B_COUNT + 4);
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    sa_after_previous();
+    const sa_ready ready = sa_after_previous();
+    const sa_data C = ready(C_in), H = ready(H_in), D = ready(D_in);
 
     // D^T as KCH operand tiles of PARTS M rows x 64 columns (k): rows n < M hold b1(D(k,n)), rows M + n hold b2, ...
     // (eight k of one n per step: coalesced loads, eight in flight, and one conflict-free 16-byte store per part; element by
@@ -390,7 +391,7 @@ gemm_tc_kernel(int64_t J, sa_data C, int64_t ldc, sa_data H, int64_t ldh, sa_dat
                     const int64_t row0 = (int64_t(blockIdx.x) + (q / G::KCH) * gridDim.x) * TC_BM + r0;
                     const sa_data src = C + (int(q % G::KCH) * TC_KC + 4 * int(qf));
 #pragma unroll
-                    for (int i = 0; i < NR; ++i) b[i] = (src + min(row0 + 16 * i, J - 1) * ldc).ld4_once();   // rows past the end re-read the last row
+                    for (int i = 0; i < NR; ++i) b[i] = (src + min(row0 + 16 * i, J - 1) * ldc).ld4_once_here();   // rows past the end re-read the last row
                 }
             };
             auto convert = [&](const float4 (&b)[NR], int64_t q) -> bool {
@@ -439,9 +440,9 @@ gemm_tc_kernel(int64_t J, sa_data C, int64_t ldc, sa_data H, int64_t ldh, sa_dat
                     const int64_t row0 = (int64_t(blockIdx.x) + (q / G::KCH) * gridDim.x) * TC_BM + r0 + half * (TC_BM / 2);
                     const int col = int(q % G::KCH) * TC_KC + 4 * int(qf);
 #pragma unroll
-                    for (int i = 0; i < HR; ++i) b[i] = (C + (col + min(row0 + 16 * i, J - 1) * ldc)).ld4_once();
+                    for (int i = 0; i < HR; ++i) b[i] = (C + (col + min(row0 + 16 * i, J - 1) * ldc)).ld4_once_here();
 #pragma unroll
-                    for (int i = 0; i < HR; ++i) b[HR + i] = (H + (col + min(row0 + 16 * i, J - 1) * ldh)).ld4_once();
+                    for (int i = 0; i < HR; ++i) b[HR + i] = (H + (col + min(row0 + 16 * i, J - 1) * ldh)).ld4_once_here();
                 }
             };
             auto convert = [&](const float4 (&b)[NR], int64_t q, auto upper) -> bool {

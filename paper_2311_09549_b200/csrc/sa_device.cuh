@@ -14,53 +14,92 @@
 // fp32 numbers that an earlier kernel on the stream may have written: dense operands, temporaries, partial sums.  A kernel may
 // start while that one is still running (sa_launch), so they are not constant for its lifetime, which is what __ldg,
 // ld.global.nc and `const float *__restrict__` promise: the compiler may move such loads up across the wait, and the read-only
-// path need not see the new values.  These loads are coherent, and volatile like the wait, so that they stay behind it.  Work
-// lists and the tensor's arrays (sa_values: its values) are never written by a kernel; they take the read-only path.
-struct sa_data {
+// path need not see the new values.  A kernel takes them as sa_input; what sa_after_previous returns turns that into sa_data,
+// whose loads are coherent and take the number that the wait gave as an operand (unused, no instruction), so that they stay
+// behind it and are otherwise free to move: with all of them volatile, their order fixed, kernel 1 on 60 K nonzeros
+// in long rows (K = L = 128) took 24.1 us instead of 20.5.  (The _here loads are volatile where a loop's loads are placed by
+// hand: the rows in flight of the order-3 kernel and the dense stage, and kernel 8's rows of C, which spill when left free.)
+// Work lists and the tensor's arrays (sa_values: its values) are never written by a kernel; they take the read-only path.
+struct sa_input {
     const float *p;
-    __host__ __device__ __forceinline__ sa_data(const float *q = nullptr) : p(q) {}
-    __device__ __forceinline__ sa_data operator+(int64_t n) const { return p + n; }
-    __device__ __forceinline__ sa_data plus_bytes(uint64_t n) const { return reinterpret_cast<const float *>(reinterpret_cast<const char *>(p) + n); }
+    __host__ __device__ __forceinline__ sa_input(const float *q) : p(q) {}
+};
+struct sa_values {
+    const float *p;
+    __host__ __device__ __forceinline__ sa_values(const float *q) : p(q) {}
+};
+struct sa_ready;
+class sa_data {
+    uint32_t ready;
+    __device__ __forceinline__ sa_data(const float *q, uint32_t r) : ready(r), p(q) {}
+    friend struct sa_ready;
+
+public:
+    const float *p;
+    __device__ __forceinline__ sa_data operator+(int64_t n) const { return sa_data(p + n, ready); }
+    __device__ __forceinline__ sa_data plus_bytes(uint64_t n) const
+    {
+        return sa_data(reinterpret_cast<const float *>(reinterpret_cast<const char *>(p) + n), ready);
+    }
     __device__ __forceinline__ float ld() const
     {
         float v;
-        asm volatile("ld.global.f32 %0, [%1];" : "=f"(v) : "l"(p));
+        asm("ld.global.f32 %0, [%1];" : "=f"(v) : "l"(p), "r"(ready));
         return v;
     }
     __device__ __forceinline__ float ld_cs() const             // read once: evict first
     {
         float v;
-        asm volatile("ld.global.cs.f32 %0, [%1];" : "=f"(v) : "l"(p));
+        asm("ld.global.cs.f32 %0, [%1];" : "=f"(v) : "l"(p), "r"(ready));
         return v;
     }
     __device__ __forceinline__ float2 ld2() const
     {
         float2 v;
-        asm volatile("ld.global.v2.f32 {%0,%1}, [%2];" : "=f"(v.x), "=f"(v.y) : "l"(p));
+        asm("ld.global.v2.f32 {%0,%1}, [%2];" : "=f"(v.x), "=f"(v.y) : "l"(p), "r"(ready));
         return v;
     }
     __device__ __forceinline__ float4 ld4() const
     {
         float4 v;
-        asm volatile("ld.global.v4.f32 {%0,%1,%2,%3}, [%4];" : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w) : "l"(p));
+        asm("ld.global.v4.f32 {%0,%1,%2,%3}, [%4];" : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w) : "l"(p), "r"(ready));
         return v;
     }
     __device__ __forceinline__ float4 ld4_cs() const
     {
         float4 v;
-        asm volatile("ld.global.cs.v4.f32 {%0,%1,%2,%3}, [%4];" : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w) : "l"(p));
+        asm("ld.global.cs.v4.f32 {%0,%1,%2,%3}, [%4];" : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w) : "l"(p), "r"(ready));
         return v;
     }
     __device__ __forceinline__ float4 ld4_once() const         // not kept in L1
+    {
+        float4 v;
+        asm("ld.global.L1::no_allocate.v4.f32 {%0,%1,%2,%3}, [%4];" : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w) : "l"(p), "r"(ready));
+        return v;
+    }
+    // the same in its place among the other volatile statements
+    __device__ __forceinline__ float2 ld2_here() const
+    {
+        float2 v;
+        asm volatile("ld.global.v2.f32 {%0,%1}, [%2];" : "=f"(v.x), "=f"(v.y) : "l"(p));
+        return v;
+    }
+    __device__ __forceinline__ float4 ld4_here() const
+    {
+        float4 v;
+        asm volatile("ld.global.v4.f32 {%0,%1,%2,%3}, [%4];" : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w) : "l"(p));
+        return v;
+    }
+    __device__ __forceinline__ float4 ld4_once_here() const
     {
         float4 v;
         asm volatile("ld.global.L1::no_allocate.v4.f32 {%0,%1,%2,%3}, [%4];" : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w) : "l"(p));
         return v;
     }
 };
-struct sa_values {
-    const float *p;
-    __host__ __device__ __forceinline__ sa_values(const float *q) : p(q) {}
+struct sa_ready {
+    uint32_t token;
+    __device__ __forceinline__ sa_data operator()(sa_input in) const { return sa_data(in.p, token); }
 };
 
 // Streaming (evict-first) stores for output tiles that are written once and never re-read, so
@@ -118,7 +157,12 @@ static inline sa_limits sa_make_limits(const sa_tensor *t, int64_t gather_rows, 
 // 100 K (K = L = 128) 55 / 87 / 51, order 3 on 8 M nonzeros and the same kernel 1 176 / 194 / 169.  One call after another:
 // kernel 1 on 6 M nonzeros 234 / 236 / 233, kernel 2 on 60 K (three launches) 18.4 / 13.8 / 12.3, kernel 7 on 60 K 12.6 / 11.9 /
 // 9.5, order 3 on 20 K (one launch, the one that is slower so) 10.3 / 7.7 / 8.1.
-__device__ __forceinline__ void sa_after_previous() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ sa_ready sa_after_previous()
+{
+    sa_ready r;
+    asm volatile("griddepcontrol.wait;\n\tmov.u32 %0, 0;" : "=r"(r.token) : : "memory");
+    return r;
+}
 
 // The arguments convert as they do in a call (not by a cast: a pointer in the wrong place does not compile).
 template <typename T>
@@ -137,7 +181,7 @@ static inline cudaError_t sa_launch(void (*kernel)(Params...), dim3 grid, unsign
     cfg.stream = stream;
     cfg.attrs = &attr;
     cfg.numAttrs = 1;
-    static_assert(!(std::is_same<Params, const float *>::value || ...), "fp32 inputs are sa_data or sa_values");
+    static_assert(!(std::is_same<Params, const float *>::value || ...), "fp32 inputs are sa_input or sa_values");
     return cudaLaunchKernelEx(&cfg, kernel, args...);
 }
 
@@ -191,11 +235,11 @@ __device__ __forceinline__ void cp_async_wait() { asm volatile("cp.async.wait_gr
 // are zeroed 256 float4 per block.  Fixed summation order: deterministic.  192 partials of 4 KB: 13 us with 64 columns per
 // block throughout, 7.5 us.
 static __global__ void __launch_bounds__(256)
-sa_fixup_kernel(const sa_fix *__restrict__ fix, unsigned n_big, unsigned n_sum, unsigned n_fix, sa_data partial,
+sa_fixup_kernel(const sa_fix *__restrict__ fix, unsigned n_big, unsigned n_sum, unsigned n_fix, sa_input partial_in,
                 float *__restrict__ out, int shift)
 {
     __shared__ float4 red[256];
-    sa_after_previous();
+    const sa_data partial = sa_after_previous()(partial_in);
     const unsigned big_blocks = n_big << (shift - 4), sum_blocks = (n_sum - n_big) << (shift - 6);
     unsigned b = blockIdx.x;
     if (b >= big_blocks + sum_blocks) {
@@ -231,7 +275,7 @@ sa_fixup_kernel(const sa_fix *__restrict__ fix, unsigned n_big, unsigned n_sum, 
 // The same for rows of at most 128 floats (8, 16 or 32 float4): the first n_big entries (the builder puts the longest
 // first) take a block each as above, the others a warp each, which is all that a few partial rows can use.
 static __global__ void __launch_bounds__(256)
-sa_fixup_rows_kernel(const sa_fix *__restrict__ fix, int n_fix, int n_big, sa_data partial, float *__restrict__ out,
+sa_fixup_rows_kernel(const sa_fix *__restrict__ fix, int n_fix, int n_big, sa_input partial_in, float *__restrict__ out,
                      int row_floats)
 {
     __shared__ float4 red[256];
@@ -240,7 +284,7 @@ sa_fixup_rows_kernel(const sa_fix *__restrict__ fix, int n_fix, int n_big, sa_da
     const int entry = big ? int(blockIdx.x) : n_big + (int(blockIdx.x) - n_big) * 8 + int(threadIdx.x >> 5);
     if (entry >= n_fix) return;                        // whole warps of the last block
     const sa_fix e = fix[entry];
-    sa_after_previous();
+    const sa_data partial = sa_after_previous()(partial_in);
     const int who = big ? int(threadIdx.x) : lane, P = (big ? 256 : 32) / W;
     const int col = who % W, phase = who / W;
     float4 s = make_float4(0.f, 0.f, 0.f, 0.f);

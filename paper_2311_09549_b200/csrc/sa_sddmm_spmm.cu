@@ -31,7 +31,7 @@ struct sd_cfg {
 template <int K, int L, int CTAS>
 __global__ void __launch_bounds__(256, CTAS)
 sddmm_spmm_kernel(const sa_item *__restrict__ items, int64_t n_items, const int32_t *__restrict__ pos,
-                  const int2 *__restrict__ nz, sa_data C, uint32_t ldc, sa_data D, uint32_t ldd, sa_data E, uint32_t lde,
+                  const int2 *__restrict__ nz, sa_input C_in, uint32_t ldc, sa_input D_in, uint32_t ldd, sa_input E_in, uint32_t lde,
                   float *__restrict__ out, float *__restrict__ partial, float *__restrict__ sampled, const sa_limits lim)
 {
     using G = sd_cfg<K, L>;
@@ -55,12 +55,6 @@ sddmm_spmm_kernel(const sa_item *__restrict__ items, int64_t n_items, const int3
         if (!SA_CHK(lim.status, e >= 0 && e <= end, 44, e)) e = end;
         return e;
     };
-    auto load_c = [&](float4 (&x)[DQ], int row) {
-        if (row < rend) {
-#pragma unroll
-            for (int q = 0; q < DQ; ++q) x[q] = (C + (uint32_t(row) * ldc + 32u * q + 4u * l)).ld4();
-        }
-    };
     int b = row_end(r), bn = row_end(r + 1);
     int2 rec[U];
 #pragma unroll
@@ -68,12 +62,18 @@ sddmm_spmm_kernel(const sa_item *__restrict__ items, int64_t n_items, const int3
         rec[u] = make_int2(0, 0);
         if (p + u < end) rec[u] = __ldg(nz + p + u);
     }
-    sa_after_previous();
+    const sa_ready ready = sa_after_previous();
+    const sa_data C = ready(C_in), Dl = ready(D_in) + 4 * l, El = ready(E_in) + 4 * l;
+    auto load_c = [&](float4 (&x)[DQ], int row) {
+        if (row < rend) {
+#pragma unroll
+            for (int q = 0; q < DQ; ++q) x[q] = (C + (uint32_t(row) * ldc + 32u * q + 4u * l)).ld4();
+        }
+    };
     load_c(c, r);
     if (G::AHEAD) load_c(cn, r + 1);
 #pragma unroll
     for (int q = 0; q < EQ; ++q) acc[q] = make_float4(0.f, 0.f, 0.f, 0.f);
-    const sa_data Dl = D + 4 * l, El = E + 4 * l;
     const uint32_t d_bytes = ldd * 4u, e_bytes = lde * 4u;
     for (;;) {
         while (p == b && r < rend) {                  // the row is complete (or empty: +0)

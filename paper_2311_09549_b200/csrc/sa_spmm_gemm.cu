@@ -48,15 +48,16 @@ __device__ __forceinline__ void load_D(float *Ds, sa_data D, int64_t ldd)
 template <int L, int M, bool HAD>
 __global__ void __launch_bounds__(256, 3)
 spmm_gemm_left_kernel(const sa_item *__restrict__ items, int64_t n_items, const int32_t *__restrict__ pos,
-                      const int32_t *__restrict__ crd, sa_values vals, sa_data C, int64_t ldc, sa_data H, int64_t ldh, sa_data D,
-                      int64_t ldd, float *__restrict__ out, float *__restrict__ partial, const sa_limits lim)
+                      const int32_t *__restrict__ crd, sa_values vals, sa_input C_in, int64_t ldc, sa_input H_in, int64_t ldh,
+                      sa_input D_in, int64_t ldd, float *__restrict__ out, float *__restrict__ partial, const sa_limits lim)
 {
     constexpr int LV4 = L / 128, MV = M / 32;
     extern __shared__ __align__(16) float smem[];
     float *Ds = smem;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     float *Ts = smem + L * M + warp * L;
-    sa_after_previous();
+    const sa_ready ready = sa_after_previous();
+    const sa_data C = ready(C_in), H = ready(H_in), D = ready(D_in);
     load_D<L, M>(Ds, D, ldd);
     __syncthreads();
     for (int64_t idx = int64_t(blockIdx.x) * SA_WARPS_PER_CTA + warp; idx < n_items;
@@ -159,7 +160,7 @@ struct gemm_bf16_cfg {
 
 template <int L, int M>
 __global__ void __launch_bounds__(256, 1)
-gemm_bf16x3_kernel(int64_t J, sa_data C, int64_t ldc, sa_data D, int64_t ldd, float *__restrict__ Eout)
+gemm_bf16x3_kernel(int64_t J, sa_input C_in, int64_t ldc, sa_input D_in, int64_t ldd, float *__restrict__ Eout)
 {
     using G = gemm_bf16_cfg<L, M>;
     extern __shared__ __align__(16) float smem[];
@@ -169,7 +170,8 @@ gemm_bf16x3_kernel(int64_t J, sa_data C, int64_t ldc, sa_data D, int64_t ldd, fl
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int g = lane >> 2, t = lane & 3;
     const int wr = warp >> 1, wc = warp & 1;           // warp tile: rows 32*wr.., columns (M/2)*wc..
-    sa_after_previous();
+    const sa_ready ready = sa_after_previous();
+    const sa_data C = ready(C_in), D = ready(D_in);
     for (int x = threadIdx.x; x < (L / 2) * M; x += 256) {
         const int p = x / M, m = x % M;
         uint32_t h, l;
@@ -269,7 +271,7 @@ gemm_bf16x3_kernel(int64_t J, sa_data C, int64_t ldc, sa_data D, int64_t ldd, fl
 template <int W>
 __global__ void __launch_bounds__(256)
 spmm_kernel(const sa_item *__restrict__ items, int64_t n_items, unsigned ctas_per_part, const int32_t *__restrict__ pos,
-            const int2 *__restrict__ nz, sa_data E, int64_t J, int M, float *__restrict__ out, float *__restrict__ partial,
+            const int2 *__restrict__ nz, sa_input E_in, int64_t J, int M, float *__restrict__ out, float *__restrict__ partial,
             const sa_limits lim)
 {
     constexpr int LPR = W / 4, U = 8;                       // lanes per row, nonzeros per step
@@ -277,7 +279,6 @@ spmm_kernel(const sa_item *__restrict__ items, int64_t n_items, unsigned ctas_pe
     const unsigned part = blockIdx.x / ctas_per_part, block = blockIdx.x - part * ctas_per_part;
     const int l = threadIdx.x % LPR;
     const int64_t idx = (int64_t(block) * 256 + threadIdx.x) / LPR;
-    E = E + (int64_t(part) * J * W + 4 * l);
     int r = 0, rend = 0, p0 = 0, end = 0, dest = -1;
     if (idx < n_items) {
         const int4 ia = __ldg(reinterpret_cast<const int4 *>(items + idx));          // out_row, row_end, -, -
@@ -308,7 +309,7 @@ spmm_kernel(const sa_item *__restrict__ items, int64_t n_items, unsigned ctas_pe
     };
     float4 acc = zero;
     int2 rec = fetch(0);
-    sa_after_previous();
+    const sa_data E = sa_after_previous()(E_in) + (int64_t(part) * J * W + 4 * l);
     while (r < rend && b == p0) { store_row(zero); next_row(); }      // empty rows
     for (int c = 0; c < steps; c += U) {
         float4 e[U];
@@ -349,7 +350,7 @@ spmm_kernel(const sa_item *__restrict__ items, int64_t n_items, unsigned ctas_pe
 template <int M>
 __global__ void __launch_bounds__(256)
 fiber_spmm_kernel(const sa_item *__restrict__ items, int64_t n_items, const int32_t *__restrict__ pos,
-                  const int2 *__restrict__ nz, sa_data E, int64_t lde, float *__restrict__ out, float *__restrict__ partial,
+                  const int2 *__restrict__ nz, sa_input E_in, int64_t lde, float *__restrict__ out, float *__restrict__ partial,
                   const sa_limits lim)
 {
     constexpr int LPR = M / 4, NG = 32 / LPR;
@@ -391,7 +392,7 @@ fiber_spmm_kernel(const sa_item *__restrict__ items, int64_t n_items, const int3
     int xn;
     float vn;
     fetch(0, xn, vn);
-    sa_after_previous();
+    const sa_data E = sa_after_previous()(E_in);
     for (int c = 0; c < maxlen; c += 8) {
         const int x = xn;
         const float v = vn;

@@ -84,7 +84,7 @@ struct rowvec<4> {
     float x[4];
     __device__ __forceinline__ void load(sa_data p)
     {
-        const float4 v = p.ld4();
+        const float4 v = p.ld4_here();
         x[0] = v.x; x[1] = v.y; x[2] = v.z; x[3] = v.w;
     }
     __device__ __forceinline__ void store_shared(uint32_t a) const
@@ -97,7 +97,7 @@ struct rowvec<2> {
     float x[2];
     __device__ __forceinline__ void load(sa_data p)
     {
-        const float2 v = p.ld2();
+        const float2 v = p.ld2_here();
         x[0] = v.x; x[1] = v.y;
     }
     __device__ __forceinline__ void store_shared(uint32_t a) const
@@ -166,7 +166,7 @@ __device__ __forceinline__ void had_flush(float (&hacc)[4], const float *__restr
         const int x = x0 + lane / LANES;
         if (x < n) {
             const float *r = ring + (row0 + x) * RS;
-            const float4 c = (C + __float_as_uint(r[M]) + m).ld4();
+            const float4 c = (C + __float_as_uint(r[M]) + m).ld4_here();
             const float4 v = *reinterpret_cast<const float4 *>(r + m);
             hacc[0] = fmaf(v.x, c.x, hacc[0]);
             hacc[1] = fmaf(v.y, c.y, hacc[1]);
@@ -280,10 +280,10 @@ __device__ __forceinline__ void ttmc_accumulate(const float (&acc)[cfg<L, M>::MT
 template <int L, int M, bool HAD, bool TTMC = false>
 __device__ __forceinline__ void ttm3_warp_task(const sa_unit3 *__restrict__ units, int u0, int nu,
                                                const int32_t *__restrict__ crd_j, const int32_t *__restrict__ crd_k,
-                                               sa_values vals, const uint32_t *__restrict__ endbits, sa_data C, uint32_t ldc,
-                                               sa_data D, uint32_t ldd, unsigned char *__restrict__ wsm,
+                                               sa_values vals, const uint32_t *__restrict__ endbits, sa_input C_in, uint32_t ldc,
+                                               sa_input D_in, uint32_t ldd, unsigned char *__restrict__ wsm,
                                                float (&acc)[cfg<L, M>::MT][cfg<L, M>::NT][4], float (&hacc)[4], const bool keep,
-                                               float *__restrict__ out, const dbg_limits &lim, const bool first, const ttmc_sink *sink = nullptr)
+                                               float *__restrict__ out, const dbg_limits &lim, const ttmc_sink *sink = nullptr)
 {
     using K = cfg<L, M>;
     constexpr int VEC = K::VEC, DEPTH = K::DEPTH;
@@ -342,11 +342,11 @@ __device__ __forceinline__ void ttm3_warp_task(const sa_unit3 *__restrict__ unit
     int fq = load_sf(0);                                // next fiber this stream parks
     if (!SA_CHK(lim.status, uint32_t(fq) <= lim.n_fibers, 4, fq)) fq = 0;
     int jreg = __ldg(crd_j + fq + c);                   // C rows of the next eight fibers of the stream, one per lane
-    const sa_data dlane = D + c * VEC;
     const uint32_t row_bytes = ldd * 4u;
     cp_async_wait<DEPTH - 2>();
     __syncwarp();
-    if (first) sa_after_previous();                      // up to here only the tensor and its lists were read
+    const sa_ready ready = sa_after_previous();          // up to here only the tensor and its lists were read
+    const sa_data C = ready(C_in), dlane = ready(D_in) + c * VEC;
     rowvec<VEC> buf[8];                                  // rows of the round about to be consumed
     {
         const uint4 ka = lds128(s_kv), kb = lds128(s_kv + 16);
@@ -511,7 +511,7 @@ template <int L, int M, int NCTA, bool HAD>
 __global__ void __launch_bounds__(32 * SA_TTM3_WARPS, NCTA)
 ttm3_kernel(const sa_unit3 *__restrict__ units, const int32_t *__restrict__ task_start, int64_t n_tasks, int n_group_ctas,
             const int32_t *__restrict__ crd_j, const int32_t *__restrict__ crd_k, sa_values vals,
-            const uint32_t *__restrict__ endbits, sa_data C, uint32_t ldc, sa_data D, uint32_t ldd, float *__restrict__ out, float *__restrict__ partial,
+            const uint32_t *__restrict__ endbits, sa_input C, uint32_t ldc, sa_input D, uint32_t ldd, float *__restrict__ out, float *__restrict__ partial,
             const dbg_limits lim)
 {
     using K = cfg<L, M>;
@@ -528,7 +528,7 @@ ttm3_kernel(const sa_unit3 *__restrict__ units, const int32_t *__restrict__ task
     int u0 = 0, u1 = 0;
     if (task < n_tasks) { u0 = task_start[task]; u1 = task_start[task + 1]; }
     if (u1 > u0)
-        ttm3_warp_task<L, M, HAD>(units, u0, u1 - u0, crd_j, crd_k, vals, endbits, C, ldc, D, ldd, wsm, acc, hacc, group, out, lim, true);
+        ttm3_warp_task<L, M, HAD>(units, u0, u1 - u0, crd_j, crd_k, vals, endbits, C, ldc, D, ldd, wsm, acc, hacc, group, out, lim);
     if (!group) return;                 // whole small slices: every tile was stored when its unit ended
     if (HAD) {
         // the warps hold partial rows of the same slice: sum them in a fixed order
@@ -584,8 +584,8 @@ template <int L, int M, int NCTA>
 __global__ void __launch_bounds__(32 * SA_TTM3_WARPS, NCTA)
 ttmc3_fused_kernel(const sa_unit3 *__restrict__ units, const int32_t *__restrict__ task_start, int64_t n_tasks, int n_group_ctas,
                    const int32_t *__restrict__ crd_j, const int32_t *__restrict__ crd_k, sa_values vals,
-                   const uint32_t *__restrict__ endbits, sa_data C, uint32_t ldc, sa_data D, uint32_t ldd, sa_data C3, uint32_t ldc3,
-                   int L3, float *__restrict__ partials, const dbg_limits lim)
+                   const uint32_t *__restrict__ endbits, sa_input C, uint32_t ldc, sa_input D, uint32_t ldd, sa_input C3_in,
+                   uint32_t ldc3, int L3, float *__restrict__ partials, const dbg_limits lim)
 {
     using K = cfg<L, M>;
     constexpr int TILE = L * M;
@@ -596,10 +596,9 @@ ttmc3_fused_kernel(const sa_unit3 *__restrict__ units, const int32_t *__restrict
     float *accs = reinterpret_cast<float *>(smem + SA_TTM3_WARPS * K::WARP_BYTES);
     const int n_acc = L3 * TILE;
     for (int x = threadIdx.x; x < n_acc; x += 32 * SA_TTM3_WARPS) accs[x] = 0.f;
-    sa_after_previous();
+    const sa_data C3 = sa_after_previous()(C3_in);
     __syncthreads();
-    ttmc_sink sink;
-    sink.C3 = C3; sink.ldc3 = ldc3; sink.L3 = L3; sink.accs = accs;
+    const ttmc_sink sink{C3, ldc3, L3, accs};
     const int64_t n_block_tasks = (n_tasks + SA_TTM3_WARPS - 1) / SA_TTM3_WARPS;
     for (int64_t bt = blockIdx.x; bt < n_block_tasks; bt += gridDim.x) {
         const int64_t task = bt * SA_TTM3_WARPS + warp;
@@ -611,7 +610,7 @@ ttmc3_fused_kernel(const sa_unit3 *__restrict__ units, const int32_t *__restrict
         if (task < n_tasks) { u0 = task_start[task]; u1 = task_start[task + 1]; }
         if (u1 > u0)
             ttm3_warp_task<L, M, false, true>(units, u0, u1 - u0, crd_j, crd_k, vals, endbits, C, ldc, D, ldd, wsm, acc, hacc, group,
-                                              nullptr, lim, false, &sink);
+                                              nullptr, lim, &sink);
         if (!group) continue;              // whole small slices: added to the accumulator when their units ended
         // the block's warps hold partial temporaries of the same slice: sum them, then one rank-1 update
         __syncthreads();                   // every warp is done with its shared-memory region

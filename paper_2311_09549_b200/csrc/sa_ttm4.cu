@@ -318,8 +318,8 @@ __global__ void __launch_bounds__(32 * F4_WARPS, SA_F4_CTAS)
 ttm4_fused_kernel(const int4 *__restrict__ pieces, const int4 *__restrict__ supers, const sa_item *__restrict__ items,
                   const int32_t *__restrict__ pos1, const int32_t *__restrict__ crd0, const int32_t *__restrict__ crd_j,
                   const int32_t *__restrict__ pos2, const int32_t *__restrict__ pos3, const int32_t *__restrict__ crd_k,
-                  const int2 *__restrict__ nz, sa_data C, uint32_t ldc, sa_data D, uint32_t ldd, sa_data E, uint32_t lde,
-                  sa_data T2L, float *__restrict__ out, float *__restrict__ partial, const f4_limits lim)
+                  const int2 *__restrict__ nz, sa_input C_in, uint32_t ldc, sa_input D_in, uint32_t ldd, sa_input E_in, uint32_t lde,
+                  sa_input T2L_in, float *__restrict__ out, float *__restrict__ partial, const f4_limits lim)
 {
     extern __shared__ __align__(16) unsigned char f4_smem[];
     float *park = reinterpret_cast<float *>(f4_smem);
@@ -340,7 +340,8 @@ ttm4_fused_kernel(const int4 *__restrict__ pieces, const int4 *__restrict__ supe
 #pragma unroll
         for (int x = 0; x < 4; ++x) acc[nt][x] = 0.f;
     if (threadIdx.x == 0) ctr[pa.x & 1] = __ldg(supers + pa.x).x;
-    sa_after_previous();
+    const sa_ready ready = sa_after_previous();
+    const sa_data C = ready(C_in), D = ready(D_in), E = ready(E_in), T2L = ready(T2L_in);
     __syncthreads();
     for (int sup = pa.x; sup < pa.y; ++sup) {
         const int4 S = __ldg(supers + sup);                // first item, one past the last, first subtree, one past the last

@@ -127,7 +127,7 @@ __device__ __forceinline__ void sl_issue(const sl_cursor &cur, uint32_t stage, i
 
 __global__ void __launch_bounds__(256, 2)
 ttm4_slice_kernel(const sa_item *__restrict__ items, int64_t n_items, const int32_t *__restrict__ crd_j,
-                  sa_data T2, sa_data C, uint32_t ldc, float *__restrict__ out, float *__restrict__ partial, const fis_limits lim)
+                  sa_input T2_in, sa_input C_in, uint32_t ldc, float *__restrict__ out, float *__restrict__ partial, const fis_limits lim)
 {
     extern __shared__ __align__(16) float sl_smem[];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, g = lane >> 2, t = lane & 3;
@@ -137,7 +137,8 @@ ttm4_slice_kernel(const sa_item *__restrict__ items, int64_t n_items, const int3
     prod.n = int64_t(blockIdx.x) * SA_WARPS_PER_CTA + warp;
     sl_load_item(prod, items, n_items, stride, lim);
     cons = next = prod;
-    sa_after_previous();
+    const sa_ready ready = sa_after_previous();
+    const sa_data T2 = ready(T2_in), C = ready(C_in);
     if (!cons.live) return;
     // the first SL_DEPTH - 1 groups go out before anything is consumed
 #pragma unroll
@@ -230,13 +231,14 @@ template <bool CONTIG>
 __global__ void __launch_bounds__(256, 4)
 ttm4_subtree_kernel(const sa_item *__restrict__ items, int64_t n_items, const int32_t *__restrict__ pos2,
                     const int32_t *__restrict__ pos3, const int32_t *__restrict__ crd_k, const int2 *__restrict__ nz,
-                    sa_data D, int64_t ldd, sa_data E, int64_t lde, float *__restrict__ T2, const fis_limits lim)
+                    sa_input D_in, int64_t ldd, sa_input E_in, int64_t lde, float *__restrict__ T2, const fis_limits lim)
 {
     extern __shared__ __align__(16) float sub_smem[];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int64_t idx = int64_t(blockIdx.x) * SA_WARPS_PER_CTA + warp;
     if (idx >= n_items) return;
-    sa_after_previous();                    // here: further down it would part loads that are in flight together (2 us)
+    const sa_ready ready = sa_after_previous();     // here: further down it would part loads that are in flight together (2 us)
+    const sa_data D = ready(D_in), E = ready(E_in);
     const sa_item it = items[idx];
     if (!SA_CHK(lim.status, it.f0 >= 0 && it.f1 - it.f0 <= SA_SUB_MAX_F3 && it.f1 <= lim.n_fibers && it.out_row >= 0 &&
                                 it.row_end - it.out_row <= SA_SUB_MAX_ROWS && it.row_end <= lim.n_subtrees && it.p0 >= 0 && it.p1 <= lim.nnz,

@@ -29,10 +29,11 @@ constexpr int TTMC_MAX_CHUNKS = 512;
 constexpr int TTMC_STEP = 64;
 template <int L>
 __global__ void __launch_bounds__(256)
-ttmc3_partial_kernel(int64_t I, int chunk, int cols, sa_data T, sa_data C, uint32_t ldc, float *__restrict__ P)
+ttmc3_partial_kernel(int64_t I, int chunk, int cols, sa_input T_in, sa_input C_in, uint32_t ldc, float *__restrict__ P)
 {
     __shared__ __align__(16) float cs[TTMC_STEP * L];
-    sa_after_previous();
+    const sa_ready ready = sa_after_previous();
+    const sa_data T = ready(T_in), C = ready(C_in);
     const int col = blockIdx.x * 256 + threadIdx.x;
     const int64_t i0 = int64_t(blockIdx.y) * chunk, i1 = min(I, i0 + chunk);
     float acc[L];
@@ -72,10 +73,10 @@ ttmc3_partial_kernel(int64_t I, int chunk, int cols, sa_data T, sa_data C, uint3
 // A(x) = sum over chunks c of P(c, x), x = l * cols + col, in a fixed order: 16 phases over the chunks (64 outputs per block),
 // then the phases.  188 chunks of 4096: 17 us as one sum per thread, 8 us now.
 __global__ void __launch_bounds__(256)
-ttmc3_final_kernel(int n_chunks, int64_t n_out, sa_data P, float *__restrict__ A)
+ttmc3_final_kernel(int n_chunks, int64_t n_out, sa_input P_in, float *__restrict__ A)
 {
     __shared__ float4 red[256];
-    sa_after_previous();
+    const sa_data P = sa_after_previous()(P_in);
     const int col = threadIdx.x & 15, phase = threadIdx.x >> 4;
     const int64_t x = (int64_t(blockIdx.x) * 16 + col) * 4;               // n_out is a multiple of 64
     float4 s = make_float4(0.f, 0.f, 0.f, 0.f);

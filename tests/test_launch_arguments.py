@@ -15,7 +15,8 @@ __global__ void kernel(const int32_t *index, int32_t *status, float *out, int64_
 }
 __global__ void copy(%s in, float *out)
 {
-    sa_after_previous();
+    const sa_ready ready = sa_after_previous();
+    (void)ready;
     out[0] = %s;
 }
 cudaError_t launch(const int32_t *index, int32_t *status, float *out, const float *in)
@@ -27,7 +28,7 @@ cudaError_t launch(const int32_t *index, int32_t *status, float *out, const floa
 """
 
 
-def _compiles(tmp_path, args="index, status, out, int64_t(7)", in_type="sa_data", read="in.ld()"):
+def _compiles(tmp_path, args="index, status, out, int64_t(7)", in_type="sa_input", read="ready(in).ld()"):
     src = tmp_path / "launch.cu"
     src.write_text(SOURCE % (in_type, read, args))
     nvcc = os.environ.get("NVCC", "/usr/local/cuda/bin/nvcc")
@@ -49,7 +50,7 @@ def test_arguments_convert_only_as_in_a_call(tmp_path, args, right):
 
 
 @pytest.mark.parametrize("in_type, read, right", [
-    ("sa_data", "in.ld()", True),
+    ("sa_input", "ready(in).ld()", True),
     ("sa_values", "in.p[0]", True),
     ("const float *", "in[0]", False),                # would be read as data that nothing writes while the kernel lives
     ("const float *__restrict__", "__ldg(in)", False),
@@ -59,4 +60,9 @@ def test_numbers_that_a_kernel_may_have_written_are_not_read_as_constants(tmp_pa
     ok, log = _compiles(tmp_path, in_type=in_type, read=read)
     assert ok == right, log
     if not right:
-        assert "fp32 inputs are sa_data or sa_values" in log
+        assert "fp32 inputs are sa_input or sa_values" in log
+
+
+@pytest.mark.parametrize("read", ["in.ld()", "sa_data(in.p, 0).ld()"])
+def test_such_numbers_cannot_be_loaded_without_having_waited(tmp_path, read):
+    assert not _compiles(tmp_path, read=read)[0]
