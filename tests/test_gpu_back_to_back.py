@@ -110,3 +110,144 @@ def test_captured_calls_replay_in_order(cfg):
         graph.replay()
     torch.cuda.synchronize()
     assert torch.equal(res, want)
+
+
+# ---- library calls with nothing between them: no torch kernel stands between the one that writes and the one that reads
+
+SCHEDULES = [(cfg, None) for cfg in CONFIGS] + [(4, "ASSOC_LEFT"), (4, "ASSOC_RIGHT"), (5, "FUSED"), (5, "FISSIONED"), (6, "FUSED"),
+                                                (6, "FISSIONED"), (8, "FUSED"), (10, "ASSOC_LEFT"), (10, "ASSOC_RIGHT")]
+STEPS = 4
+
+
+def _sched(sa, name):
+    return sa.SA_SCHED_DEFAULT if name is None else getattr(sa, "SA_SCHED_" + name)
+
+
+class _Writer:
+    """A call that writes an operand of another: out = B . C . D seen as rows x cols, other numbers at every step."""
+
+    def __init__(self, sa, rows, cols, seed):
+        import torch
+        self.shape, self.rows = (rows, cols), -(-rows * cols // 64)
+        rng = np.random.default_rng(seed)
+        coords = np.stack([np.repeat(np.arange(self.rows), 4), rng.integers(0, 500, 4 * self.rows)], axis=1).astype(np.int32)
+        coords = np.unique(coords, axis=0)
+        self.t = sa.SparseTensor((self.rows, 500), coords, rng.uniform(0.5, 1.0, len(coords)).astype(np.float32), sa.SA_FMT_CSR, device=0)
+        self.sched = (sa.SA_SCHED_ASSOC_LEFT, sa.SA_SCHED_ASSOC_RIGHT)[seed % 2]
+        g = torch.Generator(device="cuda").manual_seed(seed)
+        C = torch.randn(500, 128, device="cuda", generator=g)
+        self.C = [C * s for s in (1.0, -0.5, 4.0, 0.25)]
+        self.D = torch.randn(128, 64, device="cuda", generator=g) / 16
+        self.buf = torch.zeros(self.rows, 64, device="cuda")
+        self.ws = self.t.run("spmm_gemm", [self.C[0], self.D], out=self.buf, sched=self.sched)[1]
+
+    def write(self, step):
+        self.t.run("spmm_gemm", [self.C[step], self.D], out=self.buf, sched=self.sched, workspace=self.ws)
+        return self.buf.view(-1)[:self.shape[0] * self.shape[1]].view(self.shape)
+
+
+def _apart(step):
+    import torch
+    torch.cuda.synchronize()
+    out = step()
+    torch.cuda.synchronize()
+    return out.clone()
+
+
+def _written_operands(sa, w, t, ops, sched):
+    import torch
+    out, ws = t.run(w.expr, ops, sched=sched)
+    for i, op in enumerate(ops):
+        writer = _Writer(sa, op.shape[0], op.shape[1], 10 * len(ops) + i)
+
+        def call(step, out=None, i=i, writer=writer):
+            return t.run(w.expr, ops[:i] + [writer.write(step)] + ops[i + 1:], out=out, sched=sched, workspace=ws)[0]
+        want = [_apart(lambda: call(k)) for k in range(STEPS)]
+        assert not torch.equal(want[0], want[1])
+        yield i, call, want, [torch.empty_like(out) for _ in range(STEPS)]
+
+
+def _check_written_operands(sa, w, t, ops, sched):
+    import torch
+    for i, call, want, outs in _written_operands(sa, w, t, ops, sched):
+        torch.cuda.synchronize()
+        for k in range(STEPS):
+            call(k, outs[k])
+        torch.cuda.synchronize()
+        for k in range(STEPS):
+            assert _same(w, outs[k], want[k]), "operand %d, step %d" % (i, k)
+
+
+@pytest.mark.parametrize("cfg, sched", SCHEDULES)
+def test_a_call_reads_what_the_call_before_it_writes(cfg, sched):
+    """Every operand in turn is written by a library call, with other numbers at every step, and read by the next."""
+    import paper_2311_09549_b200 as sa
+    w, t, ops = _tensor(sa, cfg)
+    _check_written_operands(sa, w, t, ops, _sched(sa, sched))
+
+
+def test_a_call_of_many_blocks_reads_what_the_call_before_it_writes():
+    """The same with more blocks on both sides than the device has SMs."""
+    import torch
+    import paper_2311_09549_b200 as sa
+    for w in (configs.make_sddmm_spmm("many-1", 61, 20_000, 30_000, 600_000, 0.8, 2_000, 64, 64),
+              configs.make_ttm3_zipf("many-6", 62, 3_000, 4_000, 5_000, 600_000, 1.0, 5.0, 32, 32)):
+        t = sa.SparseTensor(w.dims, w.coords, w.vals, sa.SA_FMT_CSR if w.fmt == "csr" else sa.SA_FMT_CSF, device=0)
+        _check_written_operands(sa, w, t, [torch.from_numpy(x).cuda() for x in w.dense], sa.SA_SCHED_DEFAULT)
+
+
+def _operand_sets(ops):
+    import torch
+    g = torch.Generator(device="cuda").manual_seed(7)
+    return [[torch.randn(x.shape, device="cuda", generator=g) for x in ops] for _ in range(STEPS)]
+
+
+@pytest.mark.parametrize("cfg, sched", SCHEDULES)
+def test_adjacent_calls_share_a_workspace_and_a_result(cfg, sched):
+    """Calls that differ in every operand, one behind the other in one workspace: first each with a result of its own, then
+    all into the same one."""
+    import torch
+    import paper_2311_09549_b200 as sa
+    w, t, ops = _tensor(sa, cfg)
+    sched = _sched(sa, sched)
+    out, ws = t.run(w.expr, ops, sched=sched)
+    sets = _operand_sets(ops)
+    want = [_apart(lambda: t.run(w.expr, s, sched=sched, workspace=ws)[0]) for s in sets]
+    outs = [torch.empty_like(out) for _ in sets]
+    for s, o in zip(sets, outs):
+        t.run(w.expr, s, out=o, sched=sched, workspace=ws)
+    torch.cuda.synchronize()
+    for k in range(STEPS):
+        assert _same(w, outs[k], want[k]), "call %d" % k
+    for last in (STEPS - 1, STEPS - 2):
+        for s in sets[:last + 1]:
+            t.run(w.expr, s, out=out, sched=sched, workspace=ws)
+        torch.cuda.synchronize()
+        assert _same(w, out, want[last])
+
+
+@pytest.mark.parametrize("cfg, sched", SCHEDULES)
+def test_captured_calls_read_what_the_call_before_them_writes(cfg, sched):
+    import torch
+    import paper_2311_09549_b200 as sa
+    w, t, ops = _tensor(sa, cfg)
+    sched = _sched(sa, sched)
+    ws = t.run(w.expr, ops, sched=sched)[1]
+    sets = _operand_sets(ops)
+    apart = [_apart(lambda: t.run(w.expr, s, sched=sched, workspace=ws)[0]) for s in sets]
+    for i, call, want, outs in _written_operands(sa, w, t, ops, sched):
+        others = [torch.empty_like(o) for o in outs]
+        graph = torch.cuda.CUDAGraph()
+        torch.cuda.synchronize()
+        with torch.cuda.graph(graph):
+            for k in range(STEPS):
+                call(k, outs[k])
+                t.run(w.expr, sets[k], out=others[k], sched=sched, workspace=ws)
+        for _ in range(2):
+            for o in outs + others:
+                o.zero_()
+            graph.replay()
+            torch.cuda.synchronize()
+            for k in range(STEPS):
+                assert _same(w, outs[k], want[k]), "operand %d, step %d" % (i, k)
+                assert _same(w, others[k], apart[k]), "operand %d, step %d" % (i, k)
