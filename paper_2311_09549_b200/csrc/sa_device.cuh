@@ -156,7 +156,7 @@ static inline sa_limits sa_make_limits(const sa_tensor *t, int64_t gather_rows, 
 // kernels of a block per SM, or with no need of L1, starting early) / as it is: row kernel on 60 K nonzeros and kernel 1 on
 // 100 K (K = L = 128) 55 / 87 / 51, order 3 on 8 M nonzeros and the same kernel 1 176 / 194 / 169.  One call after another:
 // kernel 1 on 6 M nonzeros 234 / 236 / 233, kernel 2 on 60 K (three launches) 18.4 / 13.8 / 12.3, kernel 7 on 60 K 12.6 / 11.9 /
-// 9.5, order 3 on 20 K (one launch, the one that is slower so) 10.3 / 7.7 / 8.1.
+// 7.0, order 3 on 20 K (one launch, the one that is slower so) 10.3 / 7.7 / 8.1.
 __device__ __forceinline__ sa_ready sa_after_previous()
 {
     sa_ready r;

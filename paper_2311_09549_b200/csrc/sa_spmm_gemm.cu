@@ -344,7 +344,8 @@ spmm_kernel(const sa_item *__restrict__ items, int64_t n_items, unsigned ctas_pe
 // as one stream, eight index/value pairs per load (the next eight already requested), eight row gathers in
 // flight; index, end-of-fiber bit (sign bit) and value of a nonzero come as one 8-byte record (half the load
 // wavefronts of separate index, value and bit arrays, and the L1 pipe is what this kernel saturates first); the
-// bit closes the output row.
+// bit closes the output row.  57 registers: the eight gathers of a step stay together (with 34 they did not: 12.5 M nonzeros
+// 139 -> 136 us, 60 K 9.5 -> 7.0).
 // A piece of a long fiber (dest >= 0) is split over the groups by nonzeros and summed across them at the end; a range
 // of whole fibers is split by nonzeros as well, and the parts of a fiber cut between two groups are added in order.
 template <int M>

@@ -511,8 +511,8 @@ template <int L, int M, int NCTA, bool HAD>
 __global__ void __launch_bounds__(32 * SA_TTM3_WARPS, NCTA)
 ttm3_kernel(const sa_unit3 *__restrict__ units, const int32_t *__restrict__ task_start, int64_t n_tasks, int n_group_ctas,
             const int32_t *__restrict__ crd_j, const int32_t *__restrict__ crd_k, sa_values vals,
-            const uint32_t *__restrict__ endbits, sa_input C, uint32_t ldc, sa_input D, uint32_t ldd, float *__restrict__ out, float *__restrict__ partial,
-            const dbg_limits lim)
+            const uint32_t *__restrict__ endbits, sa_input C, uint32_t ldc, sa_input D, uint32_t ldd,
+            float *__restrict__ out, float *__restrict__ partial, const dbg_limits lim)
 {
     using K = cfg<L, M>;
     constexpr int TILE = HAD ? M : L * M;

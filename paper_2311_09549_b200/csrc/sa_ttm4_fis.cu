@@ -127,7 +127,8 @@ __device__ __forceinline__ void sl_issue(const sl_cursor &cur, uint32_t stage, i
 
 __global__ void __launch_bounds__(256, 2)
 ttm4_slice_kernel(const sa_item *__restrict__ items, int64_t n_items, const int32_t *__restrict__ crd_j,
-                  sa_input T2_in, sa_input C_in, uint32_t ldc, float *__restrict__ out, float *__restrict__ partial, const fis_limits lim)
+                  sa_input T2_in, sa_input C_in, uint32_t ldc, float *__restrict__ out, float *__restrict__ partial,
+                  const fis_limits lim)
 {
     extern __shared__ __align__(16) float sl_smem[];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, g = lane >> 2, t = lane & 3;
