@@ -268,6 +268,8 @@ gemm_bf16x3_kernel(int64_t J, sa_input C_in, int64_t ldc, sa_input D_in, int64_t
 // ahead, eight gathers in flight); a group that meets a row's last nonzero stores the row.  1M x 1M, 25 M nonzeros,
 // M = 64 (E 256 MB): 783 us with one table, 709 us with two, 837 us with four (more instructions per byte
 // than the misses saved are worth); a warp per row with the columns across its lanes took 981 us.
+// The gathers are unconditional: coherent loads under a condition each cost the chain 2 % (925 us with the dense stage, 905 through
+// the read-only path, 895 so).
 template <int W>
 __global__ void __launch_bounds__(256)
 spmm_kernel(const sa_item *__restrict__ items, int64_t n_items, unsigned ctas_per_part, const int32_t *__restrict__ pos,
@@ -318,8 +320,7 @@ spmm_kernel(const sa_item *__restrict__ items, int64_t n_items, unsigned ctas_pe
         for (int u = 0; u < U; ++u) {
             const int k = __shfl_sync(SA_FULL_MASK, rec.x, u, LPR);
             vs[u] = __int_as_float(__shfl_sync(SA_FULL_MASK, rec.y, u, LPR));
-            e[u] = zero;
-            if (c + u < len) e[u] = (E + int64_t(k) * W).ld4();
+            e[u] = (E + int64_t(k) * W).ld4();                 // row 0 past the group's end, where nothing is stored any more
         }
         rec = fetch(c + U);
 #pragma unroll

@@ -728,3 +728,21 @@ def test_sddmm_spmm_ranks_32_on_both_sides_of_the_two_and_three_block_kernels(sa
     w = _wl("sddmm_spmm", "csr", (rows, 40), coords, vals, [_dense(61, 0, rows, 32), _dense(61, 1, 40, 32), _dense(61, 2, 40, 32)], (rows, 32))
     _, t = _check(sa, w)
     assert (len(sa.sa_tensor_worklist(t.handle)[1]) <= 28_416) == (rows < 28_416 * 8)
+
+
+@pytest.mark.parametrize("M", [32, 64])
+@pytest.mark.parametrize("expr", ["spmm_gemm", "spmmh_gemm"])
+def test_right_order_rows_that_do_not_refer_to_row_0_do_not_see_it(sa, expr, M):
+    """The gather loads row 0 for steps past a row's end: with NaN and infinities there every other result stays as it is."""
+    import torch
+    deg = np.array([1, 2, 7, 8, 9, 0, 15, 16, 17, 0, 0, 31, 33, 64, 200, 1, 0, 3] * 9)
+    J = 700
+    cols = np.concatenate([1 + rng.permutation(50 + i, i, J - 1)[:n] for i, n in enumerate(deg)])
+    coords = np.stack([np.repeat(np.arange(len(deg)), deg), cols], axis=1).astype(np.int32)
+    vals = np.random.RandomState(5).uniform(0.5, 1.0, len(coords)).astype(np.float32)
+    t = sa.SparseTensor((len(deg), J), coords, vals, sa.SA_FMT_CSR, device=0)
+    ops = [torch.randn(J, 128, device="cuda") for _ in range(2 if expr == "spmmh_gemm" else 1)] + [torch.randn(128, M, device="cuda")]
+    want = t.run(expr, ops, sched=sa.SA_SCHED_ASSOC_RIGHT)[0].clone()
+    ops[0][0, ::2], ops[0][0, 1::2] = float("nan"), float("inf")
+    got = t.run(expr, ops, sched=sa.SA_SCHED_ASSOC_RIGHT)[0]
+    assert torch.equal(got, want)
